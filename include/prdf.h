@@ -82,21 +82,22 @@ typedef struct {
   int check_every;     /* sweeps launched between host convergence checks, default 8 */
   int time_sweeps;     /* 1: time every rank sweep with CUDA events (stats->ms_sweep) from a host-driven
                           loop (a residual read every check_every sweeps); 0 (default): every sweep
-                          loop (Static, DF, DF-P, DT, and the FP32 stage of each) runs as one CUDA
-                          graph with the convergence test on the device, no host round trips. Both
-                          give identical results. */
+                          loop (Static, DF, DF-P, DT, and the FP32 stage of each) runs as one
+                          cooperative launch with the convergence test on the device, no host round
+                          trips (the K-column loops as CUDA graphs). Both give identical results. */
   int tile;            /* K-column calls: columns per index fetch (8, 16, 32, 64); 0 = automatic */
   double expand_pull;  /* DF / DF-P: an expansion round after a sweep runs in pull form (each vertex
                           outside the affected set looks for a frontier in-neighbour in G') when the
                           frontier's out-edges exceed expand_pull * |E|, else in push form (Alg.
                           affected). Both mark the same set. Default 1/16; >= 1 keeps the push form;
                           must be >= 0. */
-  int64_t expand_list; /* DF / DF-P / DT: a push-form round whose frontier holds at most this many
-                          vertices lists them and expands them from the list, instead of scanning
-                          every vertex's flag through the out-degree partition; the marks are the
-                          same. -1 (default): min(32768, n / 8) on graphs of at least 2^22 vertices,
-                          0 below that (where the scan is cheaper than the list's extra launches);
-                          0: never; must be >= -1. */
+  int64_t expand_list; /* DT: a closure round whose frontier holds at most this many vertices lists
+                          them and expands them from the list, instead of scanning every vertex's
+                          flag through the out-degree partition; the marks are the same. -1
+                          (default): min(32768, n / 8) on graphs of at least 2^22 vertices, 0 below
+                          that (where the scan is cheaper than the list's extra launches); 0: never;
+                          must be >= -1. (DF / DF-P rounds always expand from a list, which the
+                          sweeps write.) */
   void* stream;        /* cudaStream_t for all work; NULL = legacy default stream */
 } prdf_params;
 
@@ -108,7 +109,7 @@ typedef struct {
   int sweeps_launched;      /* sweeps issued, including those that exited at once after convergence */
   float ms_total;           /* device time of the whole call (CUDA events) */
   float ms_partition;       /* initialisation + partitioning */
-  float ms_mark;            /* initial marking (DF/DF-P) */
+  float ms_mark;            /* initial marking (DF/DF-P: its expansion counts as iteration) */
   float ms_iterate;         /* sweeps + residual + frontier expansion (incl. host convergence checks) */
   float ms_sweep;           /* device time of the first `iterations` rank sweeps (needs time_sweeps) */
   long long edges_processed;/* in-edges gathered over all sweeps (Static) */

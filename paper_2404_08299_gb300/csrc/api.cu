@@ -437,6 +437,7 @@ struct IterResult {
   int launched = 0;       // sweeps issued
   float ms_sweep = 0;     // device time of the first `iters` sweeps (time_sweeps)
   long long kernels = 0;  // kernels launched
+  long long affected = 0; // affected vertices at the first sweep (dynamic)
 };
 
 int nonempty_classes(const int64_t* cb, int nclass) {
@@ -456,32 +457,22 @@ int64_t hub_begin(const Relabel& rl);
 // rule holds for a sweep or max_iter sweeps ran: FP64, L-inf change <= tol;
 // FP32, max|dR| <= tol_rel * max R.
 //
-// Two drivers run the same kernels:
-//   - host loop: check_every sweeps are launched ahead and one residual is
-//     read; sweeps launched past convergence exit at once on the device.
-//     With time_sweeps each sweep is bracketed by CUDA events.
-//   - CUDA graph: a while node whose body is one iteration (sweep, expansion)
-//     and a one-thread check that advances the device iteration counter; the
-//     kernels find their buffers from that counter. One launch per loop, no
-//     host round trips. The instantiated graph is cached on the graph handle
-//     and rebuilt when any buffer, numbering or parameter it holds changes.
+// Two drivers run the same kernel (sweep.cu):
+//   - one cooperative launch for the whole loop, the stop test on the device;
+//   - host loop (time_sweeps): a launch per sweep and per expansion round,
+//     check_every sweeps ahead of each residual read; sweeps launched past
+//     convergence exit at once on the device. Each sweep is bracketed by CUDA
+//     events.
 struct Loop {
   bool fp32 = false, dynamic = false, expand = false, exact = true;
-  int max_iter = 0;
-  double tol = 0;
-  float tol_rel = 0;
-  SweepArgs a;      // FP64 sweep arguments (per-iteration buffers filled per launch)
-  Sweep32Args a32;  // FP32 sweep arguments
-  int64_t cb[kMaxThr + 2] = {}, cbo[kMaxThr + 2] = {};
-  int nci = 0, nco = 0;
-  int64_t pull_warp_b = 0;
-  unsigned long long fthr = ~0ull;
-  FrontList fl;              // listed small frontiers
-  int kernels_per_iter = 0;  // kernels of one iteration (without the graph's check)
+  bool init_push = false;  // the loop starts with the marked batch's expansion
+  SweepArgs<double> a;
+  SweepArgs<float> a32;
+  int64_t cb[kMaxThr + 2] = {};
 };
 
-// An expansion round lists a frontier of at most cap vertices and expands it
-// from the list (frontier.cu); larger ones take the partition kernels. The
+// A closure round of DT lists a frontier of at most cap vertices and expands
+// it from the list (frontier.cu); larger ones take the partition kernels. The
 // automatic cap is min(32768, n / 8) on graphs of at least 2^22 vertices; on
 // smaller ones the partition kernels' scan costs less than the list's extra
 // launches, so the list is off (cap 0: fl left empty).
@@ -499,178 +490,132 @@ int front_list(prdf_graph* g, const prdf_params* p, cudaStream_t s, FrontList* f
   return PRDF_OK;
 }
 
-int loop_setup(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, bool expand, int max_iter, Loop* L,
-               cudaStream_t s) {
-  const int n = g->n;
+// room for every vertex in the frontier: one entry per started kFrontChunk out-edges
+int alloc_frontier(prdf_graph* g, cudaStream_t s) {
+  return g->loop_list.reserve((size_t)g->n + (size_t)(g->m / kFrontChunk) + 1, s);
+}
+
+int alloc_loop_ctl(prdf_graph* g, cudaStream_t s) {
+  PRDF_TRY(g->loop_ctl.reserve(1, s));
+  PRDF_CUDA(cudaMemsetAsync(g->loop_ctl.p, 0, sizeof(LoopCtl), s));
+  return PRDF_OK;
+}
+
+// what both precisions share; a's precision-specific arrays are set by the caller
+template <class Real>
+int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, SweepArgs<Real>* out, cudaStream_t s) {
   const Relabel& rl = g->rl;
-  L->fp32 = fp32;
-  L->dynamic = dynamic;
-  L->expand = dynamic && expand;
-  L->exact = p->accumulate == PRDF_ACC_EXACT;
-  L->max_iter = max_iter;
-  L->tol = p->tol;
-  L->tol_rel = (float)p->tol_fp32_rel;
-  L->nci = rl.thr.n + 1;
-  begins_from_counts(rl.count, L->nci, L->cb);
-  L->kernels_per_iter = nonempty_classes(L->cb, L->nci);
-  // the highest in-degree class's rows are cut into the hub chunks of G' (a
-  // partial sum per chunk); the table and the partial buffer are made here,
-  // outside any stream capture
-  PRDF_TRY(ensure_hub(g, rl.in, g->hub_in, s));
-  const size_t nchunk = (size_t)(g->hub_in.nchunk > 0 ? g->hub_in.nchunk : 1);
-  if (g->hub_in.nchunk > 0) L->kernels_per_iter += 1;  // the highest class takes two kernels
-  if (fp32) {
-    PRDF_TRY(g->sweep_hub_part32.reserve(nchunk, s));
-    PRDF_TRY(g->resid32.reserve(2 * ((size_t)max_iter + 1), s));
-    PRDF_CUDA(cudaMemsetAsync(g->resid32.p, 0, sizeof(uint32_t) * 2 * ((size_t)max_iter + 1), s));
-    Sweep32Args& a = L->a32;
-    memset(&a, 0, sizeof(a));
-    a.off = rl.in.off.p;
-    a.adj = rl.in.adj.p;
-    a.degf = g->degf.p;
-    a.invf = g->invf.p;
-    a.alpha = (float)p->alpha;
-    a.c0 = (float)((1.0 - p->alpha) / (double)n);
-    a.self_loops = g->self_loops ? 1 : 0;
-    a.tol_rel = L->tol_rel;
-    a.multi = rl.multi_count > 0 ? rl.multi.p : nullptr;
-    a.hub = g->hub_in.view();
-    a.hub_part = g->sweep_hub_part32.p;
-    if (dynamic) {
-      a.kf = g->kf32.p;
-      a.dV = g->dV.p;
-      a.dN = g->dN.p;
-      a.wrote = g->wrote.p;
-      a.tau_f = (float)p->tau_f;
-      a.tau_p = (float)p->tau_p;
-      a.prune = p->prune;
-    }
-  } else {
-    PRDF_TRY(g->sweep_hub_part.reserve(nchunk, s));
-    PRDF_TRY(g->resid.reserve((size_t)max_iter + 1, s));
-    PRDF_CUDA(cudaMemsetAsync(g->resid.p, 0, sizeof(uint64_t) * ((size_t)max_iter + 1), s));
-    SweepArgs& a = L->a;
-    memset(&a, 0, sizeof(a));
-    a.off = rl.in.off.p;
-    a.adj = rl.in.adj.p;
-    a.degd = rl.degd.p;
-    a.inv_deg = rl.inv_deg.p;
-    a.kf = rl.kf.p;
-    a.alpha = p->alpha;
-    a.c0 = (1.0 - p->alpha) / (double)n;
-    a.self_loops = g->self_loops ? 1 : 0;
-    a.tol = p->tol;
-    a.multi = rl.multi_count > 0 ? rl.multi.p : nullptr;
-    a.hub = g->hub_in.view();
-    a.hub_part = g->sweep_hub_part.p;
-    if (dynamic) {
-      a.dV = g->dV.p;
-      a.dN = g->dN.p;
-      a.wrote = g->wrote.p;
-      // + 0.0 turns a tolerance of -0 into +0: the sweep compares products with
-      // the tolerance by their bit patterns, which order -0 below +0
-      a.tau_f = p->tau_f + 0.0;
-      a.tau_p = p->tau_p + 0.0;
-      a.prune = p->prune;
-    }
-  }
-  if (L->expand) {
-    // pull-form expansion: frontier count, thread rows below the two highest in-degree classes, warp rows above
-    L->nco = g->thr[PRDF_OUT].n + 1;
-    begins_from_counts(rl.pout_count, L->nco, L->cbo);
-    L->pull_warp_b = hub_begin(rl);
-    PRDF_TRY(g->fwork.reserve((size_t)max_iter + 1, s));
-    PRDF_CUDA(cudaMemsetAsync(g->fwork.p, 0, sizeof(unsigned long long) * ((size_t)max_iter + 1), s));
+  SweepArgs<Real>& a = *out;
+  memset(&a, 0, sizeof(a));
+  a.off = rl.in.off.p;
+  a.adj = rl.in.adj.p;
+  a.alpha = (Real)p->alpha;
+  a.c0 = (Real)((1.0 - p->alpha) / (double)g->n);
+  a.self_loops = g->self_loops ? 1 : 0;
+  a.multi = rl.multi_count > 0 ? rl.multi.p : nullptr;
+  a.m = rl.in.m;
+  a.n = g->n;
+  a.max_iter = max_iter;
+  a.ctl = g->loop_ctl.p;
+  a.hub = g->hub_in.view();
+  a.hub_part = g->sweep_hub_part.p;
+  a.hub_done = g->sweep_hub_done.p;
+  if (!L.dynamic) return PRDF_OK;
+  a.dV = g->dV.p;
+  a.dN = g->dN.p;
+  a.wrote = g->wrote.p;
+  // + 0.0 turns a tolerance of -0 into +0: the FP64 sweep compares products
+  // with the tolerance by their bit patterns, which order -0 below +0
+  a.tau_f = (Real)(p->tau_f + 0.0);
+  a.tau_p = (Real)(p->tau_p + 0.0);
+  a.prune = p->prune;
+  a.expand = L.expand ? 1 : 0;
+  a.init_push = L.init_push ? 1 : 0;
+  if (L.expand) {
+    PRDF_TRY(alloc_frontier(g, s));
+    a.ooff = rl.out.off.p;
+    a.oadj = rl.out.adj.p;
+    a.list = g->loop_list.p;
     const double lim = p->expand_pull * (double)rl.in.m;
-    L->fthr = lim >= 1.8e19 ? ~0ull : (unsigned long long)lim;
-    PRDF_TRY(front_list(g, p, s, &L->fl));  // allocated here, outside any stream capture
-    L->kernels_per_iter += nonempty_classes(L->cbo, L->nco) + (L->pull_warp_b > 0 ? 1 : 0) +
-                           (n > L->pull_warp_b ? 1 : 0) + (L->fl.list ? 2 : 0);
+    a.fthr = lim >= 1.8e19 ? ~0ull : (unsigned long long)lim;
+    a.pull_warp_b = hub_begin(rl);
   }
   return PRDF_OK;
 }
 
-// The sweep of iteration i (i >= 0: host loop, explicit buffers; i < 0:
-// graph-driven, buffers from the device counter).
-int launch_loop_sweep(prdf_graph* g, const Loop& L, int i, cudaStream_t s) {
+int loop_setup(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, bool expand, bool init_push, int max_iter,
+               Loop* L, cudaStream_t s) {
   const Relabel& rl = g->rl;
-  if (L.fp32) {
-    Sweep32Args a = L.a32;
-    // the sweep counts the out-edges of its deltaN for the expansion round after it
-    if (i >= 0) {
-      a.y = (i & 1) ? g->yb.p : g->ya.p;
-      a.yn = (i & 1) ? g->ya.p : g->yb.p;
-      a.resid = g->resid32.p + 2 * i;
-      a.prev = i > 0 ? g->resid32.p + 2 * (i - 1) : nullptr;
-      a.fw = L.expand ? g->fwork.p + i : nullptr;
-    } else {
-      a.ctl = g->ctl.p;
-      a.ya = g->ya.p;
-      a.yb = g->yb.p;
-      a.resid_base = g->resid32.p;
-      a.fw_base = L.expand ? g->fwork.p : nullptr;
-    }
-    return launch_sweep32(a, rl.thr, L.cb, L.dynamic, s);
-  }
-  SweepArgs a = L.a;
-  if (i >= 0) {
-    a.x = (i & 1) ? g->xb.p : g->xa.p;
-    a.xn = (i & 1) ? g->xa.p : g->xb.p;
-    a.resid = g->resid.p + i;
-    a.prev = i > 0 ? g->resid.p + i - 1 : nullptr;
-    a.fw = L.expand ? g->fwork.p + i : nullptr;
+  L->fp32 = fp32;
+  L->dynamic = dynamic;
+  L->expand = dynamic && expand;
+  L->init_push = L->expand && init_push;
+  L->exact = p->accumulate == PRDF_ACC_EXACT;
+  begins_from_counts(rl.count, rl.thr.n + 1, L->cb);
+  // the highest in-degree class's rows are cut into the hub chunks of G'
+  PRDF_TRY(ensure_hub(g, rl.in, g->hub_in, s));
+  const size_t nhub = (size_t)(g->hub_in.nhub > 0 ? g->hub_in.nhub : 1);
+  PRDF_TRY(g->sweep_hub_part.reserve((size_t)(g->hub_in.nchunk > 0 ? g->hub_in.nchunk : 1), s));
+  PRDF_TRY(g->sweep_hub_done.reserve(nhub, s));
+  PRDF_CUDA(cudaMemsetAsync(g->sweep_hub_done.p, 0, sizeof(uint32_t) * nhub, s));
+  if (!L->init_push) PRDF_TRY(alloc_loop_ctl(g, s));  // (with a marked batch the marking made it)
+  if (fp32) {
+    PRDF_TRY(loop_args(g, p, *L, max_iter, &L->a32, s));
+    SweepArgs<float>& a = L->a32;
+    a.xa = g->ya.p;
+    a.xb = g->yb.p;
+    a.deg = g->degf.p;
+    a.inv = g->invf.p;
+    a.kf = g->kf32.p;
+    a.tol = (float)p->tol_fp32_rel;
   } else {
-    a.ctl = g->ctl.p;
+    PRDF_TRY(loop_args(g, p, *L, max_iter, &L->a, s));
+    SweepArgs<double>& a = L->a;
     a.xa = g->xa.p;
     a.xb = g->xb.p;
-    a.resid_base = g->resid.p;
-    a.fw_base = L.expand ? g->fwork.p : nullptr;
+    a.deg = rl.degd.p;
+    a.inv = rl.inv_deg.p;
+    a.kf = rl.kf.p;
+    a.tol = p->tol;
   }
-  return launch_sweep(a, rl.thr, L.cb, L.exact, L.dynamic, s);
+  return PRDF_OK;
 }
 
-// The expansion round after sweep i (Alg. affected over the frontier deltaN
-// the sweep left), skipped on the device once the loop has converged.
-int launch_loop_expansion(prdf_graph* g, const Loop& L, int i, cudaStream_t s) {
-  if (!L.expand) return PRDF_OK;
-  const Relabel& rl = g->rl;
-  Stop st;
+int launch_loop(prdf_graph* g, const Loop& L, LoopMode mode, int it, int it_first, cudaStream_t s) {
+  const PartThr& t = g->rl.thr;
   if (L.fp32) {
-    st.r32 = g->resid32.p + 2 * (i >= 0 ? i : 0);
-    st.tol_rel = L.tol_rel;
-  } else {
-    st.r64 = g->resid.p + (i >= 0 ? i : 0);
-    st.tol = L.tol;
+    SweepArgs<float> a = L.a32;
+    a.slot = g->loop_slots.p;
+    a.mode = mode;
+    a.it0 = it;
+    a.it_first = it_first;
+    return launch_rank_loop(a, t, L.cb, L.dynamic, s);
   }
-  st.ctl = i >= 0 ? nullptr : g->ctl.p;
-  unsigned long long* fw = g->fwork.p + (i >= 0 ? i : 0);
-  PRDF_TRY(launch_expand_pull(rl.in.off.p, rl.in.adj.p, g->n, L.pull_warp_b, g->dN.p, g->dV.p, fw, L.fthr, st, s));
-  return launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, L.cbo, L.nco, g->dN.p, g->dV.p, nullptr, st, s, fw,
-                       L.fthr, L.fl);
+  SweepArgs<double> a = L.a;
+  a.slot = g->loop_slots.p;
+  a.mode = mode;
+  a.it0 = it;
+  a.it_first = it_first;
+  return launch_rank_loop(a, t, L.cb, L.exact, L.dynamic, s);
 }
 
-// stop rule of sweep i from the residual words read back
-bool loop_stopped(const Loop& L, const void* words, int i, double* delta) {
+// stop rule on a sweep's residual word
+bool loop_stopped(const Loop& L, unsigned long long word, double* delta) {
   if (L.fp32) {
-    const uint32_t* r = static_cast<const uint32_t*>(words) + 2 * i;
+    uint32_t r[2];
+    memcpy(r, &word, sizeof(r));
     float d, m;
     memcpy(&d, &r[0], 4);
     memcpy(&m, &r[1], 4);
     *delta = d;
-    return d <= L.tol_rel * m;
+    return d <= L.a32.tol * m;
   }
-  double d;
-  memcpy(&d, static_cast<const uint64_t*>(words) + i, sizeof(double));
-  *delta = d;
-  return d <= L.tol;
+  memcpy(delta, &word, sizeof(double));
+  return *delta <= L.a.tol;
 }
 
-int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, IterResult* res, cudaStream_t s) {
-  const int max_iter = L.max_iter;
+int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, int max_iter, IterResult* res, cudaStream_t s) {
   const int check = p->check_every > 0 ? p->check_every : 8;
-  const bool timed = p->time_sweeps != 0;
-  const size_t wsz = L.fp32 ? 2 * sizeof(uint32_t) : sizeof(uint64_t);
-  const void* resid_dev = L.fp32 ? (const void*)g->resid32.p : (const void*)g->resid.p;
   std::vector<cudaEvent_t> ev;
   struct EvGuard {
     std::vector<cudaEvent_t>& v;
@@ -678,55 +623,95 @@ int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, IterResult
       for (auto e : v) cudaEventDestroy(e);
     }
   } guard{ev};
+  const int window = check < max_iter ? check : max_iter;
+  PRDF_TRY(g->loop_slots.reserve((size_t)window + 1, s));
+  if (L.init_push) PRDF_TRY(launch_loop(g, L, kLoopPush, 0, 0, s));
+  // slot 0 holds the sweep before the window, slots 1.. the window's
+  std::vector<LoopSlot> slots((size_t)window + 1);
+  std::vector<unsigned long long> resid;
   int launched = 0;
   bool done = false;
+  double d;
   while (launched < max_iter && !done) {
-    const int upto = (launched + check < max_iter) ? launched + check : max_iter;
-    for (int i = launched; i < upto; ++i) {
-      if (timed) {
-        cudaEvent_t e0, e1;
-        PRDF_CUDA(cudaEventCreate(&e0));
-        ev.push_back(e0);
-        PRDF_CUDA(cudaEventCreate(&e1));
-        ev.push_back(e1);
-        PRDF_CUDA(cudaEventRecord(e0, s));
-      }
-      PRDF_TRY(launch_loop_sweep(g, L, i, s));
-      if (timed) PRDF_CUDA(cudaEventRecord(ev.back(), s));  // the sweep alone, not its expansion
-      PRDF_TRY(launch_loop_expansion(g, L, i, s));
+    const int cnt = max_iter - launched < window ? max_iter - launched : window;
+    if (launched)
+      PRDF_CUDA(cudaMemcpyAsync(g->loop_slots.p, g->loop_slots.p + window, sizeof(LoopSlot), cudaMemcpyDeviceToDevice,
+                                s));
+    PRDF_CUDA(cudaMemsetAsync(g->loop_slots.p + 1, 0, sizeof(LoopSlot) * (size_t)cnt, s));
+    for (int i = launched; i < launched + cnt; ++i) {
+      cudaEvent_t e0, e1;
+      PRDF_CUDA(cudaEventCreate(&e0));
+      ev.push_back(e0);
+      PRDF_CUDA(cudaEventCreate(&e1));
+      ev.push_back(e1);
+      PRDF_CUDA(cudaEventRecord(e0, s));
+      PRDF_TRY(launch_loop(g, L, kLoopSweep, i, launched, s));
+      PRDF_CUDA(cudaEventRecord(e1, s));  // the sweep alone, not its expansion
+      if (L.expand) PRDF_TRY(launch_loop(g, L, kLoopExpand, i, launched, s));
     }
-    launched = upto;
-    PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, (const char*)resid_dev + wsz * (launched - 1), wsz,
+    PRDF_CUDA(cudaMemcpyAsync(slots.data(), g->loop_slots.p + 1, sizeof(LoopSlot) * (size_t)cnt,
                               cudaMemcpyDeviceToHost, s));
     PRDF_CUDA(cudaStreamSynchronize(s));
-    double d;
-    done = loop_stopped(L, g->ws.host_i64, 0, &d);
+    for (int i = 0; i < cnt; ++i) resid.push_back(slots[(size_t)i].resid);
+    launched += cnt;
+    done = loop_stopped(L, resid.back(), &d);
   }
-  std::vector<uint64_t> hr((size_t)launched);
-  PRDF_CUDA(cudaMemcpyAsync(hr.data(), resid_dev, wsz * launched, cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
   int k = launched - 1;
   res->converged = 0;
-  for (int i = 0; i < launched; ++i) {
-    double d;
-    if (loop_stopped(L, hr.data(), i, &d)) {
+  for (int i = 0; i < launched; ++i)
+    if (loop_stopped(L, resid[(size_t)i], &d)) {
       k = i;
       res->converged = 1;
       break;
     }
-  }
-  loop_stopped(L, hr.data(), k, &res->final_delta);
+  loop_stopped(L, resid[(size_t)k], &res->final_delta);
   res->iters = k + 1;
-  res->final_buf = (k & 1) ? 0 : 1;  // sweep k wrote the second buffer if k is even
   res->launched = launched;
-  res->kernels = (long long)launched * L.kernels_per_iter;
+  res->kernels = (long long)launched * (L.expand ? 2 : 1) + (L.init_push ? 1 : 0);
   res->ms_sweep = 0;
-  if (timed)
-    for (int i = 0; i < res->iters; ++i) {
-      float ms = 0;
-      PRDF_CUDA(cudaEventElapsedTime(&ms, ev[2 * i], ev[2 * i + 1]));
-      res->ms_sweep += ms;
+  for (int i = 0; i < res->iters; ++i) {
+    float ms = 0;
+    PRDF_CUDA(cudaEventElapsedTime(&ms, ev[2 * (size_t)i], ev[2 * (size_t)i + 1]));
+    res->ms_sweep += ms;
+  }
+  return PRDF_OK;
+}
+
+// One loop with the driver the parameters select: the host loop when every
+// sweep is to be timed (time_sweeps), else one launch. Synchronises the stream.
+int run_loop(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, bool expand, bool init_push, int max_iter,
+             IterResult* res, cudaStream_t s) {
+  Loop L;
+  PRDF_TRY(loop_setup(g, p, fp32, dynamic, expand, init_push, max_iter, &L, s));
+  if (p->time_sweeps) {
+    PRDF_TRY(run_host_loop(g, L, p, max_iter, res, s));
+  } else {
+    PRDF_TRY(g->loop_slots.reserve(kLoopRing, s));
+    PRDF_CUDA(cudaMemsetAsync(g->loop_slots.p, 0, sizeof(LoopSlot) * kLoopRing, s));
+    PRDF_TRY(launch_loop(g, L, kLoopAll, 0, 0, s));
+  }
+  static_assert(sizeof(LoopCtl) <= 16 * sizeof(int64_t), "the host scratch holds the loop state");
+  PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64 + 16, g->loop_ctl.p, sizeof(LoopCtl), cudaMemcpyDeviceToHost, s));
+  PRDF_CUDA(cudaStreamSynchronize(s));
+  LoopCtl h;
+  memcpy(&h, g->ws.host_i64 + 16, sizeof(h));
+  res->affected = h.aff0;
+  if (!p->time_sweeps) {
+    if (h.timeout) {
+      set_error("the rank loop gave up waiting for its blocks");
+      return PRDF_ETIMEOUT;
     }
+    if (h.iters < 1 || h.iters > max_iter) {
+      set_error("the rank loop ran %d sweeps", h.iters);
+      return PRDF_ECUDA;
+    }
+    res->converged = loop_stopped(L, h.resid, &res->final_delta) ? 1 : 0;
+    res->iters = h.iters;
+    res->launched = h.iters;
+    res->kernels = 1;
+    res->ms_sweep = 0;
+  }
+  res->final_buf = ((res->iters - 1) & 1) ? 0 : 1;  // sweep k wrote the second buffer if k is even
   return PRDF_OK;
 }
 
@@ -790,72 +775,6 @@ struct KeyWriter {
   }
   void putv(uint64_t v) { put(&v, sizeof(v)); }
 };
-
-// The same loop as one CUDA graph (see above).
-int run_graph_loop(prdf_graph* g, const Loop& L, IterResult* res, cudaStream_t s) {
-  PRDF_TRY(g->ctl.reserve(2, s));
-  PRDF_CUDA(cudaMemsetAsync(g->ctl.p, 0, 2 * sizeof(int), s));
-  // what the captured kernels hold: their arguments and the buffers of the graph-driven iteration
-  KeyWriter kw;
-  kw.putv(((uint64_t)L.fp32 << 3) | ((uint64_t)L.dynamic << 2) | ((uint64_t)L.expand << 1) | (uint64_t)L.exact);
-  kw.putv((uint64_t)L.max_iter);
-  kw.put(&L.tol, sizeof(L.tol));
-  kw.put(&L.tol_rel, sizeof(L.tol_rel));
-  if (L.fp32) kw.put(&L.a32, sizeof(L.a32));
-  else kw.put(&L.a, sizeof(L.a));
-  kw.put(L.cb, sizeof(L.cb));
-  kw.put(L.cbo, sizeof(L.cbo));
-  kw.putv((uint64_t)L.nci | ((uint64_t)L.nco << 32));
-  kw.putv((uint64_t)L.pull_warp_b);
-  kw.putv(L.fthr);
-  kw.putv((uint64_t)L.fl.cap);
-  const Relabel& rl = g->rl;
-  const void* ptrs[] = {g->ctl.p,     g->xa.p,       g->xb.p,        g->ya.p,       g->yb.p,      g->resid.p,
-                        g->resid32.p, g->fwork.p,    g->dN.p,        g->dV.p,       rl.in.off.p,  rl.in.adj.p,
-                        rl.out.off.p, rl.out.adj.p,  rl.pout.p,     g->flist.p,    g->fcnt.p};
-  kw.put(ptrs, sizeof(ptrs));
-  kw.putv(rl.version);
-  kw.putv((uint64_t)g->n);
-  const int slot = (L.fp32 ? 4 : 0) + (L.dynamic ? 2 : 0) + (L.expand ? 1 : 0);
-  PRDF_TRY(launch_while_graph(g, slot, kw.key, [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
-    int rc = launch_loop_sweep(g, L, -1, cs);
-    if (rc == PRDF_OK) rc = launch_loop_expansion(g, L, -1, cs);
-    if (rc == PRDF_OK)
-      rc = L.fp32 ? launch_iter_check32(g->ctl.p, g->resid32.p, L.tol_rel, L.max_iter, h, cs)
-                  : launch_iter_check(g->ctl.p, g->resid.p, L.tol, L.max_iter, h, cs);
-    return rc;
-  }, s));
-  PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
-  int hit = 0;
-  memcpy(&hit, g->ws.host_i64, sizeof(int));
-  if (hit < 1 || hit > L.max_iter) {
-    set_error("iteration graph ran %d sweeps", hit);
-    return PRDF_ECUDA;
-  }
-  const size_t wsz = L.fp32 ? 2 * sizeof(uint32_t) : sizeof(uint64_t);
-  const char* resid_dev = L.fp32 ? (const char*)g->resid32.p : (const char*)g->resid.p;
-  PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, resid_dev + wsz * (hit - 1), wsz, cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
-  res->converged = loop_stopped(L, g->ws.host_i64, 0, &res->final_delta) ? 1 : 0;
-  res->iters = hit;
-  const int k = hit - 1;
-  res->final_buf = (k & 1) ? 0 : 1;
-  res->launched = hit;
-  res->kernels = (long long)hit * (L.kernels_per_iter + 1);
-  res->ms_sweep = 0;
-  return PRDF_OK;
-}
-
-// One loop with the driver the parameters select: the host loop when every
-// sweep is to be timed (time_sweeps), else the CUDA graph.
-int run_loop(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, bool expand, int max_iter, IterResult* res,
-             cudaStream_t s) {
-  Loop L;
-  PRDF_TRY(loop_setup(g, p, fp32, dynamic, expand, max_iter, &L, s));
-  if (p->time_sweeps) return run_host_loop(g, L, p, res, s);
-  return run_graph_loop(g, L, res, s);
-}
 
 int auto_tile(int K) { return K >= 64 ? 64 : (K >= 32 ? 32 : (K > 8 ? 16 : 8)); }
 
@@ -1195,7 +1114,7 @@ int dynamic_fp32_stage(prdf_graph* g, const prdf_params* p, const double* prev_r
                                                      eq2 ? rl.kf.p : nullptr, g->ya.p, g->yb.p, g->degf.p, g->invf.p,
                                                      eq2 ? g->kf32.p : nullptr);
   PRDF_LAUNCH_CHECK();
-  PRDF_TRY(run_loop(g, p, true, true, expand, p->max_iter, it32, s));
+  PRDF_TRY(run_loop(g, p, true, true, expand, expand, p->max_iter, it32, s));
   k_widen_keep<<<grid_for(n, kThreads), kThreads, 0, s>>>(it32->final_buf ? g->yb.p : g->ya.p, n, g->xa.p, g->xb.p,
                                                          g->dV.p);
   PRDF_LAUNCH_CHECK();
@@ -1208,7 +1127,7 @@ int alloc_solver(prdf_graph* g, bool dynamic, cudaStream_t s) {
   PRDF_TRY(g->xb.reserve(g->n, s));
   if (dynamic) {
     PRDF_TRY(g->dV.reserve(g->n, s));
-    PRDF_TRY(g->dN.reserve(g->n, s));
+    PRDF_TRY(g->dN.reserve((size_t)g->n + 4, s));  // marked by whole words
     PRDF_TRY(g->wrote.reserve(g->n, s));
   }
   PRDF_TRY(g->counter.reserve(1, s));
@@ -1569,7 +1488,7 @@ int prdf_expand_affected(prdf_graph* g, const uint8_t* dN, uint8_t* dV, void* st
   int64_t cb[kMaxThr + 2];
   class_begins(g, PRDF_OUT, cb);
   PRDF_TRY(launch_expand(g->csr[PRDF_OUT].off.p, g->csr[PRDF_OUT].adj.p, g->P[PRDF_OUT].p, cb, g->thr[PRDF_OUT].n + 1,
-                         dN, dV, nullptr, Stop(), s));
+                         dN, dV, nullptr, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
   return PRDF_OK;
 }
@@ -1601,7 +1520,7 @@ int prdf_pagerank_static(prdf_graph* g, const prdf_params* p, const double* R0, 
     PRDF_LAUNCH_CHECK();
     PRDF_CUDA(cudaEventRecord(t.e[1], s));
     IterResult it32;
-    PRDF_TRY(run_loop(g, p, true, false, false, p->max_iter, &it32, s));
+    PRDF_TRY(run_loop(g, p, true, false, false, false, p->max_iter, &it32, s));
     iters32 = it32.iters;
     k_widen<<<grid_for(g->n, kThreads), kThreads, 0, s>>>(it32.final_buf ? g->yb.p : g->ya.p, g->n, g->xa.p);
     PRDF_LAUNCH_CHECK();
@@ -1613,7 +1532,7 @@ int prdf_pagerank_static(prdf_graph* g, const prdf_params* p, const double* R0, 
     PRDF_CUDA(cudaEventRecord(t.e[1], s));
   }
   IterResult it;
-  PRDF_TRY(run_loop(g, &p64, false, false, false, p64.max_iter, &it, s));
+  PRDF_TRY(run_loop(g, &p64, false, false, false, false, p64.max_iter, &it, s));
   k_finalize<<<grid_for(g->n, kThreads), kThreads, 0, s>>>(it.final_buf ? g->xb.p : g->xa.p, g->rl.degd.p,
                                                            g->rl.perm.p, g->n, ranks, nullptr, nullptr);
   PRDF_LAUNCH_CHECK();
@@ -1655,11 +1574,8 @@ int prdf_pagerank_dfp(prdf_graph* g, const int32_t* del_src, const int32_t* del_
   const int n = g->n;
   PRDF_CUDA(cudaEventRecord(t.e[0], s));
   // Alg. frontier: R = Rnew = R^{t-1}; partition G and G'; mark; iterate.
-  // The partitions are kept with the graph: G' by in-degree is the sweep
-  // numbering, G by out-degree (for marking) is made with it and stays valid
-  // until the graph or the thresholds change.
-  const bool pout_made = !g->rl.pout_valid;
-  PRDF_TRY(ensure_relabelled(g, true, s));
+  // The partition is kept with the graph: G' by in-degree is the sweep numbering.
+  PRDF_TRY(ensure_relabelled(g, false, s));
   Relabel& rl = g->rl;
   bool kf_made = false;
   if (p->prune && rl.kf_alpha != p->alpha) {
@@ -1676,17 +1592,12 @@ int prdf_pagerank_dfp(prdf_graph* g, const int32_t* del_src, const int32_t* del_
   PRDF_CUDA(cudaMemsetAsync(g->dV.p, 0, (size_t)n, s));
   PRDF_CUDA(cudaMemsetAsync(g->dN.p, 0, (size_t)n, s));
   PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n, s));
-  PRDF_TRY(launch_initial_affected(del_src, del_dst, del_mask, n_del, ins_src, ins_mask, n_ins, rl.inv.p, g->dV.p,
-                                   g->dN.p, s));
-  int64_t cbo[kMaxThr + 2];
-  begins_from_counts(rl.pout_count, g->thr[PRDF_OUT].n + 1, cbo);
-  FrontList fl;
-  PRDF_TRY(front_list(g, p, s, &fl));
-  PRDF_TRY(launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, cbo, g->thr[PRDF_OUT].n + 1, g->dN.p, g->dV.p,
-                         nullptr, Stop(), s, nullptr, 0, fl));
-  PRDF_TRY(count_flags(g->dV.p, n, g->counter.p, s));
+  // the batch's sources go into the first frontier list, which the loop expands before its first sweep
+  PRDF_TRY(alloc_loop_ctl(g, s));
+  PRDF_TRY(alloc_frontier(g, s));
+  PRDF_TRY(launch_mark_batch(del_src, del_dst, del_mask, n_del, ins_src, ins_mask, n_ins, rl.inv.p, rl.out.off.p,
+                             g->dV.p, g->dN.p, g->loop_ctl.p, g->loop_list.p, s));
   PRDF_CUDA(cudaEventRecord(t.e[2], s));
-  PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64 + 8, g->counter.p, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   IterResult it, it32;
   prdf_params p64 = *p;
   long long kernels32 = 0;
@@ -1697,8 +1608,9 @@ int prdf_pagerank_dfp(prdf_graph* g, const int32_t* del_src, const int32_t* del_
     p64.max_iter = p->max_iter - it32.iters > 0 ? p->max_iter - it32.iters : 1;
     kernels32 = it32.kernels + 3;
   }
-  PRDF_TRY(run_loop(g, &p64, false, true, true, p64.max_iter, &it, s));  // synchronises the stream
-  const long long aff0 = (long long)g->ws.host_i64[8];
+  const bool mixed = p->precision == PRDF_FP32_REFINE;
+  PRDF_TRY(run_loop(g, &p64, false, true, true, !mixed, p64.max_iter, &it, s));  // synchronises the stream
+  const long long aff0 = mixed ? it32.affected : it.affected;
   k_finalize<<<grid_for(n, kThreads), kThreads, 0, s>>>(it.final_buf ? g->xb.p : g->xa.p, rl.degd.p, rl.perm.p, n,
                                                        ranks, g->dV.p, dV_out);
   PRDF_LAUNCH_CHECK();
@@ -1719,9 +1631,8 @@ int prdf_pagerank_dfp(prdf_graph* g, const int32_t* del_src, const int32_t* del_
     stats->ms_sweep = it.ms_sweep + it32.ms_sweep;
     stats->edges_processed = -1;
     stats->affected_initial = aff0;
-    // (out-degree partition) + init (+ Eq. 2 factor) + initial marking + expand + count + sweeps/expands + finalize
-    stats->kernel_launches = (pout_made ? 5 : 0) + 1 + (kf_made ? 1 : 0) + (n_del + n_ins > 0 ? 1 : 0) +
-                             nonempty_classes(cbo, g->thr[PRDF_OUT].n + 1) + (fl.list ? 2 : 0) + 1 + kernels32 + it.kernels + 1;
+    // init (+ Eq. 2 factor) + initial marking + loops + finalize
+    stats->kernel_launches = 1 + (kf_made ? 1 : 0) + (n_del + n_ins > 0 ? 1 : 0) + kernels32 + it.kernels + 1;
   }
   return PRDF_OK;
 }
@@ -1761,8 +1672,7 @@ int prdf_pagerank_dt(prdf_graph* g, const int32_t* del_src, const int32_t* del_d
   begins_from_counts(rl.pout_count, nco, cbo);
   FrontList fl;
   PRDF_TRY(front_list(g, p, s, &fl));
-  PRDF_TRY(launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, cbo, nco, g->dN.p, g->dV.p, nullptr, Stop(), s,
-                         nullptr, 0, fl));
+  PRDF_TRY(launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, cbo, nco, g->dN.p, g->dV.p, nullptr, s, fl));
   // reachability closure over G^t: the frontier starts as every affected vertex; each
   // round marks the vertices it reaches that were not yet affected, which form the
   // next frontier, until a round adds none (the affected count stops changing)
@@ -1772,8 +1682,7 @@ int prdf_pagerank_dt(prdf_graph* g, const int32_t* del_src, const int32_t* del_d
   uint8_t* next = g->dF.p;
   for (int round = 0; round < n; ++round) {
     PRDF_CUDA(cudaMemsetAsync(next, 0, (size_t)n, s));
-    PRDF_TRY(launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, cbo, nco, front, g->dV.p, next, Stop(), s, nullptr,
-                           0, fl));
+    PRDF_TRY(launch_expand(rl.out.off.p, rl.out.adj.p, rl.pout.p, cbo, nco, front, g->dV.p, next, s, fl));
     PRDF_TRY(count_flags(next, n, g->counter.p, s));
     kernels += nonempty_classes(cbo, nco) + 1 + (fl.list ? 2 : 0);
     unsigned long long added = 0;
@@ -1797,7 +1706,7 @@ int prdf_pagerank_dt(prdf_graph* g, const int32_t* del_src, const int32_t* del_d
     q.max_iter = p->max_iter - it32.iters > 0 ? p->max_iter - it32.iters : 1;
     kernels += it32.kernels + 3;
   }
-  PRDF_TRY(run_loop(g, &q, false, true, false, q.max_iter, &it, s));  // synchronises the stream
+  PRDF_TRY(run_loop(g, &q, false, true, false, false, q.max_iter, &it, s));  // synchronises the stream
   const long long aff = (long long)g->ws.host_i64[8];
   k_finalize<<<grid_for(n, kThreads), kThreads, 0, s>>>(it.final_buf ? g->xb.p : g->xa.p, rl.degd.p, rl.perm.p, n,
                                                        ranks, g->dV.p, dV_out);
@@ -1857,7 +1766,7 @@ int prdf_pagerank_ppr(prdf_graph* g, const double* S, int K, double* R, const pr
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
   PRDF_TRY(ensure_hub(g, g->rl.in, g->hub_in, s));
   const KOp op{g->rl.in.off.p, g->rl.in.adj.p, g->pin32.p, g->pin64.p, hub_begin(g->rl), &g->hub_in, g->S64.p, true,
-               8};
+               0};
   KSolve ks;
   ks.kernels = 1;
   double* Rfinal = nullptr;
@@ -1955,7 +1864,7 @@ int prdf_pagerank_backward(prdf_graph* g, const double* R, const double* G, int 
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
   PRDF_TRY(ensure_hub(g, g->rl.out, g->hub_out, s));
   const KOp op{g->rl.out.off.p, g->rl.out.adj.p, g->pout32.p, g->pout64.p, hub_begin(g->rl), &g->hub_out, g->S64.p,
-               false, 12};
+               false, 4};
   KSolve ks;
   ks.kernels = 1;
   double* lam = nullptr;

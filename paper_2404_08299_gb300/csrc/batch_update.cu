@@ -617,7 +617,7 @@ int update_csr_small(int32_t n, const Csr& old, const int32_t* del_rows, const i
   const int64_t ni = ws.host_i64[1], kc = ws.host_i64[2], dm = ws.host_i64[3];
   out.m = old.m + dm;
   PRDF_TRY(out.off.alloc((size_t)n + 1, s));
-  PRDF_TRY(out.adj.alloc((size_t)(out.m > 0 ? out.m : 1), s));
+  PRDF_TRY(out.adj.alloc((size_t)out.m + kAdjPad, s));
   if (weighted) PRDF_TRY(out.w.alloc((size_t)(out.m > 0 ? out.m : 1), s));
   else out.w.release();
   k_new_offsets<<<grid_for((int64_t)n + 1, kThreads), kThreads, 0, s>>>(n, old.off.p, changed, kc, c_shift, out.off.p);
@@ -715,7 +715,7 @@ int update_csr(int32_t n, const Csr& old, const int32_t* del_rows, const int32_t
   PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, out.off.p + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
   out.m = ws.host_i64[0];
-  PRDF_TRY(out.adj.alloc((size_t)(out.m > 0 ? out.m : 1), s));
+  PRDF_TRY(out.adj.alloc((size_t)out.m + kAdjPad, s));
   if (weighted) PRDF_TRY(out.w.alloc((size_t)(out.m > 0 ? out.m : 1), s));
   else out.w.release();
   // the changed rows (those with batch entries), ascending

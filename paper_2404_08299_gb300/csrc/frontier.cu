@@ -36,73 +36,6 @@ __global__ void k_initial_affected(const int32_t* __restrict__ del_src, const in
   }
 }
 
-// The sweep this round follows already met its loop's stop rule: the round does nothing.
-__device__ __forceinline__ bool converged(const Stop& st) {
-  const int it = st.ctl ? st.ctl[0] : 0;
-  if (st.r64) return bitsd(st.r64[it]) <= st.tol;
-  if (st.r32) {
-    const uint32_t* r = st.r32 + 2 * it;
-    return __uint_as_float(r[0]) <= st.tol_rel * __uint_as_float(r[1]);
-  }
-  return false;
-}
-
-// this round's frontier out-edge counter (one per sweep; the graph-driven loop indexes it by ctl[0])
-__device__ __forceinline__ const unsigned long long* round_fw(const unsigned long long* fw, const Stop& st) {
-  return fw ? fw + (st.ctl ? st.ctl[0] : 0) : nullptr;
-}
-
-// Direction of one expansion round, chosen on the device: the pull form when
-// the frontier's out-edges (*fw) exceed fthr, else the push form.
-__device__ __forceinline__ bool pull_chosen(const unsigned long long* fw, unsigned long long fthr) {
-  return fw && *fw > fthr;
-}
-
-// Pull form of one expansion round over G' (the same marks as the push form,
-// since w is an out-neighbour of u exactly when u is an in-neighbour of w): a
-// vertex outside dV joins it when an in-neighbour is in the frontier. Only
-// w's own thread (or warp) reads or writes dV[w]; the scan stops at the first
-// frontier in-neighbour.
-__global__ void __launch_bounds__(kThreads) k_pull_thread(const int64_t* __restrict__ off,
-                                                          const int32_t* __restrict__ adj, int64_t begin, int64_t end,
-                                                          const uint8_t* __restrict__ dN, uint8_t* __restrict__ dV,
-                                                          const unsigned long long* fw, unsigned long long fthr,
-                                                          const Stop st) {
-  if (converged(st) || !pull_chosen(round_fw(fw, st), fthr)) return;
-  for (int64_t w = begin + blockIdx.x * (int64_t)kThreads + threadIdx.x; w < end; w += (int64_t)gridDim.x * kThreads) {
-    if (dV[w]) continue;
-    const int64_t e = off[w + 1];
-    for (int64_t j = off[w]; j < e; ++j)
-      if (dN[adj[j]]) {
-        dV[w] = 1;
-        break;
-      }
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) k_pull_warp(const int64_t* __restrict__ off,
-                                                        const int32_t* __restrict__ adj, int64_t begin, int64_t end,
-                                                        const uint8_t* __restrict__ dN, uint8_t* __restrict__ dV,
-                                                        const unsigned long long* fw, unsigned long long fthr,
-                                                        const Stop st) {
-  if (converged(st) || !pull_chosen(round_fw(fw, st), fthr)) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  for (int64_t w = begin + warp; w < end; w += nwarps) {
-    if (dV[w]) continue;  // the same value on every lane
-    const int64_t b = off[w], e = off[w + 1];
-    for (int64_t j0 = b; j0 < e; j0 += 32) {
-      const int64_t j = j0 + lane;
-      const bool hit = j < e && dN[adj[j]];
-      if (__any_sync(0xffffffffu, hit)) {
-        if (lane == 0) dV[w] = 1;
-        break;
-      }
-    }
-  }
-}
-
 // Mark the targets of edges [j0, e) of one row, `step` apart, kU per lane in
 // flight: the index loads of a round issue together, then their flag loads.
 template <int kU>
@@ -137,10 +70,9 @@ __global__ void __launch_bounds__(kThreads) k_expand_group(const int64_t* __rest
                                                            const int32_t* __restrict__ adj,
                                                            const int32_t* __restrict__ P, int64_t begin, int64_t end,
                                                            const uint8_t* __restrict__ dN, uint8_t* __restrict__ dV,
-                                                           uint8_t* __restrict__ dF, const Stop st,
-                                                           const unsigned long long* fw, unsigned long long fthr,
-                                                           const unsigned int* lcnt, unsigned int cap) {
-  if (converged(st) || pull_chosen(round_fw(fw, st), fthr) || listed(lcnt, cap)) return;
+                                                           uint8_t* __restrict__ dF, const unsigned int* lcnt,
+                                                           unsigned int cap) {
+  if (listed(lcnt, cap)) return;
   const int lane = (G == 1) ? 0 : (threadIdx.x & (G - 1));
   const int64_t gid = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / G;
   const int64_t ng = ((int64_t)gridDim.x * kThreads) / G;
@@ -157,10 +89,9 @@ __global__ void __launch_bounds__(kThreads) k_expand_block(const int64_t* __rest
                                                            const int32_t* __restrict__ adj,
                                                            const int32_t* __restrict__ P, int64_t begin, int64_t end,
                                                            const uint8_t* __restrict__ dN, uint8_t* __restrict__ dV,
-                                                           uint8_t* __restrict__ dF, const Stop st,
-                                                           const unsigned long long* fw, unsigned long long fthr,
-                                                           const unsigned int* lcnt, unsigned int cap) {
-  if (converged(st) || pull_chosen(round_fw(fw, st), fthr) || listed(lcnt, cap)) return;
+                                                           uint8_t* __restrict__ dF, const unsigned int* lcnt,
+                                                           unsigned int cap) {
+  if (listed(lcnt, cap)) return;
   const int64_t S = gridDim.y, y = blockIdx.y;
   for (int64_t i = begin + blockIdx.x; i < end; i += gridDim.x) {
     const int32_t u = P[i];
@@ -182,9 +113,7 @@ __global__ void __launch_bounds__(kThreads) k_expand_block(const int64_t* __rest
 // and the class kernels run as before. The marks are the same either way.
 __global__ void __launch_bounds__(kThreads) k_frontier_list(const uint8_t* __restrict__ dN, int64_t n,
                                                             int32_t* __restrict__ list, unsigned int* __restrict__ cnt,
-                                                            unsigned int cap, const Stop st,
-                                                            const unsigned long long* fw, unsigned long long fthr) {
-  if (converged(st) || pull_chosen(round_fw(fw, st), fthr)) return;
+                                                            unsigned int cap) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = n >> 2;  // whole 4-flag words; the tail is read by thread 0
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -227,10 +156,7 @@ __global__ void __launch_bounds__(kThreads) k_expand_list(const int64_t* __restr
                                                           const int32_t* __restrict__ adj,
                                                           const int32_t* __restrict__ list,
                                                           const unsigned int* __restrict__ cnt, unsigned int cap,
-                                                          uint8_t* __restrict__ dV, uint8_t* __restrict__ dF,
-                                                          const Stop st, const unsigned long long* fw,
-                                                          unsigned long long fthr) {
-  if (converged(st) || pull_chosen(round_fw(fw, st), fthr)) return;
+                                                          uint8_t* __restrict__ dV, uint8_t* __restrict__ dF) {
   const unsigned int c = *cnt;
   if (c > cap) return;
   for (unsigned int k = blockIdx.x; k < c; k += gridDim.x) {
@@ -260,16 +186,14 @@ int launch_initial_affected(const int32_t* del_src, const int32_t* del_dst, cons
 }
 
 int launch_expand(const int64_t* off, const int32_t* adj, const int32_t* P, const int64_t* cb, int nclass,
-                  const uint8_t* dN, uint8_t* dV, uint8_t* dF, const Stop& st, cudaStream_t s,
-                  const unsigned long long* fw, unsigned long long fthr, const FrontList& fl) {
+                  const uint8_t* dN, uint8_t* dV, uint8_t* dF, cudaStream_t s, const FrontList& fl) {
   const int maxg = kSMs * 8;
   const unsigned int* lcnt = fl.list ? fl.cnt : nullptr;
   if (fl.list) {
     const int64_t n = cb[nclass];
     PRDF_CUDA(cudaMemsetAsync(fl.cnt, 0, sizeof(unsigned int), s));
-    k_frontier_list<<<grid_for(n / 4 + 1, kThreads, kSMs * 4), kThreads, 0, s>>>(dN, n, fl.list, fl.cnt, fl.cap, st,
-                                                                                fw, fthr);
-    k_expand_list<<<kSMs * 8, kThreads, 0, s>>>(off, adj, fl.list, fl.cnt, fl.cap, dV, dF, st, fw, fthr);
+    k_frontier_list<<<grid_for(n / 4 + 1, kThreads, kSMs * 4), kThreads, 0, s>>>(dN, n, fl.list, fl.cnt, fl.cap);
+    k_expand_list<<<kSMs * 8, kThreads, 0, s>>>(off, adj, fl.list, fl.cnt, fl.cap, dV, dF);
   }
   for (int c = 0; c < nclass; ++c) {
     const int64_t b = cb[c], e = cb[c + 1];
@@ -277,30 +201,16 @@ int launch_expand(const int64_t* off, const int32_t* adj, const int32_t* P, cons
     const int64_t cnt = e - b;
     const int kind = (nclass == 4) ? c : (c == nclass - 1 ? 3 : c);
     switch (kind) {
-      case 0: k_expand_group<1><<<grid_for(cnt, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, st, fw, fthr, lcnt, fl.cap); break;
-      case 1: k_expand_group<8><<<grid_for(cnt * 8, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, st, fw, fthr, lcnt, fl.cap); break;
-      case 2: k_expand_group<32><<<grid_for(cnt * 32, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, st, fw, fthr, lcnt, fl.cap); break;
+      case 0: k_expand_group<1><<<grid_for(cnt, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, lcnt, fl.cap); break;
+      case 1: k_expand_group<8><<<grid_for(cnt * 8, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, lcnt, fl.cap); break;
+      case 2: k_expand_group<32><<<grid_for(cnt * 32, kThreads, maxg), kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, lcnt, fl.cap); break;
       default: {
         const dim3 grid(grid_for(cnt, 1, maxg / kExpandSlices), kExpandSlices);
-        k_expand_block<<<grid, kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, st, fw, fthr, lcnt, fl.cap);
+        k_expand_block<<<grid, kThreads, 0, s>>>(off, adj, P, b, e, dN, dV, dF, lcnt, fl.cap);
         break;
       }
     }
   }
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
-
-int launch_expand_pull(const int64_t* in_off, const int32_t* in_adj, int64_t n, int64_t warp_begin,
-                       const uint8_t* dN, uint8_t* dV, const unsigned long long* fw, unsigned long long fthr,
-                       const Stop& st, cudaStream_t s) {
-  const int maxg = kSMs * 8;
-  if (warp_begin > 0)
-    k_pull_thread<<<grid_for(warp_begin, kThreads, maxg), kThreads, 0, s>>>(in_off, in_adj, 0, warp_begin, dN, dV, fw,
-                                                                            fthr, st);
-  if (n > warp_begin)
-    k_pull_warp<<<grid_for((n - warp_begin) * 32, kThreads, maxg), kThreads, 0, s>>>(in_off, in_adj, warp_begin, n,
-                                                                                      dN, dV, fw, fthr, st);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }

@@ -37,10 +37,12 @@ int partition_by_degree(const int64_t* off, int64_t n, const PartThr& t, int32_t
 int partition_list(const int64_t* off, const int32_t* in, int64_t n, const PartThr& t, bool desc, int32_t* P,
                    int64_t* counts_host, Workspace& ws, cudaStream_t s);
 
+constexpr int kAdjPad = 4;
+
 // A device CSR with optional float weights.
 struct Csr {
   DBuf<int64_t> off;  // n + 1
-  DBuf<int32_t> adj;  // m
+  DBuf<int32_t> adj;  // m (+ kAdjPad in the sweep numbering: 16-byte loads may reach past the last entry)
   DBuf<float> w;      // m or empty
   int64_t m = 0;
 };
@@ -108,83 +110,98 @@ struct PprHub {
   const int64_t* chunk_j0;
   const int64_t* hub_first;
 };
-// Per-sweep arguments of the pull rank kernels (Alg. update).
+// ---- the rank loop (sweep.cu) ----
+
+// Row shapes of a class of the sweep: a lane per row (no gather: in-degree <=
+// 1, the row is [v]), a lane per row, 4, 8 or 16 lanes per row, a warp per row.
+enum RowKind { kRowSelf = 0, kRowThread, kRow4, kRow8, kRow16, kRowWarp };
+
+// A class of the sweep cut into units of `rows` rows: unit unit0 + k holds
+// rows [begin + k * rows, +rows) below end.
+struct SweepClass {
+  int64_t begin, end;
+  uint32_t unit0;
+  int rows, kind;
+};
+
+// Counters of one sweep and its expansion round.
+struct LoopSlot {
+  unsigned long long resid;  // FP64: L-inf change (bits); FP32: low word max |dR|, high word max R (bits)
+  unsigned long long fw;     // out-edges of the vertices the sweep put into deltaN
+  unsigned int units;        // units handed out beyond the first of each warp
+  unsigned int nlist;        // frontier entries
+  unsigned long long pad;
+};
+constexpr int kLoopRing = 4;  // slots of the whole-loop kernel (a power of two)
+
+// State and result of a loop.
+struct LoopCtl {
+  unsigned long long bar;    // arrivals at the grid barrier
+  unsigned long long resid;  // residual word of the last sweep
+  int iters;                 // sweeps run
+  int timeout;               // a block gave up waiting at the grid barrier
+  unsigned int nlist0;       // frontier entries of the initial marking
+  unsigned int aff0;         // affected vertices at the first sweep
+};
+
+enum LoopMode { kLoopAll = 0, kLoopSweep, kLoopExpand, kLoopPush };
+
+// A frontier entry (v, k) stands for out-edges [k, k + 1) * kFrontChunk of v.
+constexpr int kFrontChunk = 1024;
+
+// Arguments of the rank loop, Real = double (FP64 sweeps) or float (FP32
+// stage of the mixed-precision solves).
+template <class Real>
 struct SweepArgs {
   const int64_t* off;      // in-CSR offsets of G'
-  const int32_t* adj;      // in-CSR sources
-  const double* x;         // x[u] = R[u] / |out(u)| of the previous iteration
-  double* xn;              // next x
-  const double* degd;      // |out(v)| (self-loop included), as a double
-  const double* inv_deg;   // 1 / |out(v)|
-  const double* kf;        // DF-P: 1 / (1 - alpha / |out(v)|) (Eq. 2's self-loop factor)
-  double alpha, c0;        // damping, (1 - alpha) / n
+  const int32_t* adj;      // in-CSR sources (padded: 16-byte loads may reach past the last entry)
+  Real* xa;                // x[u] = R[u] / |out(u)|; even sweeps read xa and write xb
+  Real* xb;
+  const Real* deg;         // |out(v)| (self-loop included)
+  const Real* inv;         // 1 / |out(v)|
+  const Real* kf;          // DF-P: 1 / (1 - alpha / |out(v)|) (Eq. 2's self-loop factor)
+  Real alpha, c0;          // damping, (1 - alpha) / n
+  Real tol;                // FP64: stop at L-inf change <= tol; FP32: at max |dR| <= tol * max R
   int self_loops;          // every vertex has exactly one self-loop (graph built with PRDF_ADD_SELF_LOOPS)
   const uint32_t* multi;   // null, or a bit per vertex: set for the in-degree <= 1 classes' vertices that
                            // gained in-edges since the numbering was made (they read their row)
-  uint64_t* resid;         // L-inf change of this sweep (bits of a non-negative double), atomic max
-  const uint64_t* prev;    // L-inf change of the previous sweep, or null on the first sweep
-  double tol;              // the sweep exits at once if *prev <= tol (already converged)
-  // DF / DF-P only
-  // device-driven iteration (CUDA graph): when ctl is set the kernel takes
-  // x/xn/resid/prev for iteration it = ctl[0] from xa/xb/resid_base instead
-  const int* ctl;
-  const double* xa;
-  double* xb;
-  uint64_t* resid_base;
+  int64_t m;               // in-edges
+  int32_t n;
+  int max_iter;
+  int mode, it0, it_first; // LoopMode; single phases: the iteration, and the one slot[1] stands for
+  LoopSlot* slot;
+  LoopCtl* ctl;
+  // chunks of the highest in-degree class's rows, one partial sum and one
+  // arrival counter (zero between sweeps) each
+  PprHub hub;
+  uint4* hub_part;
+  uint32_t* hub_done;
+  // units: hub chunks, then the classes (filled by the launcher)
+  SweepClass cls[kMaxThr + 1];
+  int ncls;
+  uint32_t units;
+  // DF / DF-P / DT
   uint8_t* dV;             // affected flags (read; cleared on prune)
   uint8_t* dN;             // expand flags (set when the change exceeds tau_f)
   uint8_t* wrote;          // 1 where this vertex's slot in xn was written by the previous sweep
-  double tau_f, tau_p;
+  Real tau_f, tau_p;
   int prune;               // DF-P (Eq. 2, prune) or DF (Eq. 1)
-  unsigned long long* fw;  // null, or: += out-edges of the vertices this sweep puts into deltaN
-  unsigned long long* fw_base;  // graph-driven loop: fw of iteration it is fw_base + it
-  // Static: chunks of the highest in-degree class's rows (nchunk = 0: none)
-  // and one partial sum per chunk (4 words)
-  PprHub hub;
-  uint4* hub_part;
+  int expand;              // an expansion round after each sweep
+  int init_push;           // the marked batch's frontier list is expanded before the first sweep
+  const int64_t* ooff;     // G (push form)
+  const int32_t* oadj;
+  int2* list;              // frontier entries of the round (room for n + m / kFrontChunk + 1)
+  unsigned long long fthr; // the round runs in pull form when the frontier's out-edges exceed this
+  int64_t pull_warp_b;     // pull form: rows from here on take a warp each
 };
-
-// FP32 stage of the mixed-precision sweeps (sweep32.cu): Static (Eq. 1 on
-// every vertex) or DF / DF-P (Eq. 1 / Eq. 2 on the affected vertices, with
-// the prune and expand flags of Alg. update).
-struct Sweep32Args {
-  const int64_t* off;      // in-CSR offsets of G' (class-contiguous numbering)
-  const int32_t* adj;      // in-CSR sources
-  const float* y;          // y[u] = R[u] / |out(u)| in FP32
-  float* yn;               // next y
-  const float* degf;       // |out(v)| as float
-  const float* invf;       // 1 / |out(v)| as float
-  float alpha, c0;
-  int self_loops;
-  const uint32_t* multi;   // as in SweepArgs
-  uint32_t* resid;         // [0]: max |r - R[v]|, [1]: max r of this sweep (FP32 bits, atomic max)
-  const uint32_t* prev;    // previous sweep's pair, or null
-  float tol_rel;           // the sweep exits at once if prev[0] <= tol_rel * prev[1]
-  // device-driven iteration (CUDA graph): when ctl is set the kernel takes
-  // y/yn/resid/prev for iteration it = ctl[0] from ya/yb/resid_base instead
-  const int* ctl;
-  const float* ya;
-  float* yb;
-  uint32_t* resid_base;
-  // DF / DF-P only (same meaning as in SweepArgs)
-  const float* kf;         // Eq. 2 factor 1 / (1 - alpha / |out(v)|) as float
-  uint8_t* dV;
-  uint8_t* dN;
-  uint8_t* wrote;
-  float tau_f, tau_p;
-  int prune;
-  unsigned long long* fw;       // as in SweepArgs
-  unsigned long long* fw_base;
-  // chunks of the highest in-degree class's rows (nchunk = 0: a block per row)
-  // and one compensated partial sum (s, e) per chunk
-  PprHub hub;
-  float2* hub_part;
-};
-int launch_sweep32(const Sweep32Args& a, const PartThr& t, const int64_t* class_begin, bool dynamic, cudaStream_t s);
-// One-thread check of the graph-driven FP32 loop: it = ctl[0]; stop when
-// r32[2 it] <= tol_rel * r32[2 it + 1] or it + 1 >= max_iter; ctl[0] = it + 1.
-int launch_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
-                        cudaGraphConditionalHandle h, cudaStream_t s);
+int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t* cb, bool exact, bool dynamic,
+                     cudaStream_t s);
+int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s);
+// initialAffected (Alg. affected) in the sweep numbering: dV, dN and the frontier list of the first push
+// (dN padded to whole 32-bit words)
+int launch_mark_batch(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
+                      const int32_t* ins_src, const uint8_t* ins_mask, int64_t n_ins, const int32_t* inv,
+                      const int64_t* ooff, uint8_t* dV, uint8_t* dN, LoopCtl* ctl, int2* list, cudaStream_t s);
 
 // K-column personalised PageRank (ppr.cu), row-major [n, K] in the class-contiguous numbering.
 struct Ppr32Args {
@@ -269,54 +286,30 @@ int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, c
 int ppr_narrow(const double* x, int64_t cnt, float* y, cudaStream_t s);
 int ppr_widen(const float* y, int64_t cnt, double* x, cudaStream_t s);
 
-// One-thread iteration check of the graph-driven loop: it = ctl[0]; stop when
-// resid[it] <= tol or it + 1 >= max_iter; ctl[0] = it + 1; sets the while condition.
+// One-thread checks of the graph-driven K-column loops: it = ctl[0]; stop when
+// resid[it] <= tol (FP64) or resid[2 it] <= tol_rel * resid[2 it + 1] (FP32),
+// or it + 1 >= max_iter; ctl[0] = it + 1; sets the while condition.
 int launch_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
                       cudaGraphConditionalHandle h, cudaStream_t s);
-
-// Launch one rank sweep (all degree classes) for Static (dynamic = false) or DF/DF-P.
-int launch_sweep(const SweepArgs& a, const PartThr& t, const int64_t* class_begin, bool exact, bool dynamic,
-                 cudaStream_t s);
-
-// Stop rule of the loop an expansion round belongs to, read on the device so
-// that rounds launched after the converged sweep do nothing. FP64 loops:
-// r64[it] <= tol; FP32 stage: r32[2 it] <= tol_rel * r32[2 it + 1]; neither
-// set: the round always runs. it = ctl[0] in the graph-driven loop, else 0
-// (r64 / r32 then point at this sweep's slot).
-struct Stop {
-  const uint64_t* r64 = nullptr;
-  double tol = 0;
-  const uint32_t* r32 = nullptr;
-  float tol_rel = 0;
-  const int* ctl = nullptr;
-};
+int launch_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
+                        cudaGraphConditionalHandle h, cudaStream_t s);
 
 // Alg. affected kernels (frontier.cu). map (nullable): vertex id -> flag index.
 int launch_initial_affected(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
                             const int32_t* ins_src, const uint8_t* ins_mask, int64_t n_ins, const int32_t* map,
                             uint8_t* dV, uint8_t* dN, cudaStream_t s);
-// expandAffected over the out-degree partition; skipped on the device when the
-// stop rule st holds, and when fw (nullable; this round's counter, indexed by
-// st.ctl in the graph-driven loop) is given, also when *fw > fthr (the pull
-// form runs instead). dF (nullable): also mark in dF every vertex that was not
-// yet in dV (one round of Dynamic Traversal's reachability closure).
-// fl (optional scratch): a frontier of at most fl.cap vertices is listed and
-// expanded from the list, without the partition kernels' scan of every vertex.
+// expandAffected over the out-degree partition. dF (nullable): also mark in
+// dF every vertex that was not yet in dV (one round of Dynamic Traversal's
+// reachability closure). fl (optional scratch): a frontier of at most fl.cap
+// vertices is listed and expanded from the list, without the partition
+// kernels' scan of every vertex.
 struct FrontList {
   int32_t* list = nullptr;      // cap entries
   unsigned int* cnt = nullptr;  // one counter
   unsigned int cap = 0;
 };
 int launch_expand(const int64_t* off, const int32_t* adj, const int32_t* P, const int64_t* cb, int nclass,
-                  const uint8_t* dN, uint8_t* dV, uint8_t* dF, const Stop& st, cudaStream_t s,
-                  const unsigned long long* fw = nullptr, unsigned long long fthr = 0,
-                  const FrontList& fl = FrontList());
-// The same round in pull form over G' (in_off/in_adj; rows from warp_begin on
-// take a warp each): marks only if *fw, the frontier's out-edges (counted by
-// the sweep before it), exceeds fthr.
-int launch_expand_pull(const int64_t* in_off, const int32_t* in_adj, int64_t n, int64_t warp_begin,
-                       const uint8_t* dN, uint8_t* dV, const unsigned long long* fw, unsigned long long fthr,
-                       const Stop& st, cudaStream_t s);
+                  const uint8_t* dN, uint8_t* dV, uint8_t* dF, cudaStream_t s, const FrontList& fl = FrontList());
 int count_flags(const uint8_t* f, int64_t n, unsigned long long* dev_out, cudaStream_t s);
 
 }  // namespace prdf
@@ -338,8 +331,8 @@ struct prdf_graph {
   // solver scratch
   prdf::DBuf<double> xa, xb;
   prdf::PprHubTable hub_in, hub_out;  // chunk tables of G' (Static sweep, K-column forward) and G (adjoint)
-  prdf::DBuf<uint4> sweep_hub_part;   // FP64 sweeps: one exact partial sum per chunk of G's hub rows
-  prdf::DBuf<float2> sweep_hub_part32;  // FP32 sweeps: one compensated partial sum per chunk
+  prdf::DBuf<uint4> sweep_hub_part;     // rank sweeps: one partial sum per chunk of G's hub rows
+  prdf::DBuf<uint32_t> sweep_hub_done;  // and one arrival counter per hub row
   prdf::DBuf<float2> ppr_part;        // chunk partial sums of one column tile (FP32 sweeps)
   prdf::DBuf<double> ppr_part64;      // chunk partial sums of one column tile (FP64 steps)
   prdf::DBuf<float> ya, yb, degf, invf;  // FP32 stage state and degrees (class-contiguous numbering)
@@ -350,16 +343,17 @@ struct prdf_graph {
   prdf::DBuf<uint8_t> dF;  // Dynamic Traversal: next frontier of the closure
   prdf::DBuf<unsigned long long> counter;
   prdf::DBuf<unsigned long long> chk;  // input checks: bad-id flag, bad-rank flag, rank sum (double bits)
-  prdf::DBuf<unsigned long long> fwork;  // frontier out-edges of each expansion round
-  prdf::DBuf<int32_t> flist;             // a small frontier listed for its expansion round (frontier.cu)
+  prdf::DBuf<prdf::LoopCtl> loop_ctl;    // state of a rank loop
+  prdf::DBuf<prdf::LoopSlot> loop_slots; // its per-sweep counters
+  prdf::DBuf<int2> loop_list;            // DF / DF-P: frontier entries of an expansion round
+  prdf::DBuf<int32_t> flist;             // DT: a small frontier listed for its closure round (frontier.cu)
   prdf::DBuf<unsigned int> fcnt;         // its size
-  prdf::DBuf<int> ctl;               // device iteration counter of the graph-driven loop
+  prdf::DBuf<int> ctl;               // device iteration counter of the graph-driven K-column loops
   cudaStream_t cap_stream = nullptr; // private stream used to capture graph bodies
-  // instantiated loops (CUDA graphs), one per kind of loop, each with the
-  // arguments and buffers it was captured for: sweep loops at fp32 * 4 +
-  // dynamic * 2 + expand; K-column loops from 8 on
-  cudaGraphExec_t loop_exec[16] = {};
-  std::vector<uint64_t> loop_key[16];
+  // instantiated K-column loops (CUDA graphs), one per kind of loop, each
+  // with the arguments and buffers it was captured for
+  cudaGraphExec_t loop_exec[8] = {};
+  std::vector<uint64_t> loop_key[8];
   prdf::Relabel rl;                  // class-contiguous copy used by the sweeps
   // weighted graphs: transition probabilities P_uv = w_uv / sum_k w_uk
   bool ppr_valid = false;

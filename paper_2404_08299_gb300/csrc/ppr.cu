@@ -670,6 +670,24 @@ __global__ void k_widen_n(const float* __restrict__ y, int64_t cnt, double* __re
     x[i] = (double)y[i];
 }
 
+// stop checks of the graph-driven loops
+__global__ void k_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
+                             cudaGraphConditionalHandle h) {
+  const int it = ctl[0];
+  const bool done = bitsd(resid_base[it]) <= tol || it + 1 >= max_iter;
+  ctl[0] = it + 1;
+  cudaGraphSetConditional(h, done ? 0u : 1u);
+}
+
+__global__ void k_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
+                               cudaGraphConditionalHandle h) {
+  const int it = ctl[0];
+  const uint32_t* r = resid_base + 2 * it;
+  const bool done = __uint_as_float(r[0]) <= tol_rel * __uint_as_float(r[1]) || it + 1 >= max_iter;
+  ctl[0] = it + 1;
+  cudaGraphSetConditional(h, done ? 0u : 1u);
+}
+
 template <int LPE>
 void launch32_tile(const Ppr32Args& a, const PprHub& h, float2* part, int64_t hub_b, int64_t n, int c0, int tile,
                    cudaStream_t s) {
@@ -697,6 +715,20 @@ void launch64_tile(const Ppr64Args& a, const PprHub& h, double* part, int64_t hu
 }
 
 }  // namespace
+
+int launch_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
+                      cudaGraphConditionalHandle h, cudaStream_t s) {
+  k_iter_check<<<1, 1, 0, s>>>(ctl, resid_base, tol, max_iter, h);
+  PRDF_LAUNCH_CHECK();
+  return PRDF_OK;
+}
+
+int launch_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
+                        cudaGraphConditionalHandle h, cudaStream_t s) {
+  k_iter_check32<<<1, 1, 0, s>>>(ctl, resid_base, tol_rel, max_iter, h);
+  PRDF_LAUNCH_CHECK();
+  return PRDF_OK;
+}
 
 int launch_ppr32_sweep(const Ppr32Args& a, int tile, int64_t n, int64_t hub_begin, const PprHub& h, float2* part,
                        cudaStream_t s) {

@@ -147,7 +147,7 @@ int permute_csr(const Csr& src, const int32_t* perm, const int32_t* inv, int32_t
   PRDF_TRY(dst.off.alloc((size_t)n + 1, s));
   PRDF_TRY(exclusive_scan_i64(len.p, n, dst.off.p, ws, s));
   dst.m = src.m;
-  PRDF_TRY(dst.adj.alloc(src.m > 0 ? (size_t)src.m : 1, s));
+  PRDF_TRY(dst.adj.alloc((size_t)src.m + kAdjPad, s));
   if (src.w.p) PRDF_TRY(dst.w.alloc(src.m > 0 ? (size_t)src.m : 1, s));
   else dst.w.release();
   if (src.m > 0)

@@ -1,243 +1,147 @@
-// Synchronous, pull-based, atomics-free rank sweeps (Alg. update of
-// arXiv 2404.08299) for Static (Eq. 1, every vertex) and DF / DF-P
-// (Eq. 1 / Eq. 2 on affected vertices, with prune and expand flags).
+// Synchronous, pull-based rank sweeps (Alg. update of arXiv 2404.08299) for
+// Static (Eq. 1, every vertex) and DF / DF-P (Eq. 1 / Eq. 2 on the affected
+// vertices, with prune and expand flags), the expansion rounds between them
+// (Alg. affected), and the loop around both, in FP64 and in FP32.
 //
-// State: x[u] = R[u] / |out(u)|, so a sweep gathers one FP64 value per
-// in-edge. The sweeps run on the class-contiguous numbering (relabel.cu):
-// class c is the id range [begin, end). Vertices are split by in-degree class (the paper's thread- and
-// block-per-vertex kernels, refined into narrower classes so the lanes of a
-// warp carry similar work): each vertex is processed by a group of G lanes
-// (G = 1, 4, 16, 32) or by a whole block. The L-inf change of the sweep is
-// reduced in the epilogue (warp max, block max, one 64-bit atomic max per
-// block on the bit pattern of a non-negative double); rank writes stay one
+// One persistent kernel runs a whole loop: k_rank_loop is launched
+// cooperatively with as many blocks as fit the GPU, every sweep and every
+// expansion round is one phase of it, and a grid barrier separates phases.
+// Before, each in-degree class of each sweep was a kernel of its own inside a
+// CUDA graph (eight launches a sweep, up to eight more an expansion round,
+// and a graph to build anew after every batch update).
+//
+// State: x[u] = R[u] / |out(u)|, so a sweep gathers one value per in-edge.
+// The sweeps run on the class-contiguous numbering (relabel.cu): class c is
+// the id range [begin, end). A class is cut into units of rows that warps
+// fetch from a counter, long rows first, so that the tail of one class is
+// filled with the work of the next. A unit goes through batches of 32 rows
+// (the affected ones only, in DF / DF-P): groups of G lanes (G = 4, 8, 16, 32
+// by class) sum the batch's rows one after the other, each group keeping the
+// sum of its s-th row in its s-th lane, and the epilogue then runs once with
+// a row in every lane. The epilogue costs some hundred instructions, FP64
+// ones among them (which GB300 issues at about 1.6 a clock per SM whatever
+// the number of active lanes), so it is shared by 32 rows instead of running
+// in one lane per row.
+//
+// The L-inf change of the sweep is reduced per block and with one atomic max
+// per block on the bit pattern of a non-negative value; rank writes stay one
 // plain store per vertex.
-//
-// GB300 issues FP64 instructions at ~1.6 per clock per SM, so gathered
-// values stay in 64-bit integer registers and are summed exactly on the
-// integer pipes (common.cuh); FP64 arithmetic is limited to a few
-// instructions per vertex.
-//
-// A sweep whose predecessor already met the tolerance exits at once, so the
-// host can launch several sweeps ahead of its convergence check.
+#include <cstring>
+
 #include "internal.cuh"
 
 namespace prdf {
 
 namespace {
 
-constexpr int kThreads = 256;
-// four blocks of 256 threads per SM (64 registers a thread): the sweeps are
-// bound by the latency of their gathers, so resident warps matter more than
-// registers (at 70 registers a thread the DF-P warp kernel ran 3 blocks per SM
-// and took 1.5x the time of the same work at 64). The block-per-vertex kernel
-// and the 8-indices-per-lane group need more registers and keep three.
-constexpr int kMinBlocks = 4;
+// Two blocks of 512 threads per SM at 64 registers: the sweeps are bound by
+// the latency and the rate of their gathers, so resident warps matter more
+// than registers, and few blocks keep the grid barrier short.
+constexpr int kThreads = 512;
+constexpr int kMinBlocks = 2;
+constexpr int kWarps = kThreads / 32;
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kMaxWords = 8;  // a unit holds at most 8 x 32 rows
 
-// Exact accumulator (4 x 32-bit words, 2^-124 resolution) or plain FP64.
-template <bool EXACT>
-struct Acc;
+// ------------------------------------------------------ precision traits ----
 
-template <>
-struct Acc<true> {
+// gathered state: coherent loads (the buffers are written in the same kernel,
+// a grid barrier earlier), kept in L2 (evict-last)
+__device__ __forceinline__ uint64_t ld_state(const double* p, uint64_t pol) {
+  uint64_t v;
+  asm volatile("ld.global.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_state(const float* p, uint64_t pol) {
+  uint32_t v;
+  asm volatile("ld.global.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ float ld_const(const float* p, uint64_t pol) {
+  float v;
+  asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+  return v;
+}
+
+// Exact accumulator (4 x 32-bit words, 2^-124 resolution).
+struct AccExact {
   Fix4 v;
   __device__ __forceinline__ void add(uint64_t xb) { v.add(xb); }
   // add_w1: only for terms with in_w1 (the common window, three-word add)
   __device__ __forceinline__ static bool in_w1(uint64_t xb) { return Fix4::in_w1(xb); }
   __device__ __forceinline__ void add_w1(uint64_t xb) { v.add_w1(xb); }
-  __device__ __forceinline__ void merge(const Acc& o) { v.add4(o.v.w0, o.v.w1, o.v.w2, o.v.w3); }
-  __device__ __forceinline__ Acc shfl_up(int o) const {
-    Acc r;
-    r.v.w0 = __shfl_up_sync(0xffffffffu, v.w0, o);
-    r.v.w1 = __shfl_up_sync(0xffffffffu, v.w1, o);
-    r.v.w2 = __shfl_up_sync(0xffffffffu, v.w2, o);
-    r.v.w3 = __shfl_up_sync(0xffffffffu, v.w3, o);
-    return r;
-  }
-  __device__ __forceinline__ Acc shfl_idx(int l) const {
-    Acc r;
-    r.v.w0 = __shfl_sync(0xffffffffu, v.w0, l);
-    r.v.w1 = __shfl_sync(0xffffffffu, v.w1, l);
-    r.v.w2 = __shfl_sync(0xffffffffu, v.w2, l);
-    r.v.w3 = __shfl_sync(0xffffffffu, v.w3, l);
-    return r;
-  }
   template <int G>
   __device__ __forceinline__ void group_reduce() { v.template group_reduce<G>(); }
   __device__ __forceinline__ double value() const { return v.to_double(); }
-  __device__ __forceinline__ void to_shared(uint32_t* s) const { v.store(s); }
-  __device__ __forceinline__ void from_shared(const uint32_t* s) { v.add_words(s); }
+  __device__ __forceinline__ uint4 pack() const { return make_uint4(v.w0, v.w1, v.w2, v.w3); }
+  __device__ __forceinline__ void merge(const uint4& p) { v.add4(p.x, p.y, p.z, p.w); }
 };
 
-template <>
-struct Acc<false> {
+// plain FP64 additions
+struct AccPlain {
   double v = 0;
   __device__ __forceinline__ void add(uint64_t xb) { v += bitsd(xb); }
   __device__ __forceinline__ static bool in_w1(uint64_t) { return true; }
   __device__ __forceinline__ void add_w1(uint64_t xb) { v += bitsd(xb); }
-  __device__ __forceinline__ void merge(const Acc& o) { v += o.v; }
-  __device__ __forceinline__ Acc shfl_up(int o) const {
-    Acc r;
-    r.v = __shfl_up_sync(0xffffffffu, v, o);
-    return r;
+  template <int G>
+  __device__ __forceinline__ void group_reduce() {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   }
-  __device__ __forceinline__ Acc shfl_idx(int l) const {
-    Acc r;
-    r.v = __shfl_sync(0xffffffffu, v, l);
-    return r;
+  __device__ __forceinline__ double value() const { return v; }
+  __device__ __forceinline__ uint4 pack() const {
+    const uint64_t b = dbits(v);
+    return make_uint4((uint32_t)b, (uint32_t)(b >> 32), 0u, 0u);
+  }
+  __device__ __forceinline__ void merge(const uint4& p) { v += bitsd(((uint64_t)p.y << 32) | p.x); }
+};
+
+// FP32 sum compensated by Kahan-Babuska (TwoSum of every term, errors summed
+// separately): value = s + e
+struct AccKahan {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void addf(float y) {
+    const float t = s + y;
+    const float bp = t - s;
+    e += (s - (t - bp)) + (y - bp);
+    s = t;
+  }
+  __device__ __forceinline__ void add(uint32_t b) { addf(__uint_as_float(b)); }
+  __device__ __forceinline__ static bool in_w1(uint32_t) { return true; }
+  __device__ __forceinline__ void add_w1(uint32_t b) { addf(__uint_as_float(b)); }
+  __device__ __forceinline__ void merge2(float s2, float e2) {
+    addf(s2);
+    e += e2;
   }
   template <int G>
   __device__ __forceinline__ void group_reduce() {
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const float s2 = __shfl_xor_sync(kFull, s, o);
+      const float e2 = __shfl_xor_sync(kFull, e, o);
+      merge2(s2, e2);
+    }
   }
-  __device__ __forceinline__ double value() const { return v; }
-  __device__ __forceinline__ void to_shared(uint32_t* s) const {
-    const uint64_t b = dbits(v);
-    s[0] = (uint32_t)b;
-    s[1] = (uint32_t)(b >> 32);
+  __device__ __forceinline__ float value() const { return s + e; }
+  __device__ __forceinline__ uint4 pack() const {
+    return make_uint4(__float_as_uint(s), __float_as_uint(e), 0u, 0u);
   }
-  __device__ __forceinline__ void from_shared(const uint32_t* s) {
-    v += bitsd(((uint64_t)s[1] << 32) | s[0]);
-  }
+  __device__ __forceinline__ void merge(const uint4& p) { merge2(__uint_as_float(p.x), __uint_as_float(p.y)); }
 };
 
-// Per-lane gather over row [b, e) of G' with stride G and U loads in flight.
-template <int G, int U, bool EXACT>
-__device__ __forceinline__ void gather_row(const SweepArgs& a, int64_t b, int64_t e, int lane, int32_t v,
-                                           Acc<EXACT>& acc, uint64_t& xself, uint64_t pf, uint64_t pl) {
-  for (int64_t j0 = b + lane; j0 < e; j0 += (int64_t)G * U) {
-    int32_t u[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t j = j0 + (int64_t)k * G;
-      u[k] = j < e ? ld_stream_i32(a.adj + j, pf) : -1;
-    }
-    uint64_t xv[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) xv[k] = u[k] >= 0 ? ld_gather_b64(a.x + u[k], pl) : 0ull;
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      if (u[k] >= 0) acc.add(xv[k]);
-      xself = (u[k] == v) ? xv[k] : xself;
-    }
-  }
-}
-
-// Vectorised variant for a row handled by NT lanes: 16-byte index loads for
-// the aligned body (KV of them in flight per lane), scalar head and tail;
-// row_indices issues a row's first indices, gather_row_from consumes them.
-// (A warp kernel that loaded the next row's first indices a turn ahead needed
-// 76 registers, ran three blocks per SM instead of four and was 4 % slower.)
-template <int KV>
-struct RowIdx {
-  int64_t ba = 0, ea = 0;  // aligned body [ba, ea)
-  int32_t uh = -1;         // this lane's head or tail entry (the unaligned ends), -1: none
-  int4 u4[KV];             // this lane's first body indices
+template <class A>
+struct Prec64 {
+  using Real = double;
+  using Bits = uint64_t;
+  using Acc = A;
 };
-
-template <int NT, int KV>
-__device__ __forceinline__ void row_indices(const SweepArgs& a, int64_t b, int64_t e, int lane, uint64_t pf,
-                                            RowIdx<KV>& r) {
-  int64_t ba = (b + 3) & ~(int64_t)3;
-  if (ba > e) ba = e;
-  const int64_t ea = ba + ((e - ba) & ~(int64_t)3);
-  r.ba = ba;
-  r.ea = ea;
-  const int64_t nh = ba - b, nt = e - ea;
-  int64_t j = -1;
-  if (lane < nh) j = b + lane;
-  else if (lane >= 4 && lane < 4 + nt) j = ea + (lane - 4);
-  r.uh = j >= 0 ? ld_stream_i32(a.adj + j, pf) : -1;
-#pragma unroll
-  for (int k = 0; k < KV; ++k) {
-    const int64_t q = ba + 4 * (int64_t)lane + 4 * (int64_t)NT * k;
-    r.u4[k] = q < ea ? ld_stream_i32x4(a.adj + q, pf) : make_int4(-1, -1, -1, -1);
-  }
-}
-
-// The head / tail term's gather is issued with the body's first gathers and
-// added after them, so the row costs one gather round trip before its first
-// add. The body loads the next chunk's indices while this chunk's gathers are
-// in flight; the loop runs the same trip count on all NT lanes, so each warp
-// is converged at the vote below.
-template <int NT, int KV, bool EXACT, bool SELF = true>
-__device__ __forceinline__ void gather_row_from(const SweepArgs& a, const RowIdx<KV>& r, int lane, int32_t v,
-                                                Acc<EXACT>& acc, uint64_t& xself, uint64_t pf, uint64_t pl) {
-  const int64_t ba = r.ba, ea = r.ea;
-  const int32_t uh = r.uh;
-  const int64_t step = 4 * (int64_t)NT * KV;
-  int4 u4[KV];
-#pragma unroll
-  for (int k = 0; k < KV; ++k) u4[k] = r.u4[k];
-  uint64_t xh = uh >= 0 ? ld_gather_b64(a.x + uh, pl) : 0ull;
-  bool head = uh >= 0;  // the head term is still to be added
-  for (int64_t base = ba; base < ea; base += step) {
-    const int64_t q0 = base + 4 * (int64_t)lane;
-    uint64_t xv[4 * KV];
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-      xv[4 * k + 0] = u4[k].x >= 0 ? ld_gather_b64(a.x + u4[k].x, pl) : 0ull;
-      xv[4 * k + 1] = u4[k].y >= 0 ? ld_gather_b64(a.x + u4[k].y, pl) : 0ull;
-      xv[4 * k + 2] = u4[k].z >= 0 ? ld_gather_b64(a.x + u4[k].z, pl) : 0ull;
-      xv[4 * k + 3] = u4[k].w >= 0 ? ld_gather_b64(a.x + u4[k].w, pl) : 0ull;
-    }
-    int4 nx[KV];
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-      const int64_t q = q0 + step + 4 * (int64_t)NT * k;
-      nx[k] = q < ea ? ld_stream_i32x4(a.adj + q, pf) : make_int4(-1, -1, -1, -1);
-    }
-    if (head) {
-      acc.add(xh);
-      if (SELF) xself = (uh == v) ? xh : xself;
-      head = false;
-    }
-    bool w1 = true;
-#pragma unroll
-    for (int k = 0; k < KV; ++k)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) w1 = w1 && (u4[k].x < 0 || Acc<EXACT>::in_w1(xv[4 * k + q]));
-    if (__all_sync(0xffffffffu, w1)) {
-#pragma unroll
-      for (int k = 0; k < KV; ++k) {
-        if (u4[k].x < 0) continue;  // a whole int4 is valid or not
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc.add_w1(xv[4 * k + q]);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < KV; ++k) {
-        if (u4[k].x < 0) continue;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc.add(xv[4 * k + q]);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-      if (u4[k].x < 0) continue;
-      if (SELF) {
-        xself = (u4[k].x == v) ? xv[4 * k + 0] : xself;
-        xself = (u4[k].y == v) ? xv[4 * k + 1] : xself;
-        xself = (u4[k].z == v) ? xv[4 * k + 2] : xself;
-        xself = (u4[k].w == v) ? xv[4 * k + 3] : xself;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < KV; ++k) u4[k] = nx[k];
-  }
-  if (head) {  // rows without a body chunk
-    acc.add(xh);
-    if (SELF) xself = (uh == v) ? xh : xself;
-  }
-}
-
-template <int NT, int KV, bool EXACT, bool SELF = true>
-__device__ __forceinline__ void gather_row_vec(const SweepArgs& a, int64_t b, int64_t e, int lane, int32_t v,
-                                               Acc<EXACT>& acc, uint64_t& xself, uint64_t pf, uint64_t pl) {
-  RowIdx<KV> r;
-  row_indices<NT, KV>(a, b, e, lane, pf, r);
-  gather_row_from<NT, KV, EXACT, SELF>(a, r, lane, v, acc, xself, pf, pl);
-}
+using PExact = Prec64<AccExact>;
+using PPlain = Prec64<AccPlain>;
+struct PKahan {
+  using Real = float;
+  using Bits = uint32_t;
+  using Acc = AccKahan;
+};
 
 // Exact integer value of an out-degree held as a double (an integer below
 // 2^53), decoded from its bit pattern on the integer pipes; 0 for 0.
@@ -247,579 +151,953 @@ __device__ __forceinline__ uint64_t degree_of(double d) {
   const uint64_t mant = (b & 0x000FFFFFFFFFFFFFull) | (1ull << 52);
   return e >= 0 ? mant >> (52 - e) : 0ull;
 }
+__device__ __forceinline__ uint64_t degree_of(float d) { return (uint64_t)d; }
+
+// What a warp carries through a sweep: largest |r - R[v]|, (FP32) largest r,
+// out-edges put into deltaN, affected vertices seen.
+struct Tally {
+  uint64_t dmax = 0;
+  uint32_t rmax = 0;
+  uint64_t fw = 0;
+  unsigned int aff = 0;
+};
+
+// ---------------------------------------------------------- per sweep ----
+template <class P>
+struct Ctx {
+  const typename P::Real* x;
+  typename P::Real* xn;
+  LoopSlot* slot;  // this sweep's
+  uint64_t pf, pl;
+  int lane;
+};
+
+// Frontier entries of one vertex: one per kFrontChunk out-edges.
+__device__ __forceinline__ unsigned int front_entries(uint64_t deg) {
+  return (unsigned int)((deg + kFrontChunk - 1) / kFrontChunk);
+}
+
+// The lanes with flag set append their vertices to the frontier list (all
+// lanes call it): warp-aggregated, one entry per kFrontChunk out-edges.
+__device__ __forceinline__ void append_frontier(bool flag, int32_t v, uint64_t deg, unsigned int* count, int2* list,
+                                                int lane) {
+  if (!__any_sync(kFull, flag)) return;
+  const unsigned int c = flag ? front_entries(deg) : 0u;
+  unsigned int incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int t = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += t;
+  }
+  unsigned int base = 0;
+  if (lane == 31) base = atomicAdd(count, incl);
+  base = __shfl_sync(kFull, base, 31) + incl - c;
+  for (unsigned int k = 0; k < c; ++k) list[base + k] = make_int2(v, (int)k);
+}
 
 // Vertex epilogue: Eq. 1 (Static, DF) or Eq. 2 (DF-P), prune / expand flags,
-// next x, and this vertex's |r - R[v]| as bits. GB300's FP64 pipe is narrow,
-// so FP64 instructions are kept to those that need FP64 rounding: three on the
-// Static path (r, |r - R[v]| as one FMA, next x); on the DF-P path also
-// Eq. 2's two extra steps, R[v] and the threshold tau * max(r, R[v]). The
-// maximum and the comparisons run on the bit patterns of the non-negative
-// doubles (integer instructions, the same order as the FP64 comparison; a
-// negative threshold's pattern is negative as int64, so it orders below every
-// non-negative value, as in FP64).
+// next x, and this vertex's |r - R[v]| into the tally. GB300's FP64 pipe is
+// narrow, so the FP64 form keeps to what needs FP64 rounding; the maximum and
+// the comparisons run on the bit patterns of the non-negative doubles
+// (integer instructions, the same order as the FP64 comparison; a negative
+// threshold's pattern is negative as int64, so it orders below every
+// non-negative value, as in FP64). Returns whether v joins deltaN.
 template <bool DYN>
-__device__ __forceinline__ uint64_t finish_vertex(const SweepArgs& a, int32_t v, double c, uint64_t xself_b,
-                                                  uint64_t pf, uint64_t& fwsum, uint8_t dn_old) {
-  const double xself = bitsd(xself_b);
-  const double d = ld_stream_f64(a.degd + v, pf);
+__device__ __forceinline__ bool finish(const SweepArgs<double>& a, const Ctx<PExact>& c, int32_t v, double sum,
+                                       double xself, bool dn_old, Tally& t, uint64_t& deg) {
+  const double d = ld_stream_f64(a.deg + v, c.pf);
+  const double iv = ld_stream_f64(a.inv + v, c.pf);
   double r;
   if (DYN && a.prune) {
     // Eq. 2: the self-loop term is solved in closed form (factor precomputed per vertex)
-    r = ld_stream_f64(a.kf + v, pf) * (a.c0 + a.alpha * (c - xself));
+    r = ld_stream_f64(a.kf + v, c.pf) * (a.c0 + a.alpha * (sum - xself));
   } else {
-    r = fma(a.alpha, c, a.c0);  // Eq. 1
+    r = fma(a.alpha, sum, a.c0);  // Eq. 1
   }
   // |r - R[v]| with R[v] = x[v] * |out(v)| of the previous iteration, one rounding
   const double dr = fabs(fma(xself, -d, r));
+  bool front = false;
   if (DYN) {
     const uint64_t rb = dbits(r), ob = dbits(xself * d), drb = dbits(dr);
     const double m = bitsd(rb > ob ? rb : ob);  // max(r, R[v])
     const int64_t tp = (int64_t)dbits(a.tau_p * m);
     const int64_t tf = a.tau_f == a.tau_p ? tp : (int64_t)dbits(a.tau_f * m);
     if (a.prune && (int64_t)drb <= tp) a.dV[v] = 0;
-    // deltaN holds exactly this sweep's expand set: set or cleared for every vertex; the out-edges of
-    // the set are counted for the choice of the expansion round's direction
-    // (dn_old: the vertex's deltaN flag before this sweep, read ahead; no load on this path)
-    if ((int64_t)drb > tf) {
-      if (!dn_old) a.dN[v] = 1;
-      fwsum += degree_of(d);
-    } else if (dn_old) {
-      a.dN[v] = 0;
+    // deltaN holds exactly this sweep's expand set: set or cleared for every vertex
+    front = (int64_t)drb > tf;
+    if (front != dn_old) a.dN[v] = front ? 1 : 0;
+    if (front) {
+      deg = degree_of(d);
+      t.fw += deg;
     }
     a.wrote[v] = 1;
   }
-  a.xn[v] = r * ld_stream_f64(a.inv_deg + v, pf);
-  return dbits(dr);
+  c.xn[v] = r * iv;
+  const uint64_t db = dbits(dr);
+  t.dmax = db > t.dmax ? db : t.dmax;
+  return front;
+}
+template <bool DYN>
+__device__ __forceinline__ bool finish(const SweepArgs<double>& a, const Ctx<PPlain>& c, int32_t v, double sum,
+                                       double xself, bool dn_old, Tally& t, uint64_t& deg) {
+  const Ctx<PExact> e{c.x, c.xn, c.slot, c.pf, c.pl, c.lane};
+  return finish<DYN>(a, e, v, sum, xself, dn_old, t, deg);
+}
+// the same in FP32, with Alg. update's prune and expand tests evaluated in FP32
+template <bool DYN>
+__device__ __forceinline__ bool finish(const SweepArgs<float>& a, const Ctx<PKahan>& c, int32_t v, float sum,
+                                       float xself, bool dn_old, Tally& t, uint64_t& deg) {
+  const float d = ld_const(a.deg + v, c.pf);
+  const float iv = ld_const(a.inv + v, c.pf);
+  const float rold = xself * d;
+  float r;
+  if (DYN && a.prune) r = ld_const(a.kf + v, c.pf) * fmaf(a.alpha, sum - xself, a.c0);  // Eq. 2
+  else r = fmaf(a.alpha, sum, a.c0);                                                      // Eq. 1
+  const float dr = fabsf(r - rold);
+  bool front = false;
+  if (DYN) {
+    const float m = fmaxf(r, rold);
+    if (a.prune && dr <= a.tau_p * m) a.dV[v] = 0;
+    front = dr > a.tau_f * m;
+    if (front != dn_old) a.dN[v] = front ? 1 : 0;
+    if (front) {
+      deg = degree_of(d);
+      t.fw += deg;
+    }
+    a.wrote[v] = 1;
+  }
+  c.xn[v] = r * iv;
+  const uint32_t db = __float_as_uint(dr), rb = __float_as_uint(r);
+  t.dmax = db > (uint32_t)t.dmax ? db : t.dmax;
+  t.rmax = rb > t.rmax ? rb : t.rmax;
+  return front;
 }
 
-// per-iteration pointers of the graph-driven loop
-__device__ __forceinline__ SweepArgs resolve(const SweepArgs& in) {
-  if (!in.ctl) return in;
-  SweepArgs a = in;
-  const int it = in.ctl[0];
-  a.x = (it & 1) ? in.xb : in.xa;
-  a.xn = (it & 1) ? const_cast<double*>(in.xa) : in.xb;
-  a.resid = in.resid_base + it;
-  a.prev = it > 0 ? in.resid_base + it - 1 : nullptr;
-  a.fw = in.fw_base ? in.fw_base + it : nullptr;
-  return a;
-}
-
-__global__ void k_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
-                             cudaGraphConditionalHandle h) {
-  const int it = ctl[0];
-  const bool done = bitsd(resid_base[it]) <= tol || it + 1 >= max_iter;
-  ctl[0] = it + 1;
-  cudaGraphSetConditional(h, done ? 0u : 1u);
-}
+__device__ __forceinline__ double as_real(uint64_t b) { return bitsd(b); }
+__device__ __forceinline__ float as_real(uint32_t b) { return __uint_as_float(b); }
 
 // DF / DF-P: an unaffected vertex keeps its rank; its slot in xn is stale
 // only if the previous sweep wrote it (then copy it through). It is not in
 // this sweep's expand set, so its deltaN flag is cleared (the sweep keeps
 // deltaN exact without a separate clearing pass).
-__device__ __forceinline__ bool skip_unaffected(const SweepArgs& a, int32_t v) {
-  if (a.dV[v]) return false;
-  if (a.wrote[v]) {
-    a.xn[v] = a.x[v];
+template <class P>
+__device__ __forceinline__ void skip_vertex(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int32_t v, bool wr,
+                                            bool dn) {
+  if (wr) {
+    c.xn[v] = as_real(ld_state(c.x + v, c.pl));
     a.wrote[v] = 0;
   }
-  if (a.dN[v]) a.dN[v] = 0;
-  return true;
+  if (dn) a.dN[v] = 0;
 }
 
-// The three flags of a vertex, read ahead of its turn: a vertex's flags change
-// during a sweep only in its own epilogue or skip, so a read issued earlier in
-// the sweep sees the values of the previous sweep, which is what the skip and
-// the epilogue need, and the loads leave the critical path.
-struct Flags {
-  uint8_t dv = 1, wr = 0, dn = 0;
+// The rows of one unit, [vb, ve) with at most 256 rows. Static: all of them.
+// DF / DF-P: the affected ones, compacted over the whole unit (the flags of
+// 256 rows are read at once, a bit mask per 32 rows is kept in the lanes), so
+// that a batch is 32 affected rows however thinly they are spread; the others
+// are copied through.
+template <class P, bool DYN>
+struct UnitRows {
+  int64_t vb;
+  int nact;
+  uint32_t mdv, mdn;  // lane i: affected / deltaN bits of rows vb + 32 i ..
+  int excl;           // lane i: affected rows before word i
+
+  __device__ __forceinline__ UnitRows(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb_, int64_t ve,
+                                      Tally& t)
+      : vb(vb_), mdv(0), mdn(0), excl(0) {
+    if (!DYN) {
+      nact = (int)(ve - vb);
+      return;
+    }
+    uint32_t mwr = 0;
+    uint8_t dv[kMaxWords], wr[kMaxWords], dn[kMaxWords];
+#pragma unroll
+    for (int i = 0; i < kMaxWords; ++i) {
+      const int64_t v = vb + 32 * i + c.lane;
+      const bool in = v < ve;
+      dv[i] = in ? a.dV[v] : (uint8_t)0;
+      wr[i] = in ? a.wrote[v] : (uint8_t)0;
+      dn[i] = in ? a.dN[v] : (uint8_t)0;
+    }
+#pragma unroll
+    for (int i = 0; i < kMaxWords; ++i) {
+      const uint32_t b0 = __ballot_sync(kFull, dv[i] != 0), b1 = __ballot_sync(kFull, wr[i] != 0),
+                     b2 = __ballot_sync(kFull, dn[i] != 0);
+      if (c.lane == i) {
+        mdv = b0;
+        mwr = b1;
+        mdn = b2;
+      }
+    }
+    // unaffected rows with something to undo
+    uint32_t todo = __ballot_sync(kFull, ((mwr | mdn) & ~mdv) != 0);
+    while (todo) {
+      const int i = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const uint32_t w = __shfl_sync(kFull, mwr & ~mdv, i), d = __shfl_sync(kFull, mdn & ~mdv, i);
+      const bool bw = (w >> c.lane) & 1u, bd = (d >> c.lane) & 1u;
+      if (bw || bd) skip_vertex(a, c, (int32_t)(vb + 32 * i + c.lane), bw, bd);
+    }
+    const int cnt = __popc(mdv);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < kMaxWords; o <<= 1) {
+      const int u = __shfl_up_sync(kFull, incl, o);
+      if (c.lane >= o) incl += u;
+    }
+    excl = incl - cnt;
+    nact = __shfl_sync(kFull, incl, kMaxWords - 1);
+    if (c.lane == 0) t.aff += (unsigned int)nact;
+  }
+
+  // the k-th row (0 <= k < nact; any k on lanes that hold no row) and its deltaN flag
+  __device__ __forceinline__ int32_t row(int k, bool& dn) const {
+    if (!DYN) {
+      dn = false;
+      return (int32_t)(vb + k);
+    }
+    int w = 0, before = 0;
+#pragma unroll
+    for (int i = 1; i < kMaxWords; ++i) {
+      const int e = __shfl_sync(kFull, excl, i);
+      if (e <= k) {
+        w = i;
+        before = e;
+      }
+    }
+    const uint32_t m = __shfl_sync(kFull, mdv, w);
+    const uint32_t d = __shfl_sync(kFull, mdn, w);
+    int r = k - before;  // the r-th set bit of m
+    int pos = 0;
+#pragma unroll
+    for (int half = 16; half > 0; half >>= 1) {
+      const int low = __popc((m >> pos) & ((1u << half) - 1u));
+      if (r >= low) {
+        r -= low;
+        pos += half;
+      }
+    }
+    dn = (d >> pos) & 1u;
+    return (int32_t)(vb + 32 * w + pos);
+  }
 };
-__device__ __forceinline__ Flags load_flags(const SweepArgs& a, int32_t v) {
-  Flags f;
-  f.dv = a.dV[v];
-  f.wr = a.wrote[v];
-  f.dn = a.dN[v];
-  return f;
-}
-// skip_unaffected with the flags read ahead
-__device__ __forceinline__ void skip_vertex(const SweepArgs& a, int32_t v, const Flags& f) {
-  if (f.wr) {
-    a.xn[v] = a.x[v];
-    a.wrote[v] = 0;
-  }
-  if (f.dn) a.dN[v] = 0;
+
+// One row per lane, its offsets known: the epilogue of a batch.
+template <class P, bool DYN>
+__device__ __forceinline__ void finish_batch(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, bool have,
+                                             int32_t v, typename P::Real sum, typename P::Real xself, bool dn,
+                                             Tally& t) {
+  bool front = false;
+  uint64_t deg = 0;
+  if (have) front = finish<DYN>(a, c, v, sum, xself, dn, t, deg);
+  if (DYN && a.expand) append_frontier(front, v, deg, &c.slot->nlist, a.list, c.lane);
 }
 
-__device__ __forceinline__ void block_max_to(uint64_t dmax, uint64_t* out) {
-  __shared__ uint64_t sh[32];
-  dmax = warp_max_u64(dmax);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = dmax;
-  __syncthreads();
-  if (wid == 0) {
-    uint64_t x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
-    x = warp_max_u64(x);
-    if (lane == 0 && x) atomicMax((unsigned long long*)out, (unsigned long long)x);
+// Sum of the gathered terms of one step into acc: one vote picks the
+// three-word add when every gathered term of the warp's step is in the common
+// window.
+template <class P, int U>
+__device__ __forceinline__ void add_terms(typename P::Acc& acc, const int32_t (&u)[U],
+                                          const typename P::Bits (&xv)[U]) {
+  bool w1 = true;
+#pragma unroll
+  for (int k = 0; k < U; ++k) w1 = w1 && (u[k] < 0 || P::Acc::in_w1(xv[k]));
+  if (__all_sync(kFull, w1)) {
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (u[k] >= 0) acc.add_w1(xv[k]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (u[k] >= 0) acc.add(xv[k]);
   }
 }
 
-// Sweep epilogue of a block: the L-inf change (max) and, for DF / DF-P, the
-// out-edges of the vertices put into deltaN (sum, when fw is given).
-template <bool DYN>
-__device__ __forceinline__ void block_epilogue(const SweepArgs& a, uint64_t dmax, uint64_t fwsum) {
-  block_max_to(dmax, a.resid);
-  if (DYN && a.fw) {
-    __shared__ uint64_t shs[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    fwsum = (uint64_t)warp_sum_i64((int64_t)fwsum);
-    __syncthreads();  // shs is written after every warp left block_max_to's shared reads
-    if (lane == 0) shs[wid] = fwsum;
-    __syncthreads();
-    if (wid == 0) {
-      uint64_t x = lane < (int)(blockDim.x >> 5) ? shs[lane] : 0;
-      x = (uint64_t)warp_sum_i64((int64_t)x);
-      if (lane == 0 && x) atomicAdd((unsigned long long*)a.fw, (unsigned long long)x);
+// Four entries of a row, positions j .. j + 3 (a multiple of four) of the
+// sequence at base (16-byte aligned), those outside [lo, hi) masked by -1.
+__device__ __forceinline__ int4 load4(const int32_t* base, int j, int hi, uint64_t pf) {
+  return j < hi ? ld_stream_i32x4(base + j, pf) : make_int4(-1, -1, -1, -1);
+}
+__device__ __forceinline__ void mask4(const int4& q, int j, int lo, int hi, int32_t (&u)[4]) {
+  u[0] = (j + 0 >= lo && j + 0 < hi) ? q.x : -1;
+  u[1] = (j + 1 >= lo && j + 1 < hi) ? q.y : -1;
+  u[2] = (j + 2 >= lo && j + 2 < hi) ? q.z : -1;
+  u[3] = (j + 3 >= lo && j + 3 < hi) ? q.w : -1;
+}
+
+// G lanes per row, a 16-byte index load each per step. The row's entries are
+// read from the 16-byte boundary below its first one (positions in a row are
+// 32-bit, counted from that boundary). While the gathers of one step are in
+// flight the indices of the next step load: the next chunk of the same rows,
+// or the first chunk of the groups' next rows, whose offsets are already in
+// the lanes, so a step waits for one round trip. The offsets of the next
+// batch load before the batch.
+template <class P, int G, bool DYN>
+__device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb,
+                                           int64_t ve, Tally& t) {
+  using Bits = typename P::Bits;
+  constexpr int NG = 32 / G;
+  const int lane = c.lane, sub = lane & (G - 1), src0 = lane & ~(G - 1);
+  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
+  const int nact = rows.nact;
+  if (nact == 0) return;
+
+  // lane's row of the batch at k0: group g takes rows g * S .. g * S + S - 1
+  struct Batch {
+    int32_t v;  // row, its deltaN flag in the sign bit
+    int len;
+    int64_t b;
+  };
+  auto steps = [&](int k0) { return ((nact - k0 < 32 ? nact - k0 : 32) + NG - 1) / NG; };
+  auto in_batch = [&](int k0) {
+    const int S = steps(k0);
+    return sub < S && (lane / G) * S + sub < (nact - k0 < 32 ? nact - k0 : 32);
+  };
+  auto load_batch = [&](int k0) {
+    Batch r;
+    const bool have = in_batch(k0);
+    bool dn;
+    const int32_t v = rows.row(have ? k0 + (lane / G) * steps(k0) + sub : 0, dn);
+    r.v = dn ? (v | INT32_MIN) : v;
+    r.b = 0;
+    r.len = 0;
+    if (have) {
+      r.b = ld_stream_i64(a.off + v, c.pf);
+      r.len = (int)(ld_stream_i64(a.off + v + 1, c.pf) - r.b);
     }
-  }
-}
+    return r;
+  };
 
-// Work item of a group: list entry, vertex, its row of G' and the first
-// G*U indices of the row (this lane's share), and (DF / DF-P) its flags.
-template <int U>
-struct Item {
-  int32_t v;
-  int64_t b, e;
-  int32_t u[U];
-  Flags f;
-  bool self_only;  // the row is [v] (in-degree <= 1 class, no in-edges added since the numbering)
-};
-
-// G lanes per vertex (G = 1, 4, 16), U indices per lane per round. The loop is
-// uniform across each warp (a warp owns 32/G consecutive list entries per
-// step), so the group shuffles always see all 32 lanes. Software pipeline:
-// the list entry of the item two steps ahead (and its affected flag) and the
-// offsets, first indices and other flags of the next item are loaded while
-// the current item's gathers are in flight, so a step costs about one memory
-// round trip instead of four. With self-loops on every vertex, a row of length 1 is [v] itself and needs
-// no offsets or indices.
-template <int G, int U, bool EXACT, bool DYN, bool SELF1>
-__global__ void __launch_bounds__(kThreads, U >= 8 ? 3 : kMinBlocks) k_sweep_group(const SweepArgs a_in, int64_t begin,
-                                                                                  int64_t end) {
-  const SweepArgs a = resolve(a_in);
-  if (a.prev && bitsd(*a.prev) <= a.tol) return;
-  const uint64_t pf = policy_evict_first(), pl = policy_evict_last();
-  constexpr int kGroupsPerWarp = 32 / G;
-  const int lane = (G == 1) ? 0 : (threadIdx.x & (G - 1));
-  const int gw = (threadIdx.x & 31) / G;  // group within warp
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int64_t step = nwarps * kGroupsPerWarp;
-  uint64_t dmax = 0, fwsum = 0;
-
-  auto load_v = [&](int64_t i) -> int32_t { return i < end ? (int32_t)i : -1; };
-  auto load_dv = [&](int32_t v) -> uint8_t { return (DYN && v >= 0) ? a.dV[v] : (uint8_t)1; };
-  // DF / DF-P: the row of an unaffected vertex is not read
-  auto load_item = [&](int32_t v, uint8_t dv, Item<U>& it) {
-    it.v = v;
-    it.b = 0;
-    it.e = 0;
-    it.f = Flags();
-    if (DYN && v >= 0) {
-      it.f.dv = dv;
-      it.f.wr = a.wrote[v];
-      it.f.dn = a.dN[v];
-    }
-    const bool live = v >= 0 && dv;
-    // the row is [v] unless a batch gave the vertex in-edges (its bit in multi)
-    const bool self_only = SELF1 && !(live && a.multi && ((a.multi[v >> 5] >> (v & 31)) & 1u));
-    it.self_only = self_only;
-    if (live) {
-      if (self_only) {
-        it.b = 0;
-        it.e = 1;
+  Batch cur = load_batch(0);
+  for (int k0 = 0; k0 < nact; k0 += 32) {
+    Batch nxt = cur;
+    if (k0 + 32 < nact) nxt = load_batch(k0 + 32);
+    const int S = steps(k0);
+    typename P::Acc saved, acc;
+    bool hit = false, myhit = false;
+    // the group's row: entries [lo, hi) from base; this lane's position j
+    int64_t rb = __shfl_sync(kFull, cur.b, src0);
+    int lo = (int)(rb & 3), hi = lo + __shfl_sync(kFull, cur.len, src0), j = 4 * sub;
+    const int32_t* base = a.adj + (rb & ~(int64_t)3);
+    int4 q = load4(base, j, hi, c.pf);
+    for (int s = 0; s < S;) {
+      int32_t u[4];
+      mask4(q, j, lo, hi, u);
+      Bits xv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
+      // the next step's indices
+      const bool more = __any_sync(kFull, j - 4 * sub + 4 * G < hi);
+      if (more) {
+        j += 4 * G;
+        lo = 0;
       } else {
-        it.b = ld_stream_i64(a.off + v, pf);
-        it.e = ld_stream_i64(a.off + v + 1, pf);
+        const int src = src0 + s + 1;  // (past the last row: any lane, no entries)
+        rb = __shfl_sync(kFull, cur.b, src & 31);
+        const int len = __shfl_sync(kFull, cur.len, src & 31);
+        lo = (int)(rb & 3);
+        hi = s + 1 < S ? lo + len : 0;
+        j = 4 * sub;
+        base = a.adj + (rb & ~(int64_t)3);
+      }
+      q = load4(base, j, hi, c.pf);
+      if (G < 32 && !a.self_loops) {
+        const int32_t rv = __shfl_sync(kFull, cur.v, src0 + s) & INT32_MAX;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) myhit = myhit || u[k] == rv;
+      }
+      add_terms<P>(acc, u, xv);
+      if (!more) {
+        acc.template group_reduce<G>();
+        if (sub == s) saved = acc;
+        acc = typename P::Acc();
+        if (G < 32 && !a.self_loops) {
+          // graphs without self-loops on every vertex: x[v] counts only when the row holds v
+          const uint32_t m = __ballot_sync(kFull, myhit) >> src0;
+          if (sub == s) hit = (m & ((1u << (G & 31)) - 1u)) != 0;
+          myhit = false;
+        }
+        ++s;
       }
     }
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t j = it.b + lane + (int64_t)k * G;
-      if (self_only) it.u[k] = (live && k == 0 && lane == 0) ? v : -1;
-      else it.u[k] = (live && j < it.e) ? ld_stream_i32(a.adj + j, pf) : -1;
-    }
-  };
-
-  // The row offsets run one more step ahead (offsets of the item two steps
-  // ahead, indices of the next), so a step waits for one round trip. In DF /
-  // DF-P the affected flag runs three steps ahead, so that offsets and indices
-  // are loaded only for affected vertices.
-  constexpr bool kOffAhead = !DYN && !SELF1;
-  constexpr bool kDynAhead = DYN && !SELF1;
-  auto load_off = [&](int32_t v, int64_t& b, int64_t& e) {
-    b = v >= 0 ? ld_stream_i64(a.off + v, pf) : 0;
-    e = v >= 0 ? ld_stream_i64(a.off + v + 1, pf) : 0;
-  };
-  auto load_idx = [&](int32_t v, int64_t b, int64_t e, Item<U>& it) {
-    it.v = v;
-    it.b = b;
-    it.e = e;
-    it.f = Flags();
-    it.self_only = false;
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t j = b + lane + (int64_t)k * G;
-      it.u[k] = (v >= 0 && j < e) ? ld_stream_i32(a.adj + j, pf) : -1;
-    }
-  };
-
-  int64_t base = begin + warp * kGroupsPerWarp;
-  Item<U> cur;
-  {
-    const int32_t v0 = load_v(base + gw);
-    load_item(v0, load_dv(v0), cur);
-  }
-  int32_t v_next = load_v(base + step + gw);
-  uint8_t dv_next = load_dv(v_next);
-  int64_t nb = 0, ne = 0;  // kOffAhead, kDynAhead: row offsets of v_next (when affected)
-  if (kOffAhead) load_off(v_next, nb, ne);
-  int32_t v_n2 = -1;  // kDynAhead: the list entry two steps ahead and its affected flag
-  uint8_t dv_n2 = 0;
-  if (kDynAhead) {
-    load_off((v_next >= 0 && dv_next) ? v_next : -1, nb, ne);
-    v_n2 = load_v(base + 2 * step + gw);
-    dv_n2 = load_dv(v_n2);
-  }
-  for (; base < end; base += step) {
-    // gathers of the current item
-    uint64_t xv[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) xv[k] = cur.u[k] >= 0 ? ld_gather_b64(a.x + cur.u[k], pl) : 0ull;
-    // prefetch: next item's row, first indices and flags, and the list entry (and flag) after it
-    Item<U> nxt;
-    if (kOffAhead) {
-      load_idx(v_next, nb, ne, nxt);
-      v_next = load_v(base + 2 * step + gw);
-      load_off(v_next, nb, ne);
-    } else if (kDynAhead) {
-      const bool live = v_next >= 0 && dv_next;
-      load_idx(live ? v_next : -1, nb, ne, nxt);
-      nxt.v = v_next;
-      if (v_next >= 0) {
-        nxt.f.dv = dv_next;
-        nxt.f.wr = a.wrote[v_next];
-        nxt.f.dn = a.dN[v_next];
-      }
-      v_next = v_n2;
-      dv_next = dv_n2;
-      load_off((v_next >= 0 && dv_next) ? v_next : -1, nb, ne);
-      v_n2 = load_v(base + 3 * step + gw);
-      dv_n2 = load_dv(v_n2);
-    } else {
-      load_item(v_next, dv_next, nxt);
-      v_next = load_v(base + 2 * step + gw);
-      dv_next = load_dv(v_next);
-    }
-
-    // the warp is converged here (uniform loop): one vote picks the
-    // three-word add when every gathered term of the step is in the common window
-    bool w1 = true;
-#pragma unroll
-    for (int k = 0; k < U; ++k) w1 = w1 && (cur.u[k] < 0 || Acc<EXACT>::in_w1(xv[k]));
-    const bool all_w1 = __all_sync(0xffffffffu, w1);
-    bool active = cur.v >= 0;
-    if (DYN && active && !cur.f.dv) {
-      if (lane == 0) skip_vertex(a, cur.v, cur.f);
-      active = false;
-    }
-    if (SELF1 && cur.self_only) {
-      // row [v] (one lane per item): the in-neighbour sum is the single term x[v], exactly
-      if (active) {
-        const uint64_t db = finish_vertex<DYN>(a, cur.v, bitsd(xv[0]), xv[0], pf, fwsum, cur.f.dn);
-        dmax = db > dmax ? db : dmax;
-      }
-      cur = nxt;
-      continue;
-    }
-    // DF / DF-P: a step in which no item of the warp is affected (most steps of
-    // the first sweeps after a small batch) has nothing to reduce. (Every lane
-    // reaches the vote: only the SELF1 form leaves the step early, per lane.)
-    if (DYN && !SELF1 && !__any_sync(0xffffffffu, active)) {
-      cur = nxt;
-      continue;
-    }
-    Acc<EXACT> acc;
-    uint64_t xself = 0;
-    if (active) {
-      if (all_w1) {
-#pragma unroll
-        for (int k = 0; k < U; ++k)
-          if (cur.u[k] >= 0) acc.add_w1(xv[k]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < U; ++k)
-          if (cur.u[k] >= 0) acc.add(xv[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < U; ++k) xself = (cur.u[k] == cur.v) ? xv[k] : xself;
-      // rest of a row longer than G*U (rows that grew past their class's bound in a batch update)
-      if (cur.e - cur.b > (int64_t)G * U)
-        gather_row<G, U, EXACT>(a, cur.b + (int64_t)G * U, cur.e, lane, cur.v, acc, xself, pf, pl);
-    }
-    if (G > 1) {
-      acc.template group_reduce<G>();
-#pragma unroll
-      for (int o = G / 2; o > 0; o >>= 1) {
-        const uint64_t t = __shfl_xor_sync(0xffffffffu, xself, o);
-        xself = t > xself ? t : xself;
-      }
-    }
-    if (active && lane == 0) {
-      const uint64_t db = finish_vertex<DYN>(a, cur.v, acc.value(), xself, pf, fwsum, cur.f.dn);
-      dmax = db > dmax ? db : dmax;
-    }
+    const bool have = in_batch(k0);
+    const int32_t v = cur.v & INT32_MAX;
+    const Bits xs = have && (G == 32 || a.self_loops || hit) ? ld_state(c.x + v, c.pl) : Bits(0);
+    finish_batch<P, DYN>(a, c, have, v, saved.value(), as_real(xs), cur.v < 0, t);
     cur = nxt;
   }
-  block_epilogue<DYN>(a, dmax, fwsum);
 }
 
-// one warp per vertex, 16-byte index loads; the next vertex's list entry, row
-// offsets and (DF / DF-P) flags are loaded while the current row is gathered
-template <int KV, bool EXACT, bool DYN>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep_warp(const SweepArgs a_in, int64_t begin, int64_t end) {
-  const SweepArgs a = resolve(a_in);
-  if (a.prev && bitsd(*a.prev) <= a.tol) return;
-  const uint64_t pf = policy_evict_first(), pl = policy_evict_last();
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  uint64_t dmax = 0, fwsum = 0;
-  int64_t i = begin + warp;
-  int32_t v = i < end ? (int32_t)i : -1;
-  int64_t b = v >= 0 ? ld_stream_i64(a.off + v, pf) : 0, e = v >= 0 ? ld_stream_i64(a.off + v + 1, pf) : 0;
-  Flags f;
-  if (DYN && v >= 0) f = load_flags(a, v);
-  for (; i < end; i += nwarps) {
-    const int64_t inx = i + nwarps;
-    const int32_t vn = inx < end ? (int32_t)inx : -1;
-    bool active = true;
-    if (DYN && !f.dv) {
-      if (lane == 0) skip_vertex(a, v, f);
-      active = false;
+// One row per lane, U indices in flight (short rows).
+template <class P, int U, bool DYN>
+__device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb, int64_t ve,
+                                         Tally& t) {
+  using Bits = typename P::Bits;
+  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
+  const int nact = rows.nact;
+  if (nact == 0) return;
+  struct Row {
+    int32_t v;
+    int len;
+    int64_t b;
+    bool have, dn;
+  };
+  auto load_row = [&](int k0) {
+    Row r;
+    r.have = k0 + c.lane < nact;
+    r.v = rows.row(r.have ? k0 + c.lane : 0, r.dn);
+    r.b = 0;
+    r.len = 0;
+    if (r.have) {
+      r.b = ld_stream_i64(a.off + r.v, c.pf);
+      r.len = (int)(ld_stream_i64(a.off + r.v + 1, c.pf) - r.b);
     }
-    Acc<EXACT> acc;
-    // x[v], for R[v] of the previous iteration = x[v] * |out(v)|, issued ahead of the gathers
-    uint64_t xself = (active && lane == 0) ? ld_gather_b64(a.x + v, pl) : 0ull;
-    if (active) gather_row_vec<32, KV, EXACT, false>(a, b, e, lane, v, acc, xself, pf, pl);
-    const int64_t bn = vn >= 0 ? ld_stream_i64(a.off + vn, pf) : 0, en = vn >= 0 ? ld_stream_i64(a.off + vn + 1, pf) : 0;
-    Flags fn;
-    if (DYN && vn >= 0) fn = load_flags(a, vn);
-    if (active) acc.template group_reduce<32>();  // active is the same on every lane (one row per warp)
-    if (active && lane == 0) {
-      const uint64_t db = finish_vertex<DYN>(a, v, acc.value(), xself, pf, fwsum, f.dn);
-      dmax = db > dmax ? db : dmax;
+    return r;
+  };
+  auto load_idx = [&](const Row& r, int32_t (&u)[U]) {
+#pragma unroll
+    for (int k = 0; k < U; ++k) u[k] = k < r.len ? ld_stream_i32(a.adj + r.b + k, c.pf) : -1;
+  };
+  // offsets two batches ahead, indices one ahead
+  Row cur = load_row(0), nxt;
+  int32_t u[U];
+  load_idx(cur, u);
+  nxt.have = false;
+  nxt.len = 0;
+  nxt.b = 0;
+  nxt.v = 0;
+  nxt.dn = false;
+  if (32 < nact) nxt = load_row(32);
+  for (int k0 = 0; k0 < nact; k0 += 32) {
+    Bits xv[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
+    const Bits xs = cur.have ? ld_state(c.x + cur.v, c.pl) : Bits(0);
+    int32_t un[U];
+    load_idx(nxt, un);
+    Row far = nxt;
+    far.have = false;
+    far.len = 0;
+    if (k0 + 64 < nact) far = load_row(k0 + 64);
+    typename P::Acc acc;
+    bool hit = false;
+#pragma unroll
+    for (int k = 0; k < U; ++k) hit = hit || u[k] == cur.v;
+    add_terms<P>(acc, u, xv);
+    // rest of a row longer than U (rows that grew past their class's bound in a batch update)
+    for (int j = U; j < cur.len; ++j) {
+      const int32_t w = ld_stream_i32(a.adj + cur.b + j, c.pf);
+      acc.add(ld_state(c.x + w, c.pl));
+      hit = hit || w == cur.v;
     }
-    v = vn;
-    b = bn;
-    e = en;
-    f = fn;
+    const Bits xself = (a.self_loops || hit) ? xs : Bits(0);
+    finish_batch<P, DYN>(a, c, cur.have, cur.v, acc.value(), as_real(xself), cur.dn, t);
+    cur = nxt;
+    nxt = far;
+#pragma unroll
+    for (int k = 0; k < U; ++k) u[k] = un[k];
   }
-  block_epilogue<DYN>(a, dmax, fwsum);
 }
 
-// one block per vertex (high in-degree)
-template <int KV, bool EXACT, bool DYN>
-__global__ void __launch_bounds__(kThreads, 3) k_sweep_block(const SweepArgs a_in, int64_t begin, int64_t end) {
-  const SweepArgs a = resolve(a_in);
-  if (a.prev && bitsd(*a.prev) <= a.tol) return;
-  const uint64_t pf = policy_evict_first(), pl = policy_evict_last();
-  __shared__ uint32_t s_acc[kThreads / 32][4];
-  __shared__ int s_skip;
-  uint64_t dmax = 0, fwsum = 0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t i = begin + blockIdx.x; i < end; i += gridDim.x) {
-    const int32_t v = (int32_t)i;
-    if (DYN) {
-      if (threadIdx.x == 0) s_skip = skip_unaffected(a, v) ? 1 : 0;
-      __syncthreads();
-      const int sk = s_skip;
-      __syncthreads();
-      if (sk) continue;
+// The class of in-degree <= 1 on a graph with all self-loops: the row is [v],
+// so the in-neighbour sum is the single term x[v], exactly, and no offsets or
+// indices are read (a vertex that gained in-edges in a batch update has its
+// bit in multi and reads its row).
+template <class P, bool DYN>
+__device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb, int64_t ve,
+                                       Tally& t) {
+  using Bits = typename P::Bits;
+  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
+  const int nact = rows.nact;
+  for (int k0 = 0; k0 < nact; k0 += 32) {
+    const bool have = k0 + c.lane < nact;
+    bool dn;
+    const int32_t v = rows.row(have ? k0 + c.lane : 0, dn);
+    const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
+    typename P::Real sum = as_real(xs);
+    if (a.multi && have && ((a.multi[v >> 5] >> (v & 31)) & 1u)) {
+      typename P::Acc acc;
+      const int64_t e = a.off[v + 1];
+      for (int64_t j = a.off[v]; j < e; ++j) acc.add(ld_state(c.x + a.adj[j], c.pl));
+      sum = acc.value();
     }
-    const int64_t b = a.off[v], e = a.off[v + 1];
-    Acc<EXACT> acc;
-    // x[v] for R[v] of the previous iteration, read by the thread that finishes the vertex
-    uint64_t xb = (threadIdx.x == 0) ? ld_gather_b64(a.x + v, pl) : 0ull;
-    gather_row_vec<kThreads, KV, EXACT, false>(a, b, e, threadIdx.x, v, acc, xb, pf, pl);
+    finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), dn, t);
+  }
+}
+
+// One 1024-edge chunk of a row of the highest in-degree class. The warp that
+// finishes the last chunk of a row adds the row's partial sums and finishes
+// the vertex. With exact accumulation the partials are integers, so the
+// result is the same bits as any other split; the compensated FP32 partials
+// are added in chunk order by lanes and a fixed shuffle tree, so every run
+// gives the same bits. A hub's flags change only in its finishing warp, which
+// runs after every chunk's warp has read them, or (unaffected hubs) in the
+// warp of its first chunk, which leaves dV alone.
+template <class P, bool DYN>
+__device__ __forceinline__ void unit_hub(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t ch, Tally& t) {
+  using Bits = typename P::Bits;
+  const int lane = c.lane;
+  const int64_t h = a.hub.chunk_hub[ch];
+  const int32_t v = (int32_t)(a.hub.begin + h);
+  const int64_t jb = a.hub.chunk_j0[ch];
+  const int64_t first = a.hub.hub_first[h], last = a.hub.hub_first[h + 1];
+  if (DYN) {
+    const bool skip = __shfl_sync(kFull, lane == 0 ? (int)(a.dV[v] == 0) : 0, 0) != 0;
+    if (skip) {
+      if (ch == first && lane == 0) skip_vertex(a, c, v, a.wrote[v] != 0, a.dN[v] != 0);
+      return;
+    }
+    if (ch == first && lane == 0) t.aff += 1;
+  }
+  const int64_t row_e = a.off[v + 1];
+  const int64_t je = jb + kHubChunk < row_e ? jb + kHubChunk : row_e;
+  typename P::Acc acc;
+  const int lo0 = (int)(jb & 3), hi = lo0 + (int)(je - jb);
+  const int32_t* base = a.adj + (jb & ~(int64_t)3);
+  int4 q = load4(base, 4 * lane, hi, c.pf);
+  for (int j = 4 * lane; j - 4 * lane < hi; j += 128) {
+    int32_t u[4];
+    mask4(q, j, lo0, hi, u);
+    Bits xv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
+    q = load4(base, j + 128, hi, c.pf);
+    add_terms<P>(acc, u, xv);
+  }
+  acc.template group_reduce<32>();
+  unsigned int done = 0;
+  if (last - first > 1) {
+    if (lane == 0) {
+      __stcg(a.hub_part + ch, acc.pack());
+      __threadfence();
+      done = atomicAdd(a.hub_done + h, 1u) + 1;
+    }
+    done = __shfl_sync(kFull, done, 0);
+    if (done != (unsigned int)(last - first)) return;
+    if (lane == 0) a.hub_done[h] = 0;
+    __threadfence();
+    acc = typename P::Acc();
+    for (int64_t k = first + lane; k < last; k += 32) acc.merge(__ldcg(a.hub_part + k));
     acc.template group_reduce<32>();
-    if (lane == 0) acc.to_shared(s_acc[wid]);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      Acc<EXACT> tot;
-      for (int k = 0; k < kThreads / 32; ++k) tot.from_shared(s_acc[k]);
-      const uint64_t db = finish_vertex<DYN>(a, v, tot.value(), xb, pf, fwsum, DYN ? a.dN[v] : (uint8_t)0);
-      dmax = db > dmax ? db : dmax;
+  }
+  const bool have = lane == 0;
+  const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
+  finish_batch<P, DYN>(a, c, have, v, acc.value(), as_real(xs), DYN && have && a.dN[v] != 0, t);
+}
+
+// -------------------------------------------------------------- phases ----
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Barrier over the whole (co-resident) grid: every block adds one arrival and
+// waits until all of this barrier's are in. The wait is bounded: past the
+// limit (minutes; no sweep takes that long) the block flags the loop as timed
+// out and gives up, and so does every other block when it sees the flag.
+// Returns false after a timeout.
+constexpr unsigned long long kSpinLimit = 1ull << 28;
+
+__device__ bool grid_barrier(LoopCtl* ctl, unsigned long long& target) {
+  __shared__ int s_ok;
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&ctl->bar, 1ull);
+    int ok = 1;
+    unsigned long long spins = 0;
+    while (ld_acquire(&ctl->bar) < target) {
+      if (++spins > kSpinLimit || ((spins & 1023) == 0 && *(volatile int*)&ctl->timeout)) {
+        *(volatile int*)&ctl->timeout = 1;
+        ok = 0;
+        break;
+      }
+      if (spins > 256) __nanosleep(100);
     }
-    __syncthreads();
+    __threadfence();
+    s_ok = ok;
   }
-  block_epilogue<DYN>(a, dmax, fwsum);
+  __syncthreads();
+  return s_ok != 0;
 }
 
-// Rows of the highest in-degree class in 1024-edge chunks (the hub chunk
-// table). A warp per chunk sums the chunk's terms and stores the partial sum;
-// a warp per hub vertex adds its chunks' partials and finishes the vertex.
-// With exact accumulation the partials are integers, so the result is the
-// same bits as any other split; long rows no longer serialise on one block.
-// DF / DF-P: chunks of unaffected hubs are skipped; the finishing warp copies
-// an unaffected hub through. A hub's flag changes only in its finishing warp,
-// which runs after every chunk of the sweep has read it.
-template <bool EXACT, bool DYN>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep_hub_part(const SweepArgs a_in) {
-  const SweepArgs a = resolve(a_in);
-  if (a.prev && bitsd(*a.prev) <= a.tol) return;
-  const uint64_t pf = policy_evict_first(), pl = policy_evict_last();
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  for (int64_t c = warp; c < a.hub.nchunk; c += nwarps) {
-    const int32_t v = (int32_t)(a.hub.begin + a.hub.chunk_hub[c]);
-    if (DYN && !a.dV[v]) continue;  // the same flag on every lane
-    const int64_t jb = a.hub.chunk_j0[c];
-    const int64_t re = a.off[v + 1];
-    const int64_t je = jb + kHubChunk < re ? jb + kHubChunk : re;
-    Acc<EXACT> acc;
-    uint64_t unused = 0;
-    gather_row_vec<32, 2, EXACT, false>(a, jb, je, lane, v, acc, unused, pf, pl);
-    acc.template group_reduce<32>();
-    if (lane == 0) acc.to_shared(reinterpret_cast<uint32_t*>(a.hub_part + c));
-  }
+// the slot of sweep it: a ring of kLoopRing in the whole-loop kernel, one a
+// sweep from it_first on in the host-driven loop (slot 0: the sweep before)
+template <class Real>
+__device__ __forceinline__ LoopSlot* slot_of(const SweepArgs<Real>& a, int it) {
+  return a.slot + (a.mode == kLoopAll ? (it & (kLoopRing - 1)) : it - a.it_first + 1);
 }
 
-template <bool EXACT, bool DYN>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep_hub_finish(const SweepArgs a_in) {
-  const SweepArgs a = resolve(a_in);
-  if (a.prev && bitsd(*a.prev) <= a.tol) return;
-  const uint64_t pf = policy_evict_first(), pl = policy_evict_last();
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  uint64_t dmax = 0, fwsum = 0;
-  // a warp per hub vertex: lanes add strided chunk partials, then the warp reduces
-  for (int64_t h = warp; h < a.hub.nhub; h += nwarps) {
-    const int32_t v = (int32_t)(a.hub.begin + h);
-    if (DYN) {
-      // every lane reads the flag before lane 0 may change it
-      const bool skip = __shfl_sync(0xffffffffu, lane == 0 ? (int)(a.dV[v] == 0) : 0, 0) != 0;
-      if (skip) {
-        if (lane == 0) skip_unaffected(a, v);
-        continue;
+template <class P, bool DYN>
+__device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int it) {
+  Ctx<P> c;
+  c.x = (it & 1) ? a.xb : a.xa;
+  c.xn = (it & 1) ? a.xa : a.xb;
+  c.slot = slot_of(a, it);
+  c.pf = policy_evict_first();
+  c.pl = policy_evict_last();
+  c.lane = threadIdx.x & 31;
+  Tally t;
+  // first unit by position (consecutive units on different SMs), the rest from the counter
+  const unsigned int nw = gridDim.x * kWarps;
+  unsigned int u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  while (u < a.units) {
+    unsigned int nx = 0;
+    if (c.lane == 0) nx = atomicAdd(&c.slot->units, 1u);
+    if (u < (unsigned int)a.hub.nchunk) {
+      unit_hub<P, DYN>(a, c, u, t);
+    } else {
+      int k = 0;
+      while (k + 1 < a.ncls && u >= a.cls[k + 1].unit0) ++k;
+      const SweepClass& cl = a.cls[k];
+      const int64_t vb = cl.begin + (int64_t)(u - cl.unit0) * cl.rows;
+      const int64_t ve = vb + cl.rows < cl.end ? vb + cl.rows : cl.end;
+      switch (cl.kind) {
+        case kRowSelf: unit_self<P, DYN>(a, c, vb, ve, t); break;
+        case kRowThread: unit_thread<P, 4, DYN>(a, c, vb, ve, t); break;
+        case kRow4: unit_group<P, 4, DYN>(a, c, vb, ve, t); break;
+        case kRow8: unit_group<P, 8, DYN>(a, c, vb, ve, t); break;
+        case kRow16: unit_group<P, 16, DYN>(a, c, vb, ve, t); break;
+        default: unit_group<P, 32, DYN>(a, c, vb, ve, t); break;
       }
     }
-    Acc<EXACT> tot;
-    for (int64_t c = a.hub.hub_first[h] + lane; c < a.hub.hub_first[h + 1]; c += 32)
-      tot.from_shared(reinterpret_cast<const uint32_t*>(a.hub_part + c));
-    tot.template group_reduce<32>();
-    if (lane == 0) {
-      const uint64_t db =
-          finish_vertex<DYN>(a, v, tot.value(), ld_gather_b64(a.x + v, pl), pf, fwsum, DYN ? a.dN[v] : (uint8_t)0);
-      dmax = db > dmax ? db : dmax;
-    }
+    u = nw + __shfl_sync(kFull, nx, 0);
   }
-  block_epilogue<DYN>(a, dmax, fwsum);
+  // block maxima and sums
+  __shared__ unsigned long long s_max, s_fw;
+  __shared__ unsigned int s_r, s_aff;
+  if (threadIdx.x == 0) {
+    s_max = 0;
+    s_fw = 0;
+    s_r = 0;
+    s_aff = 0;
+  }
+  __syncthreads();
+  const uint64_t dm = warp_max_u64(t.dmax);
+  if (c.lane == 0 && dm) atomicMax(&s_max, (unsigned long long)dm);
+  if (sizeof(typename P::Real) == 4) {
+    const uint32_t rm = __reduce_max_sync(kFull, t.rmax);
+    if (c.lane == 0 && rm) atomicMax(&s_r, rm);
+  }
+  if (DYN) {
+    const uint64_t f = (uint64_t)warp_sum_i64((int64_t)t.fw);
+    if (c.lane == 0 && f) atomicAdd(&s_fw, (unsigned long long)f);
+    if (c.lane == 0 && t.aff) atomicAdd(&s_aff, t.aff);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sizeof(typename P::Real) == 8) {
+      if (s_max) atomicMax(&c.slot->resid, s_max);
+    } else {
+      uint32_t* r = reinterpret_cast<uint32_t*>(&c.slot->resid);
+      if (s_max) atomicMax(r, (uint32_t)s_max);
+      if (s_r) atomicMax(r + 1, s_r);
+    }
+    if (DYN && s_fw) atomicAdd(&c.slot->fw, s_fw);
+    if (DYN && it == 0 && s_aff) atomicAdd(&a.ctl->aff0, s_aff);
+  }
 }
 
-// Kernel shape of class c: the last class is block-per-vertex, the one before
-// it warp-per-vertex; lower classes by their upper degree bound.
-enum Kind { kT1 = 0, kT4, kG4, kG8, kG16, kG16U8, kWarp, kBlock };
-
-Kind class_kind(const PartThr& t, int c) {
-  const int C = t.n + 1;
-  if (c == C - 1) return kBlock;
-  if (c == C - 2 && C >= 3) return kWarp;
-  const int64_t hi = t.thr[c];
-  if (hi <= 1) return kT1;
-  if (hi <= 4) return kT4;
-  if (hi <= 16) return kG4;
-  if (hi <= 32) return kG8;
-  // 16 lanes; 8 indices per lane only when every row of the class is longer than 64
-  if (hi <= 128) return (c > 0 && t.thr[c - 1] >= 64) ? kG16U8 : kG16;
-  return kWarp;
+// stop rule on a sweep's residual word: FP64, L-inf change <= tol; FP32, max|dR| <= tol * max R
+__device__ __forceinline__ bool stopped(unsigned long long resid, double tol) { return bitsd(resid) <= tol; }
+__device__ __forceinline__ bool stopped(unsigned long long resid, float tol) {
+  return __uint_as_float((uint32_t)resid) <= tol * __uint_as_float((uint32_t)(resid >> 32));
 }
 
-// The sweep kernels use almost no shared memory: give the unified L1 /
-// shared storage to L1, which holds the gathered x of the hottest sources.
-template <typename K>
-void prefer_l1(K k) {
-  // a preference the driver declines is not an error: clear what this call set
-  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 0) != cudaSuccess) cudaGetLastError();
-}
-
-template <bool EXACT, bool DYN>
-bool prefer_l1_all() {
-  prefer_l1(k_sweep_group<1, 1, EXACT, DYN, true>);
-  prefer_l1(k_sweep_group<1, 1, EXACT, DYN, false>);
-  prefer_l1(k_sweep_group<1, 4, EXACT, DYN, false>);
-  prefer_l1(k_sweep_group<4, 4, EXACT, DYN, false>);
-  prefer_l1(k_sweep_group<8, 4, EXACT, DYN, false>);
-  prefer_l1(k_sweep_group<16, 4, EXACT, DYN, false>);
-  prefer_l1(k_sweep_group<16, 8, EXACT, DYN, false>);
-  prefer_l1(k_sweep_warp<2, EXACT, DYN>);
-  prefer_l1(k_sweep_block<4, EXACT, DYN>);
-  prefer_l1(k_sweep_hub_part<EXACT, DYN>);
-  return true;
-}
-
-template <bool EXACT, bool DYN>
-int launch_all(const SweepArgs& a, const PartThr& t, const int64_t* cb, cudaStream_t s) {
-  static const bool carveout_set = prefer_l1_all<EXACT, DYN>();
-  (void)carveout_set;
-  const int maxg = kSMs * 8;
-  const int C = t.n + 1;
-  for (int c = 0; c < C; ++c) {
-    const int64_t b = cb[c], e = cb[c + 1];
-    if (e <= b) continue;
-    const int64_t cnt = e - b;
-    const Kind kind = class_kind(t, c);
-    // a class holding only rows of length <= 1 on a graph with all self-loops: the row is [v]
-    const bool self1 = a.self_loops && kind == kT1 && t.thr[c] <= 1;
-    switch (kind) {
-      case kT1:
-        if (self1) k_sweep_group<1, 1, EXACT, DYN, true><<<grid_for(cnt, kThreads, maxg), kThreads, 0, s>>>(a, b, e);
-        else k_sweep_group<1, 1, EXACT, DYN, false><<<grid_for(cnt, kThreads, maxg), kThreads, 0, s>>>(a, b, e);
-        break;
-      case kT4: k_sweep_group<1, 4, EXACT, DYN, false><<<grid_for(cnt, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      case kG4: k_sweep_group<4, 4, EXACT, DYN, false><<<grid_for(cnt * 4, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      case kG8: k_sweep_group<8, 4, EXACT, DYN, false><<<grid_for(cnt * 8, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      case kG16: k_sweep_group<16, 4, EXACT, DYN, false><<<grid_for(cnt * 16, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      case kG16U8: k_sweep_group<16, 8, EXACT, DYN, false><<<grid_for(cnt * 16, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      case kWarp: k_sweep_warp<2, EXACT, DYN><<<grid_for(cnt * 32, kThreads, maxg), kThreads, 0, s>>>(a, b, e); break;
-      default:
-        if (a.hub.nchunk > 0 && a.hub.begin == b && a.hub.nhub == cnt && a.hub_part) {
-          k_sweep_hub_part<EXACT, DYN><<<grid_for(a.hub.nchunk * 32, kThreads, maxg), kThreads, 0, s>>>(a);
-          k_sweep_hub_finish<EXACT, DYN><<<grid_for(cnt * 32, kThreads, maxg), kThreads, 0, s>>>(a);
-        } else {
-          k_sweep_block<4, EXACT, DYN><<<grid_for(cnt, 1, maxg), kThreads, 0, s>>>(a, b, e);
+// Push form of an expansion round from the frontier list the sweep (or the
+// initial marking) left: dV[w] = 1 for every out-neighbour w. A warp takes up
+// to 32 entries and walks their edges as one sequence, so short rows share a
+// step; a long row is several entries (kFrontChunk edges each) on different
+// warps. A flag already set is not stored again.
+template <class Real>
+__device__ void push_round(const SweepArgs<Real>& a, const unsigned int* count) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int total = __ldcg(count);
+  const unsigned int nw = gridDim.x * kWarps;
+  const unsigned int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const unsigned int per = (total + nw - 1) / nw;
+  const unsigned int epw = per < 1 ? 1 : (per > 32 ? 32 : per);
+  for (unsigned int base = w * epw; base < total; base += nw * epw) {
+    int64_t b = 0;
+    unsigned int len = 0;
+    if ((unsigned int)lane < epw && base + lane < total) {
+      const int2 en = __ldcg(a.list + base + lane);
+      const int64_t rb = a.ooff[en.x] + (int64_t)en.y * kFrontChunk, re = a.ooff[en.x + 1];
+      b = rb;
+      len = (unsigned int)(re - rb < kFrontChunk ? re - rb : kFrontChunk);
+    }
+    unsigned int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int x = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += x;
+    }
+    const unsigned int excl = incl - len;
+    const unsigned int edges = __shfl_sync(kFull, incl, 31);
+    constexpr int kU = 4;
+    for (unsigned int e0 = 0; e0 < edges; e0 += 32 * kU) {
+      int32_t t[kU];
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        const unsigned int e = e0 + 32 * k + lane;
+        int lo = 0;  // the last entry that starts at or before e
+#pragma unroll
+        for (int half = 16; half > 0; half >>= 1) {
+          const unsigned int s = __shfl_sync(kFull, excl, lo + half);
+          if (s <= e) lo += half;
         }
-        break;
+        const int64_t rb = __shfl_sync(kFull, b, lo);
+        const unsigned int st = __shfl_sync(kFull, excl, lo);
+        t[k] = e < edges ? __ldg(a.oadj + rb + (e - st)) : -1;
+      }
+      uint8_t f[kU];
+#pragma unroll
+      for (int k = 0; k < kU; ++k) f[k] = t[k] >= 0 ? a.dV[t[k]] : (uint8_t)1;
+#pragma unroll
+      for (int k = 0; k < kU; ++k)
+        if (!f[k]) a.dV[t[k]] = 1;
     }
   }
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
 }
+
+// Pull form over G' (the same marks, since w is an out-neighbour of u exactly
+// when u is an in-neighbour of w): a vertex outside dV joins it when an
+// in-neighbour is in the frontier. Only w's own thread (or warp) reads or
+// writes dV[w]; the scan stops at the first frontier in-neighbour. Rows below
+// pull_warp_b take a thread each, the others a warp.
+template <class Real>
+__device__ void pull_round(const SweepArgs<Real>& a) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = (int64_t)gridDim.x * kWarps;
+  const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (int64_t w = a.pull_warp_b + warp; w < a.n; w += nw) {
+    if (__shfl_sync(kFull, lane == 0 ? (int)a.dV[w] : 0, 0)) continue;
+    const int64_t b = a.off[w], e = a.off[w + 1];
+    for (int64_t j0 = b; j0 < e; j0 += 32) {
+      const int64_t j = j0 + lane;
+      const bool hit = j < e && a.dN[a.adj[j]];
+      if (__any_sync(kFull, hit)) {
+        if (lane == 0) a.dV[w] = 1;
+        break;
+      }
+    }
+  }
+  for (int64_t w = warp * 32 + lane; w < a.pull_warp_b; w += nw * 32) {
+    if (a.dV[w]) continue;
+    const int64_t e = a.off[w + 1];
+    for (int64_t j = a.off[w]; j < e; ++j)
+      if (a.dN[a.adj[j]]) {
+        a.dV[w] = 1;
+        break;
+      }
+  }
+}
+
+// The expansion round after a sweep: pull when the frontier's out-edges
+// exceed fthr, else push.
+template <class Real>
+__device__ __forceinline__ void expand_round(const SweepArgs<Real>& a, LoopSlot* slot) {
+  if (__ldcg(&slot->fw) > a.fthr) pull_round(a);
+  else push_round(a, &slot->nlist);
+}
+
+// mode kLoopAll: the whole loop (cooperative launch): [initial push], then
+// sweep, barrier, stop test, [expansion, barrier] until the stop rule holds or
+// max_iter sweeps ran. The other modes run one phase of iteration it0 as a
+// launch of its own (the host-driven loop): a phase past convergence exits at
+// once.
+template <class P, bool DYN>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) k_rank_loop(const __grid_constant__ SweepArgs<typename P::Real> a) {
+  if (a.mode == kLoopPush) {
+    if (DYN) push_round(a, &a.ctl->nlist0);
+    return;
+  }
+  if (a.mode == kLoopSweep) {
+    if (a.it0 > 0 && stopped(__ldcg(&slot_of(a, a.it0 - 1)->resid), a.tol)) return;
+    sweep<P, DYN>(a, a.it0);
+    return;
+  }
+  if (a.mode == kLoopExpand) {
+    LoopSlot* sl = slot_of(a, a.it0);
+    if (DYN && !stopped(__ldcg(&sl->resid), a.tol)) expand_round(a, sl);
+    return;
+  }
+  unsigned long long target = 0;
+  if (DYN && a.init_push) {
+    push_round(a, &a.ctl->nlist0);
+    if (!grid_barrier(a.ctl, target)) return;
+  }
+  for (int it = 0;; ++it) {
+    sweep<P, DYN>(a, it);
+    if (!grid_barrier(a.ctl, target)) return;
+    LoopSlot* sl = slot_of(a, it);
+    const unsigned long long resid = __ldcg(&sl->resid);
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (stopped(resid, a.tol) || it + 1 >= a.max_iter) {
+      if (first) {
+        a.ctl->iters = it + 1;
+        a.ctl->resid = resid;
+      }
+      return;
+    }
+    // the slot of sweep it + 2, which the sweep before this one used: a
+    // barrier separates both from here
+    if (first) *slot_of(a, it + 2) = LoopSlot();
+    if (DYN && a.expand) {
+      expand_round(a, sl);
+      if (!grid_barrier(a.ctl, target)) return;
+    }
+  }
+}
+
+// Effective sources of a batch into dN and the first frontier list, targets
+// of effective deletions into dV (initialAffected, Alg. affected, in the
+// sweep numbering).
+__global__ void k_mark_batch(const int32_t* __restrict__ del_src, const int32_t* __restrict__ del_dst,
+                             const uint8_t* __restrict__ del_mask, int64_t n_del, const int32_t* __restrict__ ins_src,
+                             const uint8_t* __restrict__ ins_mask, int64_t n_ins, const int32_t* __restrict__ inv,
+                             const int64_t* __restrict__ ooff, uint8_t* __restrict__ dV, uint8_t* __restrict__ dN,
+                             LoopCtl* __restrict__ ctl, int2* __restrict__ list) {
+  const int lane = threadIdx.x & 31;
+  const int64_t tot = n_del + n_ins, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < tot; base += stride) {
+    const int64_t i = base + lane;
+    int32_t u = -1;
+    if (i < n_del) {
+      if (!del_mask || del_mask[i]) {
+        u = inv[del_src[i]];
+        dV[inv[del_dst[i]]] = 1;
+      }
+    } else if (i < tot) {
+      if (!ins_mask || ins_mask[i - n_del]) u = inv[ins_src[i - n_del]];
+    }
+    // first to set the flag appends the vertex (flags are read by words: the array is padded to them)
+    bool mine = false;
+    if (u >= 0) {
+      const uint32_t bit = 1u << (8 * (u & 3));
+      mine = !(atomicOr(reinterpret_cast<uint32_t*>(dN + (u & ~3)), bit) & bit);
+    }
+    const uint64_t deg = mine ? (uint64_t)(ooff[u + 1] - ooff[u]) : 0;
+    append_frontier(mine, u, deg, &ctl->nlist0, list, lane);
+  }
+}
+
+// Kernel shape of class c by its upper degree bound; the last class runs in
+// hub chunks and the one before it a warp per row.
+int class_kind(const PartThr& t, int c, bool self_loops) {
+  const int C = t.n + 1;
+  if (c == C - 2 && C >= 3) return kRowWarp;
+  const int64_t hi = t.thr[c];
+  if (hi <= 1 && self_loops) return kRowSelf;
+  if (hi <= 4) return kRowThread;
+  if (hi <= 16) return kRow4;
+  if (hi <= 32) return kRow8;
+  if (hi <= 128) return kRow16;
+  return kRowWarp;
+}
+
+template <class P, bool DYN>
+struct Launcher {
+  using Args = SweepArgs<typename P::Real>;
+  // co-resident blocks of the loop kernel on the current device
+  static int max_blocks(int* out) {
+    auto k = k_rank_loop<P, DYN>;
+    int dev = 0, sms = 0, per = 0;
+    PRDF_CUDA(cudaGetDevice(&dev));
+    PRDF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // almost no shared memory: the unified L1 / shared storage goes to L1, which
+    // holds the gathered x of the hottest sources (a preference the driver
+    // declines is not an error)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 0) != cudaSuccess) cudaGetLastError();
+    PRDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kThreads, 0));
+    if (per < 1 || sms < 1) {
+      set_error("the sweep kernel does not fit this device");
+      return PRDF_ECUDA;
+    }
+    *out = per * sms;
+    return PRDF_OK;
+  }
+
+  // units of rows per class, long rows first
+  static int plan(Args& a, const PartThr& t, const int64_t* cb, int max_b) {
+    const int C = t.n + 1;
+    const int64_t n = cb[C];
+    const double warps = (double)max_b * kWarps;
+    // a unit's share of the sweep: about an eighth of a warp's work, at least
+    // two short steps, at most a few thousand edges
+    double target = ((double)a.m + 6.0 * (double)n) / (warps * 8.0);
+    if (target < 96) target = 96;
+    if (target > 4096) target = 4096;
+    int64_t units = a.hub.nchunk;
+    a.ncls = 0;
+    for (int c = C - 2; c >= 0; --c) {
+      const int64_t cnt = cb[c + 1] - cb[c];
+      if (cnt <= 0) continue;
+      const int kind = class_kind(t, c, a.self_loops != 0);
+      const double lo = c > 0 ? (double)t.thr[c - 1] + 1 : 1, hi = (double)t.thr[c];
+      const double deg = (lo + hi) / 2 < 2.5 * lo ? (lo + hi) / 2 : 2.5 * lo;
+      const int least = kind == kRowWarp ? 1 : kind == kRow16 ? 2 : kind == kRow8 ? 4 : kind == kRow4 ? 8 : 32;
+      int rows = least;
+      while (rows < 32 * kMaxWords && 2 * rows * (deg + 6) <= target) rows *= 2;
+      SweepClass& k = a.cls[a.ncls++];
+      k.begin = cb[c];
+      k.end = cb[c + 1];
+      k.unit0 = (uint32_t)units;
+      k.rows = rows;
+      k.kind = kind;
+      units += (cnt + rows - 1) / rows;
+    }
+    if (units >= (int64_t)UINT32_MAX / 2) {
+      set_error("too many work units");
+      return PRDF_EINVAL;
+    }
+    a.units = (uint32_t)units;
+    return PRDF_OK;
+  }
+
+  static int run(Args a, const PartThr& t, const int64_t* cb, cudaStream_t s) {
+    int max_b = 0;
+    PRDF_TRY(max_blocks(&max_b));
+    PRDF_TRY(plan(a, t, cb, max_b));
+    // few units: few blocks, and a shorter barrier
+    int64_t blocks = ((int64_t)a.units + kWarps - 1) / kWarps;
+    if (blocks > max_b) blocks = max_b;
+    if (blocks < 1) blocks = 1;
+    if (a.mode != kLoopAll) {
+      k_rank_loop<P, DYN><<<(unsigned)(a.mode == kLoopSweep ? blocks : max_b), kThreads, 0, s>>>(a);
+      PRDF_LAUNCH_CHECK();
+      return PRDF_OK;
+    }
+    void* args[] = {&a};
+    PRDF_CUDA(cudaLaunchCooperativeKernel((const void*)k_rank_loop<P, DYN>, dim3((unsigned)blocks), dim3(kThreads),
+                                          args, 0, s));
+    return PRDF_OK;
+  }
+};
 
 }  // namespace
 
-int launch_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
-                      cudaGraphConditionalHandle h, cudaStream_t s) {
-  k_iter_check<<<1, 1, 0, s>>>(ctl, resid_base, tol, max_iter, h);
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
+int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t* cb, bool exact, bool dynamic,
+                     cudaStream_t s) {
+  if (exact) return dynamic ? Launcher<PExact, true>::run(a, t, cb, s) : Launcher<PExact, false>::run(a, t, cb, s);
+  return dynamic ? Launcher<PPlain, true>::run(a, t, cb, s) : Launcher<PPlain, false>::run(a, t, cb, s);
 }
 
-int launch_sweep(const SweepArgs& a, const PartThr& t, const int64_t* class_begin, bool exact, bool dynamic,
-                 cudaStream_t s) {
-  if (exact) return dynamic ? launch_all<true, true>(a, t, class_begin, s) : launch_all<true, false>(a, t, class_begin, s);
-  return dynamic ? launch_all<false, true>(a, t, class_begin, s) : launch_all<false, false>(a, t, class_begin, s);
+int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s) {
+  return dynamic ? Launcher<PKahan, true>::run(a, t, cb, s) : Launcher<PKahan, false>::run(a, t, cb, s);
+}
+
+int launch_mark_batch(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
+                      const int32_t* ins_src, const uint8_t* ins_mask, int64_t n_ins, const int32_t* inv,
+                      const int64_t* ooff, uint8_t* dV, uint8_t* dN, LoopCtl* ctl, int2* list, cudaStream_t s) {
+  if (n_del + n_ins == 0) return PRDF_OK;
+  k_mark_batch<<<grid_for(n_del + n_ins, 256), 256, 0, s>>>(del_src, del_dst, del_mask, n_del, ins_src, ins_mask,
+                                                           n_ins, inv, ooff, dV, dN, ctl, list);
+  PRDF_LAUNCH_CHECK();
+  return PRDF_OK;
 }
 
 }  // namespace prdf
