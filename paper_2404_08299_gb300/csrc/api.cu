@@ -463,6 +463,8 @@ int64_t hub_begin(const Relabel& rl);
 //     check_every sweeps ahead of each residual read; sweeps launched past
 //     convergence exit at once on the device. Each sweep is bracketed by CUDA
 //     events.
+constexpr int64_t kChunkSmallM = 1ll << 22;
+
 struct Loop {
   bool fp32 = false, dynamic = false, expand = false, exact = true;
   bool init_push = false;  // the loop starts with the marked batch's expansion
@@ -517,9 +519,15 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
   a.n = g->n;
   a.max_iter = max_iter;
   a.ctl = g->loop_ctl.p;
-  a.hub = g->hub_in.view();
-  a.hub_part = g->sweep_hub_part.p;
-  a.hub_done = g->sweep_hub_done.p;
+  const SweepChunks& ch = g->sweep_chunks;
+  a.chunks = ch.chunks.p;
+  a.nchunk = ch.rows > 0 ? ch.first.p + ch.rows : nullptr;
+  a.max_chunks = ch.max_chunks;
+  a.chunk_class = ch.first_class;
+  a.chunk_size = ch.size;
+  a.chunks_per_unit = ch.size < kHubChunk ? 1 : 4;
+  a.hub_part = ch.part.p;
+  a.hub_done = ch.done.p;
   if (!L.dynamic) return PRDF_OK;
   a.dV = g->dV.p;
   a.dN = g->dN.p;
@@ -529,6 +537,10 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
   a.tau_f = (Real)(p->tau_f + 0.0);
   a.tau_p = (Real)(p->tau_p + 0.0);
   a.prune = p->prune;
+  // the class before the chunk table's is listed in four parts (sweep.cu)
+  const int64_t parts = ch.first_class > 0 ? L.cb[ch.first_class] - L.cb[ch.first_class - 1] : 0;
+  PRDF_TRY(g->loop_act.reserve((size_t)(g->n + 3 * parts), s));
+  a.act = g->loop_act.p;
   a.expand = L.expand ? 1 : 0;
   a.init_push = L.init_push ? 1 : 0;
   if (L.expand) {
@@ -538,8 +550,28 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
     a.list = g->loop_list.p;
     const double lim = p->expand_pull * (double)rl.in.m;
     a.fthr = lim >= 1.8e19 ? ~0ull : (unsigned long long)lim;
-    a.pull_warp_b = hub_begin(rl);
   }
+  return PRDF_OK;
+}
+
+// The rows of the highest in-degree class are cut into chunks of 1024 edges
+// summed by different warps. On graphs with little work per warp a sweep
+// lasts as long as its longest chain of gathers, so there the class below
+// (a warp per row otherwise, up to 4096 edges) is cut as well, into chunks of
+// 512 edges.
+int ensure_sweep_chunks(prdf_graph* g, const int64_t* cb, cudaStream_t s) {
+  SweepChunks& t = g->sweep_chunks;
+  if (!t.valid || t.version != g->rl.version) {
+    const int C = g->rl.thr.n + 1;
+    const bool small = g->rl.in.m < kChunkSmallM && C >= 3;
+    t.valid = false;
+    t.first_class = small ? C - 2 : C - 1;
+    t.size = small ? 512 : (int)kHubChunk;
+    PRDF_TRY(build_chunks(g->rl.in.off.p, cb[t.first_class], g->n, g->rl.in.m, t.size, t, g->ws, s));
+    t.version = g->rl.version;
+    t.valid = true;
+  }
+  if (t.rows > 0) PRDF_CUDA(cudaMemsetAsync(t.done.p, 0, sizeof(uint32_t) * (size_t)t.rows, s));
   return PRDF_OK;
 }
 
@@ -552,12 +584,7 @@ int loop_setup(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, boo
   L->init_push = L->expand && init_push;
   L->exact = p->accumulate == PRDF_ACC_EXACT;
   begins_from_counts(rl.count, rl.thr.n + 1, L->cb);
-  // the highest in-degree class's rows are cut into the hub chunks of G'
-  PRDF_TRY(ensure_hub(g, rl.in, g->hub_in, s));
-  const size_t nhub = (size_t)(g->hub_in.nhub > 0 ? g->hub_in.nhub : 1);
-  PRDF_TRY(g->sweep_hub_part.reserve((size_t)(g->hub_in.nchunk > 0 ? g->hub_in.nchunk : 1), s));
-  PRDF_TRY(g->sweep_hub_done.reserve(nhub, s));
-  PRDF_CUDA(cudaMemsetAsync(g->sweep_hub_done.p, 0, sizeof(uint32_t) * nhub, s));
+  PRDF_TRY(ensure_sweep_chunks(g, L->cb, s));
   if (!L->init_push) PRDF_TRY(alloc_loop_ctl(g, s));  // (with a marked batch the marking made it)
   if (fp32) {
     PRDF_TRY(loop_args(g, p, *L, max_iter, &L->a32, s));
@@ -645,6 +672,7 @@ int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, int max_it
       PRDF_CUDA(cudaEventCreate(&e1));
       ev.push_back(e1);
       PRDF_CUDA(cudaEventRecord(e0, s));
+      if (L.dynamic) PRDF_TRY(launch_loop(g, L, kLoopScan, i, launched, s));
       PRDF_TRY(launch_loop(g, L, kLoopSweep, i, launched, s));
       PRDF_CUDA(cudaEventRecord(e1, s));  // the sweep alone, not its expansion
       if (L.expand) PRDF_TRY(launch_loop(g, L, kLoopExpand, i, launched, s));
@@ -667,7 +695,7 @@ int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, int max_it
   loop_stopped(L, resid[(size_t)k], &res->final_delta);
   res->iters = k + 1;
   res->launched = launched;
-  res->kernels = (long long)launched * (L.expand ? 2 : 1) + (L.init_push ? 1 : 0);
+  res->kernels = (long long)launched * (1 + (L.dynamic ? 1 : 0) + (L.expand ? 1 : 0)) + (L.init_push ? 1 : 0);
   res->ms_sweep = 0;
   for (int i = 0; i < res->iters; ++i) {
     float ms = 0;
@@ -1126,9 +1154,10 @@ int alloc_solver(prdf_graph* g, bool dynamic, cudaStream_t s) {
   PRDF_TRY(g->xa.reserve(g->n, s));
   PRDF_TRY(g->xb.reserve(g->n, s));
   if (dynamic) {
-    PRDF_TRY(g->dV.reserve(g->n, s));
-    PRDF_TRY(g->dN.reserve((size_t)g->n + 4, s));  // marked by whole words
-    PRDF_TRY(g->wrote.reserve(g->n, s));
+    // read and marked by whole words
+    PRDF_TRY(g->dV.reserve((size_t)g->n + 32, s));
+    PRDF_TRY(g->dN.reserve((size_t)g->n + 32, s));
+    PRDF_TRY(g->wrote.reserve((size_t)g->n + 32, s));
   }
   PRDF_TRY(g->counter.reserve(1, s));
   return PRDF_OK;

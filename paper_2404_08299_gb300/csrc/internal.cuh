@@ -100,7 +100,7 @@ struct Relabel {
 };
 
 // Rows of the highest in-degree class are cut into chunks of kHubChunk edges
-// (used by the K-column calls and by the Static sweep): chunk c covers edges
+// by the K-column calls: chunk c covers edges
 // [chunk_j0[c], +kHubChunk) of vertex begin + chunk_hub[c]; the chunks of
 // hub i are [hub_first[i], hub_first[i + 1]) in row order.
 constexpr int64_t kHubChunk = 1024;
@@ -116,12 +116,35 @@ struct PprHub {
 // 1, the row is [v]), a lane per row, 4, 8 or 16 lanes per row, a warp per row.
 enum RowKind { kRowSelf = 0, kRowThread, kRow4, kRow8, kRow16, kRowWarp };
 
-// A class of the sweep cut into units of `rows` rows: unit unit0 + k holds
-// rows [begin + k * rows, +rows) below end.
+// A class of the sweep: its rows, their shape, about how long they are, and
+// the fewest rows a unit of work takes. In DF / DF-P the affected rows are
+// listed from act + list on; the rows of the warp-per-row class are listed in
+// four parts by their length (entries k .. k + 3, parts 0 to 3, longest first).
 struct SweepClass {
-  int64_t begin, end;
-  uint32_t unit0;
-  int rows, kind;
+  int64_t begin, end, list;
+  float deg;
+  int least, kind, part;  // part: -1 whole class
+};
+constexpr int kMaxCls = kMaxThr + 4;
+
+// A chunk of a long row of the sweep: entries [j0, j0 + len) of vertex v;
+// chunks [first, first + parts) are the row's, row its index in the table.
+struct alignas(16) SweepChunk {
+  int64_t j0;
+  int32_t len, v;
+  int32_t first, parts, row, pad;
+};
+// Owner of the chunk table of the sweep's long rows [begin, n) of G'.
+struct SweepChunks {
+  int64_t rows = 0, max_chunks = 0;
+  int first_class = 0, size = 0;
+  DBuf<uint32_t> cnt;
+  DBuf<int64_t> first;       // rows + 1: exclusive scan of the chunk counts, first[rows] = number of chunks
+  DBuf<SweepChunk> chunks;
+  DBuf<uint4> part;          // partial sum of a chunk
+  DBuf<uint32_t> done;       // chunks of a row that arrived
+  uint64_t version = 0;      // numbering version it was built for
+  bool valid = false;
 };
 
 // Counters of one sweep and its expansion round.
@@ -130,7 +153,7 @@ struct LoopSlot {
   unsigned long long fw;     // out-edges of the vertices the sweep put into deltaN
   unsigned int units;        // units handed out beyond the first of each warp
   unsigned int nlist;        // frontier entries
-  unsigned long long pad;
+  unsigned int act[kMaxCls];  // DF / DF-P: affected rows of each class
 };
 constexpr int kLoopRing = 4;  // slots of the whole-loop kernel (a power of two)
 
@@ -144,7 +167,7 @@ struct LoopCtl {
   unsigned int aff0;         // affected vertices at the first sweep
 };
 
-enum LoopMode { kLoopAll = 0, kLoopSweep, kLoopExpand, kLoopPush };
+enum LoopMode { kLoopAll = 0, kLoopScan, kLoopSweep, kLoopExpand, kLoopPush };
 
 // A frontier entry (v, k) stands for out-edges [k, k + 1) * kFrontChunk of v.
 constexpr int kFrontChunk = 1024;
@@ -171,15 +194,18 @@ struct SweepArgs {
   int mode, it0, it_first; // LoopMode; single phases: the iteration, and the one slot[1] stands for
   LoopSlot* slot;
   LoopCtl* ctl;
-  // chunks of the highest in-degree class's rows, one partial sum and one
-  // arrival counter (zero between sweeps) each
-  PprHub hub;
+  // chunk table of the classes from chunk_class on: a partial sum per chunk
+  // and an arrival counter (zero between sweeps) per row
+  const SweepChunk* chunks;
+  const int64_t* nchunk;   // number of chunks (device), null: none
+  int64_t max_chunks;
+  int chunk_class, chunk_size;
+  uint32_t chunks_per_unit;
   uint4* hub_part;
   uint32_t* hub_done;
-  // units: hub chunks, then the classes (filled by the launcher)
-  SweepClass cls[kMaxThr + 1];
+  // the other classes (filled by the launcher)
+  SweepClass cls[kMaxCls];
   int ncls;
-  uint32_t units;
   // DF / DF-P / DT
   uint8_t* dV;             // affected flags (read; cleared on prune)
   uint8_t* dN;             // expand flags (set when the change exceeds tau_f)
@@ -192,11 +218,15 @@ struct SweepArgs {
   const int32_t* oadj;
   int2* list;              // frontier entries of the round (room for n + m / kFrontChunk + 1)
   unsigned long long fthr; // the round runs in pull form when the frontier's out-edges exceed this
-  int64_t pull_warp_b;     // pull form: rows from here on take a warp each
+  int32_t* act;            // affected rows of the classes (SweepClass::list)
+  int64_t scan_end;        // rows outside the chunk table
+  int scan_rows;           // of them a warp scans at a time (a power of two, 32 to 1024)
 };
 int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t* cb, bool exact, bool dynamic,
                      cudaStream_t s);
 int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s);
+int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, SweepChunks& t, Workspace& ws,
+                 cudaStream_t s);
 // initialAffected (Alg. affected) in the sweep numbering: dV, dN and the frontier list of the first push
 // (dN padded to whole 32-bit words)
 int launch_mark_batch(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
@@ -331,8 +361,7 @@ struct prdf_graph {
   // solver scratch
   prdf::DBuf<double> xa, xb;
   prdf::PprHubTable hub_in, hub_out;  // chunk tables of G' (Static sweep, K-column forward) and G (adjoint)
-  prdf::DBuf<uint4> sweep_hub_part;     // rank sweeps: one partial sum per chunk of G's hub rows
-  prdf::DBuf<uint32_t> sweep_hub_done;  // and one arrival counter per hub row
+  prdf::SweepChunks sweep_chunks;     // chunk table of the rank sweeps
   prdf::DBuf<float2> ppr_part;        // chunk partial sums of one column tile (FP32 sweeps)
   prdf::DBuf<double> ppr_part64;      // chunk partial sums of one column tile (FP64 steps)
   prdf::DBuf<float> ya, yb, degf, invf;  // FP32 stage state and degrees (class-contiguous numbering)
@@ -346,6 +375,7 @@ struct prdf_graph {
   prdf::DBuf<prdf::LoopCtl> loop_ctl;    // state of a rank loop
   prdf::DBuf<prdf::LoopSlot> loop_slots; // its per-sweep counters
   prdf::DBuf<int2> loop_list;            // DF / DF-P: frontier entries of an expansion round
+  prdf::DBuf<int32_t> loop_act;          // DF / DF-P / DT: affected rows of a sweep
   prdf::DBuf<int32_t> flist;             // DT: a small frontier listed for its closure round (frontier.cu)
   prdf::DBuf<unsigned int> fcnt;         // its size
   prdf::DBuf<int> ctl;               // device iteration counter of the graph-driven K-column loops

@@ -41,7 +41,7 @@ constexpr int kThreads = 512;
 constexpr int kMinBlocks = 2;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kMaxWords = 8;  // a unit holds at most 8 x 32 rows
+constexpr int kMaxRows = 256;  // rows of a unit at most
 
 // ------------------------------------------------------ precision traits ----
 
@@ -290,106 +290,20 @@ __device__ __forceinline__ void skip_vertex(const SweepArgs<typename P::Real>& a
   if (dn) a.dN[v] = 0;
 }
 
-// The rows of one unit, [vb, ve) with at most 256 rows. Static: all of them.
-// DF / DF-P: the affected ones, compacted over the whole unit (the flags of
-// 256 rows are read at once, a bit mask per 32 rows is kept in the lanes), so
-// that a batch is 32 affected rows however thinly they are spread; the others
-// are copied through.
+// The k-th row of a class: every vertex of it (Static), or the k-th affected
+// one (DF / DF-P, listed by the scan phase), with its deltaN flag.
 template <class P, bool DYN>
-struct UnitRows {
-  int64_t vb;
-  int nact;
-  uint32_t mdv, mdn;  // lane i: affected / deltaN bits of rows vb + 32 i ..
-  int excl;           // lane i: affected rows before word i
-
-  __device__ __forceinline__ UnitRows(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb_, int64_t ve,
-                                      Tally& t)
-      : vb(vb_), mdv(0), mdn(0), excl(0) {
-    if (!DYN) {
-      nact = (int)(ve - vb);
-      return;
-    }
-    uint32_t mwr = 0;
-    uint8_t dv[kMaxWords], wr[kMaxWords], dn[kMaxWords];
-#pragma unroll
-    for (int i = 0; i < kMaxWords; ++i) {
-      const int64_t v = vb + 32 * i + c.lane;
-      const bool in = v < ve;
-      dv[i] = in ? a.dV[v] : (uint8_t)0;
-      wr[i] = in ? a.wrote[v] : (uint8_t)0;
-      dn[i] = in ? a.dN[v] : (uint8_t)0;
-    }
-#pragma unroll
-    for (int i = 0; i < kMaxWords; ++i) {
-      const uint32_t b0 = __ballot_sync(kFull, dv[i] != 0), b1 = __ballot_sync(kFull, wr[i] != 0),
-                     b2 = __ballot_sync(kFull, dn[i] != 0);
-      if (c.lane == i) {
-        mdv = b0;
-        mwr = b1;
-        mdn = b2;
-      }
-    }
-    // unaffected rows with something to undo
-    uint32_t todo = __ballot_sync(kFull, ((mwr | mdn) & ~mdv) != 0);
-    while (todo) {
-      const int i = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const uint32_t w = __shfl_sync(kFull, mwr & ~mdv, i), d = __shfl_sync(kFull, mdn & ~mdv, i);
-      const bool bw = (w >> c.lane) & 1u, bd = (d >> c.lane) & 1u;
-      if (bw || bd) skip_vertex(a, c, (int32_t)(vb + 32 * i + c.lane), bw, bd);
-    }
-    const int cnt = __popc(mdv);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < kMaxWords; o <<= 1) {
-      const int u = __shfl_up_sync(kFull, incl, o);
-      if (c.lane >= o) incl += u;
-    }
-    excl = incl - cnt;
-    nact = __shfl_sync(kFull, incl, kMaxWords - 1);
-    if (c.lane == 0) t.aff += (unsigned int)nact;
-  }
-
-  // the k-th row (0 <= k < nact; any k on lanes that hold no row) and its deltaN flag
-  __device__ __forceinline__ int32_t row(int k, bool& dn) const {
-    if (!DYN) {
-      dn = false;
-      return (int32_t)(vb + k);
-    }
-    int w = 0, before = 0;
-#pragma unroll
-    for (int i = 1; i < kMaxWords; ++i) {
-      const int e = __shfl_sync(kFull, excl, i);
-      if (e <= k) {
-        w = i;
-        before = e;
-      }
-    }
-    const uint32_t m = __shfl_sync(kFull, mdv, w);
-    const uint32_t d = __shfl_sync(kFull, mdn, w);
-    int r = k - before;  // the r-th set bit of m
-    int pos = 0;
-#pragma unroll
-    for (int half = 16; half > 0; half >>= 1) {
-      const int low = __popc((m >> pos) & ((1u << half) - 1u));
-      if (r >= low) {
-        r -= low;
-        pos += half;
-      }
-    }
-    dn = (d >> pos) & 1u;
-    return (int32_t)(vb + 32 * w + pos);
-  }
-};
+__device__ __forceinline__ int32_t row_at(const SweepArgs<typename P::Real>& a, int64_t k) {
+  return DYN ? __ldcg(a.act + k) : (int32_t)k;
+}
 
 // One row per lane, its offsets known: the epilogue of a batch.
 template <class P, bool DYN>
 __device__ __forceinline__ void finish_batch(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, bool have,
-                                             int32_t v, typename P::Real sum, typename P::Real xself, bool dn,
-                                             Tally& t) {
+                                             int32_t v, typename P::Real sum, typename P::Real xself, Tally& t) {
   bool front = false;
   uint64_t deg = 0;
-  if (have) front = finish<DYN>(a, c, v, sum, xself, dn, t, deg);
+  if (have) front = finish<DYN>(a, c, v, sum, xself, DYN && a.dN[v] != 0, t, deg);
   if (DYN && a.expand) append_frontier(front, v, deg, &c.slot->nlist, a.list, c.lane);
 }
 
@@ -425,132 +339,223 @@ __device__ __forceinline__ void mask4(const int4& q, int j, int lo, int hi, int3
   u[3] = (j + 3 >= lo && j + 3 < hi) ? q.w : -1;
 }
 
-// G lanes per row, a 16-byte index load each per step. The row's entries are
-// read from the 16-byte boundary below its first one (positions in a row are
-// 32-bit, counted from that boundary). While the gathers of one step are in
-// flight the indices of the next step load: the next chunk of the same rows,
-// or the first chunk of the groups' next rows, whose offsets are already in
-// the lanes, so a step waits for one round trip. The offsets of the next
-// batch load before the batch.
+// Sums of up to 32 rows, one after the other by groups of G lanes; row s of a
+// group is described by its lane s (b: first entry, len, and v when the graph
+// has vertices without self-loop), S rows at most per group. A 16-byte index
+// load a lane and step: the row's entries are read from the 16-byte boundary
+// below its first one (positions in a row are 32-bit, counted from that
+// boundary). While the gathers of one step are in flight the indices of the
+// next step load: the next chunk of the same rows, or the first chunk of the
+// groups' next rows, whose offsets are already in the lanes, so a step waits
+// for one round trip. On return lane s of each group holds the sum of row s
+// in saved (and in hit whether the row holds v itself).
+template <class P, int G>
+__device__ __forceinline__ void sum_rows(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int S, int64_t b,
+                                         int len, int32_t v, typename P::Acc& saved, bool& hit) {
+  using Bits = typename P::Bits;
+  const int lane = c.lane, sub = lane & (G - 1), src0 = lane & ~(G - 1);
+  typename P::Acc acc;
+  bool myhit = false;
+  // the group's row: entries [lo, hi) from base; this lane's position j
+  int64_t rb = __shfl_sync(kFull, b, src0);
+  int lo = (int)(rb & 3), hi = lo + __shfl_sync(kFull, len, src0), j = 4 * sub;
+  const int32_t* base = a.adj + (rb & ~(int64_t)3);
+  int4 q = load4(base, j, hi, c.pf);
+  for (int s = 0; s < S;) {
+    int32_t u[4];
+    mask4(q, j, lo, hi, u);
+    Bits xv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
+    // the next step's indices
+    const bool more = __any_sync(kFull, j - 4 * sub + 4 * G < hi);
+    if (more) {
+      j += 4 * G;
+      lo = 0;
+    } else {
+      const int src = (src0 + s + 1) & 31;  // (past the last row: any lane, no entries)
+      rb = __shfl_sync(kFull, b, src);
+      const int l = __shfl_sync(kFull, len, src);
+      lo = (int)(rb & 3);
+      hi = s + 1 < S ? lo + l : 0;
+      j = 4 * sub;
+      base = a.adj + (rb & ~(int64_t)3);
+    }
+    q = load4(base, j, hi, c.pf);
+    if (G < 32 && !a.self_loops) {
+      const int32_t rv = __shfl_sync(kFull, v, src0 + s) & INT32_MAX;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) myhit = myhit || u[k] == rv;
+    }
+    add_terms<P>(acc, u, xv);
+    if (!more) {
+      acc.template group_reduce<G>();
+      if (sub == s) saved = acc;
+      acc = typename P::Acc();
+      if (G < 32 && !a.self_loops) {
+        const uint32_t m = __ballot_sync(kFull, myhit) >> src0;
+        if (sub == s) hit = (m & ((1u << (G & 31)) - 1u)) != 0;
+        myhit = false;
+      }
+      ++s;
+    }
+  }
+}
+
+// A unit: the rows at positions [kb, ke) of a class, G lanes per row, in
+// batches of up to 32. The offsets of the next batch and the row ids of the
+// one after it load before the batch.
 template <class P, int G, bool DYN>
-__device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb,
-                                           int64_t ve, Tally& t) {
+__device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t kb,
+                                           int64_t ke, Tally& t) {
   using Bits = typename P::Bits;
   constexpr int NG = 32 / G;
-  const int lane = c.lane, sub = lane & (G - 1), src0 = lane & ~(G - 1);
-  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
-  const int nact = rows.nact;
-  if (nact == 0) return;
-
-  // lane's row of the batch at k0: group g takes rows g * S .. g * S + S - 1
+  const int lane = c.lane, sub = lane & (G - 1);
+  const int nact = (int)(ke - kb);
   struct Batch {
-    int32_t v;  // row, its deltaN flag in the sign bit
+    int32_t v;
     int len;
     int64_t b;
   };
+  // lane's row of the batch at k0: group g takes rows g * S .. g * S + S - 1
   auto steps = [&](int k0) { return ((nact - k0 < 32 ? nact - k0 : 32) + NG - 1) / NG; };
   auto in_batch = [&](int k0) {
     const int S = steps(k0);
     return sub < S && (lane / G) * S + sub < (nact - k0 < 32 ? nact - k0 : 32);
   };
-  auto load_batch = [&](int k0) {
+  auto load_v = [&](int k0) {
+    return k0 < nact && in_batch(k0) ? row_at<P, DYN>(a, kb + k0 + (lane / G) * steps(k0) + sub) : -1;
+  };
+  auto load_off = [&](int32_t v) {
     Batch r;
-    const bool have = in_batch(k0);
-    bool dn;
-    const int32_t v = rows.row(have ? k0 + (lane / G) * steps(k0) + sub : 0, dn);
-    r.v = dn ? (v | INT32_MIN) : v;
+    r.v = v;
     r.b = 0;
     r.len = 0;
-    if (have) {
+    if (v >= 0) {
       r.b = ld_stream_i64(a.off + v, c.pf);
       r.len = (int)(ld_stream_i64(a.off + v + 1, c.pf) - r.b);
     }
     return r;
   };
 
-  Batch cur = load_batch(0);
+  int32_t vn = load_v(32);
+  Batch cur = load_off(load_v(0));
   for (int k0 = 0; k0 < nact; k0 += 32) {
-    Batch nxt = cur;
-    if (k0 + 32 < nact) nxt = load_batch(k0 + 32);
-    const int S = steps(k0);
-    typename P::Acc saved, acc;
-    bool hit = false, myhit = false;
-    // the group's row: entries [lo, hi) from base; this lane's position j
-    int64_t rb = __shfl_sync(kFull, cur.b, src0);
-    int lo = (int)(rb & 3), hi = lo + __shfl_sync(kFull, cur.len, src0), j = 4 * sub;
-    const int32_t* base = a.adj + (rb & ~(int64_t)3);
-    int4 q = load4(base, j, hi, c.pf);
-    for (int s = 0; s < S;) {
-      int32_t u[4];
-      mask4(q, j, lo, hi, u);
-      Bits xv[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
-      // the next step's indices
-      const bool more = __any_sync(kFull, j - 4 * sub + 4 * G < hi);
-      if (more) {
-        j += 4 * G;
-        lo = 0;
-      } else {
-        const int src = src0 + s + 1;  // (past the last row: any lane, no entries)
-        rb = __shfl_sync(kFull, cur.b, src & 31);
-        const int len = __shfl_sync(kFull, cur.len, src & 31);
-        lo = (int)(rb & 3);
-        hi = s + 1 < S ? lo + len : 0;
-        j = 4 * sub;
-        base = a.adj + (rb & ~(int64_t)3);
-      }
-      q = load4(base, j, hi, c.pf);
-      if (G < 32 && !a.self_loops) {
-        const int32_t rv = __shfl_sync(kFull, cur.v, src0 + s) & INT32_MAX;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) myhit = myhit || u[k] == rv;
-      }
-      add_terms<P>(acc, u, xv);
-      if (!more) {
-        acc.template group_reduce<G>();
-        if (sub == s) saved = acc;
-        acc = typename P::Acc();
-        if (G < 32 && !a.self_loops) {
-          // graphs without self-loops on every vertex: x[v] counts only when the row holds v
-          const uint32_t m = __ballot_sync(kFull, myhit) >> src0;
-          if (sub == s) hit = (m & ((1u << (G & 31)) - 1u)) != 0;
-          myhit = false;
-        }
-        ++s;
-      }
-    }
+    const Batch nxt = load_off(vn);
+    vn = load_v(k0 + 64);
+    typename P::Acc saved;
+    bool hit = false;
+    sum_rows<P, G>(a, c, steps(k0), cur.b, cur.len, cur.v, saved, hit);
     const bool have = in_batch(k0);
-    const int32_t v = cur.v & INT32_MAX;
-    const Bits xs = have && (G == 32 || a.self_loops || hit) ? ld_state(c.x + v, c.pl) : Bits(0);
-    finish_batch<P, DYN>(a, c, have, v, saved.value(), as_real(xs), cur.v < 0, t);
+    // graphs without self-loops on every vertex: x[v] counts only when the row
+    // holds v (rows of a warp or more always took x[v])
+    const Bits xs = have && (G == 32 || a.self_loops || hit) ? ld_state(c.x + cur.v, c.pl) : Bits(0);
+    finish_batch<P, DYN>(a, c, have, cur.v, saved.value(), as_real(xs), t);
     cur = nxt;
   }
 }
 
+// A unit of chunks of the long rows (the chunk table), a warp per chunk one
+// after the other. A row of one chunk is finished like any other. The chunks
+// of a longer row leave their sums in hub_part; the warp that sums the last
+// of them (an arrival counter per row) adds the row's partial sums and
+// finishes the vertex. With exact accumulation the partials are integers, so
+// the result is the same bits as any other split; the compensated FP32
+// partials are added in chunk order by lanes and a fixed shuffle tree, so
+// every run gives the same bits. DF / DF-P: a row's flags change only in its
+// finishing warp, which runs after every chunk's warp has read them, or
+// (unaffected rows) in the warp of its first chunk, which leaves dV alone.
+template <class P, bool DYN>
+__device__ __forceinline__ void unit_chunks(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t cb,
+                                            int cnt, Tally& t) {
+  using Bits = typename P::Bits;
+  const int lane = c.lane;
+  SweepChunk k = {};
+  if (lane < cnt) {
+    const int4* p = reinterpret_cast<const int4*>(a.chunks + cb + lane);
+    const int4 p0 = __ldg(p), p1 = __ldg(p + 1);
+    k.j0 = (int64_t)(((uint64_t)(uint32_t)p0.y << 32) | (uint32_t)p0.x);
+    k.len = p0.z;
+    k.v = p0.w;
+    k.first = p1.x;
+    k.parts = p1.y;
+    k.row = p1.z;
+  }
+  int64_t ch = cb + lane;
+  int nact = cnt;
+  bool have = lane < cnt;
+  if (DYN) {
+    const bool act = have && a.dV[k.v] != 0;
+    if (have && ch == k.first) {
+      if (act) t.aff += 1;
+      else skip_vertex(a, c, k.v, a.wrote[k.v] != 0, a.dN[k.v] != 0);
+    }
+    // affected chunks to the first lanes
+    const uint32_t m = __ballot_sync(kFull, act);
+    nact = __popc(m);
+    if (nact == 0) return;
+    int src = 0;
+    uint32_t rest = m;
+    for (int i = 0; i < nact; ++i) {
+      const int l = __ffs(rest) - 1;
+      rest &= rest - 1;
+      if (lane == i) src = l;
+    }
+    k.j0 = __shfl_sync(kFull, k.j0, src);
+    k.len = __shfl_sync(kFull, k.len, src);
+    k.v = __shfl_sync(kFull, k.v, src);
+    k.first = __shfl_sync(kFull, k.first, src);
+    k.parts = __shfl_sync(kFull, k.parts, src);
+    k.row = __shfl_sync(kFull, k.row, src);
+    ch = cb + src;
+    have = lane < nact;
+  }
+  typename P::Acc saved;
+  bool hit = false;
+  sum_rows<P, 32>(a, c, nact, k.j0, k.len, 0, saved, hit);
+  bool fin = have;
+  if (have && k.parts > 1) {
+    __stcg(a.hub_part + ch, saved.pack());
+    __threadfence();
+    fin = atomicAdd(a.hub_done + k.row, 1u) + 1 == (unsigned int)k.parts;
+    if (fin) a.hub_done[k.row] = 0;
+    __threadfence();
+  }
+  uint32_t need = __ballot_sync(kFull, fin && have && k.parts > 1);
+  __syncwarp();
+  while (need) {
+    const int l = __ffs(need) - 1;
+    need &= need - 1;
+    const int first = __shfl_sync(kFull, k.first, l), parts = __shfl_sync(kFull, k.parts, l);
+    typename P::Acc acc;
+    for (int i = lane; i < parts; i += 32) acc.merge(__ldcg(a.hub_part + first + i));
+    acc.template group_reduce<32>();
+    if (lane == l) saved = acc;
+  }
+  const Bits xs = fin ? ld_state(c.x + k.v, c.pl) : Bits(0);
+  finish_batch<P, DYN>(a, c, fin, k.v, saved.value(), as_real(xs), t);
+}
+
 // One row per lane, U indices in flight (short rows).
 template <class P, int U, bool DYN>
-__device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb, int64_t ve,
-                                         Tally& t) {
+__device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t kb,
+                                            int64_t ke, Tally& t) {
   using Bits = typename P::Bits;
-  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
-  const int nact = rows.nact;
-  if (nact == 0) return;
+  const int nact = (int)(ke - kb);
   struct Row {
     int32_t v;
     int len;
     int64_t b;
-    bool have, dn;
   };
-  auto load_row = [&](int k0) {
+  auto load_v = [&](int k0) { return k0 + c.lane < nact ? row_at<P, DYN>(a, kb + k0 + c.lane) : -1; };
+  auto load_off = [&](int32_t v) {
     Row r;
-    r.have = k0 + c.lane < nact;
-    r.v = rows.row(r.have ? k0 + c.lane : 0, r.dn);
+    r.v = v;
     r.b = 0;
     r.len = 0;
-    if (r.have) {
-      r.b = ld_stream_i64(a.off + r.v, c.pf);
-      r.len = (int)(ld_stream_i64(a.off + r.v + 1, c.pf) - r.b);
+    if (v >= 0) {
+      r.b = ld_stream_i64(a.off + v, c.pf);
+      r.len = (int)(ld_stream_i64(a.off + v + 1, c.pf) - r.b);
     }
     return r;
   };
@@ -558,27 +563,22 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
 #pragma unroll
     for (int k = 0; k < U; ++k) u[k] = k < r.len ? ld_stream_i32(a.adj + r.b + k, c.pf) : -1;
   };
-  // offsets two batches ahead, indices one ahead
-  Row cur = load_row(0), nxt;
+  // row ids three batches ahead, offsets two, indices one
+  const int32_t v0 = load_v(0), v1 = load_v(32);
+  int32_t vf = load_v(64);
+  Row cur = load_off(v0), nxt = load_off(v1);
   int32_t u[U];
   load_idx(cur, u);
-  nxt.have = false;
-  nxt.len = 0;
-  nxt.b = 0;
-  nxt.v = 0;
-  nxt.dn = false;
-  if (32 < nact) nxt = load_row(32);
   for (int k0 = 0; k0 < nact; k0 += 32) {
+    const bool have = k0 + c.lane < nact;
     Bits xv[U];
 #pragma unroll
     for (int k = 0; k < U; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
-    const Bits xs = cur.have ? ld_state(c.x + cur.v, c.pl) : Bits(0);
+    const Bits xs = have ? ld_state(c.x + cur.v, c.pl) : Bits(0);
     int32_t un[U];
     load_idx(nxt, un);
-    Row far = nxt;
-    far.have = false;
-    far.len = 0;
-    if (k0 + 64 < nact) far = load_row(k0 + 64);
+    const Row far = load_off(vf);
+    vf = load_v(k0 + 96);
     typename P::Acc acc;
     bool hit = false;
 #pragma unroll
@@ -591,7 +591,7 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
       hit = hit || w == cur.v;
     }
     const Bits xself = (a.self_loops || hit) ? xs : Bits(0);
-    finish_batch<P, DYN>(a, c, cur.have, cur.v, acc.value(), as_real(xself), cur.dn, t);
+    finish_batch<P, DYN>(a, c, have, cur.v, acc.value(), as_real(xself), t);
     cur = nxt;
     nxt = far;
 #pragma unroll
@@ -604,15 +604,14 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
 // indices are read (a vertex that gained in-edges in a batch update has its
 // bit in multi and reads its row).
 template <class P, bool DYN>
-__device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t vb, int64_t ve,
-                                       Tally& t) {
+__device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t kb,
+                                          int64_t ke, Tally& t) {
   using Bits = typename P::Bits;
-  const UnitRows<P, DYN> rows(a, c, vb, ve, t);
-  const int nact = rows.nact;
-  for (int k0 = 0; k0 < nact; k0 += 32) {
-    const bool have = k0 + c.lane < nact;
-    bool dn;
-    const int32_t v = rows.row(have ? k0 + c.lane : 0, dn);
+  int32_t vn = kb + c.lane < ke ? row_at<P, DYN>(a, kb + c.lane) : 0;
+  for (int64_t k0 = kb; k0 < ke; k0 += 32) {
+    const bool have = k0 + c.lane < ke;
+    const int32_t v = vn;
+    vn = k0 + 32 + c.lane < ke ? row_at<P, DYN>(a, k0 + 32 + c.lane) : 0;
     const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
     typename P::Real sum = as_real(xs);
     if (a.multi && have && ((a.multi[v >> 5] >> (v & 31)) & 1u)) {
@@ -621,68 +620,8 @@ __device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, 
       for (int64_t j = a.off[v]; j < e; ++j) acc.add(ld_state(c.x + a.adj[j], c.pl));
       sum = acc.value();
     }
-    finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), dn, t);
+    finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), t);
   }
-}
-
-// One 1024-edge chunk of a row of the highest in-degree class. The warp that
-// finishes the last chunk of a row adds the row's partial sums and finishes
-// the vertex. With exact accumulation the partials are integers, so the
-// result is the same bits as any other split; the compensated FP32 partials
-// are added in chunk order by lanes and a fixed shuffle tree, so every run
-// gives the same bits. A hub's flags change only in its finishing warp, which
-// runs after every chunk's warp has read them, or (unaffected hubs) in the
-// warp of its first chunk, which leaves dV alone.
-template <class P, bool DYN>
-__device__ __forceinline__ void unit_hub(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t ch, Tally& t) {
-  using Bits = typename P::Bits;
-  const int lane = c.lane;
-  const int64_t h = a.hub.chunk_hub[ch];
-  const int32_t v = (int32_t)(a.hub.begin + h);
-  const int64_t jb = a.hub.chunk_j0[ch];
-  const int64_t first = a.hub.hub_first[h], last = a.hub.hub_first[h + 1];
-  if (DYN) {
-    const bool skip = __shfl_sync(kFull, lane == 0 ? (int)(a.dV[v] == 0) : 0, 0) != 0;
-    if (skip) {
-      if (ch == first && lane == 0) skip_vertex(a, c, v, a.wrote[v] != 0, a.dN[v] != 0);
-      return;
-    }
-    if (ch == first && lane == 0) t.aff += 1;
-  }
-  const int64_t row_e = a.off[v + 1];
-  const int64_t je = jb + kHubChunk < row_e ? jb + kHubChunk : row_e;
-  typename P::Acc acc;
-  const int lo0 = (int)(jb & 3), hi = lo0 + (int)(je - jb);
-  const int32_t* base = a.adj + (jb & ~(int64_t)3);
-  int4 q = load4(base, 4 * lane, hi, c.pf);
-  for (int j = 4 * lane; j - 4 * lane < hi; j += 128) {
-    int32_t u[4];
-    mask4(q, j, lo0, hi, u);
-    Bits xv[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
-    q = load4(base, j + 128, hi, c.pf);
-    add_terms<P>(acc, u, xv);
-  }
-  acc.template group_reduce<32>();
-  unsigned int done = 0;
-  if (last - first > 1) {
-    if (lane == 0) {
-      __stcg(a.hub_part + ch, acc.pack());
-      __threadfence();
-      done = atomicAdd(a.hub_done + h, 1u) + 1;
-    }
-    done = __shfl_sync(kFull, done, 0);
-    if (done != (unsigned int)(last - first)) return;
-    if (lane == 0) a.hub_done[h] = 0;
-    __threadfence();
-    acc = typename P::Acc();
-    for (int64_t k = first + lane; k < last; k += 32) acc.merge(__ldcg(a.hub_part + k));
-    acc.template group_reduce<32>();
-  }
-  const bool have = lane == 0;
-  const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
-  finish_batch<P, DYN>(a, c, have, v, acc.value(), as_real(xs), DYN && have && a.dN[v] != 0, t);
 }
 
 // -------------------------------------------------------------- phases ----
@@ -731,8 +670,171 @@ __device__ __forceinline__ LoopSlot* slot_of(const SweepArgs<Real>& a, int it) {
   return a.slot + (a.mode == kLoopAll ? (it & (kLoopRing - 1)) : it - a.it_first + 1);
 }
 
+// Units of a sweep: the chunk units, then each class cut by `rows`. Classes
+// without rows have no units.
+struct Plan {
+  uint32_t unit0[kMaxCls];
+  int64_t begin[kMaxCls], end[kMaxCls];
+  int rows[kMaxCls];
+  uint32_t chunk_units, total;
+};
+
+// Cuts the classes (Static: whole, DF / DF-P: their affected rows) into units
+// of about an eighth of a warp's share of the sweep, at least two short steps
+// and at most a few thousand edges (so that a unit's start-up latency is paid
+// for, and the last units of a sweep are short). Lane k of the block's first
+// warp takes class k.
+template <bool DYN, class Real>
+__device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSlot* slot, Plan* plan) {
+  if (threadIdx.x < 32) {
+    const int k = threadIdx.x;
+    const bool in = k < a.ncls;
+    const int64_t cnt = !in ? 0 : DYN ? (int64_t)__ldcg(&slot->act[k]) : a.cls[k].end - a.cls[k].begin;
+    const unsigned int nchunk = a.nchunk ? (unsigned int)__ldg(a.nchunk) : 0u;
+    const float per = in ? a.cls[k].deg + 6.f : 0.f;
+    float cost = (float)cnt * per;
+    if (k == 31) cost = (float)nchunk * (float)a.chunk_size;
+    const float all = warp_sum_f32(cost);
+    float target = all / (8.f * (float)(gridDim.x * kWarps));
+    target = fminf(fmaxf(target, 96.f), 4096.f);
+    int rows = in ? a.cls[k].least : 1;
+    while (rows < kMaxRows && 2.f * rows * per <= target) rows *= 2;
+    const unsigned int units = (unsigned int)((cnt + rows - 1) / rows);
+    unsigned int incl = units;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int x = __shfl_up_sync(kFull, incl, o);
+      if (k >= o) incl += x;
+    }
+    const unsigned int cu = (nchunk + a.chunks_per_unit - 1) / a.chunks_per_unit;
+    if (in) {
+      plan->unit0[k] = cu + incl - units;
+      plan->begin[k] = DYN ? a.cls[k].list : a.cls[k].begin;
+      plan->end[k] = plan->begin[k] + cnt;
+      plan->rows[k] = rows;
+    }
+    if (k == 31) {
+      plan->chunk_units = cu;
+      plan->total = cu + incl;
+    }
+  }
+  __syncthreads();
+}
+
+constexpr int64_t kLong0 = 2048, kLong1 = 1024, kLong2 = 512;
+
+// DF / DF-P: lists the affected rows of every class outside the chunk table,
+// in id order within a stretch of 1024 (a.act + class begin, counts in the
+// sweep's slot), and copies the unaffected ones through. A sweep then works
+// on full batches of affected rows, however thinly they are spread, at the
+// cost of one pass over the flag bytes.
+template <class P>
+__device__ __forceinline__ void scan(const SweepArgs<typename P::Real>& a, int it) {
+  Ctx<P> c;
+  c.x = (it & 1) ? a.xb : a.xa;
+  c.xn = (it & 1) ? a.xa : a.xb;
+  c.slot = slot_of(a, it);
+  c.pf = policy_evict_first();
+  c.pl = policy_evict_last();
+  c.lane = threadIdx.x & 31;
+  const int lane = c.lane;
+  const int64_t nw = (int64_t)gridDim.x * kWarps;
+  const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  unsigned int aff = 0;
+  const bool parts = a.ncls > 0 && a.cls[0].part == 0;
+  const int64_t n = parts ? a.cls[0].begin : a.scan_end;
+  if (parts) {
+    // rows of 129 to 4096 edges: by length, so that the sweep can start with
+    // the longest; few vertices, so 32 rows a step spread them over the warps
+    for (int64_t v0 = n + warp * 32; v0 < a.scan_end; v0 += nw * 32) {
+      const int64_t v = v0 + lane;
+      int part = -1;
+      if (v < a.scan_end) {
+        const bool dv = a.dV[v] != 0, wr = a.wrote[v] != 0, dn = a.dN[v] != 0;
+        const int64_t len = __ldg(a.off + v + 1) - __ldg(a.off + v);
+        if (dv) part = len > kLong0 ? 0 : len > kLong1 ? 1 : len > kLong2 ? 2 : 3;
+        else if (wr || dn) skip_vertex(a, c, (int32_t)v, wr, dn);
+      }
+      uint32_t b[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) b[p] = __ballot_sync(kFull, part == p);
+      const uint32_t all = b[0] | b[1] | b[2] | b[3];
+      if (!all) continue;
+      if (lane == 0) aff += __popc(all);
+      const uint32_t mine = lane == 0 ? b[0] : lane == 1 ? b[1] : lane == 2 ? b[2] : b[3];
+      unsigned int at = 0;
+      if (lane < 4 && mine) at = atomicAdd(&c.slot->act[lane], (unsigned int)__popc(mine));
+      at = __shfl_sync(kFull, at, part < 0 ? 0 : part);
+      const uint32_t same = __shfl_sync(kFull, mine, part < 0 ? 0 : part);
+      if (part >= 0) a.act[a.cls[part].list + at + __popc(same & ((1u << lane) - 1u))] = (int32_t)v;
+    }
+  }
+  for (int64_t v0 = warp * a.scan_rows; v0 < n; v0 += nw * a.scan_rows) {
+    // lane's word: rows v0 + 32 lane ..
+    uint32_t mdv = 0, mwr = 0, mdn = 0;
+    const int64_t w0 = v0 + 32 * lane;
+    if (32 * lane < a.scan_rows && w0 < n) {
+      const uint4 f[6] = {*reinterpret_cast<const uint4*>(a.dV + w0),    *reinterpret_cast<const uint4*>(a.dV + w0 + 16),
+                          *reinterpret_cast<const uint4*>(a.wrote + w0), *reinterpret_cast<const uint4*>(a.wrote + w0 + 16),
+                          *reinterpret_cast<const uint4*>(a.dN + w0),    *reinterpret_cast<const uint4*>(a.dN + w0 + 16)};
+      // four flag bytes (0 or 1) to four bits
+      auto bits4 = [](uint32_t x) { return ((x * 0x10204080u) >> 28) & 0xFu; };
+      auto bits16 = [&](const uint4& q) {
+        return bits4(q.x) | bits4(q.y) << 4 | bits4(q.z) << 8 | bits4(q.w) << 12;
+      };
+      const uint32_t in = n - w0 >= 32 ? kFull : (1u << (int)(n - w0)) - 1u;
+      mdv = (bits16(f[0]) | bits16(f[1]) << 16) & in;
+      mwr = (bits16(f[2]) | bits16(f[3]) << 16) & in;
+      mdn = (bits16(f[4]) | bits16(f[5]) << 16) & in;
+    }
+    uint32_t todo = __ballot_sync(kFull, ((mwr | mdn) & ~mdv) != 0);
+    while (todo) {
+      const int i = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const uint32_t w = __shfl_sync(kFull, mwr & ~mdv, i), d = __shfl_sync(kFull, mdn & ~mdv, i);
+      const bool bw = (w >> lane) & 1u, bd = (d >> lane) & 1u;
+      if (bw || bd) skip_vertex(a, c, (int32_t)(v0 + 32 * i + lane), bw, bd);
+    }
+    if (!__any_sync(kFull, mdv != 0)) continue;
+    aff += __popc(mdv);
+    for (int k = 0; k < a.ncls; ++k) {  // (one class, but for the stretches that hold a class bound)
+      const int64_t cb = a.cls[k].begin - v0, ce = a.cls[k].end - v0;
+      if (ce <= 0 || cb >= a.scan_rows || a.cls[k].part >= 0) continue;
+      // rows of this class among the word's: bits [lo, hi)
+      const int lo = (int)(cb - 32 * lane < 0 ? 0 : cb - 32 * lane > 32 ? 32 : cb - 32 * lane);
+      const int hi = (int)(ce - 32 * lane < 0 ? 0 : ce - 32 * lane > 32 ? 32 : ce - 32 * lane);
+      uint32_t m = mdv;
+      m &= lo >= 32 ? 0u : kFull << lo;
+      m &= hi >= 32 ? kFull : (1u << hi) - 1u;
+      const int cnt = __popc(m);
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += x;
+      }
+      unsigned int base = 0;
+      if (lane == 31 && incl) base = atomicAdd(&c.slot->act[k], (unsigned int)incl);
+      base = __shfl_sync(kFull, base, 31);
+      int32_t* out = a.act + a.cls[k].list + base;
+      uint32_t some = __ballot_sync(kFull, m != 0);
+      while (some) {
+        const int i = __ffs(some) - 1;
+        some &= some - 1;
+        const uint32_t w = __shfl_sync(kFull, m, i);
+        const int at = __shfl_sync(kFull, incl - cnt, i);
+        if ((w >> lane) & 1u) out[at + __popc(w & ((1u << lane) - 1u))] = (int32_t)(v0 + 32 * i + lane);
+      }
+    }
+  }
+  if (it == 0) {
+    aff = __reduce_add_sync(kFull, aff);
+    if (lane == 0 && aff) atomicAdd(&a.ctl->aff0, aff);
+  }
+}
+
 template <class P, bool DYN>
-__device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int it) {
+__device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int it, const Plan* plan) {
   Ctx<P> c;
   c.x = (it & 1) ? a.xb : a.xa;
   c.xn = (it & 1) ? a.xa : a.xb;
@@ -741,27 +843,32 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
   c.pl = policy_evict_last();
   c.lane = threadIdx.x & 31;
   Tally t;
-  // first unit by position (consecutive units on different SMs), the rest from the counter
+  // First unit by position (consecutive units on different SMs). The others
+  // come from a counter, or by position again when there are few per warp: the
+  // counter is one address, and thousands of warps asking at once wait for
+  // one another longer than a short sweep lasts.
   const unsigned int nw = gridDim.x * kWarps;
-  unsigned int u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  while (u < a.units) {
-    unsigned int nx = 0;
-    if (c.lane == 0) nx = atomicAdd(&c.slot->units, 1u);
-    if (u < (unsigned int)a.hub.nchunk) {
-      unit_hub<P, DYN>(a, c, u, t);
+  const bool counted = plan->total > 4 * nw;
+  for (unsigned int u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < plan->total;) {
+    unsigned int nx = u;
+    if (counted && c.lane == 0) nx = atomicAdd(&c.slot->units, 1u);
+    if (u < plan->chunk_units) {
+      const unsigned int nchunk = (unsigned int)__ldg(a.nchunk);
+      const unsigned int cb = u * a.chunks_per_unit;
+      const unsigned int cnt = nchunk - cb < a.chunks_per_unit ? nchunk - cb : a.chunks_per_unit;
+      unit_chunks<P, DYN>(a, c, cb, (int)cnt, t);
     } else {
       int k = 0;
-      while (k + 1 < a.ncls && u >= a.cls[k + 1].unit0) ++k;
-      const SweepClass& cl = a.cls[k];
-      const int64_t vb = cl.begin + (int64_t)(u - cl.unit0) * cl.rows;
-      const int64_t ve = vb + cl.rows < cl.end ? vb + cl.rows : cl.end;
-      switch (cl.kind) {
-        case kRowSelf: unit_self<P, DYN>(a, c, vb, ve, t); break;
-        case kRowThread: unit_thread<P, 4, DYN>(a, c, vb, ve, t); break;
-        case kRow4: unit_group<P, 4, DYN>(a, c, vb, ve, t); break;
-        case kRow8: unit_group<P, 8, DYN>(a, c, vb, ve, t); break;
-        case kRow16: unit_group<P, 16, DYN>(a, c, vb, ve, t); break;
-        default: unit_group<P, 32, DYN>(a, c, vb, ve, t); break;
+      while (k + 1 < a.ncls && u >= plan->unit0[k + 1]) ++k;
+      const int64_t kb = plan->begin[k] + (int64_t)(u - plan->unit0[k]) * plan->rows[k];
+      const int64_t ke = kb + plan->rows[k] < plan->end[k] ? kb + plan->rows[k] : plan->end[k];
+      switch (a.cls[k].kind) {
+        case kRowSelf: unit_self<P, DYN>(a, c, kb, ke, t); break;
+        case kRowThread: unit_thread<P, 4, DYN>(a, c, kb, ke, t); break;
+        case kRow4: unit_group<P, 4, DYN>(a, c, kb, ke, t); break;
+        case kRow8: unit_group<P, 8, DYN>(a, c, kb, ke, t); break;
+        case kRow16: unit_group<P, 16, DYN>(a, c, kb, ke, t); break;
+        default: unit_group<P, 32, DYN>(a, c, kb, ke, t); break;
       }
     }
     u = nw + __shfl_sync(kFull, nx, 0);
@@ -865,34 +972,113 @@ __device__ void push_round(const SweepArgs<Real>& a, const unsigned int* count) 
 
 // Pull form over G' (the same marks, since w is an out-neighbour of u exactly
 // when u is an in-neighbour of w): a vertex outside dV joins it when an
-// in-neighbour is in the frontier. Only w's own thread (or warp) reads or
-// writes dV[w]; the scan stops at the first frontier in-neighbour. Rows below
-// pull_warp_b take a thread each, the others a warp.
+// in-neighbour is in the frontier. Only w's own lanes read or write dV[w]; the
+// scan of a row stops at its first frontier in-neighbour. A warp takes the
+// rows of a class outside dV among 32, G lanes per row with four entries each
+// in flight (a lane per row and serial loads before: the longest rows of 128
+// entries set the round's time).
+template <class Real, int G>
+__device__ __forceinline__ void pull_rows(const SweepArgs<Real>& a, int64_t vb, int64_t ve, int64_t warp, int64_t nw,
+                                          uint64_t pf) {
+  const int lane = threadIdx.x & 31, sub = lane & (G - 1), grp = lane / G;
+  constexpr int NG = 32 / G;
+  int64_t v = vb + warp * 32 + lane;
+  bool out = v < ve && a.dV[v] == 0;
+  for (int64_t v0 = vb + warp * 32; v0 < ve; v0 += nw * 32) {
+    v = v0 + lane;
+    uint32_t m = __ballot_sync(kFull, out);
+    const int64_t w = v + nw * 32;  // the next rows' flags load ahead
+    out = w < ve && a.dV[w] == 0;
+    if (!m) continue;
+    int64_t b = 0;
+    int len = 0;
+    if ((m >> lane) & 1u) {
+      b = ld_stream_i64(a.off + v, pf);
+      len = (int)(ld_stream_i64(a.off + v + 1, pf) - b);
+    }
+    while (m) {
+      // the next NG rows, one per group
+      int r = -1;
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        const int l = m ? __ffs(m) - 1 : -1;
+        m &= m - 1;  // (0 stays 0)
+        if (g == grp) r = l;
+      }
+      const int64_t rb = __shfl_sync(kFull, b, r < 0 ? 0 : r);
+      const int rl = __shfl_sync(kFull, len, r < 0 ? 0 : r);
+      const int lo = (int)(rb & 3);
+      const int32_t* base = a.adj + (rb & ~(int64_t)3);
+      int hi = r < 0 ? 0 : lo + rl;
+      bool hit = false;
+      for (int j = 4 * sub; __any_sync(kFull, j - 4 * sub < hi); j += 4 * G) {
+        int32_t u[4];
+        mask4(load4(base, j, hi, pf), j, lo, hi, u);
+        uint8_t f[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f[k] = u[k] >= 0 ? a.dN[u[k]] : (uint8_t)0;
+        const uint32_t any = __ballot_sync(kFull, (f[0] | f[1] | f[2] | f[3]) != 0);
+        const uint32_t mine = G == 32 ? any : (any >> (lane & ~(G - 1))) & ((1u << (G & 31)) - 1u);
+        if (mine) {
+          hit = true;
+          hi = 0;  // this group is done
+        }
+      }
+      if (hit && sub == 0) a.dV[v0 + r] = 1;
+    }
+  }
+}
+
+// one vertex of the in-degree <= 1 class
+template <class Real>
+__device__ __forceinline__ void pull_self(const SweepArgs<Real>& a, int64_t v) {
+  if (a.dV[v]) return;
+  bool hit = a.dN[v] != 0;
+  if (!hit && a.multi && ((a.multi[v >> 5] >> (v & 31)) & 1u)) {
+    const int64_t e = a.off[v + 1];
+    for (int64_t j = a.off[v]; j < e && !hit; ++j) hit = a.dN[a.adj[j]] != 0;
+  }
+  if (hit) a.dV[v] = 1;
+}
+
 template <class Real>
 __device__ void pull_round(const SweepArgs<Real>& a) {
   const int lane = threadIdx.x & 31;
+  const uint64_t pf = policy_evict_first();
   const int64_t nw = (int64_t)gridDim.x * kWarps;
   const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  for (int64_t w = a.pull_warp_b + warp; w < a.n; w += nw) {
-    if (__shfl_sync(kFull, lane == 0 ? (int)a.dV[w] : 0, 0)) continue;
-    const int64_t b = a.off[w], e = a.off[w + 1];
-    for (int64_t j0 = b; j0 < e; j0 += 32) {
-      const int64_t j = j0 + lane;
-      const bool hit = j < e && a.dN[a.adj[j]];
-      if (__any_sync(kFull, hit)) {
-        if (lane == 0) a.dV[w] = 1;
+  pull_rows<Real, 32>(a, a.scan_end, a.n, warp, nw, pf);
+  for (int k = 0; k < a.ncls; ++k) {
+    const SweepClass& cl = a.cls[k];
+    if (cl.part > 0) continue;  // (the class's other parts list the same rows)
+    switch (cl.kind) {
+      case kRowSelf:
+        // the row is [v], so v joins when it is in the frontier itself: 16 flags
+        // at a time inside the class, its ragged ends and the vertices that
+        // gained in-edges one by one
+        {
+          const int64_t wb = (cl.begin + 15) >> 4, we = cl.end >> 4;
+          for (int64_t w = wb + warp * 32 + lane; w < we; w += nw * 32) {
+            const uint4 d = reinterpret_cast<const uint4*>(a.dV)[w], f = reinterpret_cast<const uint4*>(a.dN)[w];
+            const uint4 o = make_uint4(d.x | f.x, d.y | f.y, d.z | f.z, d.w | f.w);
+            if (o.x != d.x || o.y != d.y || o.z != d.z || o.w != d.w) reinterpret_cast<uint4*>(a.dV)[w] = o;
+            if (a.multi && ((a.multi[w >> 1] >> (16 * (w & 1))) & 0xFFFFu))
+              for (int64_t v = 16 * w; v < 16 * w + 16; ++v) pull_self(a, v);
+          }
+          if (warp == 0) {
+            const int64_t b0 = cl.begin, b1 = wb * 16 < cl.end ? wb * 16 : cl.end;
+            for (int64_t v = b0 + lane; v < b1; v += 32) pull_self(a, v);
+            const int64_t e0 = we * 16 > b1 ? we * 16 : b1;
+            for (int64_t v = e0 + lane; v < cl.end; v += 32) pull_self(a, v);
+          }
+        }
         break;
-      }
+      case kRowThread:
+      case kRow4: pull_rows<Real, 4>(a, cl.begin, cl.end, warp, nw, pf); break;
+      case kRow8: pull_rows<Real, 8>(a, cl.begin, cl.end, warp, nw, pf); break;
+      case kRow16: pull_rows<Real, 16>(a, cl.begin, cl.end, warp, nw, pf); break;
+      default: pull_rows<Real, 32>(a, cl.begin, cl.end, warp, nw, pf); break;
     }
-  }
-  for (int64_t w = warp * 32 + lane; w < a.pull_warp_b; w += nw * 32) {
-    if (a.dV[w]) continue;
-    const int64_t e = a.off[w + 1];
-    for (int64_t j = a.off[w]; j < e; ++j)
-      if (a.dN[a.adj[j]]) {
-        a.dV[w] = 1;
-        break;
-      }
   }
 }
 
@@ -911,13 +1097,19 @@ __device__ __forceinline__ void expand_round(const SweepArgs<Real>& a, LoopSlot*
 // once.
 template <class P, bool DYN>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) k_rank_loop(const __grid_constant__ SweepArgs<typename P::Real> a) {
+  __shared__ Plan plan;
   if (a.mode == kLoopPush) {
     if (DYN) push_round(a, &a.ctl->nlist0);
     return;
   }
-  if (a.mode == kLoopSweep) {
+  if (a.mode == kLoopScan || a.mode == kLoopSweep) {
     if (a.it0 > 0 && stopped(__ldcg(&slot_of(a, a.it0 - 1)->resid), a.tol)) return;
-    sweep<P, DYN>(a, a.it0);
+    if (a.mode == kLoopScan) {
+      if (DYN) scan<P>(a, a.it0);
+      return;
+    }
+    make_plan<DYN>(a, slot_of(a, a.it0), &plan);
+    sweep<P, DYN>(a, a.it0, &plan);
     return;
   }
   if (a.mode == kLoopExpand) {
@@ -930,10 +1122,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_rank_loop(const __grid
     push_round(a, &a.ctl->nlist0);
     if (!grid_barrier(a.ctl, target)) return;
   }
+  if (!DYN) make_plan<DYN>(a, a.slot, &plan);
   for (int it = 0;; ++it) {
-    sweep<P, DYN>(a, it);
-    if (!grid_barrier(a.ctl, target)) return;
     LoopSlot* sl = slot_of(a, it);
+    if (DYN) {
+      scan<P>(a, it);
+      if (!grid_barrier(a.ctl, target)) return;
+      make_plan<DYN>(a, sl, &plan);
+    }
+    sweep<P, DYN>(a, it, &plan);
+    if (!grid_barrier(a.ctl, target)) return;
     const unsigned long long resid = __ldcg(&sl->resid);
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     if (stopped(resid, a.tol) || it + 1 >= a.max_iter) {
@@ -985,8 +1183,40 @@ __global__ void k_mark_batch(const int32_t* __restrict__ del_src, const int32_t*
   }
 }
 
+// Chunk table: a row is cut into ceil(len / size) chunks (one when empty).
+__global__ void k_chunk_count(const int64_t* __restrict__ off, int64_t begin, int64_t rows, int size,
+                              uint32_t* __restrict__ cnt) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t d = off[begin + i + 1] - off[begin + i];
+    cnt[i] = d > 0 ? (uint32_t)((d + size - 1) / size) : 1u;
+  }
+}
+
+__global__ void k_chunk_fill(const int64_t* __restrict__ off, int64_t begin, int64_t rows, int size,
+                             const int64_t* __restrict__ first, SweepChunk* __restrict__ chunks) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = warp; i < rows; i += nwarps) {
+    const int64_t b = off[begin + i], e = off[begin + i + 1], f = first[i];
+    const int parts = (int)(first[i + 1] - f);
+    for (int p = lane; p < parts; p += 32) {
+      const int64_t j0 = b + (int64_t)p * size;
+      SweepChunk k;
+      k.j0 = j0;
+      k.len = (int)(e - j0 < size ? e - j0 : size);
+      k.v = (int32_t)(begin + i);
+      k.first = (int32_t)f;
+      k.parts = parts;
+      k.row = (int32_t)i;
+      k.pad = 0;
+      chunks[f + p] = k;
+    }
+  }
+}
+
 // Kernel shape of class c by its upper degree bound; the last class runs in
-// hub chunks and the one before it a warp per row.
+// chunks and the one before it a warp per row (or in chunks).
 int class_kind(const PartThr& t, int c, bool self_loops) {
   const int C = t.n + 1;
   if (c == C - 2 && C >= 3) return kRowWarp;
@@ -1021,53 +1251,51 @@ struct Launcher {
     return PRDF_OK;
   }
 
-  // units of rows per class, long rows first
-  static int plan(Args& a, const PartThr& t, const int64_t* cb, int max_b) {
-    const int C = t.n + 1;
-    const int64_t n = cb[C];
-    const double warps = (double)max_b * kWarps;
-    // a unit's share of the sweep: about an eighth of a warp's work, at least
-    // two short steps, at most a few thousand edges
-    double target = ((double)a.m + 6.0 * (double)n) / (warps * 8.0);
-    if (target < 96) target = 96;
-    if (target > 4096) target = 4096;
-    int64_t units = a.hub.nchunk;
+  // classes outside the chunk table, long rows first
+  static void classes(Args& a, const PartThr& t, const int64_t* cb) {
     a.ncls = 0;
-    for (int c = C - 2; c >= 0; --c) {
+    a.scan_end = cb[a.chunk_class];
+    int64_t extra = a.n;  // lists of the parts of the longest rows follow the n first entries
+    for (int c = a.chunk_class - 1; c >= 0; --c) {
       const int64_t cnt = cb[c + 1] - cb[c];
       if (cnt <= 0) continue;
-      const int kind = class_kind(t, c, a.self_loops != 0);
       const double lo = c > 0 ? (double)t.thr[c - 1] + 1 : 1, hi = (double)t.thr[c];
-      const double deg = (lo + hi) / 2 < 2.5 * lo ? (lo + hi) / 2 : 2.5 * lo;
-      const int least = kind == kRowWarp ? 1 : kind == kRow16 ? 2 : kind == kRow8 ? 4 : kind == kRow4 ? 8 : 32;
-      int rows = least;
-      while (rows < 32 * kMaxWords && 2 * rows * (deg + 6) <= target) rows *= 2;
-      SweepClass& k = a.cls[a.ncls++];
+      SweepClass k;
       k.begin = cb[c];
       k.end = cb[c + 1];
-      k.unit0 = (uint32_t)units;
-      k.rows = rows;
-      k.kind = kind;
-      units += (cnt + rows - 1) / rows;
+      k.list = cb[c];
+      k.kind = class_kind(t, c, a.self_loops != 0);
+      k.deg = (float)((lo + hi) / 2 < 2.5 * lo ? (lo + hi) / 2 : 2.5 * lo);
+      k.least = k.kind == kRowWarp ? 1 : k.kind == kRow16 ? 2 : k.kind == kRow8 ? 4 : k.kind == kRow4 ? 8 : 32;
+      k.part = -1;
+      if (DYN && c == a.chunk_class - 1 && k.kind == kRowWarp) {
+        const float deg[4] = {1.4f * kLong0, 1.4f * kLong1, 1.4f * kLong2, 250.f};
+        for (int p = 0; p < 4; ++p) {
+          k.part = p;
+          k.deg = deg[p];
+          k.list = p < 3 ? extra : cb[c];
+          if (p < 3) extra += cnt;
+          a.cls[a.ncls++] = k;
+        }
+        continue;
+      }
+      a.cls[a.ncls++] = k;
     }
-    if (units >= (int64_t)UINT32_MAX / 2) {
-      set_error("too many work units");
-      return PRDF_EINVAL;
-    }
-    a.units = (uint32_t)units;
-    return PRDF_OK;
   }
 
   static int run(Args a, const PartThr& t, const int64_t* cb, cudaStream_t s) {
     int max_b = 0;
     PRDF_TRY(max_blocks(&max_b));
-    PRDF_TRY(plan(a, t, cb, max_b));
-    // few units: few blocks, and a shorter barrier
-    int64_t blocks = ((int64_t)a.units + kWarps - 1) / kWarps;
+    classes(a, t, cb);
+    // small graphs: few blocks, and a shorter barrier
+    int64_t blocks = ((a.m + 8 * (int64_t)a.n) / 64 + kWarps - 1) / kWarps;
     if (blocks > max_b) blocks = max_b;
     if (blocks < 1) blocks = 1;
+    // rows a warp scans at a time: 1024, fewer when that leaves warps idle
+    a.scan_rows = 1024;
+    while (a.scan_rows > 32 && a.scan_end < (int64_t)a.scan_rows * blocks * kWarps) a.scan_rows /= 2;
     if (a.mode != kLoopAll) {
-      k_rank_loop<P, DYN><<<(unsigned)(a.mode == kLoopSweep ? blocks : max_b), kThreads, 0, s>>>(a);
+      k_rank_loop<P, DYN><<<(unsigned)blocks, kThreads, 0, s>>>(a);
       PRDF_LAUNCH_CHECK();
       return PRDF_OK;
     }
@@ -1088,6 +1316,33 @@ int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t
 
 int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s) {
   return dynamic ? Launcher<PKahan, true>::run(a, t, cb, s) : Launcher<PKahan, false>::run(a, t, cb, s);
+}
+
+int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, SweepChunks& t, Workspace& ws,
+                 cudaStream_t s) {
+  t.rows = n - begin;
+  t.max_chunks = 0;
+  if (t.rows <= 0) {
+    t.rows = 0;
+    return PRDF_OK;
+  }
+  // the number of chunks stays on the device; the table has room for the most there can be
+  t.max_chunks = t.rows + m / size;
+  if (t.max_chunks >= INT32_MAX) {
+    set_error("too many row chunks");
+    return PRDF_EINVAL;
+  }
+  PRDF_TRY(t.cnt.reserve((size_t)t.rows, s));
+  PRDF_TRY(t.first.reserve((size_t)t.rows + 1, s));
+  PRDF_TRY(t.chunks.reserve((size_t)t.max_chunks, s));
+  PRDF_TRY(t.part.reserve((size_t)t.max_chunks, s));
+  PRDF_TRY(t.done.reserve((size_t)t.rows, s));
+  k_chunk_count<<<grid_for(t.rows, 256), 256, 0, s>>>(off, begin, t.rows, size, t.cnt.p);
+  PRDF_LAUNCH_CHECK();
+  PRDF_TRY(exclusive_scan_u32(t.cnt.p, t.rows, t.first.p, ws, s));
+  k_chunk_fill<<<grid_for(t.rows * 32, 256), 256, 0, s>>>(off, begin, t.rows, size, t.first.p, t.chunks.p);
+  PRDF_LAUNCH_CHECK();
+  return PRDF_OK;
 }
 
 int launch_mark_batch(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
