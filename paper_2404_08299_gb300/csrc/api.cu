@@ -96,33 +96,23 @@ __global__ void k_widen_keep(const float* __restrict__ y, int32_t n, double* __r
   }
 }
 
-// dst[i, :] = src[perm[i], :] for [n, K] row-major matrices
+// dst[i, c] = scale * src[perm[i], c] for c < K, 0 for K <= c < Kp (row-major, [n, Kp] from [n, K])
 __global__ void k_rows_gather(const double* __restrict__ src, const int32_t* __restrict__ perm, int64_t n, int K,
-                              double* __restrict__ dst) {
-  const int64_t cnt = n * K;
+                              int Kp, double scale, double* __restrict__ dst) {
+  const int64_t cnt = n * Kp;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / K, c = t - i * K;
-    dst[t] = src[(int64_t)perm[i] * K + c];
+    const int64_t i = t / Kp, c = t - i * Kp;
+    dst[t] = c < K ? scale * src[(int64_t)perm[i] * K + c] : 0.0;
   }
 }
 
-// dst[perm[i], :] = scale * src[i, :]
+// dst[perm[i], c] = scale * src[i, c] ([n, K] from [n, Kp])
 __global__ void k_rows_scatter(const double* __restrict__ src, const int32_t* __restrict__ perm, int64_t n, int K,
-                               double* __restrict__ dst, double scale = 1.0) {
+                               int Kp, double* __restrict__ dst, double scale) {
   const int64_t cnt = n * K;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t / K, c = t - i * K;
-    dst[(int64_t)perm[i] * K + c] = scale * src[t];
-  }
-}
-
-// dst[i, :] = scale * src[perm[i], :]
-__global__ void k_rows_gather_scaled(const double* __restrict__ src, const int32_t* __restrict__ perm, int64_t n,
-                                     int K, double scale, double* __restrict__ dst) {
-  const int64_t cnt = n * K;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / K, c = t - i * K;
-    dst[t] = scale * src[(int64_t)perm[i] * K + c];
+    dst[(int64_t)perm[i] * K + c] = scale * src[i * Kp + c];
   }
 }
 
@@ -446,8 +436,6 @@ int nonempty_classes(const int64_t* cb, int nclass) {
   return k;
 }
 
-int ensure_hub(prdf_graph* g, const Csr& c, PprHubTable& t, cudaStream_t s);
-int64_t hub_begin(const Relabel& rl);
 
 // ----------------------------------------------------------- the loop ----
 // One loop of synchronous sweeps, Alg. static (every vertex, Eq. 1) or
@@ -567,7 +555,9 @@ int ensure_sweep_chunks(prdf_graph* g, const int64_t* cb, cudaStream_t s) {
     t.valid = false;
     t.first_class = small ? C - 2 : C - 1;
     t.size = small ? 512 : (int)kHubChunk;
-    PRDF_TRY(build_chunks(g->rl.in.off.p, cb[t.first_class], g->n, g->rl.in.m, t.size, t, g->ws, s));
+    PRDF_TRY(build_chunks(g->rl.in.off.p, cb[t.first_class], g->n, g->rl.in.m, t.size, 0, t, g->ws, s));
+    PRDF_TRY(t.part.reserve((size_t)t.max_chunks, s));
+    PRDF_TRY(t.done.reserve((size_t)t.rows, s));
     t.version = g->rl.version;
     t.valid = true;
   }
@@ -743,68 +733,8 @@ int run_loop(prdf_graph* g, const prdf_params* p, bool fp32, bool dynamic, bool 
   return PRDF_OK;
 }
 
-// Launch on s the cached while-loop graph of `slot`, first building it when
-// it was made for another key: a conditional while node whose body is
-// recorded by body(capture stream, conditional handle) (the body ends with a
-// one-thread check that sets the condition).
-template <class Body>
-int launch_while_graph(prdf_graph* g, int slot, const std::vector<uint64_t>& key, Body body, cudaStream_t s) {
-  if (!g->loop_exec[slot] || g->loop_key[slot] != key) {
-    if (g->loop_exec[slot]) {
-      cudaGraphExecDestroy(g->loop_exec[slot]);
-      g->loop_exec[slot] = nullptr;
-    }
-    if (!g->cap_stream) PRDF_CUDA(cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    PRDF_CUDA(cudaGraphCreate(&graph, 0));
-    cudaGraphConditionalHandle h;
-    cudaError_t e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
-    alignas(cudaGraphNodeParams) unsigned char np_storage[sizeof(cudaGraphNodeParams)];
-    memset(np_storage, 0, sizeof(np_storage));
-    cudaGraphNodeParams& np = *reinterpret_cast<cudaGraphNodeParams*>(np_storage);
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = h;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    cudaGraphNode_t node;
-    if (e == cudaSuccess) e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
-    cudaGraph_t bodyg = e == cudaSuccess ? np.conditional.phGraph_out[0] : nullptr;
-    if (e == cudaSuccess)
-      e = cudaStreamBeginCaptureToGraph(g->cap_stream, bodyg, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
-    int rc = PRDF_OK;
-    if (e == cudaSuccess) {
-      rc = body(g->cap_stream, h);
-      cudaGraph_t captured = nullptr;
-      cudaError_t e2 = cudaStreamEndCapture(g->cap_stream, &captured);
-      if (e == cudaSuccess) e = e2;
-    }
-    cudaGraphExec_t exec = nullptr;
-    if (e == cudaSuccess && rc == PRDF_OK) e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (rc != PRDF_OK) return rc;
-    if (e != cudaSuccess) {
-      set_error("building the iteration graph: %s", cudaGetErrorString(e));
-      return PRDF_ECUDA;
-    }
-    g->loop_exec[slot] = exec;
-    g->loop_key[slot] = key;
-  }
-  PRDF_CUDA(cudaGraphLaunch(g->loop_exec[slot], s));
-  return PRDF_OK;
-}
-
-// key words of a graph: the raw bytes of the values it was captured with
-struct KeyWriter {
-  std::vector<uint64_t> key;
-  void put(const void* p, size_t nb) {
-    const size_t at = key.size();
-    key.resize(at + (nb + 7) / 8, 0);
-    memcpy(key.data() + at, p, nb);
-  }
-  void putv(uint64_t v) { put(&v, sizeof(v)); }
-};
-
-int auto_tile(int K) { return K >= 64 ? 64 : (K >= 32 ? 32 : (K > 8 ? 16 : 8)); }
+// the narrowest column tile that holds K columns in one pass (64 at most)
+int auto_tile(int K) { return K > 32 ? 64 : (K > 16 ? 32 : (K > 8 ? 16 : 8)); }
 
 // the K-column fixed-point operator: forward pull over G' (P on in-slots) or
 // adjoint pull over G (P on out-slots)
@@ -813,263 +743,186 @@ struct KOp {
   const int32_t* adj;
   const float* p32;
   const double* p64;
-  int64_t hub_begin;  // first vertex of the two highest in-degree classes
-  const PprHubTable* hub;  // chunks of the highest class's rows of this CSR
-  const double* S64;  // right-hand side (dense [n, K]), also the start of the iteration
-  bool sparse_rhs;    // look for few non-zero rows in S64 (a teleport on a few seed vertices)
-  int slot;           // first of the four graph-cache slots of this operator's loops
+  const SweepChunks* chunks; // of the long rows
+  const double* S64;         // right-hand side (dense [n, Kp]), also the start of the iteration
+  bool sparse_rhs;           // look for few non-zero rows in S64 (a teleport on a few seed vertices)
 };
 
-int64_t hub_begin(const Relabel& rl) {
-  const int C = rl.thr.n + 1;
-  int64_t cb[kMaxThr + 2];
-  begins_from_counts(rl.count, C, cb);
-  return C >= 3 ? cb[C - 2] : cb[C - 1];
-}
-
-int64_t blk_begin(const Relabel& rl) {
-  const int C = rl.thr.n + 1;
-  int64_t cb[kMaxThr + 2];
-  begins_from_counts(rl.count, C, cb);
-  return cb[C - 1];
-}
-
-// kernels of one K-column FP32 tile: groups, warps, hub partials and hub finish
-int ppr32_kernels(int64_t hub_b, int64_t blk_b, int64_t n) {
-  return (hub_b > 0 ? 1 : 0) + (blk_b > hub_b ? 1 : 0) + (n > blk_b ? 2 : 0);
-}
-
-// chunk table of the highest in-degree class's rows of one CSR, rebuilt when the numbering changes
-int ensure_hub(prdf_graph* g, const Csr& c, PprHubTable& t, cudaStream_t s) {
-  if (t.valid && t.version == g->rl.version) return PRDF_OK;
-  PRDF_TRY(build_ppr_hub(c.off.p, blk_begin(g->rl), g->n, t, g->ws, s));
+// Chunk table of the rows of one CSR above `above` edges, wherever they are
+// (the numbering follows the in-degrees, the adjoint sums over out-rows),
+// rebuilt when the numbering or the bound changes.
+constexpr int kPprChunk = 512;
+int ppr_long_row(int tile) { return tile <= 16 ? 32 : 128; }
+int ensure_ppr_chunks(prdf_graph* g, const Csr& c, int tile, SweepChunks& t, cudaStream_t s) {
+  const int above = ppr_long_row(tile);
+  if (t.valid && t.version == g->rl.version && t.above == above) return PRDF_OK;
+  t.valid = false;
+  PRDF_TRY(build_chunks(c.off.p, 0, g->n, c.m, kPprChunk, above, t, g->ws, s));
+  t.size = kPprChunk;
+  t.above = above;
   t.version = g->rl.version;
   t.valid = true;
   return PRDF_OK;
 }
 
-// FP32 K-column solve of R = alpha P^T R + (1 - alpha) rhs from the start held
-// in *cur; on return *cur holds the result (the other buffer is scratch).
-int ppr32_solve(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, const float* rhs,
-                const int32_t* srow, float** cur, float** other, int max_iter, int* iters, long long* kernels,
-                cudaStream_t s) {
-  PRDF_TRY(g->resid32.reserve(2 * ((size_t)max_iter + 1), s));
-  PRDF_CUDA(cudaMemsetAsync(g->resid32.p, 0, sizeof(uint32_t) * 2 * ((size_t)max_iter + 1), s));
-  PRDF_TRY(g->ppr_part.reserve((size_t)(op.hub->nchunk > 0 ? op.hub->nchunk : 1) * (size_t)tile, s));
-  Ppr32Args a;
+// Arguments of a K-column loop over op from Ra (the other buffer: Rb).
+template <class T>
+int ppr_args(prdf_graph* g, const KOp& op, const prdf_params* p, int Kp, int tile, const T* P, T* Ra, T* Rb,
+             const T* rhs, const int32_t* srow, int max_iter, PprArgs<T>* out, cudaStream_t s) {
+  PprArgs<T>& a = *out;
   memset(&a, 0, sizeof(a));
+  const SweepChunks& ch = *op.chunks;
+  const size_t tiles = (size_t)((Kp + tile - 1) / tile);
   a.off = op.off;
   a.adj = op.adj;
-  a.P = op.p32;
+  a.P = P;
+  a.Ra = Ra;
+  a.Rb = Rb;
   a.S = rhs;
   a.srow = srow;
-  a.K = K;
-  a.alpha = (float)p->alpha;
-  a.beta = (float)(1.0 - p->alpha);
-  a.tol_rel = (float)p->tol_fp32_rel;
-  const int64_t hb = op.hub_begin;
-  const int check = p->check_every > 0 ? p->check_every : 8;
-  float* buf[2] = {*cur, *other};
-  const int tiles = (K + tile - 1) / tile;
-  if (!p->time_sweeps) {
-    // one CUDA graph: a while node over one sweep (every column tile) and the stop check
-    PRDF_TRY(g->ctl.reserve(2, s));
-    PRDF_CUDA(cudaMemsetAsync(g->ctl.p, 0, 2 * sizeof(int), s));
-    a.ctl = g->ctl.p;
-    a.Ra = buf[0];
-    a.Rb = buf[1];
-    a.resid_base = g->resid32.p;
-    const PprHub hv = op.hub->view();
-    KeyWriter kw;
-    kw.put(&a, sizeof(a));
-    kw.put(&hv, sizeof(hv));
-    kw.putv((uint64_t)tile | ((uint64_t)max_iter << 32));
-    kw.putv((uint64_t)hb);
-    kw.putv((uint64_t)(uintptr_t)g->ppr_part.p);
-    kw.putv((uint64_t)g->n);
-    PRDF_TRY(launch_while_graph(g, op.slot + (srow ? 1 : 0), kw.key, [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
-      int rc = launch_ppr32_sweep(a, tile, g->n, hb, hv, g->ppr_part.p, cs);
-      if (rc == PRDF_OK) rc = launch_iter_check32(g->ctl.p, g->resid32.p, a.tol_rel, max_iter, h, cs);
-      return rc;
-    }, s));
-    int hit = 0;
-    PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    PRDF_CUDA(cudaStreamSynchronize(s));
-    memcpy(&hit, g->ws.host_i64, sizeof(int));
-    if (hit < 1 || hit > max_iter) {
-      set_error("K-column graph ran %d sweeps", hit);
-      return PRDF_ECUDA;
-    }
-    const int k = hit - 1;
-    *iters = hit;
-    *cur = buf[(k + 1) & 1];
-    *other = buf[k & 1];
-    *kernels += (long long)hit * (tiles * ppr32_kernels(hb, op.hub->begin, g->n) + 1);
-    return PRDF_OK;
-  }
-  int launched = 0;
-  bool done = false;
-  while (launched < max_iter && !done) {
-    const int upto = (launched + check < max_iter) ? launched + check : max_iter;
-    for (int i = launched; i < upto; ++i) {
-      a.R = buf[i & 1];
-      a.Rn = buf[(i + 1) & 1];
-      a.resid = g->resid32.p + 2 * i;
-      a.prev = i > 0 ? g->resid32.p + 2 * (i - 1) : nullptr;
-      PRDF_TRY(launch_ppr32_sweep(a, tile, g->n, hb, op.hub->view(), g->ppr_part.p, s));
-    }
-    launched = upto;
-    PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->resid32.p + 2 * (launched - 1), 2 * sizeof(uint32_t),
-                              cudaMemcpyDeviceToHost, s));
-    PRDF_CUDA(cudaStreamSynchronize(s));
-    uint32_t h[2];
-    memcpy(h, g->ws.host_i64, sizeof(h));
-    float d, r;
-    memcpy(&d, &h[0], 4);
-    memcpy(&r, &h[1], 4);
-    done = d <= (float)p->tol_fp32_rel * r;
-  }
-  std::vector<uint32_t> hr(2 * (size_t)launched);
-  PRDF_CUDA(cudaMemcpyAsync(hr.data(), g->resid32.p, sizeof(uint32_t) * 2 * launched, cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
-  int k = launched - 1;
-  for (int i = 0; i < launched; ++i) {
-    float d, r;
-    memcpy(&d, &hr[2 * i], 4);
-    memcpy(&r, &hr[2 * i + 1], 4);
-    if (d <= (float)p->tol_fp32_rel * r) {
-      k = i;
-      break;
-    }
-  }
-  *iters = k + 1;
-  *cur = buf[(k + 1) & 1];
-  *other = buf[k & 1];
-  *kernels += (long long)launched * tiles * ppr32_kernels(hb, op.hub->begin, g->n);
+  a.K = Kp;
+  a.alpha = (T)p->alpha;
+  a.beta = (T)(1.0 - p->alpha);
+  a.inv_beta = (T)(1.0 / (1.0 - p->alpha));
+  a.tol = sizeof(T) == 4 ? (T)p->tol_fp32_rel : (T)p->tol;
+  a.max_iter = max_iter;
+  a.row_end = g->n;
+  a.row_max = ch.above;
+  a.chunks = ch.chunks.p;
+  a.nchunk = ch.rows > 0 ? ch.first.p + ch.rows : nullptr;
+  a.max_chunks = ch.max_chunks;
+  a.chunk_rows = ch.rows;
+  PRDF_TRY(g->ppr_part.reserve(tiles * (size_t)(ch.max_chunks > 0 ? ch.max_chunks : 1) * (size_t)tile, s));
+  PRDF_TRY(g->ppr_done.reserve(tiles * (size_t)(ch.rows > 0 ? ch.rows : 1), s));
+  a.part = g->ppr_part.p;
+  a.done = g->ppr_done.p;
+  PRDF_CUDA(cudaMemsetAsync(a.done, 0, sizeof(uint32_t) * tiles * (size_t)ch.rows, s));
+  PRDF_TRY(alloc_loop_ctl(g, s));
+  a.ctl = g->loop_ctl.p;
   return PRDF_OK;
 }
 
-// one FP64 Jacobi step Rn = T(R); returns max |T(R) - R|
-int ppr64_step(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, const double* rhs,
-               const int32_t* srow, const double* R, double* Rn, float* res32, double* dmax, long long* kernels,
-               cudaStream_t s) {
-  PRDF_TRY(g->resid.reserve(2, s));
-  PRDF_CUDA(cudaMemsetAsync(g->resid.p, 0, sizeof(uint64_t), s));
-  Ppr64Args a;
-  memset(&a, 0, sizeof(a));
-  a.off = op.off;
-  a.adj = op.adj;
-  a.P = op.p64;
-  a.R = R;
-  a.Rn = Rn;
-  a.S = rhs;
-  a.srow = srow;
-  a.res32 = res32;
-  a.K = K;
-  a.alpha = p->alpha;
-  a.beta = 1.0 - p->alpha;
-  a.inv_beta = 1.0 / (1.0 - p->alpha);
-  a.dmax = g->resid.p;
-  PRDF_TRY(g->ppr_part64.reserve((size_t)(op.hub->nchunk > 0 ? op.hub->nchunk : 1) * (size_t)tile, s));
-  PRDF_TRY(launch_ppr64_step(a, tile, g->n, op.hub_begin, op.hub->view(), g->ppr_part64.p, s));
-  PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->resid.p, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
-  memcpy(dmax, g->ws.host_i64, sizeof(double));
-  *kernels += (long long)((K + tile - 1) / tile) * ppr32_kernels(op.hub_begin, op.hub->begin, g->n);
+bool ppr_stopped(unsigned long long word, float tol, double* delta) {
+  uint32_t r[2];
+  memcpy(r, &word, sizeof(r));
+  float d, m;
+  memcpy(&d, &r[0], 4);
+  memcpy(&m, &r[1], 4);
+  *delta = d;
+  return d <= tol * m;
+}
+bool ppr_stopped(unsigned long long word, double tol, double* delta) {
+  memcpy(delta, &word, sizeof(double));
+  return *delta <= tol;
+}
+
+// Runs the loop of a to its stop rule: one cooperative launch, or (time_sweeps)
+// a launch per sweep from the host, check_every ahead of each residual read.
+// Iteration k writes Rb when k is even. Synchronises the stream.
+template <class T>
+int ppr_loop(prdf_graph* g, const prdf_params* p, PprArgs<T> a, int tile, int* iters, double* delta,
+             int* converged, long long* kernels, cudaStream_t s) {
+  if (!p->time_sweeps) {
+    PRDF_TRY(g->loop_slots.reserve(kLoopRing, s));
+    PRDF_CUDA(cudaMemsetAsync(g->loop_slots.p, 0, sizeof(LoopSlot) * kLoopRing, s));
+    a.slot = g->loop_slots.p;
+    a.mode = kLoopAll;
+    PRDF_TRY(launch_ppr_loop(a, tile, g->n, s));
+    *kernels += 1;
+    PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64 + 16, g->loop_ctl.p, sizeof(LoopCtl), cudaMemcpyDeviceToHost, s));
+    PRDF_CUDA(cudaStreamSynchronize(s));
+    LoopCtl h;
+    memcpy(&h, g->ws.host_i64 + 16, sizeof(h));
+    if (h.timeout) {
+      set_error("the K-column loop gave up waiting for its blocks");
+      return PRDF_ETIMEOUT;
+    }
+    if (h.iters < 1 || h.iters > a.max_iter) {
+      set_error("the K-column loop ran %d sweeps", h.iters);
+      return PRDF_ECUDA;
+    }
+    *iters = h.iters;
+    *converged = ppr_stopped(h.resid, a.tol, delta) ? 1 : 0;
+    return PRDF_OK;
+  }
+  const int check = p->check_every > 0 ? p->check_every : 8;
+  const int window = check < a.max_iter ? check : a.max_iter;
+  PRDF_TRY(g->loop_slots.reserve((size_t)window + 1, s));
+  a.slot = g->loop_slots.p;
+  a.mode = kLoopSweep;
+  std::vector<LoopSlot> slots((size_t)window);
+  int launched = 0;
+  *converged = 0;
+  while (launched < a.max_iter && !*converged) {
+    const int cnt = a.max_iter - launched < window ? a.max_iter - launched : window;
+    // slot 0 holds the sweep before the window
+    if (launched)
+      PRDF_CUDA(cudaMemcpyAsync(g->loop_slots.p, g->loop_slots.p + window, sizeof(LoopSlot), cudaMemcpyDeviceToDevice,
+                                s));
+    PRDF_CUDA(cudaMemsetAsync(g->loop_slots.p + 1, 0, sizeof(LoopSlot) * (size_t)cnt, s));
+    for (int i = launched; i < launched + cnt; ++i) {
+      a.it0 = i;
+      a.it_first = launched;
+      PRDF_TRY(launch_ppr_loop(a, tile, g->n, s));
+    }
+    *kernels += cnt;
+    PRDF_CUDA(cudaMemcpyAsync(slots.data(), g->loop_slots.p + 1, sizeof(LoopSlot) * (size_t)cnt,
+                              cudaMemcpyDeviceToHost, s));
+    PRDF_CUDA(cudaStreamSynchronize(s));
+    for (int i = 0; i < cnt && !*converged; ++i) {
+      *converged = ppr_stopped(slots[(size_t)i].resid, a.tol, delta) ? 1 : 0;
+      *iters = launched + i + 1;
+    }
+    launched += cnt;
+  }
+  return PRDF_OK;
+}
+
+// FP32 K-column solve of R = alpha P^T R + (1 - alpha) rhs from the start held
+// in *cur; on return *cur holds the result (the other buffer is scratch).
+int ppr32_solve(prdf_graph* g, const KOp& op, const prdf_params* p, int Kp, int tile, const float* rhs,
+                const int32_t* srow, float** cur, float** other, int max_iter, int* iters, long long* kernels,
+                cudaStream_t s) {
+  PprArgs<float> a;
+  PRDF_TRY(ppr_args(g, op, p, Kp, tile, op.p32, *cur, *other, rhs, srow, max_iter, &a, s));
+  double delta;
+  int conv;
+  PRDF_TRY(ppr_loop(g, p, a, tile, iters, &delta, &conv, kernels, s));
+  if (*iters & 1) {
+    float* t = *cur;
+    *cur = *other;
+    *other = t;
+  }
   return PRDF_OK;
 }
 
 // Solve X = alpha * A X + (1 - alpha) * op.S64 (A = P^T on G' or P on G) from
-// X = S64, K columns in the class-contiguous numbering; result in *out
-// (one of R64a / R64b). Mixed: FP32 solve, then iterative refinement with an
-// FP64 step for the residual and an FP32 solve for the correction.
+// X = S64, K columns (row stride Kp) in the class-contiguous numbering; result
+// in *out (one of R64a / R64b). Mixed: FP32 solve, then iterative refinement
+// with an FP64 step for the residual and an FP32 solve for the correction.
 struct KSolve {
   int iters32 = 0, steps64 = 0, converged = 0;
   double dmax = 0;
   long long kernels = 0;
 };
 
-int ksolve(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, double** out, KSolve* r,
+int ksolve(prdf_graph* g, const KOp& op, const prdf_params* p, int Kp, int tile, double** out, KSolve* r,
            cudaStream_t s) {
-  const int64_t cnt = (int64_t)g->n * K;
+  const int64_t cnt = (int64_t)g->n * Kp;
   PprSparseRhs& sp = g->ppr_rhs;
   sp.rows = 0;
+  PprArgs<double> a64;
   if (p->precision == PRDF_FP64) {
     PRDF_CUDA(cudaMemcpyAsync(g->R64a.p, op.S64, sizeof(double) * cnt, cudaMemcpyDeviceToDevice, s));
     if (op.sparse_rhs) {
-      PRDF_TRY(ppr_sparse_rhs(op.S64, g->n, K, g->ws, &sp, nullptr, s));
+      PRDF_TRY(ppr_sparse_rhs(op.S64, g->n, Kp, g->ws, &sp, nullptr, s));
       r->kernels += 2 + (sp.rows ? 1 : 0);
     }
     const double* rhs = sp.rows ? sp.Sc64.p : op.S64;
     const int32_t* srow = sp.rows ? sp.srow.p : nullptr;
-    if (!p->time_sweeps) {
-      // one CUDA graph: a while node over one FP64 Jacobi step (every column tile) and the stop check
-      const int max_iter = p->max_iter;
-      PRDF_TRY(g->resid.reserve((size_t)max_iter + 1, s));
-      PRDF_CUDA(cudaMemsetAsync(g->resid.p, 0, sizeof(uint64_t) * ((size_t)max_iter + 1), s));
-      PRDF_TRY(g->ctl.reserve(2, s));
-      PRDF_CUDA(cudaMemsetAsync(g->ctl.p, 0, 2 * sizeof(int), s));
-      PRDF_TRY(g->ppr_part64.reserve((size_t)(op.hub->nchunk > 0 ? op.hub->nchunk : 1) * (size_t)tile, s));
-      Ppr64Args pa;
-      memset(&pa, 0, sizeof(pa));
-      pa.off = op.off;
-      pa.adj = op.adj;
-      pa.P = op.p64;
-      pa.S = rhs;
-      pa.srow = srow;
-      pa.K = K;
-      pa.alpha = p->alpha;
-      pa.beta = 1.0 - p->alpha;
-      pa.inv_beta = 1.0 / (1.0 - p->alpha);
-      pa.ctl = g->ctl.p;
-      pa.Ra = g->R64a.p;
-      pa.Rb = g->R64b.p;
-      pa.dmax_base = g->resid.p;
-      const PprHub hv = op.hub->view();
-      KeyWriter kw;
-      kw.put(&pa, sizeof(pa));
-      kw.put(&hv, sizeof(hv));
-      kw.putv((uint64_t)tile | ((uint64_t)max_iter << 32));
-      kw.put(&p->tol, sizeof(p->tol));
-      kw.putv((uint64_t)op.hub_begin);
-      kw.putv((uint64_t)(uintptr_t)g->ppr_part64.p);
-      kw.putv((uint64_t)g->n);
-      PRDF_TRY(launch_while_graph(g, op.slot + 2, kw.key, [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
-        int rc = launch_ppr64_step(pa, tile, g->n, op.hub_begin, hv, g->ppr_part64.p, cs);
-        if (rc == PRDF_OK) rc = launch_iter_check(g->ctl.p, g->resid.p, p->tol, max_iter, h, cs);
-        return rc;
-      }, s));
-      int hit = 0;
-      PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-      PRDF_CUDA(cudaStreamSynchronize(s));
-      memcpy(&hit, g->ws.host_i64, sizeof(int));
-      if (hit < 1 || hit > max_iter) {
-        set_error("K-column graph ran %d steps", hit);
-        return PRDF_ECUDA;
-      }
-      PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, g->resid.p + hit - 1, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-      PRDF_CUDA(cudaStreamSynchronize(s));
-      memcpy(&r->dmax, g->ws.host_i64, sizeof(double));
-      r->steps64 += hit;
-      r->converged = r->dmax <= p->tol ? 1 : 0;
-      r->kernels += (long long)hit * (((K + tile - 1) / tile) * ppr32_kernels(op.hub_begin, op.hub->begin, g->n) + 1);
-      *out = ((hit - 1) & 1) ? g->R64a.p : g->R64b.p;  // step k writes R64b when k is even
-      return PRDF_OK;
-    }
-    double* a = g->R64a.p;
-    double* b = g->R64b.p;
-    for (int it = 0; it < p->max_iter; ++it) {
-      PRDF_TRY(ppr64_step(g, op, p, K, tile, rhs, srow, a, b, nullptr, &r->dmax, &r->kernels, s));
-      ++r->steps64;
-      double* tmp = a;
-      a = b;
-      b = tmp;
-      if (r->dmax <= p->tol) {
-        r->converged = 1;
-        break;
-      }
-    }
-    *out = a;
+    PRDF_TRY(ppr_args(g, op, p, Kp, tile, op.p64, g->R64a.p, g->R64b.p, rhs, srow, p->max_iter, &a64, s));
+    PRDF_TRY(ppr_loop(g, p, a64, tile, &r->steps64, &r->dmax, &r->converged, &r->kernels, s));
+    *out = (r->steps64 & 1) ? g->R64b.p : g->R64a.p;
     return PRDF_OK;
   }
   PRDF_TRY(g->S32.reserve(cnt, s));
@@ -1077,7 +930,7 @@ int ksolve(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, 
   PRDF_TRY(g->R32b.reserve(cnt, s));
   if (op.sparse_rhs) {
     // a teleport on few vertices: the first solve reads a 4-byte row index per vertex instead of its row
-    PRDF_TRY(ppr_sparse_rhs(op.S64, g->n, K, g->ws, &sp, g->R32a.p, s));
+    PRDF_TRY(ppr_sparse_rhs(op.S64, g->n, Kp, g->ws, &sp, g->R32a.p, s));
     r->kernels += 2 + (sp.rows ? 1 : 0);
   }
   const double* rhs64 = sp.rows ? sp.Sc64.p : op.S64;
@@ -1089,7 +942,7 @@ int ksolve(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, 
   float* cur = g->R32a.p;
   float* oth = g->R32b.p;
   int it32 = 0;
-  PRDF_TRY(ppr32_solve(g, op, p, K, tile, sp.rows ? sp.Sc32.p : g->S32.p, srow, &cur, &oth, p->max_iter, &it32,
+  PRDF_TRY(ppr32_solve(g, op, p, Kp, tile, sp.rows ? sp.Sc32.p : g->S32.p, srow, &cur, &oth, p->max_iter, &it32,
                        &r->kernels, s));
   r->iters32 += it32;
   PRDF_TRY(ppr_widen(cur, cnt, g->R64a.p, s));
@@ -1097,16 +950,16 @@ int ksolve(prdf_graph* g, const KOp& op, const prdf_params* p, int K, int tile, 
   const int kRounds = 8;
   for (int round = 0; round < kRounds; ++round) {
     // FP64 Jacobi step: T(R) and the residual (T(R) - R) / (1 - alpha), dense, in S32
-    PRDF_TRY(ppr64_step(g, op, p, K, tile, rhs64, srow, g->R64a.p, g->R64b.p, g->S32.p, &r->dmax, &r->kernels, s));
+    PRDF_TRY(ppr_args(g, op, p, Kp, tile, op.p64, g->R64a.p, g->R64b.p, rhs64, srow, 1, &a64, s));
+    a64.res32 = g->S32.p;
+    int one = 0;
+    PRDF_TRY(ppr_loop(g, p, a64, tile, &one, &r->dmax, &r->converged, &r->kernels, s));
     ++r->steps64;
-    if (r->dmax <= p->tol) {
-      r->converged = 1;
-      break;
-    }
+    if (r->converged) break;
     PRDF_CUDA(cudaMemcpyAsync(g->R32a.p, g->S32.p, sizeof(float) * cnt, cudaMemcpyDeviceToDevice, s));
     cur = g->R32a.p;
     oth = g->R32b.p;
-    PRDF_TRY(ppr32_solve(g, op, p, K, tile, g->S32.p, nullptr, &cur, &oth, p->max_iter, &it32, &r->kernels, s));
+    PRDF_TRY(ppr32_solve(g, op, p, Kp, tile, g->S32.p, nullptr, &cur, &oth, p->max_iter, &it32, &r->kernels, s));
     r->iters32 += it32;
     PRDF_TRY(ppr_add_correction(g->R64a.p, cur, cnt, s));
     r->kernels += 1;
@@ -1291,9 +1144,6 @@ void prdf_graph_destroy(prdf_graph* g) {
   if (!g) return;
   cudaStreamSynchronize(g->stream);
   cudaDeviceSynchronize();
-  for (auto& e : g->loop_exec)
-    if (e) cudaGraphExecDestroy(e);
-  if (g->cap_stream) cudaStreamDestroy(g->cap_stream);
   delete g;
 }
 
@@ -1785,25 +1635,25 @@ int prdf_pagerank_ppr(prdf_graph* g, const double* S, int K, double* R, const pr
   PRDF_CUDA(cudaEventRecord(t.e[0], s));
   PRDF_TRY(ensure_relabelled(g, false, s));
   if (!g->ppr_valid) PRDF_TRY(build_ppr_weights(g, s));
-  const int tile = p->tile ? p->tile : auto_tile(K);
-  const int64_t cnt = (int64_t)g->n * K;
+  const int tile = p->tile && K > 2 ? p->tile : auto_tile(K);
+  const int Kp = padded_cols(K);
+  const int64_t cnt = (int64_t)g->n * Kp;
   PRDF_TRY(g->S64.reserve(cnt, s));
   PRDF_TRY(g->R64a.reserve(cnt, s));
   PRDF_TRY(g->R64b.reserve(cnt, s));
-  k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(S, g->rl.perm.p, g->n, K, g->S64.p);
+  k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(S, g->rl.perm.p, g->n, K, Kp, 1.0, g->S64.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_TRY(ensure_hub(g, g->rl.in, g->hub_in, s));
-  const KOp op{g->rl.in.off.p, g->rl.in.adj.p, g->pin32.p, g->pin64.p, hub_begin(g->rl), &g->hub_in, g->S64.p, true,
-               0};
+  PRDF_TRY(ensure_ppr_chunks(g, g->rl.in, tile, g->ppr_chunks_in, s));
+  const KOp op{g->rl.in.off.p, g->rl.in.adj.p, g->pin32.p, g->pin64.p, &g->ppr_chunks_in, g->S64.p, true};
   KSolve ks;
   ks.kernels = 1;
   double* Rfinal = nullptr;
-  PRDF_TRY(ksolve(g, op, p, K, tile, &Rfinal, &ks, s));
+  PRDF_TRY(ksolve(g, op, p, Kp, tile, &Rfinal, &ks, s));
   long long kernels = ks.kernels;
   const int iters32 = ks.iters32, steps64 = ks.steps64, conv = ks.converged;
   const double dmax = ks.dmax;
-  k_rows_scatter<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(Rfinal, g->rl.perm.p, g->n, K, R);
+  k_rows_scatter<<<grid_for((int64_t)g->n * K, kThreads), kThreads, 0, s>>>(Rfinal, g->rl.perm.p, g->n, K, Kp, R, 1.0);
   PRDF_LAUNCH_CHECK();
   kernels += 1;
   PRDF_CUDA(cudaEventRecord(t.e[2], s));
@@ -1881,35 +1731,36 @@ int prdf_pagerank_backward(prdf_graph* g, const double* R, const double* G, int 
   PRDF_CUDA(cudaEventRecord(t.e[0], s));
   PRDF_TRY(ensure_relabelled(g, false, s));
   if (!g->ppr_valid) PRDF_TRY(build_ppr_weights(g, s));
-  const int tile = p->tile ? p->tile : auto_tile(K);
-  const int64_t cnt = (int64_t)g->n * K;
+  const int tile = p->tile && K > 2 ? p->tile : auto_tile(K);
+  const int Kp = padded_cols(K);
+  const int64_t cnt = (int64_t)g->n * Kp;
   const double beta = 1.0 - p->alpha;
   PRDF_TRY(g->S64.reserve(cnt, s));
   PRDF_TRY(g->R64a.reserve(cnt, s));
   PRDF_TRY(g->R64b.reserve(cnt, s));
   // lambda = alpha P lambda + G, i.e. X = alpha A X + (1 - alpha) * G / (1 - alpha) over the out-CSR
-  k_rows_gather_scaled<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(G, g->rl.perm.p, g->n, K, 1.0 / beta, g->S64.p);
+  k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(G, g->rl.perm.p, g->n, K, Kp, 1.0 / beta, g->S64.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_TRY(ensure_hub(g, g->rl.out, g->hub_out, s));
-  const KOp op{g->rl.out.off.p, g->rl.out.adj.p, g->pout32.p, g->pout64.p, hub_begin(g->rl), &g->hub_out, g->S64.p,
-               false, 4};
+  PRDF_TRY(ensure_ppr_chunks(g, g->rl.out, tile, g->ppr_chunks_out, s));
+  const KOp op{g->rl.out.off.p, g->rl.out.adj.p, g->pout32.p, g->pout64.p, &g->ppr_chunks_out, g->S64.p, false};
   KSolve ks;
   ks.kernels = 1;
   double* lam = nullptr;
-  PRDF_TRY(ksolve(g, op, p, K, tile, &lam, &ks, s));
+  PRDF_TRY(ksolve(g, op, p, Kp, tile, &lam, &ks, s));
   if (grad_S) {
-    k_rows_scatter<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(lam, g->rl.perm.p, g->n, K, grad_S, beta);
+    k_rows_scatter<<<grid_for((int64_t)g->n * K, kThreads), kThreads, 0, s>>>(lam, g->rl.perm.p, g->n, K, Kp, grad_S,
+                                                                              beta);
     PRDF_LAUNCH_CHECK();
     ks.kernels += 1;
   }
   if (grad_w) {
     PRDF_TRY(ensure_orig(g, s));  // grad_w is written in the original out-CSR's slot order
     double* Rr = (lam == g->R64a.p) ? g->R64b.p : g->R64a.p;
-    k_rows_gather_scaled<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(R, g->rl.perm.p, g->n, K, 1.0, Rr);
+    k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(R, g->rl.perm.p, g->n, K, Kp, 1.0, Rr);
     PRDF_LAUNCH_CHECK();
     PRDF_TRY(launch_grad_w(g->rl.out.off.p, g->rl.out.adj.p, g->rl.perm.p, g->csr[PRDF_OUT].off.p, lam, g->S64.p, beta,
-                           Rr, g->wsum.p, g->n, K, p->alpha, grad_w, s));
+                           Rr, g->wsum.p, g->n, Kp, p->alpha, grad_w, s));
     ks.kernels += 2;
   }
   PRDF_CUDA(cudaEventRecord(t.e[2], s));

@@ -1,8 +1,6 @@
 // Internal declarations shared by the translation units of libprdf.
 #pragma once
 
-#include <vector>
-
 #include "common.cuh"
 
 namespace prdf {
@@ -99,17 +97,8 @@ struct Relabel {
   int64_t drift = 0;                 // batch entries applied since the numbering was made
 };
 
-// Rows of the highest in-degree class are cut into chunks of kHubChunk edges
-// by the K-column calls: chunk c covers edges
-// [chunk_j0[c], +kHubChunk) of vertex begin + chunk_hub[c]; the chunks of
-// hub i are [hub_first[i], hub_first[i + 1]) in row order.
-constexpr int64_t kHubChunk = 1024;
-struct PprHub {
-  int64_t begin, nhub, nchunk;
-  const int32_t* chunk_hub;
-  const int64_t* chunk_j0;
-  const int64_t* hub_first;
-};
+constexpr int kHubChunk = 1024;  // edges of a chunk of the rank sweeps's longest rows
+
 // ---- the rank loop (sweep.cu) ----
 
 // Row shapes of a class of the sweep: a lane per row (no gather: in-degree <=
@@ -137,7 +126,7 @@ struct alignas(16) SweepChunk {
 // Owner of the chunk table of the sweep's long rows [begin, n) of G'.
 struct SweepChunks {
   int64_t rows = 0, max_chunks = 0;
-  int first_class = 0, size = 0;
+  int first_class = 0, size = 0, above = 0;
   DBuf<uint32_t> cnt;
   DBuf<int64_t> first;       // rows + 1: exclusive scan of the chunk counts, first[rows] = number of chunks
   DBuf<SweepChunk> chunks;
@@ -225,77 +214,53 @@ struct SweepArgs {
 int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t* cb, bool exact, bool dynamic,
                      cudaStream_t s);
 int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s);
-int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, SweepChunks& t, Workspace& ws,
-                 cudaStream_t s);
+// Chunk table of the rows [begin, n) longer than `above` entries (above = 0: of every row).
+int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, int above, SweepChunks& t,
+                 Workspace& ws, cudaStream_t s);
 // initialAffected (Alg. affected) in the sweep numbering: dV, dN and the frontier list of the first push
 // (dN padded to whole 32-bit words)
 int launch_mark_batch(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
                       const int32_t* ins_src, const uint8_t* ins_mask, int64_t n_ins, const int32_t* inv,
                       const int64_t* ooff, uint8_t* dV, uint8_t* dN, LoopCtl* ctl, int2* list, cudaStream_t s);
 
-// K-column personalised PageRank (ppr.cu), row-major [n, K] in the class-contiguous numbering.
-struct Ppr32Args {
-  const int64_t* off;      // in-CSR of G'
-  const int32_t* adj;
-  const float* P;          // P_uv for the in-edge slot (u -> v)
-  const float* R;          // current [n, K]
-  float* Rn;               // next [n, K]
-  const float* S;          // right-hand side [n, K] (teleport, or residual / (1 - alpha))
-  const int32_t* srow;     // null: S is dense; else S holds compact rows and row v is S[srow[v]] (-1: zero)
-  int K;
-  float alpha, beta;       // alpha, 1 - alpha
-  uint32_t* resid;         // [0] max |R_new - R|, [1] max |R_new| (FP32 bits, atomic max)
-  const uint32_t* prev;    // previous sweep's pair or null
-  float tol_rel;
-  // device-driven iteration (CUDA graph): when ctl is set, iteration it = ctl[0]
-  // reads R from Ra (even it) or Rb (odd it), writes the other, and uses the
-  // pair resid_base + 2 it (previous: resid_base + 2 (it - 1))
-  const int* ctl;
-  const float* Ra;
-  float* Rb;
-  uint32_t* resid_base;
-};
-struct Ppr64Args {
+// K-column personalised PageRank (ppr.cu): one solve of
+// R = alpha A R + beta S (A over the rows of off / adj / P), or one sweep of
+// it. T = float (FP32 sweeps) or double (FP64 Jacobi steps), row-major
+// [n, K] in the class-contiguous numbering; K here is the row stride
+// (padded_cols).
+template <class T>
+struct PprArgs {
   const int64_t* off;
   const int32_t* adj;
-  const double* P;
-  const double* R;
-  double* Rn;              // T(R)
-  const double* S;         // right-hand side, dense or compact rows as in Ppr32Args
-  const int32_t* srow;
-  float* res32;            // (T(R) - R) / (1 - alpha) in FP32, or null
-  int K;
-  double alpha, beta, inv_beta;
-  uint64_t* dmax;          // max |T(R) - R| (FP64 bits, atomic max)
-  // device-driven iteration (CUDA graph): when ctl is set, step it = ctl[0]
-  // reads R from Ra (even it) or Rb (odd it), writes the other, and puts its
-  // maximum in dmax_base + it
-  const int* ctl;
-  const double* Ra;
-  double* Rb;
-  uint64_t* dmax_base;
+  const T* P;              // P_uv of the slot
+  T* Ra;                   // even sweeps read Ra and write Rb
+  T* Rb;
+  const T* S;              // right-hand side [n, K] (teleport, or residual / (1 - alpha))
+  const int32_t* srow;     // null: S is dense; else S holds compact rows and row v is S[srow[v]] (-1: zero)
+  float* res32;            // FP64: (T(R) - R) / (1 - alpha) in FP32, or null
+  int K, tiles;
+  T alpha, beta, inv_beta; // alpha, 1 - alpha, 1 / (1 - alpha)
+  T tol;                   // FP32: stop at max|dR| <= tol * max|R|; FP64: at max|dR| <= tol
+  int max_iter, mode, it0, it_first;  // as in SweepArgs
+  LoopSlot* slot;
+  LoopCtl* ctl;
+  // rows [0, row_end) of at most row_max entries one by one, the others in the chunk table
+  int64_t row_end;
+  int row_max;
+  int rows_per_unit;
+  const SweepChunk* chunks;
+  const int64_t* nchunk;
+  int64_t max_chunks, chunk_rows;
+  uint32_t chunks_per_unit;
+  void* part;              // [tiles][max_chunks][tile] partial sums
+  uint32_t* done;          // [tiles][chunk_rows] arrivals, zero between sweeps
 };
+int launch_ppr_loop(const PprArgs<float>& a, int tile, int64_t n, cudaStream_t s);
+int launch_ppr_loop(const PprArgs<double>& a, int tile, int64_t n, cudaStream_t s);
+// row stride of the K-column state: a multiple of four columns (16-byte FP32
+// rows), except for one or two columns
+inline int padded_cols(int K) { return K <= 2 ? K : (K + 3) & ~3; }
 
-// Owner of a chunk table (PprHub above) of one CSR of the sweep numbering.
-struct PprHubTable {
-  int64_t begin = 0, nhub = 0, nchunk = 0;
-  DBuf<int32_t> chunk_hub;
-  DBuf<int64_t> chunk_j0, hub_first;
-  uint64_t version = 0;  // numbering version it was built for
-  bool valid = false;
-  PprHub view() const { return PprHub{begin, nhub, nchunk, chunk_hub.p, chunk_j0.p, hub_first.p}; }
-};
-int build_ppr_hub(const int64_t* off, int64_t begin, int64_t n, PprHubTable& t, Workspace& ws, cudaStream_t s);
-
-// FP32 sweep over tiles of `tile` columns: vertices [0, hub_begin) one per
-// slot, [hub_begin, h.begin) a warp each, the hub rows in chunks (part:
-// h.nchunk * tile float2 scratch).
-int launch_ppr32_sweep(const Ppr32Args& a, int tile, int64_t n, int64_t hub_begin, const PprHub& h, float2* part,
-                       cudaStream_t s);
-// FP64 Jacobi step over tiles of `tile` columns, same ranges as the FP32
-// sweep (part: h.nchunk * tile doubles of scratch).
-int launch_ppr64_step(const Ppr64Args& a, int tile, int64_t n, int64_t hub_begin, const PprHub& h, double* part,
-                      cudaStream_t s);
 // Sparse teleport: the rows of S (double [n, K]) with a non-zero entry. When
 // at most n / 4 rows are non-zero, srow[v] gets v's compact row (-1 for none),
 // Sc64 / Sc32 the rows in FP64 / FP32, R32 (float [n, K]) the FP32 matrix
@@ -315,14 +280,6 @@ int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, c
                   int K, double alpha, double* grad_w, cudaStream_t s);
 int ppr_narrow(const double* x, int64_t cnt, float* y, cudaStream_t s);
 int ppr_widen(const float* y, int64_t cnt, double* x, cudaStream_t s);
-
-// One-thread checks of the graph-driven K-column loops: it = ctl[0]; stop when
-// resid[it] <= tol (FP64) or resid[2 it] <= tol_rel * resid[2 it + 1] (FP32),
-// or it + 1 >= max_iter; ctl[0] = it + 1; sets the while condition.
-int launch_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
-                      cudaGraphConditionalHandle h, cudaStream_t s);
-int launch_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
-                        cudaGraphConditionalHandle h, cudaStream_t s);
 
 // Alg. affected kernels (frontier.cu). map (nullable): vertex id -> flag index.
 int launch_initial_affected(const int32_t* del_src, const int32_t* del_dst, const uint8_t* del_mask, int64_t n_del,
@@ -360,14 +317,12 @@ struct prdf_graph {
   prdf::Workspace ws;
   // solver scratch
   prdf::DBuf<double> xa, xb;
-  prdf::PprHubTable hub_in, hub_out;  // chunk tables of G' (Static sweep, K-column forward) and G (adjoint)
   prdf::SweepChunks sweep_chunks;     // chunk table of the rank sweeps
-  prdf::DBuf<float2> ppr_part;        // chunk partial sums of one column tile (FP32 sweeps)
-  prdf::DBuf<double> ppr_part64;      // chunk partial sums of one column tile (FP64 steps)
+  prdf::SweepChunks ppr_chunks_in, ppr_chunks_out;  // of G' (K-column forward) and of G (adjoint)
+  prdf::DBuf<double> ppr_part;        // K-column calls: partial sum of a chunk and column
+  prdf::DBuf<uint32_t> ppr_done;      // and arrivals per row and tile
   prdf::DBuf<float> ya, yb, degf, invf;  // FP32 stage state and degrees (class-contiguous numbering)
   prdf::DBuf<float> kf32;                // FP32 stage of DF-P: Eq. 2 factor
-  prdf::DBuf<uint32_t> resid32;
-  prdf::DBuf<uint64_t> resid;
   prdf::DBuf<uint8_t> dV, dN, wrote;
   prdf::DBuf<uint8_t> dF;  // Dynamic Traversal: next frontier of the closure
   prdf::DBuf<unsigned long long> counter;
@@ -378,12 +333,6 @@ struct prdf_graph {
   prdf::DBuf<int32_t> loop_act;          // DF / DF-P / DT: affected rows of a sweep
   prdf::DBuf<int32_t> flist;             // DT: a small frontier listed for its closure round (frontier.cu)
   prdf::DBuf<unsigned int> fcnt;         // its size
-  prdf::DBuf<int> ctl;               // device iteration counter of the graph-driven K-column loops
-  cudaStream_t cap_stream = nullptr; // private stream used to capture graph bodies
-  // instantiated K-column loops (CUDA graphs), one per kind of loop, each
-  // with the arguments and buffers it was captured for
-  cudaGraphExec_t loop_exec[8] = {};
-  std::vector<uint64_t> loop_key[8];
   prdf::Relabel rl;                  // class-contiguous copy used by the sweeps
   // weighted graphs: transition probabilities P_uv = w_uv / sum_k w_uk
   bool ppr_valid = false;

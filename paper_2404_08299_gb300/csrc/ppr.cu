@@ -1,23 +1,36 @@
 // K-column weighted personalised PageRank (an extension of Eq. 1 and
 // Alg. static): R[:, c] = alpha * P^T R[:, c] + (1 - alpha) * S[:, c] with the
 // row-stochastic P_uv = w_uv / sum_k w_uk, for K personalisation columns at
-// once. State is row-major [n, K] in the class-contiguous numbering, so one
-// index and weight fetch serves a tile of T columns (T = 2 * lanes per
-// vertex); rows above kHubDeg in-edges use a block per vertex.
+// once. State is row-major [n, Kp] in the class-contiguous numbering, Kp = K
+// rounded up to a multiple of four (padding columns stay zero), so one index
+// and weight fetch serves a tile of columns, four of them per lane.
 //
-// FP32 sweeps use a compensated dot product (each product's rounding error
-// from an FMA, TwoSum for the additions). The FP64 stage is mixed-precision
-// iterative refinement: an FP64 sweep computes the Jacobi step T(R) and the
-// residual T(R) - R; an FP32 solve of E = alpha P^T E + residual gives the
-// correction. The stop rule is the same as Static's: the L-inf change of an
-// FP64 Jacobi step <= tol.
-#include "internal.cuh"
+// FP32 sweeps sum the products of up to eight edges with FMAs and fold each
+// such sum into a compensated pair (TwoSum), so the rounding error does not
+// grow with the row length. The FP64 stage is mixed-precision iterative
+// refinement: an FP64 sweep computes the Jacobi step T(R) and the residual
+// T(R) - R; an FP32 solve of E = alpha P^T E + residual gives the correction.
+// The stop rule is the same as Static's: the L-inf change of an FP64 Jacobi
+// step <= tol.
+//
+// One persistent kernel per solve (k_ppr_loop, a cooperative launch), as in
+// sweep.cu: units of rows and row chunks of every column tile, a grid barrier
+// between sweeps, the stop test on the device. What bounds a sweep is the
+// 16-byte gathers of the rows of R (K * 4 bytes per edge through L2), so the
+// kernel is built to keep them in flight: the indices and weights of the next
+// step load (one per lane, handed round by shuffles) while this step's
+// gathers are on their way, across row and chunk bounds.
+#include <cstring>
+
+#include "loop.cuh"
 
 namespace prdf {
 
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
+constexpr unsigned kFull = 0xffffffffu;
 
 // Compensated FP32 sum (s + e): TwoSum folds each term's rounding error into e.
 struct Dot2 {
@@ -33,14 +46,29 @@ struct Dot2 {
     e += o.e;
   }
   __device__ __forceinline__ float value() const { return s + e; }
+  __device__ __forceinline__ Dot2 shfl_xor(int o) const {
+    Dot2 x;
+    x.s = __shfl_xor_sync(kFull, s, o);
+    x.e = __shfl_xor_sync(kFull, e, o);
+    return x;
+  }
+};
+// Plain FP64 sum (fixed order: edges of a slot, then slots, then chunks).
+struct Sum64 {
+  double s = 0;
+  __device__ __forceinline__ void merge(const Sum64& o) { s += o.s; }
+  __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ Sum64 shfl_xor(int o) const {
+    Sum64 x;
+    x.s = __shfl_xor_sync(kFull, s, o);
+    return x;
+  }
 };
 
-// Column accumulator of the FP32 sweeps: the products of a block of up to U
-// edges are summed with FMAs in b, and each block sum is folded into a
-// compensated pair, so the rounding error does not grow with the row length
-// (about two FP32 instructions per edge and column instead of ten for a
-// compensated product per edge).
-struct BlockSum {
+// Column accumulator: products go to b; fold() ends a block of at most eight
+// of them; sum(folded) is the total (folded: any block was ended before).
+struct Col32 {
+  using Sum = Dot2;
   Dot2 d;
   float b = 0.f;
   __device__ __forceinline__ void prod(float p, float r) { b = fmaf(p, r, b); }
@@ -48,543 +76,524 @@ struct BlockSum {
     d.add(b);
     b = 0.f;
   }
+  __device__ __forceinline__ Dot2 sum(bool folded) {
+    if (!folded) {
+      d.s = b;
+      d.e = 0.f;
+    } else {
+      d.add(b);
+    }
+    return d;
+  }
+};
+struct Col64 {
+  using Sum = Sum64;
+  Sum64 d;
+  __device__ __forceinline__ void prod(double p, double r) { d.s = fma(p, r, d.s); }
+  __device__ __forceinline__ void fold() {}
+  __device__ __forceinline__ Sum64 sum(bool) const { return d; }
 };
 
-__device__ __forceinline__ void block_max2_u32(uint32_t dmax, uint32_t rmax, uint32_t* out) {
-  __shared__ uint32_t sd[32], sr[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-    rmax = max(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    sd[wid] = dmax;
-    sr[wid] = rmax;
-  }
-  __syncthreads();
-  if (wid == 0) {
-    uint32_t x = lane < (int)(blockDim.x >> 5) ? sd[lane] : 0u;
-    uint32_t y = lane < (int)(blockDim.x >> 5) ? sr[lane] : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
-      y = max(y, __shfl_xor_sync(0xffffffffu, y, o));
-    }
-    if (lane == 0) {
-      if (x) atomicMax(out, x);
-      if (y) atomicMax(out + 1, y);
-    }
-  }
-}
-
-// per-iteration buffers of the graph-driven loops
-__device__ __forceinline__ Ppr32Args resolve_ppr32(const Ppr32Args& in) {
-  if (!in.ctl) return in;
-  Ppr32Args a = in;
-  const int it = in.ctl[0];
-  a.R = (it & 1) ? in.Rb : in.Ra;
-  a.Rn = (it & 1) ? const_cast<float*>(in.Ra) : in.Rb;
-  a.resid = in.resid_base + 2 * it;
-  a.prev = it > 0 ? in.resid_base + 2 * (it - 1) : nullptr;
-  return a;
-}
-__device__ __forceinline__ Ppr64Args resolve_ppr64(const Ppr64Args& in) {
-  if (!in.ctl) return in;
-  Ppr64Args a = in;
-  const int it = in.ctl[0];
-  a.R = (it & 1) ? in.Rb : in.Ra;
-  a.Rn = (it & 1) ? const_cast<double*>(in.Ra) : in.Rb;
-  a.dmax = in.dmax_base + it;
-  return a;
-}
-
-__device__ __forceinline__ bool ppr32_converged(const Ppr32Args& a) {
-  if (!a.prev) return false;
-  return __uint_as_float(a.prev[0]) <= a.tol_rel * __uint_as_float(a.prev[1]);
-}
-
-// ------------------------------------------------- FP32 K-column sweep ----
-// A lane owns 4 consecutive columns of a tile (one 16-byte load per gathered
-// row when K % 4 == 0), so LPE = tile / 4 lanes cover one edge and a warp
-// load serves 32 / LPE edges ("slots").
-
-struct Col4 {
-  float v[4];
+template <class T>
+struct Traits;
+template <>
+struct Traits<float> {
+  using Col = Col32;
+  static constexpr int kU = 4;          // gathers of a lane in flight
+  static constexpr int kMinBlocks = 4;  // 64 registers
+};
+template <>
+struct Traits<double> {
+  using Col = Col64;
+  static constexpr int kU = 4;
+  static constexpr int kMinBlocks = 2;  // 128 registers
 };
 
-__device__ __forceinline__ Col4 zero4() {
-  Col4 c;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) c.v[q] = 0.f;
-  return c;
-}
+template <class T>
+struct Vec4 {
+  T v[4];
+};
 
-// columns col .. col + 3 of row u (zero past K)
-__device__ __forceinline__ Col4 ld_cols(const float* R, int64_t u, int K, int col) {
-  Col4 c;
-  const float* src = R + u * K + col;
-  if ((K & 3) == 0) {  // col is a multiple of 4: 16-byte aligned
-    const float4 f = __ldg(reinterpret_cast<const float4*>(src));
-    c.v[0] = f.x;
-    c.v[1] = f.y;
-    c.v[2] = f.z;
-    c.v[3] = f.w;
+// Four columns of a row: coherent loads (R is written in the same kernel, a
+// grid barrier earlier). VEC (a row stride that is a multiple of four, every K
+// above 2): 16-byte loads, and the columns past K are the row's zero padding;
+// else `left` columns one by one. Nothing is read and zeros are returned when
+// `on` is false.
+template <bool VEC>
+__device__ __forceinline__ void ld_row(const float* src, bool on, int left, Vec4<float>& r) {
+  if (VEC) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) r.v[q] = 0.f;
+    if (on)
+      asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
+                   : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
+                   : "l"(src));
   } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) c.v[q] = col + q < K ? __ldg(src + q) : 0.f;
+    for (int q = 0; q < 4; ++q) {
+      r.v[q] = 0.f;
+      if (on && q < left) asm volatile("ld.global.f32 %0, [%1];" : "=f"(r.v[q]) : "l"(src + q));
+    }
   }
-  return c;
 }
-
-// S and the previous R of the 4 columns of vertex v, loaded before the row's
-// gathers so their latency overlaps
-struct Own4 {
-  float s[4], o[4];
-};
-__device__ __forceinline__ Own4 ppr32_own(const Ppr32Args& a, int32_t v, int col) {
-  Own4 w;
+template <bool VEC>
+__device__ __forceinline__ void ld_row(const double* src, bool on, int left, Vec4<double>& r) {
+  if (VEC) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) w.s[q] = w.o[q] = 0.f;
-  if (col >= a.K) return w;
-  const int64_t o = (int64_t)v * a.K + col;
-  // right-hand side row: dense, or (srow) the compact row of v, none when v has no teleport mass
-  const int64_t sr = a.srow ? (int64_t)a.srow[v] : (int64_t)v;
-  const float* S = sr >= 0 ? a.S + sr * a.K + col : nullptr;
-  if ((a.K & 3) == 0) {
-    const float4 o4 = *reinterpret_cast<const float4*>(a.R + o);
-    w.o[0] = o4.x; w.o[1] = o4.y; w.o[2] = o4.z; w.o[3] = o4.w;
-    if (S) {
-      const float4 s4 = *reinterpret_cast<const float4*>(S);
-      w.s[0] = s4.x; w.s[1] = s4.y; w.s[2] = s4.z; w.s[3] = s4.w;
+    for (int q = 0; q < 4; ++q) r.v[q] = 0.0;
+    if (on) {
+      asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(src));
+      asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[2]), "=d"(r.v[3]) : "l"(src + 2));
     }
   } else {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      w.s[q] = (S && col + q < a.K) ? S[q] : 0.f;
-      w.o[q] = col + q < a.K ? a.R[o + q] : 0.f;
+      r.v[q] = 0.0;
+      if (on && q < left) asm volatile("ld.global.f64 %0, [%1];" : "=d"(r.v[q]) : "l"(src + q));
     }
   }
-  return w;
+}
+__device__ __forceinline__ float ld_weight(const float* p, uint64_t pol) {
+  float v;
+  asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ double ld_weight(const double* p, uint64_t pol) { return ld_stream_f64(p, pol); }
+
+// Largest |T(R) - R| and |T(R)| a thread saw (bits).
+struct Peak {
+  uint64_t d = 0;
+  uint32_t r = 0;
+  __device__ __forceinline__ void see(float diff, float val) {
+    const uint32_t a = __float_as_uint(fabsf(diff)), b = __float_as_uint(fabsf(val));
+    d = a > (uint32_t)d ? a : d;
+    r = b > r ? b : r;
+  }
+  __device__ __forceinline__ void see(double diff, double) {
+    const uint64_t a = dbits(fabs(diff));
+    d = a > d ? a : d;
+  }
+};
+
+template <class T>
+struct Ctx {
+  const T* R;     // this lane's columns of row 0 of the current iterate
+  T* Rn;          // the next iterate
+  uint64_t pf;
+  int lane, col;
+  bool colok;     // the lane has columns
+  int left;       // columns of the matrix from col on
+};
+
+template <bool VEC, class T>
+__device__ __forceinline__ void gather(const Ctx<T>& c, int K, int32_t u, bool on, Vec4<T>& r) {
+  ld_row<VEC>(c.R + (int64_t)u * K, on && c.colok, c.left, r);
 }
 
-// new values of the 4 columns of vertex v from their accumulated sums
-__device__ __forceinline__ void ppr32_finish4(const Ppr32Args& a, int32_t v, int col, const float* acc, const Own4& w,
-                                              uint32_t& dmax, uint32_t& rmax) {
-  if (col >= a.K) return;
-  const int64_t o = (int64_t)v * a.K + col;
-  float r[4];
+// New values of the 4 columns of vertex v from their sums: Eq. 1 with the
+// teleport S, the change against the previous R, and (FP64) the residual.
+template <class T, bool VEC>
+__device__ __forceinline__ void finish_row(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, const T* sum, Peak& pk) {
+  if (!c.colok) return;
+  const int64_t o = (int64_t)v * a.K + c.col;
+  // right-hand side row: dense, or (srow) the compact row of v, none when v has no teleport mass
+  const int64_t sr = a.srow ? (int64_t)__ldg(a.srow + v) : (int64_t)v;
+  Vec4<T> s, old;
+  ld_row<VEC>(a.S + (sr >= 0 ? sr : 0) * a.K + c.col, sr >= 0, c.left, s);
+  ld_row<VEC>(c.R + (int64_t)v * a.K, true, c.left, old);
+  T t[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    r[q] = fmaf(a.alpha, acc[q], a.beta * w.s[q]);
-    if (col + q < a.K) {
-      dmax = max(dmax, __float_as_uint(fabsf(r[q] - w.o[q])));
-      rmax = max(rmax, __float_as_uint(fabsf(r[q])));
-    }
+    t[q] = fma(a.alpha, sum[q], a.beta * s.v[q]);
+    if (VEC || q < c.left) pk.see(t[q] - old.v[q], t[q]);
   }
-  if ((a.K & 3) == 0) {
-    *reinterpret_cast<float4*>(a.Rn + o) = make_float4(r[0], r[1], r[2], r[3]);
+  if (VEC) {
+    if (sizeof(T) == 4) {
+      *reinterpret_cast<float4*>(c.Rn + o) = make_float4((float)t[0], (float)t[1], (float)t[2], (float)t[3]);
+    } else {
+      reinterpret_cast<double2*>(c.Rn + o)[0] = make_double2((double)t[0], (double)t[1]);
+      reinterpret_cast<double2*>(c.Rn + o)[1] = make_double2((double)t[2], (double)t[3]);
+    }
   } else {
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (col + q < a.K) a.Rn[o + q] = r[q];
+      if (q < c.left) c.Rn[o + q] = t[q];
   }
-}
-
-// U edges of one slot in flight: edges j0 + k * stride (k < U) below e
-template <int U>
-__device__ __forceinline__ void ppr32_edges(const Ppr32Args& a, int64_t j0, int64_t stride, int64_t e, int col,
-                                            bool colok, BlockSum* acc) {
-  int32_t u[U];
-  float p[U];
+  if (sizeof(T) == 8 && a.res32) {
+    float d[4];
 #pragma unroll
-  for (int k = 0; k < U; ++k) {
-    const int64_t j = j0 + (int64_t)k * stride;
-    u[k] = j < e ? __ldg(a.adj + j) : -1;
-    p[k] = j < e ? __ldg(a.P + j) : 0.f;
-  }
-  Col4 r[U];
+    for (int q = 0; q < 4; ++q) d[q] = (float)((t[q] - old.v[q]) * a.inv_beta);
+    if (VEC) {
+      *reinterpret_cast<float4*>(a.res32 + o) = make_float4(d[0], d[1], d[2], d[3]);
+    } else {
 #pragma unroll
-  for (int k = 0; k < U; ++k) r[k] = (u[k] >= 0 && colok) ? ld_cols(a.R, u[k], a.K, col) : zero4();
-#pragma unroll
-  for (int k = 0; k < U; ++k)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q].prod(p[k], r[k].v[q]);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q].fold();
-}
-
-// merge the compensated sums of the slots of a warp (slot 0 ends with the total)
-template <int LPE>
-__device__ __forceinline__ void merge_slots(Dot2* t) {
-#pragma unroll
-  for (int o = LPE; o < 32; o <<= 1) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      Dot2 x;
-      x.s = __shfl_xor_sync(0xffffffffu, t[q].s, o);
-      x.e = __shfl_xor_sync(0xffffffffu, t[q].e, o);
-      t[q].merge(x);
+      for (int q = 0; q < 4; ++q)
+        if (q < c.left) a.res32[o + q] = d[q];
     }
   }
 }
 
-// One vertex per slot (rows of at most a few hundred edges), U edges in flight.
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr32_group(const Ppr32Args a_in, int64_t begin, int64_t end, int c0) {
-  const Ppr32Args a = resolve_ppr32(a_in);
-  if (ppr32_converged(a)) return;
+// Rows of at most a few hundred edges: LPE lanes (a slot) per row, kSlots rows
+// side by side, [vb, ve) in steps of kSlots. A slot's lanes hold a window of
+// the row's indices and weights (kE edges) and hand them round by shuffles.
+// The next window (of the same rows, or of the slots' next rows, whose offsets
+// are known a step ahead) loads while this one's rows are gathered.
+template <class T, int LPE, bool VEC>
+__device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, int32_t vb, int32_t ve, Peak& pk) {
   constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  uint32_t dmax = 0, rmax = 0;
-  // The row offsets of the next vertex a slot takes load while the current
-  // vertex's rows are gathered, so a vertex starts with its offsets known.
-  const int64_t step = nwarps * kSlots;
-  int64_t base = begin + warp * kSlots;
-  int64_t i = base + slot;
-  int64_t b = i < end ? a.off[i] : 0, e = i < end ? a.off[i + 1] : 0;
-  for (; base < end; base += step, i += step) {
-    const int64_t in = i + step;
-    const int64_t bn = in < end ? a.off[in] : 0, en = in < end ? a.off[in + 1] : 0;
-    if (i < end) {
-      const int32_t v = (int32_t)i;
-      const Own4 w = ppr32_own(a, v, col);
-      BlockSum acc[4];
-      for (int64_t j0 = b; j0 < e; j0 += U) ppr32_edges<U>(a, j0, 1, e, col, colok, acc);
-      float c[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) c[q] = acc[q].d.value();
-      ppr32_finish4(a, v, col, c, w, dmax, rmax);
+  constexpr int kEpl = LPE >= 16 ? 1 : LPE >= 8 ? 2 : 4;  // window edges per lane
+  constexpr int kE = kEpl * LPE;
+  constexpr int U = 4;
+  const int sub = c.lane & (LPE - 1), slot = c.lane / LPE, slot0 = c.lane & ~(LPE - 1);
+  // (rows above row_max are in the chunk table: length -1, nothing to do)
+  auto load_off = [&](int32_t v, int64_t& b, int& len) {
+    b = 0;
+    len = -1;
+    if (v < ve && v >= 0) {  // (v + kSlots may pass the largest id)
+      b = ld_stream_i64(a.off + v, c.pf);
+      const int64_t d = ld_stream_i64(a.off + v + 1, c.pf) - b;
+      len = d <= a.row_max ? (int)d : -1;
     }
-    b = bn;
-    e = en;
-  }
-  block_max2_u32(dmax, rmax, a.resid);
-}
-
-// One warp per vertex (mid-degree rows): the slots stride over the row, U
-// edges in flight each, and meet by shuffles.
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr32_warp(const Ppr32Args a_in, int64_t begin, int64_t end, int c0) {
-  const Ppr32Args a = resolve_ppr32(a_in);
-  if (ppr32_converged(a)) return;
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  uint32_t dmax = 0, rmax = 0;
-  // the next row's offsets load while the current row is gathered
-  int64_t i = begin + warp;
-  int64_t b = i < end ? a.off[i] : 0, e = i < end ? a.off[i + 1] : 0;
-  for (; i < end; i += nwarps) {
-    const int32_t v = (int32_t)i;
-    const int64_t in = i + nwarps;
-    const int64_t bn = in < end ? a.off[in] : 0, en = in < end ? a.off[in + 1] : 0;
-    Own4 w;
-    if (slot == 0) w = ppr32_own(a, v, col);
-    BlockSum acc[4];
-    for (int64_t j0 = b + slot; j0 < e; j0 += (int64_t)kSlots * U) ppr32_edges<U>(a, j0, kSlots, e, col, colok, acc);
-    b = bn;
-    e = en;
-    Dot2 t[4];
+  };
+  int32_t u[kEpl];
+  T p[kEpl];
+  auto load_win = [&](int64_t b, int rem) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) t[q] = acc[q].d;
-    merge_slots<LPE>(t);
-    if (slot == 0) {
-      float c[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) c[q] = t[q].value();
-      ppr32_finish4(a, v, col, c, w, dmax, rmax);
+    for (int i = 0; i < kEpl; ++i) {
+      const int e = sub + LPE * i;
+      u[i] = e < rem ? ld_stream_i32(a.adj + b + e, c.pf) : 0;
+      p[i] = e < rem ? ld_weight(a.P + b + e, c.pf) : T(0);
     }
-  }
-  block_max2_u32(dmax, rmax, a.resid);
-}
-
-// Rows of the highest in-degree class are cut into chunks of kHubChunk edges
-// handled by different warps; each chunk's compensated partial sums go to
-// part[chunk][column] and a second kernel merges them in chunk order.
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr32_hub_part(const Ppr32Args a_in, PprHub h, int c0, int tile,
-                                                             float2* __restrict__ part) {
-  const Ppr32Args a = resolve_ppr32(a_in);
-  if (ppr32_converged(a)) return;
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  for (int64_t c = warp; c < h.nchunk; c += nwarps) {
-    const int32_t v = (int32_t)(h.begin + h.chunk_hub[c]);
-    const int64_t j_begin = h.chunk_j0[c];
-    const int64_t row_end = a.off[v + 1];
-    const int64_t e = j_begin + kHubChunk < row_end ? j_begin + kHubChunk : row_end;
-    BlockSum acc[4];
-    for (int64_t j0 = j_begin + slot; j0 < e; j0 += (int64_t)kSlots * U) ppr32_edges<U>(a, j0, kSlots, e, col, colok, acc);
-    Dot2 t[4];
+  };
+  int64_t b, bn;
+  int32_t v = vb + slot;
+  int rem, ln;
+  load_off(v, b, rem);
+  load_win(b, rem);
+  load_off(v + kSlots, bn, ln);
+  typename Traits<T>::Col acc[4];
+  bool todo = rem >= 0, folded = false;
+  for (int32_t v0 = vb; v0 < ve;) {
+    const int here = rem < kE ? rem : kE;
+    const int most = __reduce_max_sync(kFull, here);
+    const bool more = __any_sync(kFull, rem > kE);
+    int32_t cu[kEpl];
+    T cp[kEpl];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) t[q] = acc[q].d;
-    merge_slots<LPE>(t);
-    if (slot == 0) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) part[c * tile + 4 * sub + q] = make_float2(t[q].s, t[q].e);
+    for (int i = 0; i < kEpl; ++i) {
+      cu[i] = u[i];
+      cp[i] = p[i];
     }
-  }
-}
-
-template <int LPE>
-__global__ void __launch_bounds__(kThreads) k_ppr32_hub_finish(const Ppr32Args a_in, PprHub h, int c0, int tile,
-                                                               const float2* __restrict__ part) {
-  const Ppr32Args a = resolve_ppr32(a_in);
-  if (ppr32_converged(a)) return;
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  uint32_t dmax = 0, rmax = 0;
-  for (int64_t base = warp * kSlots; base < h.nhub; base += nwarps * kSlots) {
-    const int64_t hi = base + slot;
-    if (hi >= h.nhub) continue;
-    Dot2 t[4];
-    for (int64_t c = h.hub_first[hi]; c < h.hub_first[hi + 1]; ++c) {
+    Vec4<T> r[U];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 x = part[c * tile + 4 * sub + q];
-        Dot2 y;
-        y.s = x.x;
-        y.e = x.y;
-        t[q].merge(y);
+    for (int k = 0; k < U; ++k)
+      gather<VEC>(c, a.K, __shfl_sync(kFull, cu[k / LPE], slot0 + k % LPE), k < here, r[k]);
+    // the next window
+    const int32_t vdone = v;
+    const bool done = todo;
+    if (more) {
+      b += kE;
+      rem = rem > kE ? rem - kE : 0;
+      load_win(b, rem);
+    } else {
+      v += kSlots;
+      b = bn;
+      rem = ln;
+      todo = ln >= 0;
+      load_win(b, rem);
+      load_off(v + kSlots, bn, ln);
+    }
+#pragma unroll
+    for (int e0 = 0; e0 < kE; e0 += U) {
+      if (e0 >= most) break;
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        const T w = __shfl_sync(kFull, cp[(e0 + k) / LPE], slot0 + (e0 + k) % LPE);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q].prod(w, r[k].v[q]);
+      }
+      if ((e0 / U) % 2 == 1 && (more || e0 + U < most)) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q].fold();
+        folded = true;
+      }
+      if (e0 + U < kE && e0 + U < most) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+          const int e = e0 + U + k;
+          gather<VEC>(c, a.K, __shfl_sync(kFull, cu[e / LPE], slot0 + e % LPE), e < here, r[k]);
+        }
       }
     }
-    float cv[4];
+    if (!more) {
+      if (done) {
+        T t[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) cv[q] = t[q].value();
-    const int32_t v = (int32_t)(h.begin + hi);
-    ppr32_finish4(a, v, col, cv, ppr32_own(a, v, col), dmax, rmax);
-  }
-  block_max2_u32(dmax, rmax, a.resid);
-}
-
-// hub chunk table: count, then fill (hub_first is the scan of the counts)
-__global__ void k_hub_count(const int64_t* __restrict__ off, int64_t begin, int64_t nhub, int64_t* __restrict__ cnt) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nhub; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t d = off[begin + i + 1] - off[begin + i];
-    cnt[i] = d > 0 ? (d + kHubChunk - 1) / kHubChunk : 0;
-  }
-}
-
-__global__ void k_hub_fill(const int64_t* __restrict__ off, int64_t begin, int64_t nhub,
-                           const int64_t* __restrict__ first, int32_t* __restrict__ chunk_hub,
-                           int64_t* __restrict__ chunk_j0) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nhub; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = off[begin + i];
-    for (int64_t c = first[i]; c < first[i + 1]; ++c) {
-      chunk_hub[c] = (int32_t)i;
-      chunk_j0[c] = b + (c - first[i]) * kHubChunk;
+        for (int q = 0; q < 4; ++q) t[q] = acc[q].sum(folded).value();
+        finish_row<T, VEC>(a, c, vdone, t, pk);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = typename Traits<T>::Col();
+      folded = false;
+      v0 += kSlots;
     }
   }
 }
 
-// ---------------------------------------------------- FP64 Jacobi step ----
-// T(R) = alpha P^T R + (1 - alpha) S for a tile of columns, with the layout of
-// the FP32 sweep (4 columns per lane, LPE = tile / 4 lanes per edge): writes
-// T(R) to Rn, the residual (T(R) - R) / (1 - alpha) as FP32 to res32 (if not
-// null) and max |T(R) - R| to *dmax (FP64 bits, atomic max). Sums are plain
-// FP64 FMAs in a fixed order (edge order within a slot, then slots, then
-// chunks), so every run gives the same bits.
-
-struct Col4d {
-  double v[4];
-};
-
-__device__ __forceinline__ Col4d zero4d() {
-  Col4d c;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) c.v[q] = 0.0;
-  return c;
-}
-
-// columns col .. col + 3 of row u (zero past K); K even: two 16-byte loads
-__device__ __forceinline__ Col4d ld_cols64(const double* R, int64_t u, int K, int col) {
-  Col4d c;
-  const double* src = R + u * K + col;
-  if ((K & 1) == 0 && col + 4 <= K) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(src));
-    const double2 b = __ldg(reinterpret_cast<const double2*>(src + 2));
-    c.v[0] = a.x;
-    c.v[1] = a.y;
-    c.v[2] = b.x;
-    c.v[3] = b.y;
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) c.v[q] = col + q < K ? __ldg(src + q) : 0.0;
-  }
-  return c;
-}
-
-template <int U>
-__device__ __forceinline__ void ppr64_edges(const Ppr64Args& a, int64_t j0, int64_t stride, int64_t e, int col,
-                                            bool colok, double* acc) {
-  int32_t u[U];
-  double p[U];
-#pragma unroll
-  for (int k = 0; k < U; ++k) {
-    const int64_t j = j0 + (int64_t)k * stride;
-    u[k] = j < e ? __ldg(a.adj + j) : -1;
-    p[k] = j < e ? __ldg(a.P + j) : 0.0;
-  }
-  Col4d r[U];
-#pragma unroll
-  for (int k = 0; k < U; ++k) r[k] = (u[k] >= 0 && colok) ? ld_cols64(a.R, u[k], a.K, col) : zero4d();
-#pragma unroll
-  for (int k = 0; k < U; ++k)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = fma(p[k], r[k].v[q], acc[q]);
-}
-
-// T(R), residual and |T(R) - R| for the 4 columns of vertex v
-__device__ __forceinline__ void ppr64_finish4(const Ppr64Args& a, int32_t v, int col, const double* acc,
-                                              uint64_t& dmax) {
-  const int64_t sr = a.srow ? (int64_t)a.srow[v] : (int64_t)v;  // as in ppr32_own
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (col + q >= a.K) break;
-    const int64_t o = (int64_t)v * a.K + col + q;
-    const double sv = sr >= 0 ? a.S[sr * a.K + col + q] : 0.0;
-    const double t = fma(a.alpha, acc[q], a.beta * sv);
-    const double d = t - a.R[o];
-    a.Rn[o] = t;
-    if (a.res32) a.res32[o] = (float)(d * a.inv_beta);
-    dmax = max(dmax, dbits(fabs(d)));
-  }
-}
-
-__device__ __forceinline__ void block_max_u64(uint64_t dmax, uint64_t* out) {
-  __shared__ uint64_t sm[32];
-  dmax = warp_max_u64(dmax);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = dmax;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint64_t x = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : 0;
-    x = warp_max_u64(x);
-    if (threadIdx.x == 0 && x) atomicMax((unsigned long long*)out, (unsigned long long)x);
-  }
-}
-
-template <int LPE>
-__device__ __forceinline__ void merge_slots64(double* t) {
+// sums of the slots of a warp meet in every slot (a fixed tree)
+template <class Sum, int LPE>
+__device__ __forceinline__ void merge_slots(Sum* t) {
 #pragma unroll
   for (int o = LPE; o < 32; o <<= 1)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) t[q] += __shfl_xor_sync(0xffffffffu, t[q], o);
+    for (int q = 0; q < 4; ++q) t[q].merge(t[q].shfl_xor(o));
 }
 
-// one vertex per slot (in-degree up to the two highest classes)
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr64_group(const Ppr64Args a_in, int64_t begin, int64_t end, int c0) {
-  const Ppr64Args a = resolve_ppr64(a_in);
+__device__ __forceinline__ void ld_part(const Dot2* p, Dot2& x) {
+  const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
+  x.s = f.x;
+  x.e = f.y;
+}
+__device__ __forceinline__ void ld_part(const Sum64* p, Sum64& x) { x.s = __ldcg(reinterpret_cast<const double*>(p)); }
+
+// Chunks of long rows (the chunk table), up to 32 a unit, a warp per chunk one
+// after the other, the slots striding over its edges. A row of one chunk is
+// finished at once; of a longer row the warp that sums the last chunk (an
+// arrival counter per row and tile) adds the row's partial sums in chunk order
+// and finishes it.
+template <class T, int LPE, bool VEC>
+__device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c, int64_t cb, int cnt, int tile_no,
+                                            Peak& pk) {
+  using Sum = typename Traits<T>::Col::Sum;
   constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  uint64_t dmax = 0;
-  for (int64_t base = begin + warp * kSlots; base < end; base += nwarps * kSlots) {
-    const int64_t i = base + slot;
-    if (i >= end) continue;
-    const int32_t v = (int32_t)i;
-    const int64_t b = a.off[v], e = a.off[v + 1];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t j0 = b; j0 < e; j0 += U) ppr64_edges<U>(a, j0, 1, e, col, colok, acc);
-    if (colok) ppr64_finish4(a, v, col, acc, dmax);
+  constexpr int U = Traits<T>::kU;
+  constexpr int W = LPE >= U ? 1 : U / LPE;  // 32-edge windows a step
+  constexpr int kE = 32 * W;                 // edges a step
+  constexpr int kPer = kE / kSlots;          // of them a slot's
+  const int lane = c.lane, sub = lane & (LPE - 1), slot = lane / LPE;
+  // lane l: chunk cb + l
+  int64_t j0 = 0;
+  int len = 0;
+  int32_t kv = 0;
+  if (lane < cnt) {
+    const int4 p0 = __ldg(reinterpret_cast<const int4*>(a.chunks + cb + lane));
+    j0 = (int64_t)(((uint64_t)(uint32_t)p0.y << 32) | (uint32_t)p0.x);
+    len = p0.z;
+    kv = p0.w;
   }
-  block_max_u64(dmax, a.dmax);
-}
-
-// a warp per vertex (mid-degree rows), slots meet by shuffles
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr64_warp(const Ppr64Args a_in, int64_t begin, int64_t end, int c0) {
-  const Ppr64Args a = resolve_ppr64(a_in);
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  uint64_t dmax = 0;
-  for (int64_t i = begin + warp; i < end; i += nwarps) {
-    const int32_t v = (int32_t)i;
-    const int64_t b = a.off[v], e = a.off[v + 1];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t j0 = b + slot; j0 < e; j0 += (int64_t)kSlots * U) ppr64_edges<U>(a, j0, kSlots, e, col, colok, acc);
-    merge_slots64<LPE>(acc);
-    if (slot == 0 && colok) ppr64_finish4(a, v, col, acc, dmax);
-  }
-  block_max_u64(dmax, a.dmax);
-}
-
-// hub rows in 1024-edge chunks: partial sums per chunk, then merged in chunk order
-template <int LPE, int U>
-__global__ void __launch_bounds__(kThreads) k_ppr64_hub_part(const Ppr64Args a_in, PprHub h, int c0, int tile,
-                                                             double* __restrict__ part) {
-  const Ppr64Args a = resolve_ppr64(a_in);
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  const bool colok = col < a.K;
-  for (int64_t c = warp; c < h.nchunk; c += nwarps) {
-    const int32_t v = (int32_t)(h.begin + h.chunk_hub[c]);
-    const int64_t jb = h.chunk_j0[c];
-    const int64_t re = a.off[v + 1];
-    const int64_t e = jb + kHubChunk < re ? jb + kHubChunk : re;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t j0 = jb + slot; j0 < e; j0 += (int64_t)kSlots * U) ppr64_edges<U>(a, j0, kSlots, e, col, colok, acc);
-    merge_slots64<LPE>(acc);
-    if (slot == 0) {
+  int32_t u[W];
+  T p[W];
+  auto load_win = [&](int64_t b, int rem) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) part[c * tile + 4 * sub + q] = acc[q];
+    for (int i = 0; i < W; ++i) {
+      const int e = lane + 32 * i;
+      u[i] = e < rem ? ld_stream_i32(a.adj + b + e, c.pf) : 0;
+      p[i] = e < rem ? ld_weight(a.P + b + e, c.pf) : T(0);
+    }
+  };
+  int64_t b = __shfl_sync(kFull, j0, 0);
+  int rem = __shfl_sync(kFull, len, 0);
+  load_win(b, rem);
+  typename Traits<T>::Col acc[4];
+  for (int s = 0; s < cnt;) {
+    int32_t cu[W];
+    T cp[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      cu[i] = u[i];
+      cp[i] = p[i];
+    }
+    const int here = rem < kE ? rem : kE;
+    const bool more = rem > kE;  // the same on every lane
+    Vec4<T> r[U];
+    // slot's i-th edge of the step is edge i * kSlots + slot
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int e = i * kSlots + slot;
+      gather<VEC>(c, a.K, __shfl_sync(kFull, cu[(i * kSlots) / 32], e & 31), e < here, r[i]);
+    }
+    if (more) {
+      b += kE;
+      rem -= kE;
+    } else {
+      const int nx = s + 1 < cnt ? s + 1 : 0;
+      b = __shfl_sync(kFull, j0, nx);
+      rem = __shfl_sync(kFull, len, nx);
+      if (s + 1 >= cnt) rem = 0;
+    }
+    load_win(b, rem);
+#pragma unroll
+    for (int i0 = 0; i0 < kPer; i0 += U) {
+      if (i0 * kSlots >= here && i0 > 0) break;
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const T w = __shfl_sync(kFull, cp[((i0 + i) * kSlots) / 32], ((i0 + i) * kSlots + slot) & 31);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q].prod(w, r[i].v[q]);
+      }
+      if ((i0 / U) % 2 == 1 || kPer == U) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q].fold();
+      }
+      if (i0 + U < kPer && (i0 + U) * kSlots < here) {
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+          const int e = (i0 + U + i) * kSlots + slot;
+          gather<VEC>(c, a.K, __shfl_sync(kFull, cu[((i0 + U + i) * kSlots) / 32], e & 31), e < here, r[i]);
+        }
+      }
+    }
+    if (more) continue;
+    Sum t[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      t[q] = acc[q].sum(true);
+      acc[q] = typename Traits<T>::Col();
+    }
+    merge_slots<Sum, LPE>(t);
+    const int4 rec = __ldg(reinterpret_cast<const int4*>(a.chunks + cb + s) + 1);  // first, parts, row
+    const int parts = rec.y;
+    const int32_t v = __shfl_sync(kFull, kv, s);
+    bool fin = true;
+    if (parts > 1) {
+      Sum* part = reinterpret_cast<Sum*>(a.part) + (int64_t)tile_no * a.max_chunks * (4 * LPE);
+      const int first = rec.x, row = rec.z;
+      if (slot == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) part[(cb + s) * (4 * LPE) + 4 * sub + q] = t[q];
+      }
+      __threadfence();
+      __syncwarp();
+      unsigned int n = 0;
+      if (lane == 0) n = atomicAdd(a.done + (int64_t)tile_no * a.chunk_rows + row, 1u) + 1;
+      n = __shfl_sync(kFull, n, 0);
+      fin = n == (unsigned int)parts;
+      if (fin) {
+        if (lane == 0) a.done[(int64_t)tile_no * a.chunk_rows + row] = 0;
+        __threadfence();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) t[q] = Sum();
+        for (int i = slot; i < parts; i += kSlots) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            Sum x;
+            ld_part(part + (int64_t)(first + i) * (4 * LPE) + 4 * sub + q, x);
+            t[q].merge(x);
+          }
+        }
+        merge_slots<Sum, LPE>(t);
+      }
+    }
+    if (fin && slot == 0) {
+      T sum[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum[q] = t[q].value();
+      finish_row<T, VEC>(a, c, v, sum, pk);
+    }
+    ++s;
+  }
+}
+
+template <class T>
+__device__ __forceinline__ LoopSlot* slot_of(const PprArgs<T>& a, int it) {
+  return a.slot + (a.mode == kLoopAll ? (it & (kLoopRing - 1)) : it - a.it_first + 1);
+}
+
+__device__ __forceinline__ bool stopped(unsigned long long resid, double tol) { return bitsd(resid) <= tol; }
+__device__ __forceinline__ bool stopped(unsigned long long resid, float tol) {
+  return __uint_as_float((uint32_t)resid) <= tol * __uint_as_float((uint32_t)(resid >> 32));
+}
+
+template <class T, int LPE, bool VEC>
+__device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
+  Ctx<T> c;
+  const T* R = (it & 1) ? a.Rb : a.Ra;
+  c.Rn = (it & 1) ? a.Ra : a.Rb;
+  c.pf = policy_evict_first();
+  c.lane = threadIdx.x & 31;
+  LoopSlot* slot = slot_of(a, it);
+  Peak pk;
+  const unsigned int nw = gridDim.x * kWarps;
+  const unsigned int nchunk = a.nchunk ? (unsigned int)__ldg(a.nchunk) : 0u;
+  const unsigned int cu = (nchunk + a.chunks_per_unit - 1) / a.chunks_per_unit;
+  const unsigned int ru = (unsigned int)((a.row_end + a.rows_per_unit - 1) / a.rows_per_unit);
+  const unsigned int per_tile = cu + ru;
+  const unsigned int total = per_tile * a.tiles;
+  const bool counted = total > 4 * nw;
+  for (unsigned int x = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; x < total;) {
+    unsigned int nx = x;
+    if (counted && c.lane == 0) nx = atomicAdd(&slot->units, 1u);
+    // the chunks of every tile first (long work), then the rows of every tile
+    const bool chunk = x < cu * a.tiles;
+    const unsigned int y = chunk ? x : x - cu * a.tiles;
+    const unsigned int per = chunk ? cu : ru;
+    const int tile_no = (int)(y / per);
+    const unsigned int un = y - (unsigned int)tile_no * per;
+    c.col = tile_no * (4 * LPE) + 4 * (c.lane & (LPE - 1));
+    c.colok = c.col < a.K;
+    c.left = a.K - c.col;
+    c.R = R + c.col;
+    if (chunk) {
+      const unsigned int cb = un * a.chunks_per_unit;
+      const unsigned int cnt = nchunk - cb < a.chunks_per_unit ? nchunk - cb : a.chunks_per_unit;
+      unit_chunks<T, LPE, VEC>(a, c, cb, (int)cnt, tile_no, pk);
+    } else {
+      // from the highest class down: long rows first
+      const int64_t ve = a.row_end - (int64_t)un * a.rows_per_unit;
+      const int64_t vb = ve > a.rows_per_unit ? ve - a.rows_per_unit : 0;
+      unit_rows<T, LPE, VEC>(a, c, (int32_t)vb, (int32_t)ve, pk);
+    }
+    x = nw + __shfl_sync(kFull, nx, 0);
+  }
+  __shared__ unsigned long long s_d;
+  __shared__ unsigned int s_r;
+  if (threadIdx.x == 0) {
+    s_d = 0;
+    s_r = 0;
+  }
+  __syncthreads();
+  const uint64_t d = warp_max_u64(pk.d);
+  const uint32_t r = __reduce_max_sync(kFull, pk.r);
+  if (c.lane == 0) {
+    if (d) atomicMax(&s_d, (unsigned long long)d);
+    if (r) atomicMax(&s_r, r);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sizeof(T) == 8) {
+      if (s_d) atomicMax(&slot->resid, s_d);
+    } else {
+      uint32_t* w = reinterpret_cast<uint32_t*>(&slot->resid);
+      if (s_d) atomicMax(w, (uint32_t)s_d);
+      if (s_r) atomicMax(w + 1, s_r);
     }
   }
 }
 
-template <int LPE>
-__global__ void __launch_bounds__(kThreads) k_ppr64_hub_finish(const Ppr64Args a_in, PprHub h, int c0, int tile,
-                                                               const double* __restrict__ part) {
-  const Ppr64Args a = resolve_ppr64(a_in);
-  constexpr int kSlots = 32 / LPE;
-  const int sub = threadIdx.x & (LPE - 1);
-  const int slot = (threadIdx.x & 31) / LPE;
-  const int64_t warp = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = c0 + 4 * sub;
-  uint64_t dmax = 0;
-  for (int64_t base = warp * kSlots; base < h.nhub; base += nwarps * kSlots) {
-    const int64_t hi = base + slot;
-    if (hi >= h.nhub) continue;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t c = h.hub_first[hi]; c < h.hub_first[hi + 1]; ++c)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] += part[c * tile + 4 * sub + q];
-    if (col < a.K) ppr64_finish4(a, (int32_t)(h.begin + hi), col, acc, dmax);
+// The whole solve (kLoopAll, cooperative launch) or one sweep of the
+// host-driven loop.
+template <class T, int LPE, bool VEC>
+__global__ void __launch_bounds__(kThreads, Traits<T>::kMinBlocks) k_ppr_loop(const __grid_constant__ PprArgs<T> a) {
+  if (a.mode == kLoopSweep) {
+    if (a.it0 > 0 && stopped(__ldcg(&slot_of(a, a.it0 - 1)->resid), a.tol)) return;
+    ppr_sweep<T, LPE, VEC>(a, a.it0);
+    return;
   }
-  block_max_u64(dmax, a.dmax);
+  unsigned long long target = 0;
+  for (int it = 0;; ++it) {
+    ppr_sweep<T, LPE, VEC>(a, it);
+    if (!grid_barrier(a.ctl, target)) return;
+    const unsigned long long resid = __ldcg(&slot_of(a, it)->resid);
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (stopped(resid, a.tol) || it + 1 >= a.max_iter) {
+      if (first) {
+        a.ctl->iters = it + 1;
+        a.ctl->resid = resid;
+      }
+      return;
+    }
+    if (first) *slot_of(a, it + 2) = LoopSlot();  // as in sweep.cu
+  }
 }
 
 // Edge gradient of L = sum_c G_c . R_c with respect to w_uv (out-slot j of
@@ -670,116 +679,57 @@ __global__ void k_widen_n(const float* __restrict__ y, int64_t cnt, double* __re
     x[i] = (double)y[i];
 }
 
-// stop checks of the graph-driven loops
-__global__ void k_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
-                             cudaGraphConditionalHandle h) {
-  const int it = ctl[0];
-  const bool done = bitsd(resid_base[it]) <= tol || it + 1 >= max_iter;
-  ctl[0] = it + 1;
-  cudaGraphSetConditional(h, done ? 0u : 1u);
-}
-
-__global__ void k_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
-                               cudaGraphConditionalHandle h) {
-  const int it = ctl[0];
-  const uint32_t* r = resid_base + 2 * it;
-  const bool done = __uint_as_float(r[0]) <= tol_rel * __uint_as_float(r[1]) || it + 1 >= max_iter;
-  ctl[0] = it + 1;
-  cudaGraphSetConditional(h, done ? 0u : 1u);
-}
-
-template <int LPE>
-void launch32_tile(const Ppr32Args& a, const PprHub& h, float2* part, int64_t hub_b, int64_t n, int c0, int tile,
-                   cudaStream_t s) {
-  const int maxg = kSMs * 8;
-  if (hub_b > 0) k_ppr32_group<LPE, 4><<<grid_for(hub_b * LPE, kThreads, maxg), kThreads, 0, s>>>(a, 0, hub_b, c0);
-  if (h.begin > hub_b)
-    k_ppr32_warp<LPE, 8><<<grid_for((h.begin - hub_b) * 32, kThreads, maxg), kThreads, 0, s>>>(a, hub_b, h.begin, c0);
-  if (n > h.begin) {
-    k_ppr32_hub_part<LPE, 8><<<grid_for(h.nchunk * 32, kThreads, maxg), kThreads, 0, s>>>(a, h, c0, tile, part);
-    k_ppr32_hub_finish<LPE><<<grid_for(h.nhub * LPE, kThreads, maxg), kThreads, 0, s>>>(a, h, c0, tile, part);
+template <class T, int LPE, bool VEC>
+int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
+  auto k = k_ppr_loop<T, LPE, VEC>;
+  int dev = 0, sms = 0, per = 0;
+  PRDF_CUDA(cudaGetDevice(&dev));
+  PRDF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  PRDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kThreads, 0));
+  if (per < 1 || sms < 1) {
+    set_error("the K-column kernel does not fit this device");
+    return PRDF_ECUDA;
   }
+  const int max_b = per * sms;
+  constexpr int kSlots = 32 / LPE;
+  a.tiles = (a.K + 4 * LPE - 1) / (4 * LPE);
+  // rows of a unit: about an eighth of a warp's share, a few steps at least
+  int64_t rows = kSlots;
+  while (rows < 8 * kSlots && rows * 8 * (int64_t)max_b * kWarps < n * a.tiles) rows *= 2;
+  a.rows_per_unit = (int)rows;
+  a.chunks_per_unit = a.max_chunks * a.tiles > 32 * (int64_t)max_b * kWarps ? 4 : 1;
+  const int64_t work = (a.row_end / rows + 1 + a.max_chunks / a.chunks_per_unit + 1) * a.tiles;
+  if (work * 2 >= (int64_t)UINT32_MAX) {
+    set_error("too many work units");
+    return PRDF_EINVAL;
+  }
+  int64_t blocks = (work + kWarps - 1) / kWarps;
+  if (blocks > max_b) blocks = max_b;
+  if (a.mode != kLoopAll) {
+    k<<<(unsigned)blocks, kThreads, 0, s>>>(a);
+    PRDF_LAUNCH_CHECK();
+    return PRDF_OK;
+  }
+  void* args[] = {&a};
+  PRDF_CUDA(cudaLaunchCooperativeKernel((const void*)k, dim3((unsigned)blocks), dim3(kThreads), args, 0, s));
+  return PRDF_OK;
 }
 
-template <int LPE>
-void launch64_tile(const Ppr64Args& a, const PprHub& h, double* part, int64_t hub_b, int64_t n, int c0, int tile,
-                   cudaStream_t s) {
-  const int maxg = kSMs * 8;
-  if (hub_b > 0) k_ppr64_group<LPE, 4><<<grid_for(hub_b * LPE, kThreads, maxg), kThreads, 0, s>>>(a, 0, hub_b, c0);
-  if (h.begin > hub_b)
-    k_ppr64_warp<LPE, 4><<<grid_for((h.begin - hub_b) * 32, kThreads, maxg), kThreads, 0, s>>>(a, hub_b, h.begin, c0);
-  if (n > h.begin) {
-    k_ppr64_hub_part<LPE, 4><<<grid_for(h.nchunk * 32, kThreads, maxg), kThreads, 0, s>>>(a, h, c0, tile, part);
-    k_ppr64_hub_finish<LPE><<<grid_for(h.nhub * LPE, kThreads, maxg), kThreads, 0, s>>>(a, h, c0, tile, part);
+template <class T>
+int run_ppr(const PprArgs<T>& a, int tile, int64_t n, cudaStream_t s) {
+  if (a.K & 3) return run_tile<T, 2, false>(a, n, s);  // one or two columns (tile 8)
+  switch (tile) {
+    case 8: return run_tile<T, 2, true>(a, n, s);
+    case 16: return run_tile<T, 4, true>(a, n, s);
+    case 32: return run_tile<T, 8, true>(a, n, s);
+    default: return run_tile<T, 16, true>(a, n, s);
   }
 }
 
 }  // namespace
 
-int launch_iter_check(int* ctl, const uint64_t* resid_base, double tol, int max_iter,
-                      cudaGraphConditionalHandle h, cudaStream_t s) {
-  k_iter_check<<<1, 1, 0, s>>>(ctl, resid_base, tol, max_iter, h);
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
-
-int launch_iter_check32(int* ctl, const uint32_t* resid_base, float tol_rel, int max_iter,
-                        cudaGraphConditionalHandle h, cudaStream_t s) {
-  k_iter_check32<<<1, 1, 0, s>>>(ctl, resid_base, tol_rel, max_iter, h);
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
-
-int launch_ppr32_sweep(const Ppr32Args& a, int tile, int64_t n, int64_t hub_begin, const PprHub& h, float2* part,
-                       cudaStream_t s) {
-  for (int c0 = 0; c0 < a.K; c0 += tile) {
-    switch (tile) {
-      case 8: launch32_tile<2>(a, h, part, hub_begin, n, c0, tile, s); break;
-      case 16: launch32_tile<4>(a, h, part, hub_begin, n, c0, tile, s); break;
-      case 32: launch32_tile<8>(a, h, part, hub_begin, n, c0, tile, s); break;
-      default: launch32_tile<16>(a, h, part, hub_begin, n, c0, tile, s); break;
-    }
-  }
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
-
-int build_ppr_hub(const int64_t* off, int64_t begin, int64_t n, PprHubTable& t, Workspace& ws, cudaStream_t s) {
-  const int64_t nhub = n - begin;
-  t.begin = begin;
-  t.nhub = nhub > 0 ? nhub : 0;
-  t.nchunk = 0;
-  if (t.nhub == 0) return PRDF_OK;
-  DBuf<int64_t> cnt;
-  PRDF_TRY(cnt.alloc((size_t)t.nhub, s));
-  PRDF_TRY(t.hub_first.alloc((size_t)t.nhub + 1, s));
-  k_hub_count<<<grid_for(t.nhub, kThreads), kThreads, 0, s>>>(off, begin, t.nhub, cnt.p);
-  PRDF_LAUNCH_CHECK();
-  PRDF_TRY(exclusive_scan_i64(cnt.p, t.nhub, t.hub_first.p, ws, s));
-  PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, t.hub_first.p + t.nhub, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  PRDF_CUDA(cudaStreamSynchronize(s));
-  t.nchunk = ws.host_i64[0];
-  PRDF_TRY(t.chunk_hub.alloc((size_t)(t.nchunk > 0 ? t.nchunk : 1), s));
-  PRDF_TRY(t.chunk_j0.alloc((size_t)(t.nchunk > 0 ? t.nchunk : 1), s));
-  k_hub_fill<<<grid_for(t.nhub, kThreads), kThreads, 0, s>>>(off, begin, t.nhub, t.hub_first.p, t.chunk_hub.p,
-                                                              t.chunk_j0.p);
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
-
-int launch_ppr64_step(const Ppr64Args& a, int tile, int64_t n, int64_t hub_begin, const PprHub& h, double* part,
-                      cudaStream_t s) {
-  for (int c0 = 0; c0 < a.K; c0 += tile) {
-    switch (tile) {
-      case 8: launch64_tile<2>(a, h, part, hub_begin, n, c0, tile, s); break;
-      case 16: launch64_tile<4>(a, h, part, hub_begin, n, c0, tile, s); break;
-      case 32: launch64_tile<8>(a, h, part, hub_begin, n, c0, tile, s); break;
-      default: launch64_tile<16>(a, h, part, hub_begin, n, c0, tile, s); break;
-    }
-  }
-  PRDF_LAUNCH_CHECK();
-  return PRDF_OK;
-}
+int launch_ppr_loop(const PprArgs<float>& a, int tile, int64_t n, cudaStream_t s) { return run_ppr(a, tile, n, s); }
+int launch_ppr_loop(const PprArgs<double>& a, int tile, int64_t n, cudaStream_t s) { return run_ppr(a, tile, n, s); }
 
 int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, const int64_t* orig_off,
                   const double* lam, const double* Gs, double g_scale, const double* Rr, const double* W, int32_t n,

@@ -28,7 +28,7 @@
 // plain store per vertex.
 #include <cstring>
 
-#include "internal.cuh"
+#include "loop.cuh"
 
 namespace prdf {
 
@@ -626,43 +626,6 @@ __device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, 
 
 // -------------------------------------------------------------- phases ----
 
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Barrier over the whole (co-resident) grid: every block adds one arrival and
-// waits until all of this barrier's are in. The wait is bounded: past the
-// limit (minutes; no sweep takes that long) the block flags the loop as timed
-// out and gives up, and so does every other block when it sees the flag.
-// Returns false after a timeout.
-constexpr unsigned long long kSpinLimit = 1ull << 28;
-
-__device__ bool grid_barrier(LoopCtl* ctl, unsigned long long& target) {
-  __shared__ int s_ok;
-  target += gridDim.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&ctl->bar, 1ull);
-    int ok = 1;
-    unsigned long long spins = 0;
-    while (ld_acquire(&ctl->bar) < target) {
-      if (++spins > kSpinLimit || ((spins & 1023) == 0 && *(volatile int*)&ctl->timeout)) {
-        *(volatile int*)&ctl->timeout = 1;
-        ok = 0;
-        break;
-      }
-      if (spins > 256) __nanosleep(100);
-    }
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 // the slot of sweep it: a ring of kLoopRing in the whole-loop kernel, one a
 // sweep from it_first on in the host-driven loop (slot 0: the sweep before)
 template <class Real>
@@ -1184,11 +1147,12 @@ __global__ void k_mark_batch(const int32_t* __restrict__ del_src, const int32_t*
 }
 
 // Chunk table: a row is cut into ceil(len / size) chunks (one when empty).
-__global__ void k_chunk_count(const int64_t* __restrict__ off, int64_t begin, int64_t rows, int size,
+__global__ void k_chunk_count(const int64_t* __restrict__ off, int64_t begin, int64_t rows, int size, int above,
                               uint32_t* __restrict__ cnt) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t d = off[begin + i + 1] - off[begin + i];
-    cnt[i] = d > 0 ? (uint32_t)((d + size - 1) / size) : 1u;
+    cnt[i] = above > 0 ? (d > above ? (uint32_t)((d + size - 1) / size) : 0u)
+                       : (d > 0 ? (uint32_t)((d + size - 1) / size) : 1u);
   }
 }
 
@@ -1318,8 +1282,8 @@ int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t*
   return dynamic ? Launcher<PKahan, true>::run(a, t, cb, s) : Launcher<PKahan, false>::run(a, t, cb, s);
 }
 
-int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, SweepChunks& t, Workspace& ws,
-                 cudaStream_t s) {
+int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, int above, SweepChunks& t,
+                 Workspace& ws, cudaStream_t s) {
   t.rows = n - begin;
   t.max_chunks = 0;
   if (t.rows <= 0) {
@@ -1327,7 +1291,7 @@ int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int si
     return PRDF_OK;
   }
   // the number of chunks stays on the device; the table has room for the most there can be
-  t.max_chunks = t.rows + m / size;
+  t.max_chunks = (above > 0 ? m / above : t.rows) + m / size + 1;
   if (t.max_chunks >= INT32_MAX) {
     set_error("too many row chunks");
     return PRDF_EINVAL;
@@ -1335,9 +1299,7 @@ int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int si
   PRDF_TRY(t.cnt.reserve((size_t)t.rows, s));
   PRDF_TRY(t.first.reserve((size_t)t.rows + 1, s));
   PRDF_TRY(t.chunks.reserve((size_t)t.max_chunks, s));
-  PRDF_TRY(t.part.reserve((size_t)t.max_chunks, s));
-  PRDF_TRY(t.done.reserve((size_t)t.rows, s));
-  k_chunk_count<<<grid_for(t.rows, 256), 256, 0, s>>>(off, begin, t.rows, size, t.cnt.p);
+  k_chunk_count<<<grid_for(t.rows, 256), 256, 0, s>>>(off, begin, t.rows, size, above, t.cnt.p);
   PRDF_LAUNCH_CHECK();
   PRDF_TRY(exclusive_scan_u32(t.cnt.p, t.rows, t.first.p, ws, s));
   k_chunk_fill<<<grid_for(t.rows * 32, 256), 256, 0, s>>>(off, begin, t.rows, size, t.first.p, t.chunks.p);
