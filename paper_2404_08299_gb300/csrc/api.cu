@@ -1124,8 +1124,7 @@ int prdf_graph_create(int32_t n, const int32_t* src, const int32_t* dst, const f
   int r = g->ws.init();
   const bool loops = (flags & PRDF_ADD_SELF_LOOPS) != 0;
   g->self_loops = loops;
-  if (r == PRDF_OK) r = build_csr(n, m0, src, dst, w, loops, false, g->csr[PRDF_OUT], g->ws, s);
-  if (r == PRDF_OK) r = build_csr(n, m0, dst, src, w, loops, false, g->csr[PRDF_IN], g->ws, s);
+  if (r == PRDF_OK) r = build_csr_pair(n, m0, src, dst, w, loops, g->csr[PRDF_OUT], g->csr[PRDF_IN], g->ws, s);
   g->m = g->csr[PRDF_OUT].m;
   if (r == PRDF_OK) r = build_relabelled(g, s);
   if (r == PRDF_OK && cudaStreamSynchronize(s) != cudaSuccess) {

@@ -495,8 +495,9 @@ __global__ void k_compact(int32_t n, int64_t m, const int64_t* __restrict__ star
 
 }  // namespace
 
-int build_csr(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, const float* w, bool self_loops,
-              bool allow_skip, Csr& out, Workspace& ws, cudaStream_t s) {
+namespace {
+int check_list(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, const float* w, bool allow_skip,
+               cudaStream_t s) {
   if (n < 1 || m0 < 0 || m0 >= (1ll << 32)) {
     set_error("build_csr: n=%d m0=%lld out of range", n, (long long)m0);
     return PRDF_EINVAL;
@@ -523,6 +524,24 @@ int build_csr(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, c
       return PRDF_EINVAL;
     }
   }
+  return PRDF_OK;
+}
+}  // namespace
+
+int build_csr_pair(int32_t n, int64_t m0, const int32_t* src, const int32_t* dst, const float* w, bool self_loops,
+                   Csr& out, Csr& in, Workspace& ws, cudaStream_t s) {
+  if (n >= 1 && m0 >= 0 && radix_pair_applies(n, m0, self_loops)) {
+    PRDF_TRY(check_list(n, m0, src, dst, w, false, s));
+    return build_csr_pair_radix(n, m0, src, dst, w, self_loops, out, in, ws, s);
+  }
+  PRDF_TRY(build_csr(n, m0, src, dst, w, self_loops, false, out, ws, s));
+  return build_csr(n, m0, dst, src, w, self_loops, false, in, ws, s);
+}
+
+int build_csr(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, const float* w, bool self_loops,
+              bool allow_skip, Csr& out, Workspace& ws, cudaStream_t s) {
+  PRDF_TRY(check_list(n, m0, rows, cols, w, allow_skip, s));
+  const int T = 256;
   if (radix_build_applies(n, m0, w, allow_skip, self_loops))
     return build_csr_radix(n, m0, rows, cols, self_loops, out, ws, s);
   const int64_t N = n;

@@ -1,7 +1,7 @@
 // CSR construction by a least-significant-digit radix sort of packed edge
-// keys: the CSR of G or of G' (Section 4.1, 4.3 of arXiv 2404.08299) from an
-// unweighted edge list, duplicates merged and one self-loop per vertex
-// (Section 3.1, 5.1.3).
+// keys: the CSRs of G and of G' (Section 4.1, 4.3 of arXiv 2404.08299) from an
+// edge list, duplicates merged and one self-loop per vertex (Section 3.1,
+// 5.1.3). Weights move with their keys; merged duplicates keep the largest.
 //
 // Key of entry (r, c): r << B | c, B = bits of n - 1, so the key order is the
 // CSR order (rows ascending, columns ascending inside a row). Eight key bits
@@ -33,6 +33,7 @@ static_assert(kRTile <= 65536 && kRK % 2 == 0, "ranks are packed two to a word")
 
 struct KeySrc {
   const uint64_t* keys;  // later passes
+  const float* w;        // weighted builds: the entries' weights, moved along with the keys
   const int32_t* rows;   // first pass: entry i < m0 is (rows[i], cols[i]),
   const int32_t* cols;   // entry m0 + v is the self-loop (v, v)
   int64_t m0;
@@ -45,6 +46,13 @@ __device__ __forceinline__ uint64_t load_key(const KeySrc& s, int64_t i) {
   if (i < s.m0) return ((uint64_t)(uint32_t)__ldcs(s.rows + i) << s.B) | (uint64_t)(uint32_t)__ldcs(s.cols + i);
   const uint64_t v = (uint64_t)(i - s.m0);
   return (v << s.B) | v;
+}
+
+// weight of entry i; 0 marks an added self-loop (given weights are positive)
+template <bool FIRST>
+__device__ __forceinline__ float load_w(const KeySrc& s, int64_t i) {
+  if (FIRST && i >= s.m0) return 0.f;
+  return __ldcs(s.w + i);
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
@@ -115,17 +123,19 @@ __global__ void __launch_bounds__(kRT) k_radix_hist(const KeySrc src, int64_t M,
   hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = c;
 }
 
-// Stable scatter of one tile by digit; goff = exclusive scan of hist.
-template <bool FIRST>
+// Stable scatter of one tile by digit; goff = exclusive scan of hist. W: the
+// weights move with their keys.
+template <bool FIRST, bool W>
 __global__ void __launch_bounds__(kRT, 3) k_radix_scatter(const KeySrc src, int64_t M, int shift,
                                                           const int64_t* __restrict__ goff, int64_t ntiles,
-                                                          uint64_t* __restrict__ out) {
+                                                          uint64_t* __restrict__ out, float* __restrict__ wout) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);          // kRTile keys
   int64_t* gbase = reinterpret_cast<int64_t*>(buf + kRTile);       // kRDigits
   uint32_t* wcnt = reinterpret_cast<uint32_t*>(gbase + kRDigits);  // kRWarps x kRDigits
   uint32_t* lstart = wcnt + kRWarps * kRDigits;                    // kRDigits
   uint32_t* wsum = lstart + kRDigits;                              // kRWarps
+  float* wbuf = reinterpret_cast<float*>(wsum + kRWarps);          // kRTile weights (W)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < kRWarps; ++k) wcnt[k * kRDigits + threadIdx.x] = 0;
@@ -178,18 +188,23 @@ __global__ void __launch_bounds__(kRT, 3) k_radix_scatter(const KeySrc src, int6
   for (int r = 0; r < kRK; ++r) {
     if (r < nv) {
       const uint32_t d = (uint32_t)(key[r] >> shift) & 0xFFu;
-      buf[lstart[d] + mine[d] + ((rank[r >> 1] >> (16 * (r & 1))) & 0xFFFFu)] = key[r];
+      const uint32_t at = lstart[d] + mine[d] + ((rank[r >> 1] >> (16 * (r & 1))) & 0xFFFFu);
+      buf[at] = key[r];
+      if (W) wbuf[at] = load_w<FIRST>(src, i0 + r * 32);
     }
   }
   __syncthreads();
   const int cnt = (int)(M - t0 < kRTile ? M - t0 : kRTile);
   for (int i = threadIdx.x; i < cnt; i += kRT) {
     const uint64_t k = buf[i];
-    __stcs(reinterpret_cast<unsigned long long*>(out) + gbase[(k >> shift) & 0xFFu] + i, k);
+    const int64_t at = gbase[(k >> shift) & 0xFFu] + i;
+    __stcs(reinterpret_cast<unsigned long long*>(out) + at, k);
+    if (W) __stcs(wout + at, wbuf[i]);
   }
 }
 
 constexpr int kRScatterSmem = kRTile * 8 + kRDigits * 8 + kRWarps * kRDigits * 4 + kRDigits * 4 + kRWarps * 4;
+constexpr int kRScatterSmemW = kRScatterSmem + kRTile * 4;
 
 // ---- merge of equal keys ----
 // A warp takes 32 * kRK consecutive sorted keys, 32 per round (coalesced);
@@ -231,13 +246,16 @@ __global__ void __launch_bounds__(kRT) k_uniq_count(const uint64_t* __restrict__
 
 // Columns of the unique keys, and off[r] = position of row r's first unique
 // key (rows without keys take the next row's start; off[n] = total).
-// woff = exclusive scan of the per-warp counts, woff[nw] = total. With urow
+// woff = exclusive scan of the per-warp counts, woff[nw] = total. kt (or null)
+// gets the keys of the transposed CSR in this CSR's order, uw (or null, zero
+// on entry) the largest weight bits of each unique key. With urow
 // (lists much shorter than n) the row of each unique key goes to urow instead
 // and k_offsets_from_rows fills off.
 __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ k, int64_t M, int B, int32_t n,
                                                    const int64_t* __restrict__ woff, int64_t nw,
                                                    int32_t* __restrict__ adj, int64_t* __restrict__ off,
-                                                   int32_t* __restrict__ urow) {
+                                                   int32_t* __restrict__ urow, uint64_t* __restrict__ kt,
+                                                   const float* __restrict__ w, uint32_t* __restrict__ uw) {
   const int lane = threadIdx.x & 31;
   const int64_t gw = ((int64_t)blockIdx.x * kRT + threadIdx.x) >> 5;
   const int64_t base = gw * (32 * kRK);
@@ -259,10 +277,13 @@ __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ 
     carry = __shfl_sync(0xffffffffu, key[r], 31);
     const bool f = i < M && (i == 0 || key[r] != prev);
     const uint32_t bal = __ballot_sync(0xffffffffu, f);
+    // duplicates keep the largest weight (positive floats order as their bits)
+    if (uw && i < M) atomicMax(uw + pos + __popc(bal & lt) - (f ? 0 : 1), __float_as_uint(__ldcs(w + i)));
     if (f) {
       const int64_t p = pos + __popc(bal & lt);
       const int64_t row = (int64_t)(key[r] >> B);
       adj[p] = (int32_t)(key[r] & cmask);
+      if (kt) kt[p] = (key[r] & cmask) << B | (uint64_t)row;
       if (urow) {
         urow[p] = (int32_t)row;
       } else {
@@ -291,13 +312,37 @@ __global__ void k_offsets_from_rows(const int32_t* __restrict__ urow, int64_t mu
   }
 }
 
+// an added self-loop without a weight of its own (0 so far) gets 1
+__global__ void k_loop_weights(float* __restrict__ w, int64_t m) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+    if (w[i] == 0.f) w[i] = 1.f;
+}
+
+// columns and row offsets of sorted keys without duplicates
+__global__ void __launch_bounds__(kRT) k_emit(const uint64_t* __restrict__ k, int64_t m, int B, int32_t n,
+                                              int32_t* __restrict__ adj, int64_t* __restrict__ off) {
+  const uint64_t cmask = (1ull << B) - 1;
+  for (int64_t i = blockIdx.x * (int64_t)kRT + threadIdx.x; i < m; i += (int64_t)gridDim.x * kRT) {
+    const uint64_t key = k[i];
+    const int64_t row = (int64_t)(key >> B);
+    adj[i] = (int32_t)(key & cmask);
+    for (int64_t q = i == 0 ? 0 : (int64_t)(k[i - 1] >> B) + 1; q <= row; ++q) off[q] = i;
+    if (i == m - 1)
+      for (int64_t q = row + 1; q <= n; ++q) off[q] = m;
+  }
+}
+
 template <bool FIRST>
-int radix_pass(const KeySrc& src, int64_t M, int shift, uint64_t* out, DBuf<uint32_t>& hist, DBuf<int64_t>& goff,
-               int64_t ntiles, Workspace& ws, cudaStream_t s) {
+int radix_pass(const KeySrc& src, int64_t M, int shift, uint64_t* out, float* wout, DBuf<uint32_t>& hist,
+               DBuf<int64_t>& goff, int64_t ntiles, Workspace& ws, cudaStream_t s) {
   k_radix_hist<FIRST><<<(unsigned)ntiles, kRT, 0, s>>>(src, M, shift, hist.p, ntiles);
   PRDF_LAUNCH_CHECK();
   PRDF_TRY(exclusive_scan_u32(hist.p, ntiles * kRDigits, goff.p, ws, s));
-  k_radix_scatter<FIRST><<<(unsigned)ntiles, kRT, kRScatterSmem, s>>>(src, M, shift, goff.p, ntiles, out);
+  if (wout)
+    k_radix_scatter<FIRST, true><<<(unsigned)ntiles, kRT, kRScatterSmemW, s>>>(src, M, shift, goff.p, ntiles, out, wout);
+  else
+    k_radix_scatter<FIRST, false><<<(unsigned)ntiles, kRT, kRScatterSmem, s>>>(src, M, shift, goff.p, ntiles, out,
+                                                                               nullptr);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }
@@ -309,42 +354,73 @@ bool radix_build_applies(int32_t n, int64_t m0, const float* w, bool allow_skip,
   return !w && !allow_skip && M > 0 && M < (1ll << 32);
 }
 
-int build_csr_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, bool self_loops, Csr& out,
-                    Workspace& ws, cudaStream_t s) {
+bool radix_pair_applies(int32_t n, int64_t m0, bool self_loops) {
+  const int64_t M = m0 + (self_loops ? n : 0);
+  return M > 0 && M < (1ll << 32) && M * 16 >= (int64_t)n;
+}
+
+namespace {
+
+int radix_smem() {
+  static bool smem_set = false;
+  if (smem_set) return PRDF_OK;
+  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
+  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
+  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmemW));
+  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmemW));
+  smem_set = true;
+  return PRDF_OK;
+}
+
+// The CSR of the list, and with `in` that of its transpose: the first CSR's
+// unique entries, in its order, are a list sorted by row, so a stable sort by
+// column alone (half the passes) gives the transposed CSR with its rows in
+// order.
+int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, const float* w, bool self_loops,
+                Csr& out, Csr* in, Workspace& ws, cudaStream_t s) {
   const int64_t M = m0 + (self_loops ? n : 0);
   int B = 1;
   while (B < 31 && ((int64_t)1 << B) < (int64_t)n) ++B;  // ids < n <= 2^B
   const int passes = (2 * B + 7) / 8;
   const int64_t ntiles = (M + kRTile - 1) / kRTile;
-  static bool smem_set = false;
-  if (!smem_set) {
-    PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
-    PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
-    smem_set = true;
-  }
+  PRDF_TRY(radix_smem());
   DBuf<uint64_t> ka, kb;
+  DBuf<float> wa, wb;
   DBuf<uint32_t> hist;
   DBuf<int64_t> goff;
   PRDF_TRY(ka.alloc((size_t)M, s));
   PRDF_TRY(kb.alloc((size_t)M, s));
+  if (w) {
+    PRDF_TRY(wa.alloc((size_t)M, s));
+    PRDF_TRY(wb.alloc((size_t)M, s));
+  }
   PRDF_TRY(hist.alloc((size_t)(ntiles * kRDigits), s));
   PRDF_TRY(goff.alloc((size_t)(ntiles * kRDigits + 1), s));
   KeySrc src;
   src.keys = nullptr;
+  src.w = w;
   src.rows = rows;
   src.cols = cols;
   src.m0 = m0;
   src.B = B;
   uint64_t* cur = ka.p;
   uint64_t* nxt = kb.p;
-  PRDF_TRY(radix_pass<true>(src, M, 0, cur, hist, goff, ntiles, ws, s));
-  for (int p = 1; p < passes; ++p) {
+  float* wcur = wa.p;
+  float* wnxt = wb.p;
+  PRDF_TRY(radix_pass<true>(src, M, 0, cur, wcur, hist, goff, ntiles, ws, s));
+  auto pass = [&](int64_t cnt, int shift) {
     src.keys = cur;
-    PRDF_TRY(radix_pass<false>(src, M, 8 * p, nxt, hist, goff, ntiles, ws, s));
+    src.w = wcur;
+    PRDF_TRY(radix_pass<false>(src, cnt, shift, nxt, wnxt, hist, goff, (cnt + kRTile - 1) / kRTile, ws, s));
     uint64_t* t = cur;
     cur = nxt;
     nxt = t;
-  }
+    float* f = wcur;
+    wcur = wnxt;
+    wnxt = f;
+    return (int)PRDF_OK;
+  };
+  for (int p = 1; p < passes; ++p) PRDF_TRY(pass(M, 8 * p));
   // merge equal keys
   const int64_t nw = ntiles * kRWarps;
   DBuf<uint32_t> wcnt;
@@ -356,20 +432,71 @@ int build_csr_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* c
   PRDF_TRY(exclusive_scan_u32(wcnt.p, nw, woff.p, ws, s));
   PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, woff.p + nw, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
-  out.m = ws.host_i64[0];
+  const int64_t m = ws.host_i64[0];
+  const size_t room = (size_t)(m > 0 ? m : 1);
+  out.m = m;
   PRDF_TRY(out.off.alloc((size_t)n + 1, s));
-  PRDF_TRY(out.adj.alloc((size_t)(out.m > 0 ? out.m : 1), s));
-  out.w.release();
+  PRDF_TRY(out.adj.alloc(room, s));
+  if (w) {
+    PRDF_TRY(out.w.alloc(room, s));
+    PRDF_CUDA(cudaMemsetAsync(out.w.p, 0, sizeof(float) * (size_t)m, s));
+  } else {
+    out.w.release();
+  }
   // a list much shorter than n leaves long runs of empty rows: their offsets
   // are found row-parallel instead of by the lanes that emit the keys
   const bool sparse = M * 16 < (int64_t)n;
   DBuf<int32_t> urow;
-  if (sparse) PRDF_TRY(urow.alloc((size_t)(out.m > 0 ? out.m : 1), s));
+  if (sparse) PRDF_TRY(urow.alloc(room, s));
   k_uniq_emit<<<(unsigned)ntiles, kRT, 0, s>>>(cur, M, B, n, woff.p, nw, out.adj.p, out.off.p,
-                                               sparse ? urow.p : nullptr);
+                                               sparse ? urow.p : nullptr, in ? nxt : nullptr, wcur,
+                                               w ? reinterpret_cast<uint32_t*>(out.w.p) : nullptr);
   if (sparse) k_offsets_from_rows<<<grid_for((int64_t)n + 1, kRT), kRT, 0, s>>>(urow.p, out.m, n, out.off.p);
+  if (w && self_loops) k_loop_weights<<<grid_for(m, kRT), kRT, 0, s>>>(out.w.p, m);
+  PRDF_LAUNCH_CHECK();
+  if (!in) return PRDF_OK;
+  uint64_t* t = cur;  // the transposed keys
+  cur = nxt;
+  nxt = t;
+  for (int p = 0; p < (B + 7) / 8; ++p) {
+    if (p == 0 && w) {
+      src.keys = cur;
+      src.w = out.w.p;
+      PRDF_TRY(radix_pass<false>(src, m, B, nxt, wnxt, hist, goff, (m + kRTile - 1) / kRTile, ws, s));
+      uint64_t* q = cur;
+      cur = nxt;
+      nxt = q;
+      float* f = wcur;
+      wcur = wnxt;
+      wnxt = f;
+    } else {
+      PRDF_TRY(pass(m, B + 8 * p));
+    }
+  }
+  in->m = m;
+  PRDF_TRY(in->off.alloc((size_t)n + 1, s));
+  PRDF_TRY(in->adj.alloc(room, s));
+  if (w) {
+    PRDF_TRY(in->w.alloc(room, s));
+    PRDF_CUDA(cudaMemcpyAsync(in->w.p, wcur, sizeof(float) * (size_t)m, cudaMemcpyDeviceToDevice, s));
+  } else {
+    in->w.release();
+  }
+  k_emit<<<grid_for(m, kRT), kRT, 0, s>>>(cur, m, B, n, in->adj.p, in->off.p);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
+}
+
+}  // namespace
+
+int build_csr_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, bool self_loops, Csr& out,
+                    Workspace& ws, cudaStream_t s) {
+  return build_radix(n, m0, rows, cols, nullptr, self_loops, out, nullptr, ws, s);
+}
+
+int build_csr_pair_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols, const float* w,
+                         bool self_loops, Csr& out, Csr& in, Workspace& ws, cudaStream_t s) {
+  return build_radix(n, m0, rows, cols, w, self_loops, out, &in, ws, s);
 }
 
 }  // namespace prdf
