@@ -116,29 +116,41 @@ __global__ void k_rows_scatter(const double* __restrict__ src, const int32_t* __
   }
 }
 
-// in-CSR weights from out-CSR weights: slot (u -> v) of row u holds w; find u in in-row v
-__global__ void k_weights_to_in(const int64_t* __restrict__ ooff, const int32_t* __restrict__ oadj,
-                                const float* __restrict__ w, int32_t n, const int64_t* __restrict__ ioff,
-                                const int32_t* __restrict__ iadj, float* __restrict__ win, int* __restrict__ bad) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int flag = 0;
-  for (int64_t u = warp; u < n; u += nwarps) {
-    for (int64_t j = ooff[u] + lane; j < ooff[u + 1]; j += 32) {
-      const float x = w[j];
-      if (!(x > 0.f) || !isfinite(x)) flag = 1;
-      const int32_t v = oadj[j];
-      int64_t lo = ioff[v], hi = ioff[v + 1];
-      while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (iadj[mid] < (int32_t)u) lo = mid + 1; else hi = mid;
-      }
-      win[lo] = x;  // (v, u) is in G' because (u, v) is in G
+// in-CSR slot of each out-CSR slot: entry (u -> v) of row u is entry u of in-row v
+// (slot null, graphs of 2^32 edges and more: the weight moves there at once)
+__global__ void k_in_slots(const int64_t* __restrict__ ooff, const int32_t* __restrict__ oadj, int32_t n, int64_t m,
+                           const int64_t* __restrict__ ioff, const int32_t* __restrict__ iadj,
+                           uint32_t* __restrict__ slot, const float* __restrict__ w, float* __restrict__ wi) {
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+    int64_t a = 0, z = n;  // the row of slot j: the last u with ooff[u] <= j
+    while (z - a > 1) {
+      const int64_t mid = (a + z) >> 1;
+      if (ooff[mid] <= j) a = mid; else z = mid;
     }
+    const int32_t v = oadj[j];
+    int64_t lo = ioff[v], hi = ioff[v + 1];
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (iadj[mid] < (int32_t)a) lo = mid + 1; else hi = mid;
+    }
+    // (v, u) is in G' because (u, v) is in G
+    if (slot) slot[j] = (uint32_t)lo;
+    else wi[lo] = w[j];
+  }
+}
+
+// in-CSR weights from out-CSR weights
+__global__ void k_weights_to_in(const float* __restrict__ w, int64_t m, const uint32_t* __restrict__ slot,
+                                float* __restrict__ wo, float* __restrict__ wi, int* __restrict__ bad) {
+  int flag = 0;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+    const float x = w[j];
+    if (!(x > 0.f) || !isfinite(x)) flag = 1;
+    wo[j] = x;
+    if (slot) wi[slot[j]] = x;
   }
   flag = __reduce_or_sync(0xffffffffu, flag);
-  if (lane == 0 && flag) atomicOr(bad, 1);
+  if ((threadIdx.x & 31) == 0 && flag) atomicOr(bad, 1);
 }
 
 // R[perm[i]] = x[i] * |out(perm[i])|; dV_out[perm[i]] = dV[i]
@@ -1249,6 +1261,7 @@ int prdf_graph_apply_batch(prdf_graph* g, const int32_t* del_src, const int32_t*
     rl.drift += nb;
     ++rl.version;
     g->orig_valid = false;
+    g->in_slot_valid = false;
     g->pvalid[0] = g->pvalid[1] = false;
     g->ppr_valid = false;
     PRDF_CUDA(cudaStreamSynchronize(s));
@@ -1301,6 +1314,7 @@ int prdf_graph_apply_batch(prdf_graph* g, const int32_t* del_src, const int32_t*
   g->csr[PRDF_IN] = static_cast<Csr&&>(nin);
   g->m = g->csr[PRDF_OUT].m;
   g->orig_valid = true;
+  g->in_slot_valid = false;
   g->pvalid[0] = g->pvalid[1] = false;
   PRDF_TRY(build_relabelled(g, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
@@ -1687,9 +1701,16 @@ int prdf_graph_set_weights(prdf_graph* g, const float* w, void* stream) {
   DBuf<int> bad;
   PRDF_TRY(bad.alloc(1, s));
   PRDF_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-  PRDF_CUDA(cudaMemcpyAsync(wo.p, w, sizeof(float) * (size_t)o.m, cudaMemcpyDeviceToDevice, s));
-  k_weights_to_in<<<grid_for((int64_t)g->n * 32, kThreads), kThreads, 0, s>>>(o.off.p, o.adj.p, w, g->n, in.off.p,
-                                                                               in.adj.p, wi.p, bad.p);
+  const bool keep = o.m < (1ll << 32);
+  if (!keep || !g->in_slot_valid) {
+    // where each edge sits in G', kept until the edges change
+    if (keep) PRDF_TRY(g->in_slot.reserve(o.m > 0 ? (size_t)o.m : 1, s));
+    k_in_slots<<<grid_for(o.m, kThreads), kThreads, 0, s>>>(o.off.p, o.adj.p, g->n, o.m, in.off.p, in.adj.p,
+                                                           keep ? g->in_slot.p : nullptr, w, wi.p);
+    PRDF_LAUNCH_CHECK();
+    g->in_slot_valid = keep;
+  }
+  k_weights_to_in<<<grid_for(o.m, kThreads), kThreads, 0, s>>>(w, o.m, keep ? g->in_slot.p : nullptr, wo.p, wi.p, bad.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaMemcpyAsync(g->ws.host_i64, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
@@ -1700,7 +1721,9 @@ int prdf_graph_set_weights(prdf_graph* g, const float* w, void* stream) {
   o.w = static_cast<DBuf<float>&&>(wo);
   in.w = static_cast<DBuf<float>&&>(wi);
   g->weighted = true;
-  PRDF_TRY(build_relabelled(g, s));
+  // the numbering does not depend on the weights: only they move
+  if (g->rl.valid) PRDF_TRY(permute_weights(g, s));
+  else PRDF_TRY(build_relabelled(g, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
   return PRDF_OK;
 }
@@ -1759,8 +1782,8 @@ int prdf_pagerank_backward(prdf_graph* g, const double* R, const double* G, int 
     k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(R, g->rl.perm.p, g->n, K, Kp, 1.0, Rr);
     PRDF_LAUNCH_CHECK();
     PRDF_TRY(launch_grad_w(g->rl.out.off.p, g->rl.out.adj.p, g->rl.perm.p, g->csr[PRDF_OUT].off.p, lam, g->S64.p, beta,
-                           Rr, g->wsum.p, g->n, Kp, p->alpha, grad_w, s));
-    ks.kernels += 2;
+                           Rr, g->wsum.p, g->n, g->m, Kp, p->alpha, grad_w, s));
+    ks.kernels += 3;
   }
   PRDF_CUDA(cudaEventRecord(t.e[2], s));
   PRDF_CUDA(cudaEventSynchronize(t.e[2]));

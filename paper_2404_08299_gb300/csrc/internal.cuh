@@ -283,7 +283,7 @@ int ppr_sparse_rhs(const double* S, int64_t n, int K, Workspace& ws, PprSparseRh
 int ppr_add_correction(double* R, const float* E, int64_t cnt, cudaStream_t s);
 int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, const int64_t* orig_off,
                   const double* lam, const double* Gs, double g_scale, const double* Rr, const double* W, int32_t n,
-                  int K, double alpha, double* grad_w, cudaStream_t s);
+                  int64_t m, int K, double alpha, double* grad_w, cudaStream_t s);
 int ppr_narrow(const double* x, int64_t cnt, float* y, cudaStream_t s);
 int ppr_widen(const float* y, int64_t cnt, double* x, cudaStream_t s);
 
@@ -315,6 +315,9 @@ struct prdf_graph {
   cudaStream_t stream = nullptr;
   prdf::Csr csr[2];                  // [PRDF_OUT] = G, [PRDF_IN] = G' in original ids (see orig_valid)
   bool orig_valid = true;            // false after a batch update until ensure_orig()
+  // in-CSR slot of each out-CSR slot (original ids), kept until the edges change; for set_weights
+  prdf::DBuf<uint32_t> in_slot;
+  bool in_slot_valid = false;
   int64_t m = 0;                     // edges of G (self-loops included)
   prdf::PartThr thr[2];              // class thresholds per CSR
   prdf::DBuf<int32_t> P[2];          // partitions
@@ -356,6 +359,8 @@ struct prdf_graph {
 namespace prdf {
 int build_relabelled(prdf_graph* g, cudaStream_t s);
 int build_ppr_weights(prdf_graph* g, cudaStream_t s);
+// the weights of the original-id CSRs into the sweep numbering's (rows in place)
+int permute_weights(prdf_graph* g, cudaStream_t s);
 // The CSRs of G and G' in original ids, derived from the sweep numbering's
 // copies when a batch update has changed those (rows come out sorted, as the
 // numbering keeps each row in original-id order).

@@ -600,30 +600,114 @@ __global__ void __launch_bounds__(kThreads, Traits<T>::kMinBlocks) k_ppr_loop(co
 // renumbered row i, vertex u = perm[i], target v = adj[j]):
 //   dL/dw_uv = (1 / W_u) * sum_c R[u, c] * (alpha * lambda[v, c] - (lambda[u, c] - G[u, c]))
 // using sum_k P_uk lambda[k] = (lambda[u] - G[u]) / alpha. The per-row constant
-// b_u = sum_c R[u, c] * (lambda[u, c] - G[u, c]) is formed once per row; one
-// warp per row, lanes over edges; written to the original out-slot order.
-__global__ void k_grad_w(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                         const int32_t* __restrict__ perm, const int64_t* __restrict__ orig_off,
-                         const double* __restrict__ lam, const double* __restrict__ Gs, double g_scale,
-                         const double* __restrict__ Rr, const double* __restrict__ W, int32_t n, int K, double alpha,
-                         double* __restrict__ grad_w) {
-  const int lane = threadIdx.x & 31;
+// b_u = sum_c R[u, c] * (lambda[u, c] - G[u, c]) is formed once per row.
+template <int L>
+__global__ void k_grad_rows(const double* __restrict__ lam, const double* __restrict__ Gs, double g_scale,
+                            const double* __restrict__ Rr, int32_t n, int K, double* __restrict__ bu) {
+  const int sub = threadIdx.x & (L - 1);
+  const int64_t row0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / L;
+  const int64_t step = ((int64_t)gridDim.x * blockDim.x) / L;
+  const int64_t last = ((int64_t)n + step - 1) / step * step;
+  for (int64_t i = row0; i < last; i += step) {  // (the same trip count on every lane)
+    double b = 0;
+    if (i < n)
+      for (int c = sub; c < K; c += L) b = fma(Rr[i * K + c], lam[i * K + c] - g_scale * Gs[i * K + c], b);
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) b += __shfl_xor_sync(kFull, b, o);
+    if (sub == 0 && i < n) bu[i] = b;
+  }
+}
+
+// A warp takes kGradChunk consecutive out-slots; L lanes (a slot) per edge,
+// columns over the lanes, four edges of a slot at a time, whose dot products
+// meet by exchanging halves (four additions for four edges instead of one per
+// edge and level: FP64 additions are what this kernel is short of after its
+// multiplications). The rows of long and short vertices cost the same per
+// edge (a lane per edge and a warp per row before: a serial walk over the
+// columns, and the longest row's walk at the end).
+constexpr int64_t kGradChunk = 512;
+template <int L>
+__global__ void __launch_bounds__(256) k_grad_w(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                const int32_t* __restrict__ perm, const int64_t* __restrict__ orig_off,
+                                                const double* __restrict__ lam, const double* __restrict__ bu,
+                                                const double* __restrict__ Rr, const double* __restrict__ W, int32_t n,
+                                                int64_t m, int K, double alpha, double* __restrict__ grad_w) {
+  constexpr int kSlots = 32 / L;
+  constexpr int kE = L < 4 ? L : 4;  // edges of a slot at a time
+  const int lane = threadIdx.x & 31, sub = lane & (L - 1), slot = lane / L;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    const double* Ri = Rr + i * K;
-    // b = sum_c R[i, c] * (lambda[i, c] - G[i, c]), lanes over columns
-    double b = 0;
-    for (int c = lane; c < K; c += 32) b = fma(Ri[c], lam[i * K + c] - g_scale * Gs[i * K + c], b);
-    b = warp_sum_f64(b);
-    const int32_t u = perm[i];
-    const double invW = 1.0 / W[i];
-    const int64_t rb = off[i], re = off[i + 1], ob = orig_off[u];
-    for (int64_t j = rb + lane; j < re; j += 32) {
-      const double* Lv = lam + (int64_t)adj[j] * K;
-      double d = 0;
-      for (int c = 0; c < K; ++c) d = fma(Ri[c], __ldg(Lv + c), d);
-      grad_w[ob + (j - rb)] = (alpha * d - b) * invW;
+  for (int64_t p0 = warp * kGradChunk; p0 < m; p0 += nwarps * kGradChunk) {
+    const int64_t pe = p0 + kGradChunk < m ? p0 + kGradChunk : m;
+    // row of the slot's first edge: the last r with off[r] <= p
+    int64_t r = 0, z = n;
+    while (z - r > 1) {
+      const int64_t mid = (r + z) >> 1;
+      if (off[mid] <= p0 + slot * kE) r = mid; else z = mid;
+    }
+    for (int64_t q0 = p0; q0 < pe; q0 += kSlots * kE) {
+      double d[kE];
+      int64_t row[kE];
+#pragma unroll
+      for (int k = 0; k < kE; ++k) {
+        const int64_t p = q0 + slot * kE + k;
+        d[k] = 0;
+        row[k] = -1;
+        if (p < pe) {
+          int steps = 0;
+          while (off[r + 1] <= p && steps < 8) {
+            ++r;
+            ++steps;
+          }
+          if (off[r + 1] <= p) {  // past a run of empty rows
+            int64_t a = r, b = n;
+            while (b - a > 1) {
+              const int64_t mid = (a + b) >> 1;
+              if (off[mid] <= p) a = mid; else b = mid;
+            }
+            r = a;
+          }
+          row[k] = r;
+          const double* Lv = lam + (int64_t)adj[p] * K;
+          const double* Ru = Rr + r * K;
+          if ((K & 1) == 0) {
+            for (int c = 2 * sub; c < K; c += 2 * L) {
+              const double2 x = __ldg(reinterpret_cast<const double2*>(Ru + c));
+              const double2 y = __ldg(reinterpret_cast<const double2*>(Lv + c));
+              d[k] = fma(x.x, y.x, d[k]);
+              d[k] = fma(x.y, y.y, d[k]);
+            }
+          } else {
+            for (int c = sub; c < K; c += L) d[k] = fma(__ldg(Ru + c), __ldg(Lv + c), d[k]);
+          }
+        }
+      }
+      // lane sub of the slot ends with the sum of edge sub % kE: exchange halves while several
+      // edges are left, then plain butterflies
+      int have = kE;
+      int mine = 0;
+#pragma unroll
+      for (int o = 1; o < kE; o <<= 1) {
+        have >>= 1;
+        const bool hi = sub & o;
+#pragma unroll
+        for (int k = 0; k < kE / 2; ++k) {
+          if (k < have) {
+            const double keep = hi ? d[2 * k + 1] : d[2 * k], give = hi ? d[2 * k] : d[2 * k + 1];
+            d[k] = keep + __shfl_xor_sync(kFull, give, o);
+          }
+        }
+        if (hi) mine += o;
+      }
+#pragma unroll
+      for (int o = kE; o < L; o <<= 1) d[0] += __shfl_xor_sync(kFull, d[0], o);
+      const int64_t p = q0 + slot * kE + mine;
+      int64_t rw = row[0];
+#pragma unroll
+      for (int k = 1; k < kE; ++k)
+        if (mine == k) rw = row[k];
+      if (sub < kE && rw >= 0 && p < pe)
+        grad_w[orig_off[perm[rw]] + (p - off[rw])] = (alpha * d[0] - bu[rw]) * (1.0 / W[rw]);
     }
   }
 }
@@ -733,9 +817,17 @@ int launch_ppr_loop(const PprArgs<double>& a, int tile, int64_t n, cudaStream_t 
 
 int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, const int64_t* orig_off,
                   const double* lam, const double* Gs, double g_scale, const double* Rr, const double* W, int32_t n,
-                  int K, double alpha, double* grad_w, cudaStream_t s) {
-  k_grad_w<<<grid_for((int64_t)n * 32, kThreads), kThreads, 0, s>>>(off, adj, perm, orig_off, lam, Gs, g_scale, Rr, W, n,
-                                                                     K, alpha, grad_w);
+                  int64_t m, int K, double alpha, double* grad_w, cudaStream_t s) {
+  DBuf<double> bu;
+  PRDF_TRY(bu.alloc((size_t)n, s));
+  const int grid = grid_for((m + kGradChunk - 1) / kGradChunk * 32, 256);
+  if (K > 8) {
+    k_grad_rows<8><<<grid_for((int64_t)n * 8, 256), 256, 0, s>>>(lam, Gs, g_scale, Rr, n, K, bu.p);
+    k_grad_w<8><<<grid, 256, 0, s>>>(off, adj, perm, orig_off, lam, bu.p, Rr, W, n, m, K, alpha, grad_w);
+  } else {
+    k_grad_rows<2><<<grid_for((int64_t)n * 2, 256), 256, 0, s>>>(lam, Gs, g_scale, Rr, n, K, bu.p);
+    k_grad_w<2><<<grid, 256, 0, s>>>(off, adj, perm, orig_off, lam, bu.p, Rr, W, n, m, K, alpha, grad_w);
+  }
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }

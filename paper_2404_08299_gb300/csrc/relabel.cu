@@ -87,17 +87,90 @@ __global__ void k_perm_rows(const int64_t* __restrict__ off, const int32_t* __re
   }
 }
 
-// sum of out-weights per row, one warp per row
-__global__ void k_row_wsum(const int64_t* __restrict__ off, const float* __restrict__ w, int32_t n,
-                           double* __restrict__ W) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = warp; v < n; v += nwarps) {
+// Weights alone of a permuted CSR whose rows are in place: slot p of new row i
+// gets w of the same entry of row perm[i]. Eight lanes per row; rows above
+// kLongRow entries (a warp's eight lanes would walk them for long) are listed
+// for k_long_weights, a block each.
+constexpr int kRowLanes = 8;
+constexpr int64_t kLongRow = 1024;
+
+__global__ void k_perm_weights(const int64_t* __restrict__ off, const float* __restrict__ w,
+                               const int32_t* __restrict__ perm, int32_t n, const int64_t* __restrict__ noff,
+                               float* __restrict__ nw, int32_t* __restrict__ longs, unsigned int* __restrict__ nlong) {
+  const int sub = threadIdx.x & (kRowLanes - 1);
+  const int64_t row0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kRowLanes;
+  const int64_t step = ((int64_t)gridDim.x * blockDim.x) / kRowLanes;
+  for (int64_t i = row0; i < n; i += step) {
+    const int64_t b = noff[i], len = noff[i + 1] - b, src = off[perm[i]];
+    if (len > kLongRow) {
+      if (sub == 0) longs[atomicAdd(nlong, 1u)] = (int32_t)i;
+      continue;
+    }
+    for (int64_t j = sub; j < len; j += kRowLanes) nw[b + j] = w[src + j];
+  }
+}
+
+__global__ void k_long_weights(const int64_t* __restrict__ off, const float* __restrict__ w,
+                               const int32_t* __restrict__ perm, const int64_t* __restrict__ noff,
+                               float* __restrict__ nw, const int32_t* __restrict__ longs,
+                               const unsigned int* __restrict__ nlong) {
+  for (unsigned int k = blockIdx.x; k < *nlong; k += gridDim.x) {
+    const int32_t i = longs[k];
+    const int64_t b = noff[i], len = noff[i + 1] - b, src = off[perm[i]];
+    for (int64_t j = threadIdx.x; j < len; j += blockDim.x) nw[b + j] = w[src + j];
+  }
+}
+
+// Sum of a row's out-weights, and P on its out-slots of the renumbered G:
+// slot j gets w_j / W (rows split over lanes as above; a fixed order, so every
+// run gives the same bits).
+__global__ void k_row_probs(const int64_t* __restrict__ off, const float* __restrict__ w, int32_t n,
+                            double* __restrict__ W, double* __restrict__ p64, float* __restrict__ p32,
+                            int32_t* __restrict__ longs, unsigned int* __restrict__ nlong) {
+  const int sub = threadIdx.x & (kRowLanes - 1);
+  const int64_t row0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kRowLanes;
+  const int64_t step = ((int64_t)gridDim.x * blockDim.x) / kRowLanes;
+  const unsigned int mask = ((1u << kRowLanes) - 1u) << (threadIdx.x & 31 & ~(kRowLanes - 1));
+  for (int64_t i = row0; i < n; i += step) {
+    const int64_t b = off[i], e = off[i + 1];
+    if (e - b > kLongRow) {
+      if (sub == 0) longs[atomicAdd(nlong, 1u)] = (int32_t)i;
+      continue;
+    }
     double s = 0;
-    for (int64_t j = off[v] + lane; j < off[v + 1]; j += 32) s += (double)w[j];
+    for (int64_t j = b + sub; j < e; j += kRowLanes) s += (double)w[j];
+#pragma unroll
+    for (int o = kRowLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+    if (sub == 0) W[i] = s;
+    for (int64_t j = b + sub; j < e; j += kRowLanes) {
+      const double p = (double)w[j] / s;
+      p64[j] = p;
+      p32[j] = (float)p;
+    }
+  }
+}
+
+__global__ void k_long_probs(const int64_t* __restrict__ off, const float* __restrict__ w, double* __restrict__ W,
+                             double* __restrict__ p64, float* __restrict__ p32, const int32_t* __restrict__ longs,
+                             const unsigned int* __restrict__ nlong) {
+  __shared__ double sh[32];
+  for (unsigned int k = blockIdx.x; k < *nlong; k += gridDim.x) {
+    const int32_t i = longs[k];
+    const int64_t b = off[i], e = off[i + 1];
+    double s = 0;
+    for (int64_t j = b + threadIdx.x; j < e; j += blockDim.x) s += (double)w[j];
     s = warp_sum_f64(s);
-    if (lane == 0) W[v] = s;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += sh[q];
+    if (threadIdx.x == 0) W[i] = s;
+    for (int64_t j = b + threadIdx.x; j < e; j += blockDim.x) {
+      const double p = (double)w[j] / s;
+      p64[j] = p;
+      p32[j] = (float)p;
+    }
   }
 }
 
@@ -109,22 +182,6 @@ __global__ void k_pin(const int32_t* __restrict__ new_src, const float* __restri
     const double p = (double)w[j] / W[new_src[j]];
     p64[j] = p;
     p32[j] = (float)p;
-  }
-}
-
-// P on the out-slots of the renumbered G: row i divides by its own W
-__global__ void k_pout(const int64_t* __restrict__ off, const float* __restrict__ w, const double* __restrict__ W,
-                       int32_t n, double* __restrict__ p64, float* __restrict__ p32) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    const double Wi = W[i];
-    for (int64_t j = off[i] + lane; j < off[i + 1]; j += 32) {
-      const double p = (double)w[j] / Wi;
-      p64[j] = p;
-      p32[j] = (float)p;
-    }
   }
 }
 
@@ -242,20 +299,46 @@ int build_relabelled(prdf_graph* g, cudaStream_t s) {
   return PRDF_OK;
 }
 
+int permute_weights(prdf_graph* g, cudaStream_t s) {
+  const int32_t n = g->n;
+  Relabel& r = g->rl;
+  DBuf<int32_t> longs;
+  DBuf<unsigned int> cnt;
+  PRDF_TRY(longs.alloc((size_t)n, s));
+  PRDF_TRY(cnt.alloc(1, s));
+  for (int which = 0; which < 2; ++which) {
+    const Csr& c = g->csr[which];
+    Csr& d = which == PRDF_OUT ? r.out : r.in;
+    PRDF_TRY(d.w.reserve(d.m > 0 ? (size_t)d.m : 1, s));
+    PRDF_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned int), s));
+    k_perm_weights<<<grid_for((int64_t)n * kRowLanes, kThreads), kThreads, 0, s>>>(c.off.p, c.w.p, r.perm.p, n, d.off.p,
+                                                                                  d.w.p, longs.p, cnt.p);
+    k_long_weights<<<kSMs * 4, kThreads, 0, s>>>(c.off.p, c.w.p, r.perm.p, d.off.p, d.w.p, longs.p, cnt.p);
+    PRDF_LAUNCH_CHECK();
+  }
+  g->ppr_valid = false;
+  return PRDF_OK;
+}
+
 int build_ppr_weights(prdf_graph* g, cudaStream_t s) {
   const int32_t n = g->n;
   const Relabel& r = g->rl;
   const int64_t m = r.in.m;
-  PRDF_TRY(g->wsum.alloc((size_t)n, s));
-  // each row holds its vertex's entries in original-id order: the same sum as over the original CSR
-  k_row_wsum<<<grid_for((int64_t)n * 32, kThreads), kThreads, 0, s>>>(r.out.off.p, r.out.w.p, n, g->wsum.p);
-  PRDF_TRY(g->pin64.alloc((size_t)m, s));
-  PRDF_TRY(g->pin32.alloc((size_t)m, s));
-  PRDF_TRY(g->pout64.alloc((size_t)m, s));
-  PRDF_TRY(g->pout32.alloc((size_t)m, s));
+  PRDF_TRY(g->wsum.reserve((size_t)n, s));
+  PRDF_TRY(g->pin64.reserve((size_t)m, s));
+  PRDF_TRY(g->pin32.reserve((size_t)m, s));
+  PRDF_TRY(g->pout64.reserve((size_t)m, s));
+  PRDF_TRY(g->pout32.reserve((size_t)m, s));
+  DBuf<int32_t> longs;
+  DBuf<unsigned int> cnt;
+  PRDF_TRY(longs.alloc((size_t)n, s));
+  PRDF_TRY(cnt.alloc(1, s));
+  PRDF_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned int), s));
+  k_row_probs<<<grid_for((int64_t)n * kRowLanes, kThreads), kThreads, 0, s>>>(r.out.off.p, r.out.w.p, n, g->wsum.p,
+                                                                             g->pout64.p, g->pout32.p, longs.p, cnt.p);
+  k_long_probs<<<kSMs * 4, kThreads, 0, s>>>(r.out.off.p, r.out.w.p, g->wsum.p, g->pout64.p, g->pout32.p, longs.p,
+                                             cnt.p);
   k_pin<<<grid_for(m, kThreads), kThreads, 0, s>>>(r.in.adj.p, r.in.w.p, g->wsum.p, m, g->pin64.p, g->pin32.p);
-  k_pout<<<grid_for((int64_t)n * 32, kThreads), kThreads, 0, s>>>(r.out.off.p, r.out.w.p, g->wsum.p, n,
-                                                                   g->pout64.p, g->pout32.p);
   PRDF_LAUNCH_CHECK();
   g->ppr_valid = true;
   return PRDF_OK;
