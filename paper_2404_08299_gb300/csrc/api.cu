@@ -256,11 +256,19 @@ __global__ void k_effective(const int32_t* __restrict__ s, const int32_t* __rest
   }
 }
 
-// ids of a batch list in the sweep numbering: out[i] = inv[a[i]]
-__global__ void k_map_ids(const int32_t* __restrict__ a, int64_t cnt, const int32_t* __restrict__ inv,
-                          int32_t* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = inv[a[i]];
+// The batch's ids in the sweep numbering: out = inv of del_src, del_dst, ins_src, ins_dst, one after the other.
+__global__ void k_map_batch(const int32_t* __restrict__ ds, const int32_t* __restrict__ dd, int64_t n_del,
+                            const int32_t* __restrict__ is, const int32_t* __restrict__ id, int64_t n_ins,
+                            const int32_t* __restrict__ inv, int32_t* __restrict__ out) {
+  const int64_t tot = 2 * (n_del + n_ins);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v;
+    if (i < n_del) v = ds[i];
+    else if (i < 2 * n_del) v = dd[i - n_del];
+    else if (i < 2 * n_del + n_ins) v = is[i - 2 * n_del];
+    else v = id[i - 2 * n_del - n_ins];
+    out[i] = inv[v];
+  }
 }
 
 // position of (u, v) (original ids) in a CSR of the sweep numbering, whose row inv[u] lists renumbered ids in
@@ -1215,20 +1223,22 @@ int prdf_graph_apply_batch(prdf_graph* g, const int32_t* del_src, const int32_t*
     int32_t* del_r_in = rows.p + n_del;    // inv[del_dst]
     int32_t* ins_r_out = rows.p + 2 * n_del;
     int32_t* ins_r_in = rows.p + 2 * n_del + n_ins;
-    if (n_del) {
-      k_map_ids<<<grid_for(n_del, kThreads), kThreads, 0, s>>>(del_src, n_del, rl.inv.p, del_r_out);
-      k_map_ids<<<grid_for(n_del, kThreads), kThreads, 0, s>>>(del_dst, n_del, rl.inv.p, del_r_in);
-    }
-    if (n_ins) {
-      k_map_ids<<<grid_for(n_ins, kThreads), kThreads, 0, s>>>(ins_src, n_ins, rl.inv.p, ins_r_out);
-      k_map_ids<<<grid_for(n_ins, kThreads), kThreads, 0, s>>>(ins_dst, n_ins, rl.inv.p, ins_r_in);
-    }
+    if (nb)
+      k_map_batch<<<grid_for(2 * nb, kThreads), kThreads, 0, s>>>(del_src, del_dst, n_del, ins_src, ins_dst, n_ins,
+                                                                 rl.inv.p, rows.p);
     PRDF_LAUNCH_CHECK();
-    Csr nout, nin;
-    PRDF_TRY(update_csr(n, rl.out, del_r_out, del_dst, n_del, ins_r_out, ins_dst, ins_w, n_ins, nout, g->ws, s,
-                        rl.perm.p, rl.inv.p));
-    PRDF_TRY(update_csr(n, rl.in, del_r_in, del_src, n_del, ins_r_in, ins_src, ins_w, n_ins, nin, g->ws, s,
-                        rl.perm.p, rl.inv.p));
+    const BatchLists lists[2] = {{del_r_out, del_dst, n_del, ins_r_out, ins_dst, n_ins},
+                                 {del_r_in, del_src, n_del, ins_r_in, ins_src, n_ins}};
+    Csr both[2];
+    {
+      Csr old[2] = {static_cast<Csr&&>(rl.out), static_cast<Csr&&>(rl.in)};
+      const int rc = update_csr_pair(n, old, lists, ins_w, both, g->ws, s, rl.perm.p, rl.inv.p);
+      rl.out = static_cast<Csr&&>(old[0]);
+      rl.in = static_cast<Csr&&>(old[1]);
+      if (rc != PRDF_OK) return rc;
+    }
+    Csr& nout = both[0];
+    Csr& nin = both[1];
     if (del_eff && n_del)
       k_effective_keyed<<<grid_for(n_del, kThreads), kThreads, 0, s>>>(del_src, del_dst, n_del, 1, rl.perm.p,
                                                                        rl.inv.p, rl.out.off.p, rl.out.adj.p,
@@ -1278,8 +1288,13 @@ int prdf_graph_apply_batch(prdf_graph* g, const int32_t* del_src, const int32_t*
   const int64_t m = old.m;
   Csr nout, nin;
   if (g->self_loops) {
-    PRDF_TRY(update_csr(n, g->csr[PRDF_OUT], del_src, del_dst, n_del, ins_src, ins_dst, ins_w, n_ins, nout, g->ws, s));
-    PRDF_TRY(update_csr(n, g->csr[PRDF_IN], del_dst, del_src, n_del, ins_dst, ins_src, ins_w, n_ins, nin, g->ws, s));
+    const BatchLists lists[2] = {{del_src, del_dst, n_del, ins_src, ins_dst, n_ins},
+                                 {del_dst, del_src, n_del, ins_dst, ins_src, n_ins}};
+    Csr both[2];
+    static_assert(PRDF_OUT == 0 && PRDF_IN == 1, "csr[] holds G, then G'");
+    PRDF_TRY(update_csr_pair(n, g->csr, lists, ins_w, both, g->ws, s));
+    nout = static_cast<Csr&&>(both[0]);
+    nin = static_cast<Csr&&>(both[1]);
   } else {
     DBuf<uint8_t> deleted;
     PRDF_TRY(deleted.alloc((size_t)m, s));

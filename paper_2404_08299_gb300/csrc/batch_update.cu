@@ -18,6 +18,8 @@
 // every comparison with an old entry uses key[entry], the batch's columns are
 // original ids, and store (original -> renumbered) maps an added column to the
 // value stored; rows stay ordered by original id.
+#include <cstring>
+
 #include "internal.cuh"
 
 namespace prdf {
@@ -134,10 +136,11 @@ __global__ void k_list_changed(int32_t n, const uint32_t* __restrict__ flag, con
 // the last one). A warp takes 256 consecutive entries (8 per lane,
 // lane-strided, so loads and stores stay coalesced) and finds its place in the
 // changed-row list once.
-__global__ void k_copy_unchanged(int32_t n, int64_t m, const int64_t* __restrict__ off,
-                                 const int64_t* __restrict__ noff, const int32_t* __restrict__ changed, int64_t k,
-                                 const int32_t* __restrict__ adj, const float* __restrict__ w,
-                                 int32_t* __restrict__ nadj, float* __restrict__ nw) {
+__device__ __forceinline__ void copy_unchanged(int32_t n, int64_t m, const int64_t* __restrict__ off,
+                                               const int64_t* __restrict__ noff, const int32_t* __restrict__ changed,
+                                               int64_t k, const int32_t* __restrict__ adj,
+                                               const float* __restrict__ w, int32_t* __restrict__ nadj,
+                                               float* __restrict__ nw) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -191,6 +194,13 @@ __global__ void k_copy_unchanged(int32_t n, int64_t m, const int64_t* __restrict
       if (nw) nw[to] = w[j];
     }
   }
+}
+
+__global__ void k_copy_unchanged(int32_t n, int64_t m, const int64_t* __restrict__ off,
+                                 const int64_t* __restrict__ noff, const int32_t* __restrict__ changed, int64_t k,
+                                 const int32_t* __restrict__ adj, const float* __restrict__ w,
+                                 int32_t* __restrict__ nadj, float* __restrict__ nw) {
+  copy_unchanged(n, m, off, noff, changed, k, adj, w, nadj, nw);
 }
 
 // length of each changed row (for the entry-parallel pass below)
@@ -310,31 +320,40 @@ __device__ void block_sort(uint64_t* k, int32_t* p, int cnt) {
 }
 
 // exclusive scan of v[0..cnt) in shared memory, in place; returns the total (every thread);
-// every thread of the block must call it
-__device__ int64_t block_scan(int64_t* v, int cnt, int64_t* tmp /* blockDim.x + 1 */) {
+// every thread of the block must call it (tmp: a word per warp and one more)
+__device__ int64_t block_scan(int64_t* v, int cnt, int64_t* tmp) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = (int)(blockDim.x >> 5);
   const int per = (cnt + blockDim.x - 1) / blockDim.x;
-  const int b = threadIdx.x * per, e = min(b + per, cnt);
+  const int b = min((int)threadIdx.x * per, cnt), e = min(b + per, cnt);
   int64_t sum = 0;
   for (int i = b; i < e; ++i) sum += v[i];
-  tmp[threadIdx.x] = sum;
+  int64_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += x;
+  }
+  if (lane == 31) tmp[wid] = incl;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t run = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int64_t x = tmp[t];
-      tmp[t] = run;
-      run += x;
+  if (wid == 0) {
+    const int64_t x = lane < nwarp ? tmp[lane] : 0;
+    int64_t t = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
     }
-    tmp[blockDim.x] = run;
+    if (lane < nwarp) tmp[lane] = t - x;
+    if (lane == 31) tmp[nwarp] = t;
   }
   __syncthreads();
-  int64_t run = tmp[threadIdx.x];
+  int64_t run = tmp[wid] + incl - sum;
+  const int64_t total = tmp[nwarp];
   for (int i = b; i < e; ++i) {
     const int64_t x = v[i];
     v[i] = run;
     run += x;
   }
-  const int64_t total = tmp[blockDim.x];
   __syncthreads();
   return total;
 }
@@ -347,29 +366,63 @@ __device__ __forceinline__ int lower_bound_u64(const uint64_t* a, int lo, int hi
   return lo;
 }
 
-// One block: sorts and deduplicates D (self-loops dropped) and I (duplicates
-// keep the maximum weight), classifies every entry against the old rows (a
-// deletion removes, an insertion adds unless the edge survives), and lists the
-// changed rows with their ranges in the sorted lists and the prefix of their
-// length changes. Outputs: d_cols, dpref (nd + 1), i_rows, i_cols, i_w, iflag,
-// ipref (ni + 1), changed, c_db, c_de, c_ib, c_ie, c_shift (kc + 1),
-// sizes = {nd, ni, kc, total length change}.
-__global__ void __launch_bounds__(kPrepThreads) k_prep_small(
-    const int64_t* __restrict__ off, const int32_t* __restrict__ adj, const int32_t* __restrict__ key,
-    const int32_t* __restrict__ del_rows, const int32_t* __restrict__ del_cols, int64_t n_del,
-    const int32_t* __restrict__ ins_rows, const int32_t* __restrict__ ins_cols, const float* __restrict__ ins_w,
-    int64_t n_ins, int nd_pow, int ni_pow, int32_t* __restrict__ d_cols, int64_t* __restrict__ dpref,
-    int32_t* __restrict__ i_rows, int32_t* __restrict__ i_cols, float* __restrict__ i_w,
-    uint32_t* __restrict__ iflag, int64_t* __restrict__ ipref, int32_t* __restrict__ changed,
-    int64_t* __restrict__ c_db, int64_t* __restrict__ c_de, int64_t* __restrict__ c_ib, int64_t* __restrict__ c_ie,
-    int64_t* __restrict__ c_shift, int64_t* __restrict__ sizes) {
+// One CSR of a small batch update (G or G'): its old rows, the batch as
+// (row, column) pairs, and what k_prep_small works out for the passes after it.
+struct SmallSide {
+  const int64_t* off;
+  const int32_t* adj;
+  const float* w;          // null: unweighted
+  int64_t m;
+  const int32_t *del_rows, *del_cols, *ins_rows, *ins_cols;
+  // sorted, deduplicated batch and prefixes of its effective entries
+  int32_t *d_cols, *i_rows, *i_cols;
+  float* i_w;
+  uint32_t* iflag;
+  int64_t *dpref, *ipref;
+  // changed rows: ids, ranges in D and I, length change and old entries before each
+  int32_t* changed;
+  int64_t *c_db, *c_de, *c_ib, *c_ie, *c_shift, *cpref;
+  int64_t* sizes;          // nd, ni, changed rows, total length change, old entries of the changed rows
+  // known to the host after k_prep_small
+  int64_t ni, kc, T;
+  int64_t* noff;
+  int32_t* nadj;
+  float* nw;
+};
+struct SmallSides {
+  SmallSide s[2];
+  const int32_t* key;      // see update_csr
+  const int32_t* store;
+  const float* ins_w;      // null: unweighted
+  int64_t n_del, n_ins;
+  int32_t n;
+};
+
+// One block per side: sorts and deduplicates D (self-loops dropped) and I
+// (duplicates keep the maximum weight), classifies every entry against the old
+// rows (a deletion removes, an insertion adds unless the edge survives), and
+// lists the changed rows with their ranges in the sorted lists and the
+// prefixes of their length changes and of their old lengths.
+__global__ void __launch_bounds__(kPrepThreads) k_prep_small(const SmallSides S, int nd_pow, int ni_pow) {
+  const SmallSide& a = S.s[blockIdx.x];
+  const int64_t* __restrict__ off = a.off;
+  const int32_t* __restrict__ adj = a.adj;
+  const int32_t* __restrict__ key = S.key;
+  const int32_t *del_rows = a.del_rows, *del_cols = a.del_cols, *ins_rows = a.ins_rows, *ins_cols = a.ins_cols;
+  const float* ins_w = S.ins_w;
+  const int64_t n_del = S.n_del, n_ins = S.n_ins;
+  int32_t *d_cols = a.d_cols, *i_rows = a.i_rows, *i_cols = a.i_cols, *changed = a.changed;
+  float* i_w = a.i_w;
+  uint32_t* iflag = a.iflag;
+  int64_t *dpref = a.dpref, *ipref = a.ipref, *c_db = a.c_db, *c_de = a.c_de, *c_ib = a.c_ib, *c_ie = a.c_ie;
+  int64_t *c_shift = a.c_shift, *sizes = a.sizes;
   extern __shared__ __align__(16) unsigned char smem[];
   uint64_t* dk = reinterpret_cast<uint64_t*>(smem);  // D keys (nd_pow)
   uint64_t* ik = dk + nd_pow;                         // I keys (ni_pow)
   uint64_t* rk = ik + ni_pow;                         // changed rows (nd_pow + ni_pow)
   int64_t* cnt = reinterpret_cast<int64_t*>(rk + nd_pow + ni_pow);  // scratch counts (nd_pow + ni_pow)
   int32_t* ip = reinterpret_cast<int32_t*>(cnt + nd_pow + ni_pow);  // I payload (ni_pow)
-  __shared__ int64_t tmp[kPrepThreads + 1];
+  __shared__ int64_t tmp[kPrepThreads / 32 + 1];
   __shared__ int s_nd, s_ni, s_kc;
   for (int i = threadIdx.x; i < nd_pow; i += blockDim.x) {
     uint64_t kk = kNoKey;
@@ -472,17 +525,35 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_small(
   __syncthreads();
   const int64_t run = block_scan(sh, (int)kc, tmp);
   for (int t = threadIdx.x; t <= kc; t += blockDim.x) c_shift[t] = t < kc ? sh[t] : run;
+  __syncthreads();
+  // and the same of their old lengths
+  for (int t = threadIdx.x; t < kc; t += blockDim.x) sh[t] = off[changed[t] + 1] - off[changed[t]];
+  __syncthreads();
+  const int64_t old = block_scan(sh, (int)kc, tmp);
+  for (int t = threadIdx.x; t <= kc; t += blockDim.x) a.cpref[t] = t < kc ? sh[t] : old;
   if (threadIdx.x == 0) {
     sizes[0] = nd;
     sizes[1] = ni;
     sizes[2] = kc;
     sizes[3] = run;
+    sizes[4] = old;
   }
 }
 
+__global__ void k_copy_unchanged_t(const SmallSides S) {
+  const SmallSide& a = S.s[blockIdx.y];
+  copy_unchanged(S.n, a.m, a.off, a.noff, a.changed, a.kc, a.adj, a.w, a.nadj, a.nw);
+}
+
 // new row offsets: noff[u] = off[u] + the length change of the changed rows before u (u in [0, n])
-__global__ void k_new_offsets(int32_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ changed,
-                              int64_t kc, const int64_t* __restrict__ c_shift, int64_t* __restrict__ noff) {
+__global__ void k_new_offsets(const SmallSides S) {
+  const SmallSide& a = S.s[blockIdx.y];
+  const int32_t n = S.n;
+  const int64_t* __restrict__ off = a.off;
+  const int32_t* __restrict__ changed = a.changed;
+  const int64_t kc = a.kc;
+  const int64_t* __restrict__ c_shift = a.c_shift;
+  int64_t* __restrict__ noff = a.noff;
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= n; u += (int64_t)gridDim.x * blockDim.x) {
     int64_t lo = 0, hi = kc;
     while (lo < hi) {
@@ -494,15 +565,20 @@ __global__ void k_new_offsets(int32_t n, const int64_t* __restrict__ off, const 
 }
 
 // surviving old entries of the changed rows (as k_move_changed, with each changed row's batch ranges given)
-__global__ void k_move_changed_t(const int32_t* __restrict__ changed, int64_t k, const int64_t* __restrict__ cpref,
-                                 int64_t T, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                 const int32_t* __restrict__ key, const float* __restrict__ w,
-                                 const int64_t* __restrict__ c_db, const int64_t* __restrict__ c_de,
-                                 const int64_t* __restrict__ c_ib, const int64_t* __restrict__ c_ie,
-                                 const int32_t* __restrict__ d_cols, const int64_t* __restrict__ dpref,
-                                 const int32_t* __restrict__ i_cols, const float* __restrict__ i_w,
-                                 const int64_t* __restrict__ ipref, const int64_t* __restrict__ noff,
-                                 int32_t* __restrict__ nadj, float* __restrict__ nw) {
+__global__ void k_move_changed_t(const SmallSides S) {
+  const SmallSide& a = S.s[blockIdx.y];
+  const int32_t* __restrict__ changed = a.changed;
+  const int64_t k = a.kc, T = a.T;
+  const int64_t *__restrict__ cpref = a.cpref, *__restrict__ off = a.off;
+  const int32_t *__restrict__ adj = a.adj, *__restrict__ key = S.key;
+  const float* __restrict__ w = a.w;
+  const int64_t *__restrict__ c_db = a.c_db, *__restrict__ c_de = a.c_de, *__restrict__ c_ib = a.c_ib,
+                *__restrict__ c_ie = a.c_ie;
+  const int32_t *__restrict__ d_cols = a.d_cols, *__restrict__ i_cols = a.i_cols;
+  const int64_t *__restrict__ dpref = a.dpref, *__restrict__ ipref = a.ipref, *__restrict__ noff = a.noff;
+  const float* __restrict__ i_w = a.i_w;
+  int32_t* __restrict__ nadj = a.nadj;
+  float* __restrict__ nw = a.nw;
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -534,15 +610,19 @@ __global__ void k_move_changed_t(const int32_t* __restrict__ changed, int64_t k,
 }
 
 // adding I entries of a small batch (thread per entry)
-__global__ void k_place_new_t(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                              const int32_t* __restrict__ key, const int32_t* __restrict__ store,
-                              const int32_t* __restrict__ changed, int64_t kc, const int64_t* __restrict__ c_db,
-                              const int64_t* __restrict__ c_ib, const int32_t* __restrict__ d_cols,
-                              const int64_t* __restrict__ c_de, const int64_t* __restrict__ dpref,
-                              const int32_t* __restrict__ i_rows, const int32_t* __restrict__ i_cols,
-                              const float* __restrict__ i_w, const uint32_t* __restrict__ iflag,
-                              const int64_t* __restrict__ ipref, int64_t ni, const int64_t* __restrict__ noff,
-                              int32_t* __restrict__ nadj, float* __restrict__ nw) {
+__global__ void k_place_new_t(const SmallSides S) {
+  const SmallSide& a = S.s[blockIdx.y];
+  const int64_t *__restrict__ off = a.off, *__restrict__ c_db = a.c_db, *__restrict__ c_de = a.c_de,
+                *__restrict__ c_ib = a.c_ib, *__restrict__ dpref = a.dpref, *__restrict__ ipref = a.ipref,
+                *__restrict__ noff = a.noff;
+  const int32_t *__restrict__ adj = a.adj, *__restrict__ key = S.key, *__restrict__ store = S.store,
+                *__restrict__ changed = a.changed, *__restrict__ d_cols = a.d_cols, *__restrict__ i_rows = a.i_rows,
+                *__restrict__ i_cols = a.i_cols;
+  const float* __restrict__ i_w = a.i_w;
+  const uint32_t* __restrict__ iflag = a.iflag;
+  const int64_t kc = a.kc, ni = a.ni;
+  int32_t* __restrict__ nadj = a.nadj;
+  float* __restrict__ nw = a.nw;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ni; q += (int64_t)gridDim.x * blockDim.x) {
     if (!iflag[q]) continue;
     const int32_t u = i_rows[q], c = i_cols[q];
@@ -570,10 +650,14 @@ int pow2_at_least(int64_t x) {
   return p;
 }
 
-int update_csr_small(int32_t n, const Csr& old, const int32_t* del_rows, const int32_t* del_cols, int64_t n_del,
-                     const int32_t* ins_rows, const int32_t* ins_cols, const float* ins_w, int64_t n_ins, Csr& out,
-                     Workspace& ws, cudaStream_t s, const int32_t* key, const int32_t* store) {
-  const bool weighted = old.w.p != nullptr;
+// Both CSRs of a small batch, each pass one launch over both sides, and one
+// host read between the preparation and the passes that need its sizes. (One
+// CSR after the other with two reads each before: a 168-edge batch on 15 M
+// edges 0.56 ms.)
+int update_pair_small(int32_t n, const Csr* old, const BatchLists* b, const float* ins_w, Csr* out, Workspace& ws,
+                      cudaStream_t s, const int32_t* key, const int32_t* store) {
+  const bool weighted = old[0].w.p != nullptr;
+  const int64_t n_del = b[0].n_del, n_ins = b[0].n_ins;
   // both lists padded to one power of two P, so the union of their rows (2P keys) sorts as a power of two
   const int P = pow2_at_least(n_del > n_ins ? n_del : (n_ins > 0 ? n_ins : 1));
   const int nd_pow = P, ni_pow = P;
@@ -587,81 +671,99 @@ int update_csr_small(int32_t n, const Csr& old, const int32_t* del_rows, const i
   }();
   (void)smem_set;
   const size_t nb = (size_t)(n_del + n_ins > 0 ? n_del + n_ins : 1);
-  DBuf<int32_t> i32;  // d_cols | i_rows | i_cols | changed
-  DBuf<int64_t> i64;  // dpref | ipref | c_db | c_de | c_ib | c_ie | c_shift | sizes
+  const size_t n32 = (size_t)n_del + 2 * (size_t)n_ins + nb + 4;
+  const size_t n64 = (size_t)n_del + 1 + (size_t)n_ins + 1 + 6 * (nb + 1) + 5;
+  const size_t nw = (size_t)(n_ins > 0 ? n_ins : 1);
+  DBuf<int32_t> i32;
+  DBuf<int64_t> i64;
   DBuf<float> iw;
   DBuf<uint32_t> iflag;
-  PRDF_TRY(i32.alloc((size_t)n_del + 2 * (size_t)n_ins + nb + 4, s));
-  PRDF_TRY(i64.alloc((size_t)n_del + 1 + (size_t)n_ins + 1 + 5 * (nb + 1) + 4, s));
-  PRDF_TRY(iw.alloc((size_t)(n_ins > 0 ? n_ins : 1), s));
-  PRDF_TRY(iflag.alloc((size_t)(n_ins > 0 ? n_ins : 1), s));
-  int32_t* d_cols = i32.p;
-  int32_t* i_rows = d_cols + n_del;
-  int32_t* i_cols = i_rows + n_ins;
-  int32_t* changed = i_cols + n_ins;
-  int64_t* dpref = i64.p;
-  int64_t* ipref = dpref + n_del + 1;
-  int64_t* c_db = ipref + n_ins + 1;
-  int64_t* c_de = c_db + (nb + 1);
-  int64_t* c_ib = c_de + (nb + 1);
-  int64_t* c_ie = c_ib + (nb + 1);
-  int64_t* c_shift = c_ie + (nb + 1);
-  int64_t* sizes = c_shift + (nb + 1);
-  k_prep_small<<<1, kPrepThreads, smem, s>>>(old.off.p, old.adj.p, key, del_rows, del_cols, n_del, ins_rows, ins_cols,
-                                             weighted ? ins_w : nullptr, n_ins, nd_pow, ni_pow, d_cols, dpref, i_rows,
-                                             i_cols, iw.p, iflag.p, ipref, changed, c_db, c_de, c_ib, c_ie, c_shift,
-                                             sizes);
+  PRDF_TRY(i32.alloc(2 * n32, s));
+  PRDF_TRY(i64.alloc(2 * n64 + 10, s));
+  PRDF_TRY(iw.alloc(2 * nw, s));
+  PRDF_TRY(iflag.alloc(2 * nw, s));
+  SmallSides S;
+  memset(&S, 0, sizeof(S));
+  S.key = key;
+  S.store = store;
+  S.ins_w = weighted ? ins_w : nullptr;
+  S.n_del = n_del;
+  S.n_ins = n_ins;
+  S.n = n;
+  for (int k = 0; k < 2; ++k) {
+    SmallSide& a = S.s[k];
+    a.off = old[k].off.p;
+    a.adj = old[k].adj.p;
+    a.w = old[k].w.p;
+    a.m = old[k].m;
+    a.del_rows = b[k].del_rows;
+    a.del_cols = b[k].del_cols;
+    a.ins_rows = b[k].ins_rows;
+    a.ins_cols = b[k].ins_cols;
+    a.d_cols = i32.p + k * n32;
+    a.i_rows = a.d_cols + n_del;
+    a.i_cols = a.i_rows + n_ins;
+    a.changed = a.i_cols + n_ins;
+    a.dpref = i64.p + 10 + k * n64;
+    a.ipref = a.dpref + n_del + 1;
+    a.c_db = a.ipref + n_ins + 1;
+    a.c_de = a.c_db + (nb + 1);
+    a.c_ib = a.c_de + (nb + 1);
+    a.c_ie = a.c_ib + (nb + 1);
+    a.c_shift = a.c_ie + (nb + 1);
+    a.cpref = a.c_shift + (nb + 1);
+    a.sizes = i64.p + 5 * k;
+    a.i_w = weighted ? iw.p + k * nw : nullptr;
+    a.iflag = iflag.p + k * nw;
+  }
+  k_prep_small<<<2, kPrepThreads, smem, s>>>(S, nd_pow, ni_pow);
   PRDF_LAUNCH_CHECK();
-  PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, sizes, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, i64.p, 10 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   PRDF_CUDA(cudaStreamSynchronize(s));
-  const int64_t ni = ws.host_i64[1], kc = ws.host_i64[2], dm = ws.host_i64[3];
-  out.m = old.m + dm;
-  PRDF_TRY(out.off.alloc((size_t)n + 1, s));
-  PRDF_TRY(out.adj.alloc((size_t)out.m + kAdjPad, s));
-  if (weighted) PRDF_TRY(out.w.alloc((size_t)(out.m > 0 ? out.m : 1), s));
-  else out.w.release();
-  k_new_offsets<<<grid_for((int64_t)n + 1, kThreads), kThreads, 0, s>>>(n, old.off.p, changed, kc, c_shift, out.off.p);
+  int64_t m = 0, T = 0, ni = 0;
+  for (int k = 0; k < 2; ++k) {
+    SmallSide& a = S.s[k];
+    const int64_t* h = ws.host_i64 + 5 * k;
+    a.ni = h[1];
+    a.kc = h[2];
+    a.T = h[4];
+    out[k].m = old[k].m + h[3];
+    if (old[k].m > m) m = old[k].m;
+    if (a.T > T) T = a.T;
+    if (a.ni > ni) ni = a.ni;
+  }
+  for (int k = 0; k < 2; ++k) {
+    PRDF_TRY(out[k].off.alloc((size_t)n + 1, s));
+    PRDF_TRY(out[k].adj.alloc((size_t)out[k].m + kAdjPad, s));
+    if (weighted) PRDF_TRY(out[k].w.alloc((size_t)(out[k].m > 0 ? out[k].m : 1), s));
+    else out[k].w.release();
+    S.s[k].noff = out[k].off.p;
+    S.s[k].nadj = out[k].adj.p;
+    S.s[k].nw = out[k].w.p;
+  }
+  k_new_offsets<<<dim3(grid_for((int64_t)n + 1, kThreads, kSMs * 16), 2), kThreads, 0, s>>>(S);
+  if (m > 0) k_copy_unchanged_t<<<dim3(grid_for((m + 7) / 8, kThreads, kSMs * 16), 2), kThreads, 0, s>>>(S);
+  if (T > 0) k_move_changed_t<<<dim3(grid_for((T + 7) / 8, kThreads, kSMs * 16), 2), kThreads, 0, s>>>(S);
+  if (ni > 0) k_place_new_t<<<dim3(grid_for(ni, kThreads), 2), kThreads, 0, s>>>(S);
   PRDF_LAUNCH_CHECK();
-  if (old.m > 0) {
-    k_copy_unchanged<<<grid_for((old.m + 7) / 8, kThreads), kThreads, 0, s>>>(
-        n, old.m, old.off.p, out.off.p, changed, kc, old.adj.p, old.w.p, out.adj.p, out.w.p);
-    PRDF_LAUNCH_CHECK();
-  }
-  if (kc > 0) {
-    DBuf<int64_t> clen, cpref;
-    PRDF_TRY(clen.alloc((size_t)kc, s));
-    PRDF_TRY(cpref.alloc((size_t)kc + 1, s));
-    k_changed_len<<<grid_for(kc, kThreads), kThreads, 0, s>>>(changed, kc, old.off.p, clen.p);
-    PRDF_LAUNCH_CHECK();
-    PRDF_TRY(exclusive_scan_i64(clen.p, kc, cpref.p, ws, s));
-    PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, cpref.p + kc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    PRDF_CUDA(cudaStreamSynchronize(s));
-    const int64_t T = ws.host_i64[0];
-    if (T > 0) {
-      k_move_changed_t<<<grid_for((T + 7) / 8, kThreads), kThreads, 0, s>>>(
-          changed, kc, cpref.p, T, old.off.p, old.adj.p, key, old.w.p, c_db, c_de, c_ib, c_ie, d_cols, dpref, i_cols,
-          weighted ? iw.p : nullptr, ipref, out.off.p, out.adj.p, out.w.p);
-      PRDF_LAUNCH_CHECK();
-    }
-  }
-  if (ni > 0) {
-    k_place_new_t<<<grid_for(ni, kThreads), kThreads, 0, s>>>(old.off.p, old.adj.p, key, store, changed, kc, c_db, c_ib,
-                                                              d_cols, c_de, dpref, i_rows, i_cols,
-                                                              weighted ? iw.p : nullptr, iflag.p, ipref, ni, out.off.p,
-                                                              out.adj.p, out.w.p);
-    PRDF_LAUNCH_CHECK();
-  }
   return PRDF_OK;
 }
 
 }  // namespace
 
+int update_csr_pair(int32_t n, const Csr* old, const BatchLists* b, const float* ins_w, Csr* out, Workspace& ws,
+                    cudaStream_t s, const int32_t* key, const int32_t* store) {
+  if (b[0].n_del <= kSmallBatch && b[0].n_ins <= kSmallBatch)
+    return update_pair_small(n, old, b, ins_w, out, ws, s, key, store);
+  for (int k = 0; k < 2; ++k)
+    PRDF_TRY(update_csr(n, old[k], b[k].del_rows, b[k].del_cols, b[k].n_del, b[k].ins_rows, b[k].ins_cols, ins_w,
+                        b[k].n_ins, out[k], ws, s, key, store));
+  return PRDF_OK;
+}
+
 int update_csr(int32_t n, const Csr& old, const int32_t* del_rows, const int32_t* del_cols, int64_t n_del,
                const int32_t* ins_rows, const int32_t* ins_cols, const float* ins_w, int64_t n_ins, Csr& out,
                Workspace& ws, cudaStream_t s, const int32_t* key, const int32_t* store) {
-  if (n_del <= kSmallBatch && n_ins <= kSmallBatch)
-    return update_csr_small(n, old, del_rows, del_cols, n_del, ins_rows, ins_cols, ins_w, n_ins, out, ws, s, key,
-                            store);
   const bool weighted = old.w.p != nullptr;
   // the batch as two small CSRs over the same rows
   Csr D, I;

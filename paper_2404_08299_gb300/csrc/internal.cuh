@@ -74,7 +74,16 @@ int build_csr_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* c
 // when key[r] == c.
 int update_csr(int32_t n, const Csr& old, const int32_t* del_rows, const int32_t* del_cols, int64_t n_del,
                const int32_t* ins_rows, const int32_t* ins_cols, const float* ins_w, int64_t n_ins, Csr& out,
-               Workspace& ws, cudaStream_t s, const int32_t* key = nullptr, const int32_t* store = nullptr);
+               Workspace& ws, cudaStream_t s, const int32_t* key, const int32_t* store);
+// The same for the CSRs of G and G' (old[k] with the lists b[k]) together.
+struct BatchLists {
+  const int32_t *del_rows, *del_cols;
+  int64_t n_del;
+  const int32_t *ins_rows, *ins_cols;
+  int64_t n_ins;
+};
+int update_csr_pair(int32_t n, const Csr* old, const BatchLists* b, const float* ins_w, Csr* out, Workspace& ws,
+                    cudaStream_t s, const int32_t* key = nullptr, const int32_t* store = nullptr);
 
 // The graph renumbered so that each in-degree class is a contiguous id range
 // (new id i = vertex perm[i], perm being the in-degree partition).
