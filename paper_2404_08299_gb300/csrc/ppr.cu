@@ -190,17 +190,28 @@ __device__ __forceinline__ void gather(const Ctx<T>& c, int K, int32_t u, bool o
   ld_row<VEC>(c.R + (int64_t)u * K, on && c.colok, c.left, r);
 }
 
+// The teleport and the previous R of the 4 columns of a vertex.
+template <class T>
+struct Own {
+  Vec4<T> s, old;
+};
+template <class T, bool VEC>
+__device__ __forceinline__ void load_own(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, Own<T>& w) {
+  const bool on = c.colok;
+  // right-hand side row: dense, or (srow) the compact row of v, none when v has no teleport mass
+  const int64_t sr = !on ? -1 : a.srow ? (int64_t)__ldg(a.srow + v) : (int64_t)v;
+  ld_row<VEC>(c.R + (int64_t)v * a.K, on, c.left, w.old);
+  ld_row<VEC>(a.S + (sr >= 0 ? sr : 0) * a.K + c.col, sr >= 0, c.left, w.s);
+}
+
 // New values of the 4 columns of vertex v from their sums: Eq. 1 with the
 // teleport S, the change against the previous R, and (FP64) the residual.
 template <class T, bool VEC>
-__device__ __forceinline__ void finish_row(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, const T* sum, Peak& pk) {
+__device__ __forceinline__ void finish_row(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, const T* sum,
+                                           const Own<T>& w, Peak& pk) {
   if (!c.colok) return;
   const int64_t o = (int64_t)v * a.K + c.col;
-  // right-hand side row: dense, or (srow) the compact row of v, none when v has no teleport mass
-  const int64_t sr = a.srow ? (int64_t)__ldg(a.srow + v) : (int64_t)v;
-  Vec4<T> s, old;
-  ld_row<VEC>(a.S + (sr >= 0 ? sr : 0) * a.K + c.col, sr >= 0, c.left, s);
-  ld_row<VEC>(c.R + (int64_t)v * a.K, true, c.left, old);
+  const Vec4<T>&s = w.s, &old = w.old;
   T t[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -330,7 +341,9 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
         T t[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) t[q] = acc[q].sum(folded).value();
-        finish_row<T, VEC>(a, c, vdone, t, pk);
+        Own<T> own;
+        load_own<T, VEC>(a, c, vdone, own);
+        finish_row<T, VEC>(a, c, vdone, t, own, pk);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[q] = typename Traits<T>::Col();
@@ -488,7 +501,9 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
       T sum[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) sum[q] = t[q].value();
-      finish_row<T, VEC>(a, c, v, sum, pk);
+      Own<T> own;
+      load_own<T, VEC>(a, c, v, own);
+      finish_row<T, VEC>(a, c, v, sum, own, pk);
     }
     ++s;
   }

@@ -111,7 +111,13 @@ __global__ void __launch_bounds__(kRT) k_radix_hist(const KeySrc src, int64_t M,
   const int nv = M <= i0 ? 0 : (M - i0 >= 32 * kRK ? kRK : (int)((M - i0 + 31) / 32));
   uint32_t d[kRK];
 #pragma unroll
-  for (int r = 0; r < kRK; ++r) d[r] = r < nv ? (uint32_t)(load_key<FIRST>(src, i0 + r * 32) >> shift) & 0xFFu : 0u;
+  for (int r = 0; r < kRK; ++r) {
+    const int64_t i = i0 + r * 32;
+    if (FIRST && src.B >= 8)  // the first digit is in the column alone
+      d[r] = r >= nv ? 0u : (i < src.m0 ? (uint32_t)__ldcs(src.cols + i) : (uint32_t)(i - src.m0)) & 0xFFu;
+    else
+      d[r] = r < nv ? (uint32_t)(load_key<FIRST>(src, i) >> shift) & 0xFFu : 0u;
+  }
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < kRK; ++r)

@@ -402,6 +402,43 @@ __device__ __forceinline__ void sum_rows(const SweepArgs<typename P::Real>& a, c
   }
 }
 
+// The other way to sum a batch: a row per lane, eight entries a step in two
+// 16-byte loads from the boundary below the row's first entry, the next step's
+// entries loading while this one's are gathered. No lanes idle past a group's
+// row and nothing to meet by shuffles, but the index loads touch a line per
+// lane.
+template <class P>
+__device__ __forceinline__ void sum_lane_rows(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t b,
+                                              int len, int32_t v, typename P::Acc& acc, bool& hit) {
+  using Bits = typename P::Bits;
+  const int lo = (int)(b & 3), hi = len > 0 ? lo + len : 0;
+  const int32_t* base = a.adj + (b & ~(int64_t)3);
+  auto load = [&](int j) { return j < hi ? ld_stream_i32x4(base + j, c.pf) : make_int4(-1, -1, -1, -1); };
+  int4 q0 = load(0), q1 = load(4);
+  for (int j = 0; __any_sync(kFull, j < hi); j += 8) {
+    int32_t u[8];
+    {
+      int32_t t[4];
+      mask4(q0, j, lo, hi, t);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) u[k] = t[k];
+      mask4(q1, j + 4, lo, hi, t);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) u[4 + k] = t[k];
+    }
+    Bits xv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
+    q0 = load(j + 8);
+    q1 = load(j + 12);
+    if (!a.self_loops) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) hit = hit || u[k] == v;
+    }
+    add_terms<P>(acc, u, xv);
+  }
+}
+
 // A unit: the rows at positions [kb, ke) of a class, G lanes per row, in
 // batches of up to 32. The offsets of the next batch and the row ids of the
 // one after it load before the batch.
@@ -445,7 +482,15 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
     vn = load_v(k0 + 64);
     typename P::Acc saved;
     bool hit = false;
-    sum_rows<P, G>(a, c, steps(k0), cur.b, cur.len, cur.v, saved, hit);
+    // rows of 5 to 32 entries: a row per lane when the batch fills most lanes
+    // (static solves, a row per lane against a group per row: 2^24 R-MAT 58.6 ->
+    // 57.6 ms, 4096^2 grid 21.8 -> 14.1 ms, mixed 2^22 13.5 -> 13.0 ms; rows of 33
+    // to 128 lose, 58.8 ms, their index loads then cost as much as the gathers);
+    // small batches of a small graph keep the groups (2^16: 1.07 against 1.25 ms)
+    if (G <= 8 && nact - k0 >= 24)
+      sum_lane_rows<P>(a, c, cur.b, cur.len, cur.v, saved, hit);
+    else
+      sum_rows<P, G>(a, c, steps(k0), cur.b, cur.len, cur.v, saved, hit);
     const bool have = in_batch(k0);
     // graphs without self-loops on every vertex: x[v] counts only when the row
     // holds v (rows of a warp or more always took x[v])
@@ -561,7 +606,7 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
   };
   auto load_idx = [&](const Row& r, int32_t (&u)[U]) {
 #pragma unroll
-    for (int k = 0; k < U; ++k) u[k] = k < r.len ? ld_stream_i32(a.adj + r.b + k, c.pf) : -1;
+    for (int k = 0; k < U; ++k) u[k] = k < r.len ? __ldg(a.adj + r.b + k) : -1;
   };
   // row ids three batches ahead, offsets two, indices one
   const int32_t v0 = load_v(0), v1 = load_v(32);
@@ -643,7 +688,7 @@ struct Plan {
 };
 
 // Cuts the classes (Static: whole, DF / DF-P: their affected rows) into units
-// of about an eighth of a warp's share of the sweep, at least two short steps
+// of about a quarter of a warp's share of the sweep, at least two short steps
 // and at most a few thousand edges (so that a unit's start-up latency is paid
 // for, and the last units of a sweep are short). Lane k of the block's first
 // warp takes class k.
@@ -658,7 +703,7 @@ __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSl
     float cost = (float)cnt * per;
     if (k == 31) cost = (float)nchunk * (float)a.chunk_size;
     const float all = warp_sum_f32(cost);
-    float target = all / (8.f * (float)(gridDim.x * kWarps));
+    float target = all / (4.f * (float)(gridDim.x * kWarps));
     target = fminf(fmaxf(target, 96.f), 4096.f);
     int rows = in ? a.cls[k].least : 1;
     while (rows < kMaxRows && 2.f * rows * per <= target) rows *= 2;
