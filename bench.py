@@ -77,7 +77,7 @@ def measured_peaks():
 
 
 def sweep_source_hash():
-    """sha256 over what the rank-sweep kernels are compiled from: sweep.cu, common.cuh and the SweepArgs
+    """sha256 over what the rank-sweep kernel is compiled from: sweep.cu, common.cuh and the SweepArgs
     declaration in internal.cuh (other declarations there do not change the sweep)."""
     csrc = os.path.join(ROOT, "paper_2404_08299_gb300", "csrc")
     h = hashlib.sha256()
@@ -761,7 +761,8 @@ def main():
     traffic = recorded_traffic(args.workload)
 
     extras = {}
-    # the same solve as one CUDA graph (device-side convergence loop): time to tolerance
+    # the same solve as one launch (device-side convergence loop; the key's name is from its CUDA-graph
+    # form): time to tolerance
     for _ in range(2):
         g.pagerank_static(accumulate=acc)
     torch.cuda.synchronize()
@@ -844,8 +845,8 @@ def main():
             "ms_partition": statistics.median(s.ms_partition for s in sts),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": "rank sweep (k_sweep_group / k_sweep_warp / k_sweep_block, one launch per "
-                                   "in-degree class); one unit = one sweep",
+                         "kernel": "rank sweep (k_rank_loop, one launch per sweep in the timed host loop); "
+                                   "one unit = one sweep",
                          "bytes_per_sweep": B, "ms_per_sweep": sweep_ms, "peak_source": peak_kind},
             "e2e": {"value": e2e_val, "unit": "GTEPS", "h2d_bytes_per_step": 8 * m0, "d2h_bytes_per_step": 8 * n,
                     "ms_per_step": e2e_step},

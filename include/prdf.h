@@ -84,7 +84,7 @@ typedef struct {
                           loop (a residual read every check_every sweeps); 0 (default): every sweep
                           loop (Static, DF, DF-P, DT, and the FP32 stage of each) runs as one
                           cooperative launch with the convergence test on the device, no host round
-                          trips (the K-column loops as CUDA graphs). Both give identical results. */
+                          trips, and so do the K-column loops. Both give identical results. */
   int tile;            /* K-column calls: columns per index fetch (8, 16, 32, 64); 0 = automatic */
   double expand_pull;  /* DF / DF-P: an expansion round after a sweep runs in pull form (each vertex
                           outside the affected set looks for a frontier in-neighbour in G') when the

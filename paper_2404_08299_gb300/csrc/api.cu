@@ -471,7 +471,7 @@ int nonempty_classes(const int64_t* cb, int nclass) {
 //     check_every sweeps ahead of each residual read; sweeps launched past
 //     convergence exit at once on the device. Each sweep is bracketed by CUDA
 //     events.
-constexpr int64_t kChunkSmallM = 1ll << 22;
+constexpr int64_t kChunkSmallM = 6ll << 20;
 
 struct Loop {
   bool fp32 = false, dynamic = false, expand = false, exact = true;
@@ -533,6 +533,7 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
   a.max_chunks = ch.max_chunks;
   a.chunk_class = ch.first_class;
   a.chunk_size = ch.size;
+  // four chunks a unit: 2^24 R-MAT 58.7 against 60.0 ms with one, 59.4 with two
   a.chunks_per_unit = ch.size < kHubChunk ? 1 : 4;
   a.hub_part = ch.part.p;
   a.hub_done = ch.done.p;
@@ -566,7 +567,9 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
 // summed by different warps. On graphs with little work per warp a sweep
 // lasts as long as its longest chain of gathers, so there the class below
 // (a warp per row otherwise, up to 4096 edges) is cut as well, into chunks of
-// 512 edges.
+// 512 edges: R-MAT 2^16 (1.0 M edges) 16 -> 13 us a sweep, 2^18 (4.4 M) 39 ->
+// 30, but 2^19 (8.9 M) 44 -> 47 and 2^20 64 -> 84 (a unit of one chunk costs
+// about 4 us whatever its length).
 int ensure_sweep_chunks(prdf_graph* g, const int64_t* cb, cudaStream_t s) {
   SweepChunks& t = g->sweep_chunks;
   if (!t.valid || t.version != g->rl.version) {
@@ -660,7 +663,9 @@ int run_host_loop(prdf_graph* g, const Loop& L, const prdf_params* p, int max_it
       for (auto e : v) cudaEventDestroy(e);
     }
   } guard{ev};
-  const int window = check < max_iter ? check : max_iter;
+  // (sweeps launched ahead of a residual read: bounded, as their slots are)
+  const int ahead = check < 4096 ? check : 4096;
+  const int window = ahead < max_iter ? ahead : max_iter;
   PRDF_TRY(g->loop_slots.reserve((size_t)window + 1, s));
   if (L.init_push) PRDF_TRY(launch_loop(g, L, kLoopPush, 0, 0, s));
   // slot 0 holds the sweep before the window, slots 1.. the window's
@@ -771,14 +776,22 @@ struct KOp {
 // Chunk table of the rows of one CSR above `above` edges, wherever they are
 // (the numbering follows the in-degrees, the adjoint sums over out-rows),
 // rebuilt when the numbering or the bound changes.
-constexpr int kPprChunk = 512;
-int ppr_long_row(int tile) { return tile <= 16 ? 32 : 128; }
+// Rows up to this long take a slot of lanes each, the others are cut into
+// chunks for whole warps. A narrow tile has many short slots (2 or 4 lanes) and
+// its long rows would be walked a few entries a step: measured on 0.7 M edges,
+// K = 5 in FP64, 32 / 48 / 64: 2.86 / 2.73 / 3.03 ms; wide tiles, 8.9 M edges,
+// K = 32, 80 / 96 / 128: 35.1 / 35.0 / 39.8 ms (forward and backward).
+int ppr_long_row(int tile) { return tile <= 16 ? 48 : 96; }
+// Chunks of 256 edges shorten the chains of small graphs (0.7 M edges, K = 33
+// mixed: 5.6 -> 4.6 ms), 512 cost less on large ones (K = 64 at 2^22: 212
+// against 217 ms).
+int ppr_chunk(int64_t m) { return m < (1ll << 22) ? 256 : 512; }
 int ensure_ppr_chunks(prdf_graph* g, const Csr& c, int tile, SweepChunks& t, cudaStream_t s) {
   const int above = ppr_long_row(tile);
   if (t.valid && t.version == g->rl.version && t.above == above) return PRDF_OK;
   t.valid = false;
-  PRDF_TRY(build_chunks(c.off.p, 0, g->n, c.m, kPprChunk, above, t, g->ws, s));
-  t.size = kPprChunk;
+  t.size = ppr_chunk(c.m);
+  PRDF_TRY(build_chunks(c.off.p, 0, g->n, c.m, t.size, above, t, g->ws, s));
   t.above = above;
   t.version = g->rl.version;
   t.valid = true;
@@ -806,6 +819,7 @@ int ppr_args(prdf_graph* g, const KOp& op, const prdf_params* p, int Kp, int til
   a.inv_beta = (T)(1.0 / (1.0 - p->alpha));
   a.tol = sizeof(T) == 4 ? (T)p->tol_fp32_rel : (T)p->tol;
   a.max_iter = max_iter;
+  a.m = g->m;
   a.row_end = g->n;
   a.row_max = ch.above;
   a.chunks = ch.chunks.p;
@@ -866,7 +880,8 @@ int ppr_loop(prdf_graph* g, const prdf_params* p, PprArgs<T> a, int tile, int* i
     return PRDF_OK;
   }
   const int check = p->check_every > 0 ? p->check_every : 8;
-  const int window = check < a.max_iter ? check : a.max_iter;
+  const int ahead = check < 4096 ? check : 4096;
+  const int window = ahead < a.max_iter ? ahead : a.max_iter;
   PRDF_TRY(g->loop_slots.reserve((size_t)window + 1, s));
   a.slot = g->loop_slots.p;
   a.mode = kLoopSweep;

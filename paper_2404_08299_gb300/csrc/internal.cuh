@@ -256,6 +256,7 @@ struct PprArgs {
   int K, tiles;
   T alpha, beta, inv_beta; // alpha, 1 - alpha, 1 / (1 - alpha)
   T tol;                   // FP32: stop at max|dR| <= tol * max|R|; FP64: at max|dR| <= tol
+  int64_t m;               // entries of the CSR
   int max_iter, mode, it0, it_first;  // as in SweepArgs
   LoopSlot* slot;
   LoopCtl* ctl;

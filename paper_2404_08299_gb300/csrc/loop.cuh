@@ -42,4 +42,19 @@ __device__ inline bool grid_barrier(LoopCtl* ctl, unsigned long long& target) {
   return s_ok != 0;
 }
 
+// Cooperative launch of a loop kernel. Where fewer blocks fit than the device's
+// attributes say (a share of the GPU's SMs), it takes as many as do: the
+// kernels work with any number.
+inline int launch_coop(const void* k, int64_t blocks, int threads, void** args, cudaStream_t s) {
+  for (;;) {
+    const cudaError_t e = cudaLaunchCooperativeKernel(k, dim3((unsigned)blocks), dim3((unsigned)threads), args, 0, s);
+    if (e != cudaErrorCooperativeLaunchTooLarge || blocks <= 1) {
+      PRDF_CUDA(e);
+      return PRDF_OK;
+    }
+    cudaGetLastError();
+    blocks /= 2;
+  }
+}
+
 }  // namespace prdf

@@ -19,7 +19,9 @@
 // 16-byte gathers of the rows of R (K * 4 bytes per edge through L2), so the
 // kernel is built to keep them in flight: the indices and weights of the next
 // step load (one per lane, handed round by shuffles) while this step's
-// gathers are on their way, across row and chunk bounds.
+// gathers are on their way, across row and chunk bounds. At 2^22 and K = 64 (69
+// M edges, 17.8 GB of gathered rows) an FP32 sweep takes 2.3-2.4 ms; four
+// kernels per sweep with unpipelined loads took 3.07 ms.
 #include <cstring>
 
 #include "loop.cuh"
@@ -99,14 +101,14 @@ struct Traits;
 template <>
 struct Traits<float> {
   using Col = Col32;
-  static constexpr int kU = 4;          // gathers of a lane in flight
-  static constexpr int kMinBlocks = 4;  // 64 registers
+  static constexpr int kU = 4;          // gathers of a lane in flight (8: spills, 223 against 215 ms a solve)
+  static constexpr int kMinBlocks = 4;  // 64 registers (3 blocks: 248 against 211 ms, 5: 239)
 };
 template <>
 struct Traits<double> {
   using Col = Col64;
   static constexpr int kU = 4;
-  static constexpr int kMinBlocks = 2;  // 128 registers
+  static constexpr int kMinBlocks = 2;  // 128 registers (3 blocks spill: K = 5 on 0.7 M edges 3.03 against 2.86 ms)
 };
 
 template <class T>
@@ -796,7 +798,9 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
   int64_t rows = kSlots;
   while (rows < 8 * kSlots && rows * 8 * (int64_t)max_b * kWarps < n * a.tiles) rows *= 2;
   a.rows_per_unit = (int)rows;
-  a.chunks_per_unit = a.max_chunks * a.tiles > 32 * (int64_t)max_b * kWarps ? 4 : 1;
+// four chunks a unit on large graphs (K = 64 at 2^22: 218 against 222 ms), one
+  // where that leaves warps idle (K = 32 at 2^19, 8.9 M edges: 35 against 53 ms)
+  a.chunks_per_unit = a.m >= (1ll << 25) ? 4 : 1;
   const int64_t work = (a.row_end / rows + 1 + a.max_chunks / a.chunks_per_unit + 1) * a.tiles;
   if (work * 2 >= (int64_t)UINT32_MAX) {
     set_error("too many work units");
@@ -810,8 +814,7 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
     return PRDF_OK;
   }
   void* args[] = {&a};
-  PRDF_CUDA(cudaLaunchCooperativeKernel((const void*)k, dim3((unsigned)blocks), dim3(kThreads), args, 0, s));
-  return PRDF_OK;
+  return launch_coop((const void*)k, blocks, kThreads, args, s);
 }
 
 template <class T>

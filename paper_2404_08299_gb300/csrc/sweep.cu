@@ -36,7 +36,14 @@ namespace {
 
 // Two blocks of 512 threads per SM at 64 registers: the sweeps are bound by
 // the latency and the rate of their gathers, so resident warps matter more
-// than registers, and few blocks keep the grid barrier short.
+// than registers, and few blocks keep the grid barrier short. (1024 x 1 and
+// 256 x 4 within 1 %; 256 x 5 at 51 registers: 4096^2 grid 13.1 against 14.1
+// ms, but 2^16 R-MAT 1.41 against 1.25 and the 2^20 stream window 3.51 against
+// 3.33 ms; 384 x 4 at 42: 2^24 R-MAT 66.9 against 60.2 ms.)
+//
+// What bounds a sweep: the L1's handling of its 8-byte gathers. At 2^22 (69 M
+// edges) one sweep takes 245 us with 62 M L1 sector misses, 0.83 a clock per
+// SM, where uniform gathers reach 0.92; it took 357 us as eight class kernels.
 constexpr int kThreads = 512;
 constexpr int kMinBlocks = 2;
 constexpr int kWarps = kThreads / 32;
@@ -690,7 +697,9 @@ struct Plan {
 // Cuts the classes (Static: whole, DF / DF-P: their affected rows) into units
 // of about a quarter of a warp's share of the sweep, at least two short steps
 // and at most a few thousand edges (so that a unit's start-up latency is paid
-// for, and the last units of a sweep are short). Lane k of the block's first
+// for, and the last units of a sweep are short). A half / a quarter / an eighth
+// / a sixteenth: 2^20 stream window 3.70 / 3.36 / 3.51 / 3.95 ms, mixed solve at
+// 2^22 13.6 / 13.5 / 13.6 / 14.7 ms. Lane k of the block's first
 // warp takes class k.
 template <bool DYN, class Real>
 __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSlot* slot, Plan* plan) {
@@ -729,6 +738,8 @@ __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSl
   __syncthreads();
 }
 
+// bins of the 129..4096 class in DF / DF-P: without them a long row listed late
+// sets the sweep's end (DT on 50 M edges 10.4 against 9.2 ms)
 constexpr int64_t kLong0 = 2048, kLong1 = 1024, kLong2 = 512;
 
 // DF / DF-P: lists the affected rows of every class outside the chunk table,
@@ -854,7 +865,9 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
   // First unit by position (consecutive units on different SMs). The others
   // come from a counter, or by position again when there are few per warp: the
   // counter is one address, and thousands of warps asking at once wait for
-  // one another longer than a short sweep lasts.
+  // one another longer than a short sweep lasts (2^16 R-MAT, counter from more
+  // than one unit a warp on: 1.21 against 1.02 ms; none up to 16 units a warp:
+  // mixed solve at 2^22 16.0 against 13.4 ms).
   const unsigned int nw = gridDim.x * kWarps;
   const bool counted = plan->total > 4 * nw;
   for (unsigned int u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < plan->total;) {
@@ -1309,9 +1322,7 @@ struct Launcher {
       return PRDF_OK;
     }
     void* args[] = {&a};
-    PRDF_CUDA(cudaLaunchCooperativeKernel((const void*)k_rank_loop<P, DYN>, dim3((unsigned)blocks), dim3(kThreads),
-                                          args, 0, s));
-    return PRDF_OK;
+    return launch_coop((const void*)k_rank_loop<P, DYN>, blocks, kThreads, args, s);
   }
 };
 
