@@ -202,6 +202,31 @@ __device__ __forceinline__ void append_frontier(bool flag, int32_t v, uint64_t d
   for (unsigned int k = 0; k < c; ++k) list[base + k] = make_int2(v, (int)k);
 }
 
+// What the epilogue of a vertex reads besides its sum: out-degree and its
+// inverse, (DF-P) the Eq. 2 factor, (DF / DF-P) the deltaN flag.
+template <class Real>
+struct Own {
+  Real d, iv, kf;
+  uint8_t dn;
+};
+__device__ __forceinline__ double ld_const(const double* p, uint64_t pol) { return ld_stream_f64(p, pol); }
+template <class P, bool DYN>
+__device__ __forceinline__ Own<typename P::Real> load_own(const SweepArgs<typename P::Real>& a, const Ctx<P>& c,
+                                                          bool have, int32_t v) {
+  Own<typename P::Real> w;
+  w.d = w.iv = w.kf = 0;
+  w.dn = 0;
+  if (have) {
+    w.d = ld_const(a.deg + v, c.pf);
+    w.iv = ld_const(a.inv + v, c.pf);
+    if (DYN) {
+      if (a.prune) w.kf = ld_const(a.kf + v, c.pf);
+      w.dn = a.dN[v];
+    }
+  }
+  return w;
+}
+
 // Vertex epilogue: Eq. 1 (Static, DF) or Eq. 2 (DF-P), prune / expand flags,
 // next x, and this vertex's |r - R[v]| into the tally. GB300's FP64 pipe is
 // narrow, so the FP64 form keeps to what needs FP64 rounding; the maximum and
@@ -211,13 +236,13 @@ __device__ __forceinline__ void append_frontier(bool flag, int32_t v, uint64_t d
 // non-negative value, as in FP64). Returns whether v joins deltaN.
 template <bool DYN>
 __device__ __forceinline__ bool finish(const SweepArgs<double>& a, const Ctx<PExact>& c, int32_t v, double sum,
-                                       double xself, bool dn_old, Tally& t, uint64_t& deg) {
-  const double d = ld_stream_f64(a.deg + v, c.pf);
-  const double iv = ld_stream_f64(a.inv + v, c.pf);
+                                       double xself, const Own<double>& w, Tally& t, uint64_t& deg) {
+  const double d = w.d, iv = w.iv;
+  const bool dn_old = w.dn != 0;
   double r;
   if (DYN && a.prune) {
     // Eq. 2: the self-loop term is solved in closed form (factor precomputed per vertex)
-    r = ld_stream_f64(a.kf + v, c.pf) * (a.c0 + a.alpha * (sum - xself));
+    r = w.kf * (a.c0 + a.alpha * (sum - xself));
   } else {
     r = fma(a.alpha, sum, a.c0);  // Eq. 1
   }
@@ -246,19 +271,19 @@ __device__ __forceinline__ bool finish(const SweepArgs<double>& a, const Ctx<PEx
 }
 template <bool DYN>
 __device__ __forceinline__ bool finish(const SweepArgs<double>& a, const Ctx<PPlain>& c, int32_t v, double sum,
-                                       double xself, bool dn_old, Tally& t, uint64_t& deg) {
+                                       double xself, const Own<double>& w, Tally& t, uint64_t& deg) {
   const Ctx<PExact> e{c.x, c.xn, c.slot, c.pf, c.pl, c.lane};
-  return finish<DYN>(a, e, v, sum, xself, dn_old, t, deg);
+  return finish<DYN>(a, e, v, sum, xself, w, t, deg);
 }
 // the same in FP32, with Alg. update's prune and expand tests evaluated in FP32
 template <bool DYN>
 __device__ __forceinline__ bool finish(const SweepArgs<float>& a, const Ctx<PKahan>& c, int32_t v, float sum,
-                                       float xself, bool dn_old, Tally& t, uint64_t& deg) {
-  const float d = ld_const(a.deg + v, c.pf);
-  const float iv = ld_const(a.inv + v, c.pf);
+                                       float xself, const Own<float>& w, Tally& t, uint64_t& deg) {
+  const float d = w.d, iv = w.iv;
+  const bool dn_old = w.dn != 0;
   const float rold = xself * d;
   float r;
-  if (DYN && a.prune) r = ld_const(a.kf + v, c.pf) * fmaf(a.alpha, sum - xself, a.c0);  // Eq. 2
+  if (DYN && a.prune) r = w.kf * fmaf(a.alpha, sum - xself, a.c0);  // Eq. 2
   else r = fmaf(a.alpha, sum, a.c0);                                                      // Eq. 1
   const float dr = fabsf(r - rold);
   bool front = false;
@@ -307,10 +332,11 @@ __device__ __forceinline__ int32_t row_at(const SweepArgs<typename P::Real>& a, 
 // One row per lane, its offsets known: the epilogue of a batch.
 template <class P, bool DYN>
 __device__ __forceinline__ void finish_batch(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, bool have,
-                                             int32_t v, typename P::Real sum, typename P::Real xself, Tally& t) {
+                                             int32_t v, typename P::Real sum, typename P::Real xself,
+                                             const Own<typename P::Real>& w, Tally& t) {
   bool front = false;
   uint64_t deg = 0;
-  if (have) front = finish<DYN>(a, c, v, sum, xself, DYN && a.dN[v] != 0, t, deg);
+  if (have) front = finish<DYN>(a, c, v, sum, xself, w, t, deg);
   if (DYN && a.expand) append_frontier(front, v, deg, &c.slot->nlist, a.list, c.lane);
 }
 
@@ -487,6 +513,7 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
   for (int k0 = 0; k0 < nact; k0 += 32) {
     const Batch nxt = load_off(vn);
     vn = load_v(k0 + 64);
+    const Own<typename P::Real> own = load_own<P, DYN>(a, c, in_batch(k0), cur.v);
     typename P::Acc saved;
     bool hit = false;
     // rows of 5 to 32 entries: a row per lane when the batch fills most lanes
@@ -502,7 +529,7 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
     // graphs without self-loops on every vertex: x[v] counts only when the row
     // holds v (rows of a warp or more always took x[v])
     const Bits xs = have && (G == 32 || a.self_loops || hit) ? ld_state(c.x + cur.v, c.pl) : Bits(0);
-    finish_batch<P, DYN>(a, c, have, cur.v, saved.value(), as_real(xs), t);
+    finish_batch<P, DYN>(a, c, have, cur.v, saved.value(), as_real(xs), own, t);
     cur = nxt;
   }
 }
@@ -562,6 +589,7 @@ __device__ __forceinline__ void unit_chunks(const SweepArgs<typename P::Real>& a
     ch = cb + src;
     have = lane < nact;
   }
+  const Own<typename P::Real> own = load_own<P, DYN>(a, c, have, k.v);
   typename P::Acc saved;
   bool hit = false;
   sum_rows<P, 32>(a, c, nact, k.j0, k.len, 0, saved, hit);
@@ -585,7 +613,7 @@ __device__ __forceinline__ void unit_chunks(const SweepArgs<typename P::Real>& a
     if (lane == l) saved = acc;
   }
   const Bits xs = fin ? ld_state(c.x + k.v, c.pl) : Bits(0);
-  finish_batch<P, DYN>(a, c, fin, k.v, saved.value(), as_real(xs), t);
+  finish_batch<P, DYN>(a, c, fin, k.v, saved.value(), as_real(xs), own, t);
 }
 
 // One row per lane, U indices in flight (short rows).
@@ -627,6 +655,7 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
 #pragma unroll
     for (int k = 0; k < U; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
     const Bits xs = have ? ld_state(c.x + cur.v, c.pl) : Bits(0);
+    const Own<typename P::Real> own = load_own<P, DYN>(a, c, have, cur.v);
     int32_t un[U];
     load_idx(nxt, un);
     const Row far = load_off(vf);
@@ -643,7 +672,7 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
       hit = hit || w == cur.v;
     }
     const Bits xself = (a.self_loops || hit) ? xs : Bits(0);
-    finish_batch<P, DYN>(a, c, have, cur.v, acc.value(), as_real(xself), t);
+    finish_batch<P, DYN>(a, c, have, cur.v, acc.value(), as_real(xself), own, t);
     cur = nxt;
     nxt = far;
 #pragma unroll
@@ -665,6 +694,7 @@ __device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, 
     const int32_t v = vn;
     vn = k0 + 32 + c.lane < ke ? row_at<P, DYN>(a, k0 + 32 + c.lane) : 0;
     const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
+    const Own<typename P::Real> own = load_own<P, DYN>(a, c, have, v);
     typename P::Real sum = as_real(xs);
     if (a.multi && have && ((a.multi[v >> 5] >> (v & 31)) & 1u)) {
       typename P::Acc acc;
@@ -672,7 +702,7 @@ __device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, 
       for (int64_t j = a.off[v]; j < e; ++j) acc.add(ld_state(c.x + a.adj[j], c.pl));
       sum = acc.value();
     }
-    finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), t);
+    finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), own, t);
   }
 }
 
