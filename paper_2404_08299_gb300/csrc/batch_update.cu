@@ -423,7 +423,6 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_small(const SmallSides S,
   int64_t* cnt = reinterpret_cast<int64_t*>(rk + nd_pow + ni_pow);  // scratch counts (nd_pow + ni_pow)
   int32_t* ip = reinterpret_cast<int32_t*>(cnt + nd_pow + ni_pow);  // I payload (ni_pow)
   __shared__ int64_t tmp[kPrepThreads / 32 + 1];
-  __shared__ int s_nd, s_ni, s_kc;
   for (int i = threadIdx.x; i < nd_pow; i += blockDim.x) {
     uint64_t kk = kNoKey;
     if (i < n_del) {
