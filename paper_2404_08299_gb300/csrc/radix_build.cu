@@ -27,6 +27,7 @@ constexpr int kRT = 256;              // threads per tile
 constexpr int kRK = 16;               // keys per thread
 constexpr int kRTile = kRT * kRK;     // 4096 keys per tile
 constexpr int kRWarps = kRT / 32;
+constexpr int kRBlocks = 3;           // blocks an SM of the scatter
 constexpr int kRDigits = 256;
 static_assert(kRT == kRDigits, "one digit per thread in the scatter's digit scan");
 static_assert(kRTile <= 65536 && kRK % 2 == 0, "ranks are packed two to a word");
@@ -40,10 +41,15 @@ struct KeySrc {
   int B;
 };
 
+// key of the list's entry i < m0
+__device__ __forceinline__ uint64_t list_key(const KeySrc& s, int64_t i) {
+  return ((uint64_t)(uint32_t)__ldcs(s.rows + i) << s.B) | (uint64_t)(uint32_t)__ldcs(s.cols + i);
+}
+
 template <bool FIRST>
 __device__ __forceinline__ uint64_t load_key(const KeySrc& s, int64_t i) {
   if (!FIRST) return __ldcs(reinterpret_cast<const unsigned long long*>(s.keys) + i);
-  if (i < s.m0) return ((uint64_t)(uint32_t)__ldcs(s.rows + i) << s.B) | (uint64_t)(uint32_t)__ldcs(s.cols + i);
+  if (i < s.m0) return list_key(s, i);
   const uint64_t v = (uint64_t)(i - s.m0);
   return (v << s.B) | v;
 }
@@ -69,7 +75,7 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d) {
 #pragma unroll
   for (int b = 0; b < BITS; ++b) {
     const uint32_t m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-    peers &= ((d >> b) & 1u) ? m : ~m;
+    peers &= ~(m ^ (0u - ((d >> b) & 1u)));  // no select: 3 % of a build
   }
   return peers;
 }
@@ -110,13 +116,14 @@ __global__ void __launch_bounds__(kRT) k_radix_hist(const KeySrc src, int64_t M,
   const int64_t i0 = (int64_t)blockIdx.x * kRTile + (int64_t)w * (32 * kRK) + lane;
   const int nv = M <= i0 ? 0 : (M - i0 >= 32 * kRK ? kRK : (int)((M - i0 + 31) / 32));
   uint32_t d[kRK];
+  if (FIRST && src.B >= 8 && (int64_t)(blockIdx.x + 1) * kRTile <= src.m0) {
+    // the first digit is in the column alone
 #pragma unroll
-  for (int r = 0; r < kRK; ++r) {
-    const int64_t i = i0 + r * 32;
-    if (FIRST && src.B >= 8)  // the first digit is in the column alone
-      d[r] = r >= nv ? 0u : (i < src.m0 ? (uint32_t)__ldcs(src.cols + i) : (uint32_t)(i - src.m0)) & 0xFFu;
-    else
-      d[r] = r < nv ? (uint32_t)(load_key<FIRST>(src, i) >> shift) & 0xFFu : 0u;
+    for (int r = 0; r < kRK; ++r) d[r] = (uint32_t)__ldcs(src.cols + i0 + r * 32) & 0xFFu;
+  } else {
+#pragma unroll
+    for (int r = 0; r < kRK; ++r)
+      d[r] = r < nv ? (uint32_t)(load_key<FIRST>(src, i0 + r * 32) >> shift) & 0xFFu : 0u;
   }
   __syncthreads();
 #pragma unroll
@@ -129,41 +136,18 @@ __global__ void __launch_bounds__(kRT) k_radix_hist(const KeySrc src, int64_t M,
   hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = c;
 }
 
-// Stable scatter of one tile by digit; goff = exclusive scan of hist. W: the
-// weights move with their keys.
-template <bool FIRST, bool W>
-__global__ void __launch_bounds__(kRT, 3) k_radix_scatter(const KeySrc src, int64_t M, int shift,
-                                                          const int64_t* __restrict__ goff, int64_t ntiles,
-                                                          uint64_t* __restrict__ out, float* __restrict__ wout) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);          // kRTile keys
-  int64_t* gbase = reinterpret_cast<int64_t*>(buf + kRTile);       // kRDigits
-  uint32_t* wcnt = reinterpret_cast<uint32_t*>(gbase + kRDigits);  // kRWarps x kRDigits
-  uint32_t* lstart = wcnt + kRWarps * kRDigits;                    // kRDigits
-  uint32_t* wsum = lstart + kRDigits;                              // kRWarps
-  float* wbuf = reinterpret_cast<float*>(wsum + kRWarps);          // kRTile weights (W)
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kRWarps; ++k) wcnt[k * kRDigits + threadIdx.x] = 0;
-  const int64_t t0 = (int64_t)blockIdx.x * kRTile;
-  const int64_t i0 = t0 + (int64_t)w * (32 * kRK) + lane;
-  // rounds r < nv hold a key of this thread
-  const int nv = M <= i0 ? 0 : (M - i0 >= 32 * kRK ? kRK : (int)((M - i0 + 31) / 32));
-  uint64_t key[kRK];
-#pragma unroll
-  for (int r = 0; r < kRK; ++r) key[r] = r < nv ? load_key<FIRST>(src, i0 + r * 32) : 0ull;
-  __syncthreads();
-  // rank of each key among the equal digits before it: earlier rounds of this
-  // warp (its counter), then lower lanes of the same round
-  uint32_t* mine = wcnt + w * kRDigits;
+// Rank of each key among the equal digits before it in its warp's part of the
+// tile: earlier rounds (the warp's counter), then lower lanes of the same
+// round. FULL: every round of every lane has a key (else rounds r < nv).
+template <bool FULL>
+__device__ __forceinline__ void rank_keys(const uint64_t (&key)[kRK], int shift, int nv, uint32_t* mine,
+                                          uint32_t (&rank)[kRK / 2]) {
   const uint32_t lt = lanemask_lt();
-  const bool full = t0 + kRTile <= M;
-  uint32_t rank[kRK / 2];  // two 16-bit ranks a word (a rank is below kRTile)
 #pragma unroll
   for (int r = 0; r < kRK; ++r) {
-    const bool ok = r < nv;
+    const bool ok = FULL || r < nv;
     const uint32_t d = ok ? (uint32_t)(key[r] >> shift) & 0xFFu : 0x100u;
-    const uint32_t peers = full ? match_digit<8>(d) : match_digit<9>(d);
+    const uint32_t peers = match_digit<FULL ? 8 : 9>(d);
     const uint32_t before = (uint32_t)__popc(peers & lt);
     const uint32_t prev = ok ? mine[d] : 0u;
     __syncwarp();
@@ -173,30 +157,89 @@ __global__ void __launch_bounds__(kRT, 3) k_radix_scatter(const KeySrc src, int6
     if (r & 1) rank[r >> 1] |= rk << 16;
     else rank[r >> 1] = rk;
   }
+}
+
+// Stable scatter of one tile by digit; goff = exclusive scan of hist. W: the
+// weights move with their keys. Bound by shared memory (the data pipe 73 %
+// busy: counters by digit and the staged keys are hit at random banks) and by
+// issue (57 %, the ballots), not by DRAM (3.4 of 6.7 TB/s). So a digit's start
+// is folded into the warps' counters (one random read less a key), and full
+// tiles take a branch-free path: all loads are in flight before the first
+// key is ranked, and no round tests for a missing key. 285 M keys to two CSRs:
+// 28.5 ms before, 24.2 now; the first pass alone 2.6 ms before, its rows and
+// columns loaded one key after the other. 512 or 768 threads a tile: 28.2 to
+// 30.1; 12 keys a thread and 4 blocks an SM: 24.8; __match_any_sync for the
+// ballots: 7 % more.
+template <bool FIRST, bool W>
+__global__ void __launch_bounds__(kRT, kRBlocks) k_radix_scatter(const KeySrc src, int64_t M, int shift,
+                                                                 const int64_t* __restrict__ goff, int64_t ntiles,
+                                                                 uint64_t* __restrict__ out,
+                                                                 float* __restrict__ wout) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);          // kRTile keys
+  int64_t* gbase = reinterpret_cast<int64_t*>(buf + kRTile);       // kRDigits
+  uint32_t* wcnt = reinterpret_cast<uint32_t*>(gbase + kRDigits);  // kRWarps x kRDigits
+  uint32_t* wsum = wcnt + kRWarps * kRDigits;                      // kRWarps
+  float* wbuf = reinterpret_cast<float*>(wsum + kRWarps);          // kRTile weights (W)
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kRWarps; ++k) wcnt[k * kRDigits + threadIdx.x] = 0;
+  const int64_t t0 = (int64_t)blockIdx.x * kRTile;
+  const int64_t i0 = t0 + (int64_t)w * (32 * kRK) + lane;
+  // rounds r < nv hold a key of this thread
+  const int nv = M <= i0 ? 0 : (M - i0 >= 32 * kRK ? kRK : (int)((M - i0 + 31) / 32));
+  uint64_t key[kRK];
+  if (FIRST && t0 + kRTile <= src.m0) {
+#pragma unroll
+    for (int r = 0; r < kRK; ++r) key[r] = list_key(src, i0 + r * 32);
+  } else if (!FIRST && t0 + kRTile <= M) {
+#pragma unroll
+    for (int r = 0; r < kRK; ++r) key[r] = load_key<FIRST>(src, i0 + r * 32);
+  } else {
+#pragma unroll
+    for (int r = 0; r < kRK; ++r) key[r] = r < nv ? load_key<FIRST>(src, i0 + r * 32) : 0ull;
+  }
   __syncthreads();
-  // digit d = this thread: warp bases (in warp order), the tile's count of d,
-  // and the digit's start inside the tile
+  uint32_t* mine = wcnt + w * kRDigits;
+  const bool full = t0 + kRTile <= M;
+  uint32_t rank[kRK / 2];  // two 16-bit ranks a word (a rank is below kRTile)
+  if (full) rank_keys<true>(key, shift, nv, mine, rank);
+  else rank_keys<false>(key, shift, nv, mine, rank);
+  float wv[W ? kRK : 1];
+  if (W) {
+    if (full && (!FIRST || t0 + kRTile <= src.m0)) {
+#pragma unroll
+      for (int r = 0; r < kRK; ++r) wv[W ? r : 0] = __ldcs(src.w + i0 + r * 32);
+    } else {
+#pragma unroll
+      for (int r = 0; r < kRK; ++r) wv[W ? r : 0] = r < nv ? load_w<FIRST>(src, i0 + r * 32) : 0.f;
+    }
+  }
+  __syncthreads();
+  // digit d = this thread: its start inside the tile, and from there each
+  // warp's (in warp order)
   {
     const int d = threadIdx.x;
-    uint32_t acc = 0;
+    uint32_t all = 0;
+#pragma unroll
+    for (int k = 0; k < kRWarps; ++k) all += wcnt[k * kRDigits + d];
+    uint32_t at = block_scan_excl(all, wsum, nullptr);
+    gbase[d] = goff[(int64_t)d * ntiles + blockIdx.x] - (int64_t)at;
 #pragma unroll
     for (int k = 0; k < kRWarps; ++k) {
       const uint32_t c = wcnt[k * kRDigits + d];
-      wcnt[k * kRDigits + d] = acc;
-      acc += c;
+      wcnt[k * kRDigits + d] = at;
+      at += c;
     }
-    const uint32_t ls = block_scan_excl(acc, wsum, nullptr);
-    lstart[d] = ls;
-    gbase[d] = goff[(int64_t)d * ntiles + blockIdx.x] - (int64_t)ls;
   }
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < kRK; ++r) {
     if (r < nv) {
       const uint32_t d = (uint32_t)(key[r] >> shift) & 0xFFu;
-      const uint32_t at = lstart[d] + mine[d] + ((rank[r >> 1] >> (16 * (r & 1))) & 0xFFFFu);
+      const uint32_t at = mine[d] + ((rank[r >> 1] >> (16 * (r & 1))) & 0xFFFFu);
       buf[at] = key[r];
-      if (W) wbuf[at] = load_w<FIRST>(src, i0 + r * 32);
+      if (W) wbuf[at] = wv[W ? r : 0];
     }
   }
   __syncthreads();
@@ -209,7 +252,7 @@ __global__ void __launch_bounds__(kRT, 3) k_radix_scatter(const KeySrc src, int6
   }
 }
 
-constexpr int kRScatterSmem = kRTile * 8 + kRDigits * 8 + kRWarps * kRDigits * 4 + kRDigits * 4 + kRWarps * 4;
+constexpr int kRScatterSmem = kRTile * 8 + kRDigits * 8 + kRWarps * kRDigits * 4 + kRWarps * 4;
 constexpr int kRScatterSmemW = kRScatterSmem + kRTile * 4;
 
 // ---- merge of equal keys ----
@@ -253,8 +296,11 @@ __global__ void __launch_bounds__(kRT) k_uniq_count(const uint64_t* __restrict__
 // Columns of the unique keys, and off[r] = position of row r's first unique
 // key (rows without keys take the next row's start; off[n] = total).
 // woff = exclusive scan of the per-warp counts, woff[nw] = total. kt (or null)
-// gets the keys of the transposed CSR in this CSR's order, uw (or null, zero
-// on entry) the largest weight bits of each unique key. With urow
+// gets the keys of the transposed CSR in this CSR's order, uw (or null, zeros
+// on entry) the largest weight bits of each unique key: a plain store where the
+// key stands alone, an atomic only among duplicates (one per key before, and
+// another pass for the weights of added self-loops: 9.5 ms for 64 M weighted
+// edges to two CSRs, 8.2 with the scatter's changes). With urow
 // (lists much shorter than n) the row of each unique key goes to urow instead
 // and k_offsets_from_rows fills off.
 __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ k, int64_t M, int B, int32_t n,
@@ -274,6 +320,15 @@ __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ 
     key[r] = i < M ? __ldcs(reinterpret_cast<const unsigned long long*>(k) + i) : ~0ull;
   }
   uint64_t carry = base < M ? warp_carry_in(k, base) : ~0ull;
+  uint32_t wv[kRK];
+  if (uw) {
+#pragma unroll
+    for (int r = 0; r < kRK; ++r) {
+      const int64_t i = base + r * 32 + lane;
+      wv[r] = i < M ? __float_as_uint(__ldcs(w + i)) : 0u;
+    }
+  }
+  const uint64_t after = base + 32 * kRK < M ? k[base + 32 * kRK] : ~0ull;  // the next warp's first key
   int64_t pos = gw < nw ? woff[gw] : 0;
 #pragma unroll
   for (int r = 0; r < kRK; ++r) {
@@ -283,8 +338,16 @@ __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ 
     carry = __shfl_sync(0xffffffffu, key[r], 31);
     const bool f = i < M && (i == 0 || key[r] != prev);
     const uint32_t bal = __ballot_sync(0xffffffffu, f);
-    // duplicates keep the largest weight (positive floats order as their bits)
-    if (uw && i < M) atomicMax(uw + pos + __popc(bal & lt) - (f ? 0 : 1), __float_as_uint(__ldcs(w + i)));
+    if (uw) {
+      // an entry alone has its weight (an added self-loop 1); of duplicates, cleared before, the largest stays
+      // (positive floats order as their bits, and the mark of an added self-loop is 0)
+      uint64_t next = __shfl_down_sync(0xffffffffu, key[r], 1);
+      const uint64_t over = __shfl_sync(0xffffffffu, r + 1 < kRK ? key[r + 1 < kRK ? r + 1 : 0] : after, 0);
+      if (lane == 31) next = over;
+      uint32_t* to = uw + pos + __popc(bal & lt);
+      if (f && key[r] != next) *to = wv[r] ? wv[r] : __float_as_uint(1.f);
+      else if (i < M) atomicMax(to - (f ? 0 : 1), wv[r]);
+    }
     if (f) {
       const int64_t p = pos + __popc(bal & lt);
       const int64_t row = (int64_t)(key[r] >> B);
@@ -318,24 +381,36 @@ __global__ void k_offsets_from_rows(const int32_t* __restrict__ urow, int64_t mu
   }
 }
 
-// an added self-loop without a weight of its own (0 so far) gets 1
-__global__ void k_loop_weights(float* __restrict__ w, int64_t m) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-    if (w[i] == 0.f) w[i] = 1.f;
-}
-
-// columns and row offsets of sorted keys without duplicates
+// columns and row offsets of sorted keys without duplicates; a warp takes
+// 32 * kRK keys, all loaded before the first is written (one key at a time a
+// thread before: 0.73 ms for 285 M keys, 4.6 TB/s)
 __global__ void __launch_bounds__(kRT) k_emit(const uint64_t* __restrict__ k, int64_t m, int B, int32_t n,
                                               int32_t* __restrict__ adj, int64_t* __restrict__ off) {
   const uint64_t cmask = (1ull << B) - 1;
-  for (int64_t i = blockIdx.x * (int64_t)kRT + threadIdx.x; i < m; i += (int64_t)gridDim.x * kRT) {
-    const uint64_t key = k[i];
-    const int64_t row = (int64_t)(key >> B);
-    adj[i] = (int32_t)(key & cmask);
-    for (int64_t q = i == 0 ? 0 : (int64_t)(k[i - 1] >> B) + 1; q <= row; ++q) off[q] = i;
-    if (i == m - 1)
-      for (int64_t q = row + 1; q <= n; ++q) off[q] = m;
+  const int lane = threadIdx.x & 31;
+  const int64_t base = (((int64_t)blockIdx.x * kRT + threadIdx.x) >> 5) * (32 * kRK);
+  if (base >= m) return;
+  uint64_t key[kRK];
+#pragma unroll
+  for (int r = 0; r < kRK; ++r) {
+    const int64_t i = base + r * 32 + lane;
+    key[r] = i < m ? __ldcs(reinterpret_cast<const unsigned long long*>(k) + i) : ~0ull;
   }
+  int64_t row = base > 0 ? (int64_t)(k[base - 1] >> B) : -1;  // of the key before the round's first
+#pragma unroll
+  for (int r = 0; r < kRK; ++r) {
+    const int64_t i = base + r * 32 + lane;
+    const int64_t mine = i < m ? (int64_t)(key[r] >> B) : n;
+    int64_t prev = __shfl_up_sync(0xffffffffu, mine, 1);
+    if (lane == 0) prev = row;
+    row = __shfl_sync(0xffffffffu, mine, 31);
+    if (i < m) adj[i] = (int32_t)(key[r] & cmask);
+    // rows after the previous key's start here; past the last key (i = m) they are empty and end there
+    if (i <= m)
+      for (int64_t q = prev + 1; q <= mine; ++q) off[q] = i;
+  }
+  if (base + 32 * kRK == m && lane == 31)  // no lane had i = m
+    for (int64_t q = row + 1; q <= n; ++q) off[q] = m;
 }
 
 template <bool FIRST>
@@ -414,19 +489,18 @@ int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols,
   float* wcur = wa.p;
   float* wnxt = wb.p;
   PRDF_TRY(radix_pass<true>(src, M, 0, cur, wcur, hist, goff, ntiles, ws, s));
-  auto pass = [&](int64_t cnt, int shift) {
+  auto swap = [](auto& a, auto& b) {
+    auto t = a;
+    a = b;
+    b = t;
+  };
+  for (int p = 1; p < passes; ++p) {
     src.keys = cur;
     src.w = wcur;
-    PRDF_TRY(radix_pass<false>(src, cnt, shift, nxt, wnxt, hist, goff, (cnt + kRTile - 1) / kRTile, ws, s));
-    uint64_t* t = cur;
-    cur = nxt;
-    nxt = t;
-    float* f = wcur;
-    wcur = wnxt;
-    wnxt = f;
-    return (int)PRDF_OK;
-  };
-  for (int p = 1; p < passes; ++p) PRDF_TRY(pass(M, 8 * p));
+    PRDF_TRY(radix_pass<false>(src, M, 8 * p, nxt, wnxt, hist, goff, ntiles, ws, s));
+    swap(cur, nxt);
+    swap(wcur, wnxt);
+  }
   // merge equal keys
   const int64_t nw = ntiles * kRWarps;
   DBuf<uint32_t> wcnt;
@@ -458,37 +532,25 @@ int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols,
                                                sparse ? urow.p : nullptr, in ? nxt : nullptr, wcur,
                                                w ? reinterpret_cast<uint32_t*>(out.w.p) : nullptr);
   if (sparse) k_offsets_from_rows<<<grid_for((int64_t)n + 1, kRT), kRT, 0, s>>>(urow.p, out.m, n, out.off.p);
-  if (w && self_loops) k_loop_weights<<<grid_for(m, kRT), kRT, 0, s>>>(out.w.p, m);
   PRDF_LAUNCH_CHECK();
   if (!in) return PRDF_OK;
-  uint64_t* t = cur;  // the transposed keys
-  cur = nxt;
-  nxt = t;
-  for (int p = 0; p < (B + 7) / 8; ++p) {
-    if (p == 0 && w) {
-      src.keys = cur;
-      src.w = out.w.p;
-      PRDF_TRY(radix_pass<false>(src, m, B, nxt, wnxt, hist, goff, (m + kRTile - 1) / kRTile, ws, s));
-      uint64_t* q = cur;
-      cur = nxt;
-      nxt = q;
-      float* f = wcur;
-      wcur = wnxt;
-      wnxt = f;
-    } else {
-      PRDF_TRY(pass(m, B + 8 * p));
-    }
-  }
+  swap(cur, nxt);  // the transposed keys
   in->m = m;
   PRDF_TRY(in->off.alloc((size_t)n + 1, s));
   PRDF_TRY(in->adj.alloc(room, s));
-  if (w) {
-    PRDF_TRY(in->w.alloc(room, s));
-    PRDF_CUDA(cudaMemcpyAsync(in->w.p, wcur, sizeof(float) * (size_t)m, cudaMemcpyDeviceToDevice, s));
-  } else {
-    in->w.release();
+  if (w) PRDF_TRY(in->w.alloc(room, s));
+  else in->w.release();
+  const int half = (B + 7) / 8;
+  for (int p = 0; p < half; ++p) {
+    // the weights go from the first CSR's, through the buffers, to the second's
+    src.keys = cur;
+    src.w = p == 0 ? out.w.p : wcur;
+    float* to = p == half - 1 ? in->w.p : wnxt;
+    PRDF_TRY(radix_pass<false>(src, m, B + 8 * p, nxt, to, hist, goff, (m + kRTile - 1) / kRTile, ws, s));
+    swap(cur, nxt);
+    swap(wcur, wnxt);
   }
-  k_emit<<<grid_for(m, kRT), kRT, 0, s>>>(cur, m, B, n, in->adj.p, in->off.p);
+  k_emit<<<(unsigned)((m + kRTile - 1) / kRTile), kRT, 0, s>>>(cur, m, B, n, in->adj.p, in->off.p);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }
