@@ -33,6 +33,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int64_t kShortMean = 4;  // K of 1 or 2: 2 lanes a row in units of at most this mean length, else 8
 
 // Compensated FP32 sum (s + e): TwoSum folds each term's rounding error into e.
 struct Dot2 {
@@ -111,49 +112,52 @@ struct Traits<double> {
   static constexpr int kMinBlocks = 2;  // 128 registers (3 blocks spill: K = 5 on 0.7 M edges 3.03 against 2.86 ms)
 };
 
-template <class T>
-struct Vec4 {
-  T v[4];
+template <class T, int Q>
+struct Vec {
+  T v[Q];
 };
 
-// Four columns of a row: coherent loads (R is written in the same kernel, a
-// grid barrier earlier). VEC (a row stride that is a multiple of four, every K
-// above 2): 16-byte loads, and the columns past K are the row's zero padding;
-// else `left` columns one by one. Nothing is read and zeros are returned when
-// `on` is false.
-template <bool VEC>
-__device__ __forceinline__ void ld_row(const float* src, bool on, int left, Vec4<float>& r) {
-  if (VEC) {
+// Q columns of a row, one load (two for four doubles): coherent, as R is
+// written in the same kernel, a grid barrier earlier. Q is 4 (a row stride that
+// is a multiple of four: every K above 2, the columns past K are the row's zero
+// padding), or the whole row of K = 1 or 2. Nothing is read and zeros are
+// returned when `on` is false.
+template <int Q>
+__device__ __forceinline__ void ld_row(const float* src, bool on, Vec<float, Q>& r) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) r.v[q] = 0.f;
-    if (on)
-      asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
-                   : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
-                   : "l"(src));
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      r.v[q] = 0.f;
-      if (on && q < left) asm volatile("ld.global.f32 %0, [%1];" : "=f"(r.v[q]) : "l"(src + q));
-    }
-  }
+  for (int q = 0; q < Q; ++q) r.v[q] = 0.f;
+  if (!on) return;
+  if constexpr (Q == 4)
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
+                 : "l"(src));
+  else if constexpr (Q == 2)
+    asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(r.v[0]), "=f"(r.v[1]) : "l"(src));
+  else
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(r.v[0]) : "l"(src));
 }
-template <bool VEC>
-__device__ __forceinline__ void ld_row(const double* src, bool on, int left, Vec4<double>& r) {
-  if (VEC) {
+template <int Q>
+__device__ __forceinline__ void ld_row(const double* src, bool on, Vec<double, Q>& r) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) r.v[q] = 0.0;
-    if (on) {
-      asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(src));
-      asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[2]), "=d"(r.v[3]) : "l"(src + 2));
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      r.v[q] = 0.0;
-      if (on && q < left) asm volatile("ld.global.f64 %0, [%1];" : "=d"(r.v[q]) : "l"(src + q));
-    }
-  }
+  for (int q = 0; q < Q; ++q) r.v[q] = 0.0;
+  if (!on) return;
+  if constexpr (Q == 1)
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(r.v[0]) : "l"(src));
+  else
+    asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(src));
+  if constexpr (Q == 4) asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(r.v[2]), "=d"(r.v[3]) : "l"(src + 2));
+}
+template <int Q>
+__device__ __forceinline__ void st_row(float* dst, const float* v) {
+  if constexpr (Q == 4) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  else if constexpr (Q == 2) *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
+  else *dst = v[0];
+}
+template <int Q>
+__device__ __forceinline__ void st_row(double* dst, const double* v) {
+  if constexpr (Q == 1) *dst = v[0];
+  else *reinterpret_cast<double2*>(dst) = make_double2(v[0], v[1]);
+  if constexpr (Q == 4) reinterpret_cast<double2*>(dst)[1] = make_double2(v[2], v[3]);
 }
 __device__ __forceinline__ float ld_weight(const float* p, uint64_t pol) {
   float v;
@@ -184,65 +188,46 @@ struct Ctx {
   uint64_t pf;
   int lane, col;
   bool colok;     // the lane has columns
-  int left;       // columns of the matrix from col on
 };
 
-template <bool VEC, class T>
-__device__ __forceinline__ void gather(const Ctx<T>& c, int K, int32_t u, bool on, Vec4<T>& r) {
-  ld_row<VEC>(c.R + (int64_t)u * K, on && c.colok, c.left, r);
+template <int Q, class T>
+__device__ __forceinline__ void gather(const Ctx<T>& c, int K, int32_t u, bool on, Vec<T, Q>& r) {
+  ld_row<Q>(c.R + (int64_t)u * K, on && c.colok, r);
 }
 
-// The teleport and the previous R of the 4 columns of a vertex.
-template <class T>
+// The teleport and the previous R of a lane's columns of a vertex.
+template <class T, int Q>
 struct Own {
-  Vec4<T> s, old;
+  Vec<T, Q> s, old;
 };
-template <class T, bool VEC>
-__device__ __forceinline__ void load_own(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, Own<T>& w) {
+template <class T, int Q>
+__device__ __forceinline__ void load_own(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, Own<T, Q>& w) {
   const bool on = c.colok;
   // right-hand side row: dense, or (srow) the compact row of v, none when v has no teleport mass
   const int64_t sr = !on ? -1 : a.srow ? (int64_t)__ldg(a.srow + v) : (int64_t)v;
-  ld_row<VEC>(c.R + (int64_t)v * a.K, on, c.left, w.old);
-  ld_row<VEC>(a.S + (sr >= 0 ? sr : 0) * a.K + c.col, sr >= 0, c.left, w.s);
+  ld_row<Q>(c.R + (int64_t)v * a.K, on, w.old);
+  ld_row<Q>(a.S + (sr >= 0 ? sr : 0) * a.K + c.col, sr >= 0, w.s);
 }
 
-// New values of the 4 columns of vertex v from their sums: Eq. 1 with the
+// New values of a lane's columns of vertex v from their sums: Eq. 1 with the
 // teleport S, the change against the previous R, and (FP64) the residual.
-template <class T, bool VEC>
+template <class T, int Q>
 __device__ __forceinline__ void finish_row(const PprArgs<T>& a, const Ctx<T>& c, int32_t v, const T* sum,
-                                           const Own<T>& w, Peak& pk) {
+                                           const Own<T, Q>& w, Peak& pk) {
   if (!c.colok) return;
   const int64_t o = (int64_t)v * a.K + c.col;
-  const Vec4<T>&s = w.s, &old = w.old;
-  T t[4];
+  T t[Q];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    t[q] = fma(a.alpha, sum[q], a.beta * s.v[q]);
-    if (VEC || q < c.left) pk.see(t[q] - old.v[q], t[q]);
+  for (int q = 0; q < Q; ++q) {
+    t[q] = fma(a.alpha, sum[q], a.beta * w.s.v[q]);
+    pk.see(t[q] - w.old.v[q], t[q]);
   }
-  if (VEC) {
-    if (sizeof(T) == 4) {
-      *reinterpret_cast<float4*>(c.Rn + o) = make_float4((float)t[0], (float)t[1], (float)t[2], (float)t[3]);
-    } else {
-      reinterpret_cast<double2*>(c.Rn + o)[0] = make_double2((double)t[0], (double)t[1]);
-      reinterpret_cast<double2*>(c.Rn + o)[1] = make_double2((double)t[2], (double)t[3]);
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (q < c.left) c.Rn[o + q] = t[q];
-  }
+  st_row<Q>(c.Rn + o, t);
   if (sizeof(T) == 8 && a.res32) {
-    float d[4];
+    float d[Q];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d[q] = (float)((t[q] - old.v[q]) * a.inv_beta);
-    if (VEC) {
-      *reinterpret_cast<float4*>(a.res32 + o) = make_float4(d[0], d[1], d[2], d[3]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < c.left) a.res32[o + q] = d[q];
-    }
+    for (int q = 0; q < Q; ++q) d[q] = (float)((t[q] - w.old.v[q]) * a.inv_beta);
+    st_row<Q>(a.res32 + o, d);
   }
 }
 
@@ -251,7 +236,7 @@ __device__ __forceinline__ void finish_row(const PprArgs<T>& a, const Ctx<T>& c,
 // the row's indices and weights (kE edges) and hand them round by shuffles.
 // The next window (of the same rows, or of the slots' next rows, whose offsets
 // are known a step ahead) loads while this one's rows are gathered.
-template <class T, int LPE, bool VEC>
+template <class T, int LPE>
 __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, int32_t vb, int32_t ve, Peak& pk) {
   constexpr int kSlots = 32 / LPE;
   constexpr int kEpl = LPE >= 16 ? 1 : LPE >= 8 ? 2 : 4;  // window edges per lane
@@ -297,10 +282,10 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
       cu[i] = u[i];
       cp[i] = p[i];
     }
-    Vec4<T> r[U];
+    Vec<T, 4> r[U];
 #pragma unroll
     for (int k = 0; k < U; ++k)
-      gather<VEC>(c, a.K, __shfl_sync(kFull, cu[k / LPE], slot0 + k % LPE), k < here, r[k]);
+      gather<4>(c, a.K, __shfl_sync(kFull, cu[k / LPE], slot0 + k % LPE), k < here, r[k]);
     // the next window
     const int32_t vdone = v;
     const bool done = todo;
@@ -321,6 +306,9 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
       if (e0 >= most) break;
 #pragma unroll
       for (int k = 0; k < U; ++k) {
+        // FP64 products are what a step is short of, and an instruction costs its 32 lanes whatever they hold:
+        // those past the longest row are left out (K = 8 on 17 M edges: 37.3 -> 34.2 ms)
+        if (sizeof(T) == 8 && k > 0 && e0 + k >= most) break;
         const T w = __shfl_sync(kFull, cp[(e0 + k) / LPE], slot0 + (e0 + k) % LPE);
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q].prod(w, r[k].v[q]);
@@ -334,7 +322,7 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
 #pragma unroll
         for (int k = 0; k < U; ++k) {
           const int e = e0 + U + k;
-          gather<VEC>(c, a.K, __shfl_sync(kFull, cu[e / LPE], slot0 + e % LPE), e < here, r[k]);
+          gather<4>(c, a.K, __shfl_sync(kFull, cu[e / LPE], slot0 + e % LPE), e < here, r[k]);
         }
       }
     }
@@ -343,9 +331,9 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
         T t[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) t[q] = acc[q].sum(folded).value();
-        Own<T> own;
-        load_own<T, VEC>(a, c, vdone, own);
-        finish_row<T, VEC>(a, c, vdone, t, own, pk);
+        Own<T, 4> own;
+        load_own<T, 4>(a, c, vdone, own);
+        finish_row<T, 4>(a, c, vdone, t, own, pk);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[q] = typename Traits<T>::Col();
@@ -355,13 +343,103 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
   }
 }
 
+// The same rows where a lane holds whole rows of R (K of 1 or 2): G lanes per
+// row, each with its own edges, so no index or weight is handed round, and the
+// lanes' sums meet at the row's end. With a lane per four columns half of the
+// lanes and three of four products were idle: K = 1 on 69 M edges, mixed 51.3
+// ms a solve before, 28.9 now; FP64 101.5 (four kernels a sweep) and 44.0. At
+// K = 4 the form above is the faster one (FP64 on 8.7 M edges 16.6 against 19.0
+// ms).
+template <class T, int Q, int G>
+__device__ __forceinline__ void unit_rows_narrow(const PprArgs<T>& a, const Ctx<T>& c, int32_t vb, int32_t ve,
+                                                 Peak& pk) {
+  constexpr int kSlots = 32 / G;
+  constexpr int U = 4;       // edges of a lane a step
+  constexpr int kE = U * G;
+  const int sub = c.lane & (G - 1), slot = c.lane / G;
+  auto load_off = [&](int32_t v, int64_t& b, int& len) {
+    b = 0;
+    len = -1;
+    if (v < ve && v >= 0) {
+      b = ld_stream_i64(a.off + v, c.pf);
+      const int64_t d = ld_stream_i64(a.off + v + 1, c.pf) - b;
+      len = d <= a.row_max ? (int)d : -1;
+    }
+  };
+  int32_t u[U];
+  T p[U];
+  auto load_win = [&](int64_t b, int rem) {
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int e = sub + G * i;
+      u[i] = e < rem ? ld_stream_i32(a.adj + b + e, c.pf) : 0;
+      p[i] = e < rem ? ld_weight(a.P + b + e, c.pf) : T(0);
+    }
+  };
+  int64_t b, bn;
+  int32_t v = vb + slot;
+  int rem, ln;
+  load_off(v, b, rem);
+  load_win(b, rem);
+  load_off(v + kSlots, bn, ln);
+  typename Traits<T>::Col acc[Q];
+  bool folded = false;
+  for (int32_t v0 = vb; v0 < ve;) {
+    const bool more = __any_sync(kFull, rem > kE);
+    Vec<T, Q> r[U];
+    T cp[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      gather<Q>(c, a.K, u[i], sub + G * i < rem, r[i]);
+      cp[i] = p[i];
+    }
+    const int32_t vdone = v;
+    const bool fin = !more && rem >= 0 && sub == 0;
+    Own<T, Q> own;
+    if (fin) load_own<T, Q>(a, c, vdone, own);
+    if (more) {
+      b += kE;
+      rem = rem > kE ? rem - kE : (rem >= 0 ? 0 : -1);
+      load_win(b, rem);
+    } else {
+      v += kSlots;
+      b = bn;
+      rem = ln;
+      load_win(b, rem);
+      load_off(v + kSlots, bn, ln);
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) acc[q].prod(cp[i], r[i].v[q]);
+    if (more) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) acc[q].fold();
+      folded = true;
+      continue;
+    }
+    T t[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      typename Traits<T>::Col::Sum x = acc[q].sum(folded);
+#pragma unroll
+      for (int o = 1; o < G; o <<= 1) x.merge(x.shfl_xor(o));
+      t[q] = x.value();
+      acc[q] = typename Traits<T>::Col();
+    }
+    if (fin) finish_row<T, Q>(a, c, vdone, t, own, pk);
+    folded = false;
+    v0 += kSlots;
+  }
+}
+
 // sums of the slots of a warp meet in every slot (a fixed tree)
-template <class Sum, int LPE>
+template <class Sum, int LPE, int Q>
 __device__ __forceinline__ void merge_slots(Sum* t) {
 #pragma unroll
   for (int o = LPE; o < 32; o <<= 1)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) t[q].merge(t[q].shfl_xor(o));
+    for (int q = 0; q < Q; ++q) t[q].merge(t[q].shfl_xor(o));
 }
 
 __device__ __forceinline__ void ld_part(const Dot2* p, Dot2& x) {
@@ -376,7 +454,7 @@ __device__ __forceinline__ void ld_part(const Sum64* p, Sum64& x) { x.s = __ldcg
 // finished at once; of a longer row the warp that sums the last chunk (an
 // arrival counter per row and tile) adds the row's partial sums in chunk order
 // and finishes it.
-template <class T, int LPE, bool VEC>
+template <class T, int LPE, int Q>
 __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c, int64_t cb, int cnt, int tile_no,
                                             Peak& pk) {
   using Sum = typename Traits<T>::Col::Sum;
@@ -409,7 +487,7 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
   int64_t b = __shfl_sync(kFull, j0, 0);
   int rem = __shfl_sync(kFull, len, 0);
   load_win(b, rem);
-  typename Traits<T>::Col acc[4];
+  typename Traits<T>::Col acc[Q];
   for (int s = 0; s < cnt;) {
     int32_t cu[W];
     T cp[W];
@@ -420,12 +498,12 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
     }
     const int here = rem < kE ? rem : kE;
     const bool more = rem > kE;  // the same on every lane
-    Vec4<T> r[U];
+    Vec<T, Q> r[U];
     // slot's i-th edge of the step is edge i * kSlots + slot
 #pragma unroll
     for (int i = 0; i < U; ++i) {
       const int e = i * kSlots + slot;
-      gather<VEC>(c, a.K, __shfl_sync(kFull, cu[(i * kSlots) / 32], e & 31), e < here, r[i]);
+      gather<Q>(c, a.K, __shfl_sync(kFull, cu[(i * kSlots) / 32], e & 31), e < here, r[i]);
     }
     if (more) {
       b += kE;
@@ -442,40 +520,41 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
       if (i0 * kSlots >= here && i0 > 0) break;
 #pragma unroll
       for (int i = 0; i < U; ++i) {
+        if (sizeof(T) == 8 && i > 0 && (i0 + i) * kSlots >= here) break;
         const T w = __shfl_sync(kFull, cp[((i0 + i) * kSlots) / 32], ((i0 + i) * kSlots + slot) & 31);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].prod(w, r[i].v[q]);
+        for (int q = 0; q < Q; ++q) acc[q].prod(w, r[i].v[q]);
       }
       if ((i0 / U) % 2 == 1 || kPer == U) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].fold();
+        for (int q = 0; q < Q; ++q) acc[q].fold();
       }
       if (i0 + U < kPer && (i0 + U) * kSlots < here) {
 #pragma unroll
         for (int i = 0; i < U; ++i) {
           const int e = (i0 + U + i) * kSlots + slot;
-          gather<VEC>(c, a.K, __shfl_sync(kFull, cu[((i0 + U + i) * kSlots) / 32], e & 31), e < here, r[i]);
+          gather<Q>(c, a.K, __shfl_sync(kFull, cu[((i0 + U + i) * kSlots) / 32], e & 31), e < here, r[i]);
         }
       }
     }
     if (more) continue;
-    Sum t[4];
+    Sum t[Q];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < Q; ++q) {
       t[q] = acc[q].sum(true);
       acc[q] = typename Traits<T>::Col();
     }
-    merge_slots<Sum, LPE>(t);
+    merge_slots<Sum, LPE, Q>(t);
     const int4 rec = __ldg(reinterpret_cast<const int4*>(a.chunks + cb + s) + 1);  // first, parts, row
     const int parts = rec.y;
     const int32_t v = __shfl_sync(kFull, kv, s);
     bool fin = true;
     if (parts > 1) {
-      Sum* part = reinterpret_cast<Sum*>(a.part) + (int64_t)tile_no * a.max_chunks * (4 * LPE);
+      Sum* part = reinterpret_cast<Sum*>(a.part) + (int64_t)tile_no * a.max_chunks * (Q * LPE);
       const int first = rec.x, row = rec.z;
       if (slot == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) part[(cb + s) * (4 * LPE) + 4 * sub + q] = t[q];
+        for (int q = 0; q < Q; ++q) part[(cb + s) * (Q * LPE) + Q * sub + q] = t[q];
       }
       __threadfence();
       __syncwarp();
@@ -487,25 +566,25 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
         if (lane == 0) a.done[(int64_t)tile_no * a.chunk_rows + row] = 0;
         __threadfence();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = Sum();
+        for (int q = 0; q < Q; ++q) t[q] = Sum();
         for (int i = slot; i < parts; i += kSlots) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < Q; ++q) {
             Sum x;
-            ld_part(part + (int64_t)(first + i) * (4 * LPE) + 4 * sub + q, x);
+            ld_part(part + (int64_t)(first + i) * (Q * LPE) + Q * sub + q, x);
             t[q].merge(x);
           }
         }
-        merge_slots<Sum, LPE>(t);
+        merge_slots<Sum, LPE, Q>(t);
       }
     }
     if (fin && slot == 0) {
-      T sum[4];
+      T sum[Q];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) sum[q] = t[q].value();
-      Own<T> own;
-      load_own<T, VEC>(a, c, v, own);
-      finish_row<T, VEC>(a, c, v, sum, own, pk);
+      for (int q = 0; q < Q; ++q) sum[q] = t[q].value();
+      Own<T, Q> own;
+      load_own<T, Q>(a, c, v, own);
+      finish_row<T, Q>(a, c, v, sum, own, pk);
     }
     ++s;
   }
@@ -521,7 +600,9 @@ __device__ __forceinline__ bool stopped(unsigned long long resid, float tol) {
   return __uint_as_float((uint32_t)resid) <= tol * __uint_as_float((uint32_t)(resid >> 32));
 }
 
-template <class T, int LPE, bool VEC>
+// LPE lanes of four columns each side by side (Q = 4); LPE = 1: a lane has the
+// whole row, Q columns.
+template <class T, int LPE, int Q>
 __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
   Ctx<T> c;
   const T* R = (it & 1) ? a.Rb : a.Ra;
@@ -546,19 +627,24 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
     const unsigned int per = chunk ? cu : ru;
     const int tile_no = (int)(y / per);
     const unsigned int un = y - (unsigned int)tile_no * per;
-    c.col = tile_no * (4 * LPE) + 4 * (c.lane & (LPE - 1));
+    c.col = tile_no * (Q * LPE) + Q * (c.lane & (LPE - 1));
     c.colok = c.col < a.K;
-    c.left = a.K - c.col;
     c.R = R + c.col;
     if (chunk) {
       const unsigned int cb = un * a.chunks_per_unit;
       const unsigned int cnt = nchunk - cb < a.chunks_per_unit ? nchunk - cb : a.chunks_per_unit;
-      unit_chunks<T, LPE, VEC>(a, c, cb, (int)cnt, tile_no, pk);
+      unit_chunks<T, LPE, Q>(a, c, cb, (int)cnt, tile_no, pk);
     } else {
       // from the highest class down: long rows first
       const int64_t ve = a.row_end - (int64_t)un * a.rows_per_unit;
       const int64_t vb = ve > a.rows_per_unit ? ve - a.rows_per_unit : 0;
-      unit_rows<T, LPE, VEC>(a, c, (int32_t)vb, (int32_t)ve, pk);
+      if constexpr (LPE > 1) {
+        unit_rows<T, LPE>(a, c, (int32_t)vb, (int32_t)ve, pk);
+      } else {
+        const int64_t len = __ldg(a.off + ve) - __ldg(a.off + vb);
+        if (len <= kShortMean * (ve - vb)) unit_rows_narrow<T, Q, 2>(a, c, (int32_t)vb, (int32_t)ve, pk);
+        else unit_rows_narrow<T, Q, 8>(a, c, (int32_t)vb, (int32_t)ve, pk);
+      }
     }
     x = nw + __shfl_sync(kFull, nx, 0);
   }
@@ -589,16 +675,16 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
 
 // The whole solve (kLoopAll, cooperative launch) or one sweep of the
 // host-driven loop.
-template <class T, int LPE, bool VEC>
+template <class T, int LPE, int Q>
 __global__ void __launch_bounds__(kThreads, Traits<T>::kMinBlocks) k_ppr_loop(const __grid_constant__ PprArgs<T> a) {
   if (a.mode == kLoopSweep) {
     if (a.it0 > 0 && stopped(__ldcg(&slot_of(a, a.it0 - 1)->resid), a.tol)) return;
-    ppr_sweep<T, LPE, VEC>(a, a.it0);
+    ppr_sweep<T, LPE, Q>(a, a.it0);
     return;
   }
   unsigned long long target = 0;
   for (int it = 0;; ++it) {
-    ppr_sweep<T, LPE, VEC>(a, it);
+    ppr_sweep<T, LPE, Q>(a, it);
     if (!grid_barrier(a.ctl, target)) return;
     const unsigned long long resid = __ldcg(&slot_of(a, it)->resid);
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
@@ -780,9 +866,9 @@ __global__ void k_widen_n(const float* __restrict__ y, int64_t cnt, double* __re
     x[i] = (double)y[i];
 }
 
-template <class T, int LPE, bool VEC>
+template <class T, int LPE, int Q>
 int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
-  auto k = k_ppr_loop<T, LPE, VEC>;
+  auto k = k_ppr_loop<T, LPE, Q>;
   int dev = 0, sms = 0, per = 0;
   PRDF_CUDA(cudaGetDevice(&dev));
   PRDF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -792,13 +878,13 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
     return PRDF_ECUDA;
   }
   const int max_b = per * sms;
-  constexpr int kSlots = 32 / LPE;
-  a.tiles = (a.K + 4 * LPE - 1) / (4 * LPE);
+  constexpr int kSlots = LPE > 1 ? 32 / LPE : 16;
+  a.tiles = (a.K + Q * LPE - 1) / (Q * LPE);
   // rows of a unit: about an eighth of a warp's share, a few steps at least
   int64_t rows = kSlots;
   while (rows < 8 * kSlots && rows * 8 * (int64_t)max_b * kWarps < n * a.tiles) rows *= 2;
   a.rows_per_unit = (int)rows;
-// four chunks a unit on large graphs (K = 64 at 2^22: 218 against 222 ms), one
+  // four chunks a unit on large graphs (K = 64 at 2^22: 218 against 222 ms), one
   // where that leaves warps idle (K = 32 at 2^19, 8.9 M edges: 35 against 53 ms)
   a.chunks_per_unit = a.m >= (1ll << 25) ? 4 : 1;
   const int64_t work = (a.row_end / rows + 1 + a.max_chunks / a.chunks_per_unit + 1) * a.tiles;
@@ -819,12 +905,13 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
 
 template <class T>
 int run_ppr(const PprArgs<T>& a, int tile, int64_t n, cudaStream_t s) {
-  if (a.K & 3) return run_tile<T, 2, false>(a, n, s);  // one or two columns (tile 8)
+  if (a.K == 1) return run_tile<T, 1, 1>(a, n, s);
+  if (a.K == 2) return run_tile<T, 1, 2>(a, n, s);
   switch (tile) {
-    case 8: return run_tile<T, 2, true>(a, n, s);
-    case 16: return run_tile<T, 4, true>(a, n, s);
-    case 32: return run_tile<T, 8, true>(a, n, s);
-    default: return run_tile<T, 16, true>(a, n, s);
+    case 8: return run_tile<T, 2, 4>(a, n, s);
+    case 16: return run_tile<T, 4, 4>(a, n, s);
+    case 32: return run_tile<T, 8, 4>(a, n, s);
+    default: return run_tile<T, 16, 4>(a, n, s);
   }
 }
 
