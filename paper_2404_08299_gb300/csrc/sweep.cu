@@ -722,15 +722,18 @@ struct Plan {
   int64_t begin[kMaxCls], end[kMaxCls];
   int rows[kMaxCls];
   uint32_t chunk_units, total;
+  bool counted;
 };
 
 // Cuts the classes (Static: whole, DF / DF-P: their affected rows) into units
-// of about a quarter of a warp's share of the sweep, at least two short steps
-// and at most a few thousand edges (so that a unit's start-up latency is paid
-// for, and the last units of a sweep are short). A half / a quarter / an eighth
-// / a sixteenth: 2^20 stream window 3.70 / 3.36 / 3.51 / 3.95 ms, mixed solve at
-// 2^22 13.6 / 13.5 / 13.6 / 14.7 ms. Lane k of the block's first
-// warp takes class k.
+// of about a quarter of a warp's share of the sweep, at least a full batch of
+// short rows and at most a few thousand edges (so that a unit's start-up
+// latency is paid for, and the last units of a sweep are short). A half / a
+// quarter / an eighth / a sixteenth: 2^20 stream window 3.70 / 3.36 / 3.51 /
+// 3.95 ms, mixed solve at 2^22 13.6 / 13.5 / 13.6 / 14.7 ms. Least cost of 96 /
+// 512 / 768 / 1024: 2^16 R-MAT 1.08 / 0.90 / 0.92 / 0.92 ms, 512^2 grid 1.37 /
+// 1.11 / 0.70 / 0.71, DF-P on a 2^20 R-MAT 3.1 / 3.1 / 3.5 / 3.5.
+// Lane k of the block's first warp takes class k.
 template <bool DYN, class Real>
 __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSlot* slot, Plan* plan) {
   if (threadIdx.x < 32) {
@@ -743,7 +746,9 @@ __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSl
     if (k == 31) cost = (float)nchunk * (float)a.chunk_size;
     const float all = warp_sum_f32(cost);
     float target = all / (4.f * (float)(gridDim.x * kWarps));
-    target = fminf(fmaxf(target, 96.f), 4096.f);
+    // rows of more than 128 edges: units of very different length
+    const bool uneven = nchunk > 0 || __any_sync(kFull, in && cnt > 0 && a.cls[k].kind == kRowWarp);
+    target = fminf(fmaxf(target, uneven ? 512.f : 768.f), 4096.f);
     int rows = in ? a.cls[k].least : 1;
     while (rows < kMaxRows && 2.f * rows * per <= target) rows *= 2;
     const unsigned int units = (unsigned int)((cnt + rows - 1) / rows);
@@ -763,6 +768,8 @@ __device__ __forceinline__ void make_plan(const SweepArgs<Real>& a, const LoopSl
     if (k == 31) {
       plan->chunk_units = cu;
       plan->total = cu + incl;
+      const float warps = (float)(gridDim.x * kWarps);
+      plan->counted = (float)(cu + incl) > 4.f * warps && all > (uneven ? 2048.f : 8192.f) * warps;
     }
   }
   __syncthreads();
@@ -893,13 +900,16 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
   c.lane = threadIdx.x & 31;
   Tally t;
   // First unit by position (consecutive units on different SMs). The others
-  // come from a counter, or by position again when there are few per warp: the
-  // counter is one address, and thousands of warps asking at once wait for
-  // one another longer than a short sweep lasts (2^16 R-MAT, counter from more
-  // than one unit a warp on: 1.21 against 1.02 ms; none up to 16 units a warp:
-  // mixed solve at 2^22 16.0 against 13.4 ms).
+  // come from a counter, or by position again where units are few or the sweep
+  // is short: the counter is one address, and thousands of warps asking at
+  // once wait for one another longer than a short sweep lasts (2^16 R-MAT,
+  // counter from more than one unit a warp on: 1.21 against 1.02 ms; none up to
+  // 16 units a warp: mixed solve at 2^22 16.0 against 13.4 ms). Without long
+  // rows the units are alike and position serves longer sweeps too: FP32
+  // frontier sweeps of a 1024^2 grid 4.1 against 3.5 ms; with them it does not
+  // (2^20 R-MAT, counter from a cost of 2048 / 4096 a warp on: 4.4 / 5.0 ms).
   const unsigned int nw = gridDim.x * kWarps;
-  const bool counted = plan->total > 4 * nw;
+  const bool counted = plan->counted;
   for (unsigned int u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < plan->total;) {
     unsigned int nx = u;
     if (counted && c.lane == 0) nx = atomicAdd(&c.slot->units, 1u);
