@@ -1041,7 +1041,7 @@ int dynamic_fp32_stage(prdf_graph* g, const prdf_params* p, const double* prev_r
   k_widen_keep<<<grid_for(n, kThreads), kThreads, 0, s>>>(it32->final_buf ? g->yb.p : g->ya.p, n, g->xa.p, g->xb.p,
                                                          g->dV.p);
   PRDF_LAUNCH_CHECK();
-  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n, s));
+  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n + 32, s));
   return PRDF_OK;
 }
 
@@ -1049,7 +1049,7 @@ int alloc_solver(prdf_graph* g, bool dynamic, cudaStream_t s) {
   PRDF_TRY(g->xa.reserve(g->n, s));
   PRDF_TRY(g->xb.reserve(g->n, s));
   if (dynamic) {
-    // read and marked by whole words
+    // read and marked by whole words, the padding after the last flag included: it is cleared with the flags
     PRDF_TRY(g->dV.reserve((size_t)g->n + 32, s));
     PRDF_TRY(g->dN.reserve((size_t)g->n + 32, s));
     PRDF_TRY(g->wrote.reserve((size_t)g->n + 32, s));
@@ -1518,9 +1518,9 @@ int prdf_pagerank_dfp(prdf_graph* g, const int32_t* del_src, const int32_t* del_
   k_init_x<<<grid_for(n, kThreads), kThreads, 0, s>>>(prev_ranks, rl.perm.p, n, rl.inv_deg.p, g->xa.p, g->xb.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_CUDA(cudaMemsetAsync(g->dV.p, 0, (size_t)n, s));
-  PRDF_CUDA(cudaMemsetAsync(g->dN.p, 0, (size_t)n, s));
-  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n, s));
+  PRDF_CUDA(cudaMemsetAsync(g->dV.p, 0, (size_t)n + 32, s));
+  PRDF_CUDA(cudaMemsetAsync(g->dN.p, 0, (size_t)n + 32, s));
+  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n + 32, s));
   // the batch's sources go into the first frontier list, which the loop expands before its first sweep
   PRDF_TRY(alloc_loop_ctl(g, s));
   PRDF_TRY(alloc_frontier(g, s));
@@ -1591,9 +1591,9 @@ int prdf_pagerank_dt(prdf_graph* g, const int32_t* del_src, const int32_t* del_d
   k_init_x<<<grid_for(n, kThreads), kThreads, 0, s>>>(prev_ranks, rl.perm.p, n, rl.inv_deg.p, g->xa.p, g->xb.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_CUDA(cudaMemsetAsync(g->dV.p, 0, (size_t)n, s));
-  PRDF_CUDA(cudaMemsetAsync(g->dN.p, 0, (size_t)n, s));
-  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n, s));
+  PRDF_CUDA(cudaMemsetAsync(g->dV.p, 0, (size_t)n + 32, s));
+  PRDF_CUDA(cudaMemsetAsync(g->dN.p, 0, (size_t)n + 32, s));
+  PRDF_CUDA(cudaMemsetAsync(g->wrote.p, 0, (size_t)n + 32, s));
   PRDF_TRY(launch_initial_affected(del_src, del_dst, del_mask, n_del, ins_src, ins_mask, n_ins, rl.inv.p, g->dV.p,
                                    g->dN.p, s));
   const int nco = g->thr[PRDF_OUT].n + 1;
