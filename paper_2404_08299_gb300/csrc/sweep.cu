@@ -953,7 +953,8 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
   if (DYN) {
     const uint64_t f = (uint64_t)warp_sum_i64((int64_t)t.fw);
     if (c.lane == 0 && f) atomicAdd(&s_fw, (unsigned long long)f);
-    if (c.lane == 0 && t.aff) atomicAdd(&s_aff, t.aff);
+    const unsigned int af = __reduce_add_sync(kFull, t.aff);  // (each lane counted the rows of its own chunks)
+    if (c.lane == 0 && af) atomicAdd(&s_aff, af);
   }
   __syncthreads();
   if (threadIdx.x == 0) {

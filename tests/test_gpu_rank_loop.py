@@ -1,0 +1,66 @@
+"""The rank loop on graphs of more than 6.3 M in-edges, where rows of 129 to 4096 entries are a warp each and longer ones
+go by four 1024-edge chunks a unit. Flags, counts and sweep numbers are the oracle's; ranks lie within 1e-12 relative of
+it (the same iteration, rounding-level differences), as in the other parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from helpers import batch_case, dev, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2404_08299_gb300 import build
+    build.build()
+    torch.cuda.init()
+
+
+PLANTED = [129, 130, 255, 257, 511, 512, 513, 514, 1023, 1024, 1025, 1026, 2047, 2048, 2049, 2050, 4095, 4096, 4097,
+           4099, 5000, 5121, 6000, 7169, 9000, 12000, 16385, 20000, 30000, 40000]
+
+
+@pytest.fixture(scope="module")
+def large():
+    """More than 6.3 M in-edges, so rows of 129 to 4096 are a warp each and longer ones go by four 1024-edge chunks a
+    unit; vertex k < len(PLANTED) has about PLANTED[k] in-edges, and a batch adds one to each."""
+    n, s, d = synth.rmat(18, 1 << 23, seed=71)
+    keep = d >= len(PLANTED)
+    s, d = s[keep], d[keep]
+    rng = np.random.default_rng(71)
+    hs = [rng.choice(np.arange(len(PLANTED), n - 100, dtype=np.int32), k, replace=False) for k in PLANTED]
+    hd = [np.full(k, v, np.int32) for v, k in enumerate(PLANTED)]
+    s, d = np.concatenate([s, *hs]).astype(np.int32), np.concatenate([d, *hd]).astype(np.int32)
+    empty = np.zeros(0, np.int32)
+    ins = (np.arange(n - len(PLANTED), n, dtype=np.int32), np.arange(len(PLANTED), dtype=np.int32))
+    case = batch_case(n, s, d, 72, 60, extra=(empty, empty, *ins))
+    assert case[1].m > 6 << 20 and (case[1].indeg > 4096).sum() >= 10
+    return case
+
+
+@pytest.mark.parametrize("kw", [{}, {"prune": 0}, {"expand_pull": 0.0}, {"expand_pull": 2.0}])
+def test_dfp_with_rows_of_several_chunks(large, kw):
+    g, og1, R0, (ds, dd, is_, id_, de, ie, dmo, imo) = large
+    args = dev(ds), dev(dd), dev(is_), R0
+    R, st, dV = g.pagerank_dfp(*args, del_mask=de, ins_mask=ie, want_dV=True, **kw)
+    Ro, sto, dVo, trace = oracle.pagerank_dfp(og1, ds, dd, is_, host(R0), del_mask=dmo, ins_mask=imo,
+                                              prune=bool(kw.get("prune", 1)))
+    assert st.affected_initial == trace[0]
+    assert st.iterations == sto.iterations and np.array_equal(host(dV), dVo)
+    assert np.max(np.abs(host(R) - Ro) / Ro) <= 1e-12
+    Rh, sth, dVh = g.pagerank_dfp(*args, del_mask=de, ins_mask=ie, want_dV=True, time_sweeps=1, check_every=3, **kw)
+    assert torch.equal(R, Rh) and torch.equal(dV, dVh) and sth.affected_initial == trace[0]
+
+
+def test_static_and_dt_with_rows_of_several_chunks(large):
+    g, og1, R0, (ds, dd, is_, id_, de, ie, dmo, imo) = large
+    R, st = g.pagerank_static()
+    Ro, sto = oracle.pagerank_static(og1)
+    assert st.iterations == sto.iterations and np.max(np.abs(host(R) - Ro) / Ro) <= 1e-12
+    R, st, dV = g.pagerank_dt(dev(ds), dev(dd), dev(is_), R0, del_mask=de, ins_mask=ie, want_dV=True)
+    Ro, sto, dVo, na, _ = oracle.pagerank_dt(og1, ds, dd, is_, host(R0), del_mask=dmo, ins_mask=imo)
+    assert st.affected_initial == na and st.iterations == sto.iterations and np.array_equal(host(dV), dVo)
+    assert np.max(np.abs(host(R) - Ro) / Ro) <= 1e-12
