@@ -1154,7 +1154,7 @@ __device__ __forceinline__ void expand_round(const SweepArgs<Real>& a, LoopSlot*
 
 // mode kLoopAll: the whole loop (cooperative launch): [initial push], then
 // sweep, barrier, stop test, [expansion, barrier] until the stop rule holds or
-// max_iter sweeps ran. The other modes run one phase of iteration it0 as a
+// max_iter sweeps ran (the last of them expands too). The other modes run one phase of iteration it0 as a
 // launch of its own (the host-driven loop): a phase past convergence exits at
 // once.
 template <class P, bool DYN>
@@ -1196,11 +1196,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_rank_loop(const __grid
     if (!grid_barrier(a.ctl, target)) return;
     const unsigned long long resid = __ldcg(&sl->resid);
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
-    if (stopped(resid, a.tol) || it + 1 >= a.max_iter) {
+    const bool done = stopped(resid, a.tol);
+    if (done || it + 1 >= a.max_iter) {
       if (first) {
         a.ctl->iters = it + 1;
         a.ctl->resid = resid;
       }
+      // a loop cut off by max_iter leaves the affected set of a next sweep, as after every sweep that did not converge
+      if (DYN && a.expand && !done) expand_round(a, sl);
       return;
     }
     // the slot of sweep it + 2, which the sweep before this one used: a

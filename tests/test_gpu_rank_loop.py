@@ -1,13 +1,13 @@
 """The rank loop on graphs of more than 6.3 M in-edges, where rows of 129 to 4096 entries are a warp each and longer ones
-go by four 1024-edge chunks a unit. Flags, counts and sweep numbers are the oracle's; ranks lie within 1e-12 relative of
-it (the same iteration, rounding-level differences), as in the other parity tests."""
+go by four 1024-edge chunks a unit, and loops that max_iter cuts off. Flags, counts and sweep numbers are the oracle's;
+ranks lie within 1e-12 relative of it (the same iteration, rounding-level differences), as in the other parity tests."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import synth
-from helpers import batch_case, dev, host
+from helpers import batch_case, dev, dynamic_case, host
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +64,23 @@ def test_static_and_dt_with_rows_of_several_chunks(large):
     Ro, sto, dVo, na, _ = oracle.pagerank_dt(og1, ds, dd, is_, host(R0), del_mask=dmo, ins_mask=imo)
     assert st.affected_initial == na and st.iterations == sto.iterations and np.array_equal(host(dV), dVo)
     assert np.max(np.abs(host(R) - Ro) / Ro) <= 1e-12
+
+
+@pytest.mark.parametrize("expand_pull", [0.0, 2.0])
+@pytest.mark.parametrize("max_iter", [1, 2, 3, 5])
+@pytest.mark.parametrize("prune", [1, 0])
+def test_dfp_stopped_by_max_iter(prune, max_iter, expand_pull):
+    """The affected set after a sweep that did not converge includes that sweep's expansion, the last one's too
+    (Alg. frontier), and the mixed solve's FP64 stage starts from it."""
+    g, og1, R0, (ds, dd, is_, id_, de, ie, dmo, imo) = dynamic_case(5, 12, 40000, 4)
+    kw = dict(del_mask=de, ins_mask=ie, want_dV=True, prune=prune, max_iter=max_iter, expand_pull=expand_pull)
+    args = dev(ds), dev(dd), dev(is_), R0
+    R, st, dV = g.pagerank_dfp(*args, **kw)
+    Ro, sto, dVo, _ = oracle.pagerank_dfp(og1, ds, dd, is_, host(R0), del_mask=dmo, ins_mask=imo, prune=bool(prune),
+                                          max_iter=max_iter)
+    assert not sto.converged and st.iterations == sto.iterations == max_iter
+    assert np.array_equal(host(dV), dVo)
+    assert np.max(np.abs(host(R) - Ro) / Ro) <= 1e-12
+    for precision in (0, 1):
+        (R, st, dV), (Rh, sth, dVh) = (g.pagerank_dfp(*args, precision=precision, time_sweeps=t, **kw) for t in (0, 1))
+        assert torch.equal(dV, dVh) and torch.equal(R, Rh)
