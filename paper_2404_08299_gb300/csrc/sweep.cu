@@ -158,7 +158,11 @@ __device__ __forceinline__ uint64_t degree_of(double d) {
   const uint64_t mant = (b & 0x000FFFFFFFFFFFFFull) | (1ull << 52);
   return e >= 0 ? mant >> (52 - e) : 0ull;
 }
-__device__ __forceinline__ uint64_t degree_of(float d) { return (uint64_t)d; }
+// The same of an FP32 out-degree: below 2^24 a float holds every integer, from there on the row's offsets are read (a
+// rounded degree would leave the row's last out-edges out of its frontier entries).
+__device__ __forceinline__ uint64_t degree_of(float d, const int64_t* ooff, int32_t v) {
+  return d < 16777216.f || !ooff ? (uint64_t)d : (uint64_t)(__ldg(ooff + v + 1) - __ldg(ooff + v));
+}
 
 // What a warp carries through a sweep: largest |r - R[v]|, (FP32) largest r,
 // out-edges put into deltaN, affected vertices seen.
@@ -293,7 +297,7 @@ __device__ __forceinline__ bool finish(const SweepArgs<float>& a, const Ctx<PKah
     front = dr > a.tau_f * m;
     if (front != dn_old) a.dN[v] = front ? 1 : 0;
     if (front) {
-      deg = degree_of(d);
+      deg = degree_of(d, a.ooff, v);
       t.fw += deg;
     }
     a.wrote[v] = 1;

@@ -1,6 +1,7 @@
 """The rank loop on graphs of more than 6.3 M in-edges, where rows of 129 to 4096 entries are a warp each and longer ones
-go by four 1024-edge chunks a unit, and loops that max_iter cuts off. Flags, counts and sweep numbers are the oracle's;
-ranks lie within 1e-12 relative of it (the same iteration, rounding-level differences), as in the other parity tests."""
+go by four 1024-edge chunks a unit, loops that max_iter cuts off, and out-degrees that a float does not hold. Flags,
+counts and sweep numbers are the oracle's; ranks lie within 1e-12 relative of it (the same iteration, rounding-level
+differences), as in the other parity tests."""
 import numpy as np
 import pytest
 import torch
@@ -17,6 +18,11 @@ def _built():
     from paper_2404_08299_gb300 import build
     build.build()
     torch.cuda.init()
+
+
+def prdf():
+    import paper_2404_08299_gb300 as p
+    return p
 
 
 PLANTED = [129, 130, 255, 257, 511, 512, 513, 514, 1023, 1024, 1025, 1026, 2047, 2048, 2049, 2050, 4095, 4096, 4097,
@@ -84,3 +90,19 @@ def test_dfp_stopped_by_max_iter(prune, max_iter, expand_pull):
     for precision in (0, 1):
         (R, st, dV), (Rh, sth, dVh) = (g.pagerank_dfp(*args, precision=precision, time_sweeps=t, **kw) for t in (0, 1))
         assert torch.equal(dV, dVh) and torch.equal(R, Rh)
+
+
+@pytest.mark.parametrize("above", [1, 1025])
+def test_fp32_frontier_of_an_out_degree_past_a_floats_integers(above):
+    """A vertex with 2^24 + above out-edges (its self-loop included), above = 1 modulo 1024, joins the frontier in an
+    FP32 sweep: every out-neighbour is marked, the last one too (DF keeps every mark)."""
+    n = (1 << 24) + above
+    hub = torch.zeros(n - 1, dtype=torch.int32, device="cuda")
+    g = prdf().Graph(n, hub, torch.arange(1, n, dtype=torch.int32, device="cuda"))
+    R0, _ = g.pagerank_static(max_iter=3)
+    e = torch.zeros(0, dtype=torch.int32, device="cuda")
+    one = torch.ones(1, dtype=torch.int32, device="cuda")
+    de, ie = g.apply_batch(e, e, one, torch.zeros_like(one))  # 1 -> hub
+    R, st, dV = g.pagerank_dfp(e, e, one, R0, ins_mask=ie, want_dV=True, prune=0, precision=1, expand_pull=2.0,
+                               max_iter=8)
+    assert int(dV.sum()) == n
