@@ -661,14 +661,11 @@ int update_pair_small(int32_t n, const Csr* old, const BatchLists* b, const floa
   const int P = pow2_at_least(n_del > n_ins ? n_del : (n_ins > 0 ? n_ins : 1));
   const int nd_pow = P, ni_pow = P;
   const size_t smem = (size_t)(nd_pow + ni_pow) * (8 + 8 + 8) + (size_t)ni_pow * 4;
-  static const bool smem_set = [] {
-    // the largest case: kSmallBatch keys per list
-    const int mx = (2 * kSmallBatch) * (8 + 8 + 8) + kSmallBatch * 4;
-    if (cudaFuncSetAttribute(k_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess)
-      cudaGetLastError();
-    return true;
-  }();
-  (void)smem_set;
+  // above the default limit, which each device keeps for itself: raised before every such launch, to the same value
+  // for every size, so that threads with batches of their own do not lower each other's
+  constexpr int kMaxSmem = 2 * kSmallBatch * (8 + 8 + 8) + kSmallBatch * 4;
+  if (smem > kDefaultSmem / 2)
+    PRDF_CUDA(cudaFuncSetAttribute(k_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   const size_t nb = (size_t)(n_del + n_ins > 0 ? n_del + n_ins : 1);
   const size_t n32 = (size_t)n_del + 2 * (size_t)n_ins + nb + 4;
   const size_t n64 = (size_t)n_del + 1 + (size_t)n_ins + 1 + 6 * (nb + 1) + 5;

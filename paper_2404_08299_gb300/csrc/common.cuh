@@ -95,6 +95,7 @@ struct DBuf {
 // ------------------------------------------------------ launch shapes ----
 
 constexpr int kSMs = 152;  // GB300: 2 dies x 76 SMs; grids are sized in multiples of this
+constexpr int kDefaultSmem = 48 * 1024;  // dynamic shared memory a block may take without a raised limit
 
 inline int grid_for(int64_t work, int per_block, int cap_blocks = kSMs * 32) {
   int64_t b = (work + per_block - 1) / per_block;

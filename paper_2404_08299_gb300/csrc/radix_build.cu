@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kRT, kRBlocks) k_radix_scatter(const KeySrc sr
 
 constexpr int kRScatterSmem = kRTile * 8 + kRDigits * 8 + kRWarps * kRDigits * 4 + kRWarps * 4;
 constexpr int kRScatterSmemW = kRScatterSmem + kRTile * 4;
+static_assert(kRScatterSmem <= kDefaultSmem, "launched without raising the limit");
 
 // ---- merge of equal keys ----
 // A warp takes 32 * kRK consecutive sorted keys, 32 per round (coalesced);
@@ -419,11 +420,15 @@ int radix_pass(const KeySrc& src, int64_t M, int shift, uint64_t* out, float* wo
   k_radix_hist<FIRST><<<(unsigned)ntiles, kRT, 0, s>>>(src, M, shift, hist.p, ntiles);
   PRDF_LAUNCH_CHECK();
   PRDF_TRY(exclusive_scan_u32(hist.p, ntiles * kRDigits, goff.p, ws, s));
-  if (wout)
+  if (wout) {
+    // above the default limit, which each device keeps for itself: set before every launch
+    PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<FIRST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   kRScatterSmemW));
     k_radix_scatter<FIRST, true><<<(unsigned)ntiles, kRT, kRScatterSmemW, s>>>(src, M, shift, goff.p, ntiles, out, wout);
-  else
+  } else {
     k_radix_scatter<FIRST, false><<<(unsigned)ntiles, kRT, kRScatterSmem, s>>>(src, M, shift, goff.p, ntiles, out,
                                                                                nullptr);
+  }
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }
@@ -442,17 +447,6 @@ bool radix_pair_applies(int32_t n, int64_t m0, bool self_loops) {
 
 namespace {
 
-int radix_smem() {
-  static bool smem_set = false;
-  if (smem_set) return PRDF_OK;
-  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
-  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmem));
-  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmemW));
-  PRDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRScatterSmemW));
-  smem_set = true;
-  return PRDF_OK;
-}
-
 // The CSR of the list, and with `in` that of its transpose: the first CSR's
 // unique entries, in its order, are a list sorted by row, so a stable sort by
 // column alone (half the passes) gives the transposed CSR with its rows in
@@ -464,7 +458,6 @@ int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols,
   while (B < 31 && ((int64_t)1 << B) < (int64_t)n) ++B;  // ids < n <= 2^B
   const int passes = (2 * B + 7) / 8;
   const int64_t ntiles = (M + kRTile - 1) / kRTile;
-  PRDF_TRY(radix_smem());
   DBuf<uint64_t> ka, kb;
   DBuf<float> wa, wb;
   DBuf<uint32_t> hist;
