@@ -72,6 +72,7 @@ __device__ __forceinline__ float ld_const(const float* p, uint64_t pol) {
 
 // Exact accumulator (4 x 32-bit words, 2^-124 resolution).
 struct AccExact {
+  static constexpr bool kAnyOrder = true;  // the sum does not depend on the order of the terms
   Fix4 v;
   __device__ __forceinline__ void add(uint64_t xb) { v.add(xb); }
   // add_w1: only for terms with in_w1 (the common window, three-word add)
@@ -86,6 +87,7 @@ struct AccExact {
 
 // plain FP64 additions
 struct AccPlain {
+  static constexpr bool kAnyOrder = false;
   double v = 0;
   __device__ __forceinline__ void add(uint64_t xb) { v += bitsd(xb); }
   __device__ __forceinline__ static bool in_w1(uint64_t) { return true; }
@@ -106,6 +108,7 @@ struct AccPlain {
 // FP32 sum compensated by Kahan-Babuska (TwoSum of every term, errors summed
 // separately): value = s + e
 struct AccKahan {
+  static constexpr bool kAnyOrder = false;
   float s = 0.f, e = 0.f;
   __device__ __forceinline__ void addf(float y) {
     const float t = s + y;
@@ -524,8 +527,13 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
     // (static solves, a row per lane against a group per row: 2^24 R-MAT 58.6 ->
     // 57.6 ms, 4096^2 grid 21.8 -> 14.1 ms, mixed 2^22 13.5 -> 13.0 ms; rows of 33
     // to 128 lose, 58.8 ms, their index loads then cost as much as the gathers);
-    // small batches of a small graph keep the groups (2^16: 1.07 against 1.25 ms)
-    if (G <= 8 && nact - k0 >= 24)
+    // small batches of a small graph keep the groups (2^16: 1.07 against 1.25 ms).
+    // In DF / DF-P a row's place in the list, and with it the size of its batch,
+    // changes from run to run, so sums that depend on the order of their terms
+    // take one form whatever the batch (as fast as by size, DF-P and DT on 2^16 to
+    // 2^24; groups throughout: DT of a 2^22 grid 14.7 against 12.4 ms)
+    constexpr bool kOneForm = DYN && !P::Acc::kAnyOrder;
+    if (G <= 8 && (kOneForm || nact - k0 >= 24))
       sum_lane_rows<P>(a, c, cur.b, cur.len, cur.v, saved, hit);
     else
       sum_rows<P, G>(a, c, steps(k0), cur.b, cur.len, cur.v, saved, hit);

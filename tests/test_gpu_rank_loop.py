@@ -1,7 +1,7 @@
 """The rank loop on graphs of more than 6.3 M in-edges, where rows of 129 to 4096 entries are a warp each and longer ones
-go by four 1024-edge chunks a unit, loops that max_iter cuts off, and out-degrees that a float does not hold. Flags,
-counts and sweep numbers are the oracle's; ranks lie within 1e-12 relative of it (the same iteration, rounding-level
-differences), as in the other parity tests."""
+go by four 1024-edge chunks a unit, loops that max_iter cuts off, out-degrees that a float does not hold, and sums that
+depend on their order. Flags, counts and sweep numbers are the oracle's; ranks lie within 1e-12 relative of it (the
+same iteration, rounding-level differences), as in the other parity tests."""
 import numpy as np
 import pytest
 import torch
@@ -106,3 +106,26 @@ def test_fp32_frontier_of_an_out_degree_past_a_floats_integers(above):
     R, st, dV = g.pagerank_dfp(e, e, one, R0, ins_mask=ie, want_dV=True, prune=0, precision=1, expand_pull=2.0,
                                max_iter=8)
     assert int(dV.sum()) == n
+
+
+def random_rows(n, lo, hi, seed):
+    """lo to hi in-edges a vertex from random sources."""
+    rng = np.random.default_rng(seed)
+    d = np.repeat(np.arange(n, dtype=np.int32), rng.integers(lo, hi + 1, n))
+    return n, rng.integers(0, n, len(d)).astype(np.int32), d
+
+
+@pytest.mark.parametrize("call", ["pagerank_dfp", "pagerank_dt"])
+@pytest.mark.parametrize("kw", [{"precision": 1}, {"accumulate": 1}, {"accumulate": 1, "prune": 0}])
+@pytest.mark.parametrize("graph", ["rows", "rmat"])
+def test_every_run_gives_the_same_bits(graph, kw, call):
+    """FP32 sums and plain FP64 sums round by the order of their terms. The affected rows are listed in an order that
+    changes from run to run, so rows of 5 to 32 entries come in batches of every size."""
+    case = batch_case(*random_rows(100003, 8, 15, 1), 3, 300) if graph == "rows" else dynamic_case(9, 20, 1 << 24, 300)
+    g, og1, R0, (ds, dd, is_, id_, de, ie, dmo, imo) = case
+    out = [getattr(g, call)(dev(ds), dev(dd), dev(is_), R0, del_mask=de, ins_mask=ie, want_dV=True,
+                            time_sweeps=int(k % 3 == 2), **kw) for k in range(9)]
+    R, st, dV = out[0]
+    for Rk, stk, dVk in out[1:]:
+        assert torch.equal(R, Rk) and torch.equal(dV, dVk)
+        assert st.iterations == stk.iterations and st.iterations_fp32 == stk.iterations_fp32
