@@ -479,6 +479,32 @@ __device__ __forceinline__ void sum_lane_rows(const SweepArgs<typename P::Real>&
   }
 }
 
+// Rows that outgrew their class. Batch updates keep the numbering until 1/64 of
+// the edges have changed, so a row of a short class can grow to that many
+// entries, and a lane or a small group would walk it for longer than the rest
+// of the sweep takes. The classes below a warp per row leave rows above these
+// lengths out of their batches and set the warp's flag; sum_grown takes them by
+// the whole warp after the unit. 100 K in-edges added to a row of 1 / 2 / 6 / 20 /
+// 60 on 8.9 M edges, a solve of 76 sweeps: 1401 / 1972 / 714 / 169 / 88 ms when
+// the batch summed them, 40.2 / 40.9 / 40.2 / 41.0 / 40.3 ms now, 38.7 with the
+// row numbered as what it is. A flag in shared memory and a second pass, as
+// registers for it in the batch loops cost every solve (a 4096^2 grid 13.5 ms
+// without, 14.2 summed within the batch, 13.2 this way).
+constexpr int kGrown = 128;     // no class of 4, 8 or 16 lanes per row is made for longer rows
+constexpr int kGrownLane = 16;  // the same for a lane per row
+__device__ __forceinline__ volatile int* grown_flag() {
+  __shared__ int flag[kWarps];
+  return flag + (threadIdx.x >> 5);
+}
+template <class Row>
+__device__ __forceinline__ void leave_grown(Row& r, int limit) {
+  if (r.len > limit) {
+    *grown_flag() = 1;
+    r.v = -1;
+    r.len = 0;
+  }
+}
+
 // A unit: the rows at positions [kb, ke) of a class, G lanes per row, in
 // batches of up to 32. The offsets of the next batch and the row ids of the
 // one after it load before the batch.
@@ -517,10 +543,12 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
 
   int32_t vn = load_v(32);
   Batch cur = load_off(load_v(0));
+  if (G < 32) leave_grown(cur, kGrown);
   for (int k0 = 0; k0 < nact; k0 += 32) {
     const Batch nxt = load_off(vn);
     vn = load_v(k0 + 64);
-    const Own<typename P::Real> own = load_own<P, DYN>(a, c, in_batch(k0), cur.v);
+    const bool have = cur.v >= 0;
+    const Own<typename P::Real> own = load_own<P, DYN>(a, c, have, cur.v);
     typename P::Acc saved;
     bool hit = false;
     // rows of 5 to 32 entries: a row per lane when the batch fills most lanes
@@ -537,12 +565,38 @@ __device__ __forceinline__ void unit_group(const SweepArgs<typename P::Real>& a,
       sum_lane_rows<P>(a, c, cur.b, cur.len, cur.v, saved, hit);
     else
       sum_rows<P, G>(a, c, steps(k0), cur.b, cur.len, cur.v, saved, hit);
-    const bool have = in_batch(k0);
     // graphs without self-loops on every vertex: x[v] counts only when the row
     // holds v (rows of a warp or more always took x[v])
     const Bits xs = have && (G == 32 || a.self_loops || hit) ? ld_state(c.x + cur.v, c.pl) : Bits(0);
     finish_batch<P, DYN>(a, c, have, cur.v, saved.value(), as_real(xs), own, t);
     cur = nxt;
+    if (G < 32) leave_grown(cur, kGrown);
+  }
+}
+
+// The rows of [kb, ke) above `limit` entries, one after the other. (A graph
+// that had a batch has every self-loop.)
+template <class P, bool DYN>
+__device__ __forceinline__ void sum_grown(const SweepArgs<typename P::Real>& a, const Ctx<P>& c, int64_t kb,
+                                          int64_t ke, int limit, Tally& t) {
+  for (int64_t k0 = kb; k0 < ke; k0 += 32) {
+    int32_t v = 0;
+    int64_t b = 0;
+    int len = 0;
+    if (k0 + c.lane < ke) {
+      v = row_at<P, DYN>(a, k0 + c.lane);
+      b = a.off[v];
+      len = (int)(a.off[v + 1] - b);
+    }
+    const bool far = len > limit;
+    const uint32_t m = __ballot_sync(kFull, far);
+    if (!m) continue;
+    const Own<typename P::Real> own = load_own<P, DYN>(a, c, far, v);
+    typename P::Acc saved;
+    bool hit = false;
+    sum_rows<P, 32>(a, c, 32 - __clz(m), b, far ? len : 0, 0, saved, hit);
+    const typename P::Bits xs = far ? ld_state(c.x + v, c.pl) : typename P::Bits(0);
+    finish_batch<P, DYN>(a, c, far, v, saved.value(), as_real(xs), own, t);
   }
 }
 
@@ -659,10 +713,11 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
   const int32_t v0 = load_v(0), v1 = load_v(32);
   int32_t vf = load_v(64);
   Row cur = load_off(v0), nxt = load_off(v1);
+  leave_grown(cur, kGrownLane);
   int32_t u[U];
   load_idx(cur, u);
   for (int k0 = 0; k0 < nact; k0 += 32) {
-    const bool have = k0 + c.lane < nact;
+    const bool have = cur.v >= 0;
     Bits xv[U];
 #pragma unroll
     for (int k = 0; k < U; ++k) xv[k] = u[k] >= 0 ? ld_state(c.x + u[k], c.pl) : Bits(0);
@@ -686,6 +741,7 @@ __device__ __forceinline__ void unit_thread(const SweepArgs<typename P::Real>& a
     const Bits xself = (a.self_loops || hit) ? xs : Bits(0);
     finish_batch<P, DYN>(a, c, have, cur.v, acc.value(), as_real(xself), own, t);
     cur = nxt;
+    leave_grown(cur, kGrownLane);
     nxt = far;
 #pragma unroll
     for (int k = 0; k < U; ++k) u[k] = un[k];
@@ -702,17 +758,22 @@ __device__ __forceinline__ void unit_self(const SweepArgs<typename P::Real>& a, 
   using Bits = typename P::Bits;
   int32_t vn = kb + c.lane < ke ? row_at<P, DYN>(a, kb + c.lane) : 0;
   for (int64_t k0 = kb; k0 < ke; k0 += 32) {
-    const bool have = k0 + c.lane < ke;
+    bool have = k0 + c.lane < ke;
     const int32_t v = vn;
     vn = k0 + 32 + c.lane < ke ? row_at<P, DYN>(a, k0 + 32 + c.lane) : 0;
     const Bits xs = have ? ld_state(c.x + v, c.pl) : Bits(0);
     const Own<typename P::Real> own = load_own<P, DYN>(a, c, have, v);
     typename P::Real sum = as_real(xs);
     if (a.multi && have && ((a.multi[v >> 5] >> (v & 31)) & 1u)) {
-      typename P::Acc acc;
-      const int64_t e = a.off[v + 1];
-      for (int64_t j = a.off[v]; j < e; ++j) acc.add(ld_state(c.x + a.adj[j], c.pl));
-      sum = acc.value();
+      const int64_t b = a.off[v], e = a.off[v + 1];
+      if (e - b > kGrownLane) {
+        *grown_flag() = 1;
+        have = false;
+      } else {
+        typename P::Acc acc;
+        for (int64_t j = b; j < e; ++j) acc.add(ld_state(c.x + a.adj[j], c.pl));
+        sum = acc.value();
+      }
     }
     finish_batch<P, DYN>(a, c, have, v, sum, as_real(xs), own, t);
   }
@@ -910,6 +971,8 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
   c.pf = policy_evict_first();
   c.pl = policy_evict_last();
   c.lane = threadIdx.x & 31;
+  if (c.lane == 0) *grown_flag() = 0;
+  __syncwarp();
   Tally t;
   // First unit by position (consecutive units on different SMs). The others
   // come from a counter, or by position again where units are few or the sweep
@@ -942,6 +1005,17 @@ __device__ __forceinline__ void sweep(const SweepArgs<typename P::Real>& a, int 
         case kRow8: unit_group<P, 8, DYN>(a, c, kb, ke, t); break;
         case kRow16: unit_group<P, 16, DYN>(a, c, kb, ke, t); break;
         default: unit_group<P, 32, DYN>(a, c, kb, ke, t); break;
+      }
+      __syncwarp();
+      if (*grown_flag()) {  // (the unit is looked up again, so that nothing is kept over it)
+        int q = 0;
+        while (q + 1 < a.ncls && u >= plan->unit0[q + 1]) ++q;
+        const int64_t gb = plan->begin[q] + (int64_t)(u - plan->unit0[q]) * plan->rows[q];
+        const int64_t ge = gb + plan->rows[q] < plan->end[q] ? gb + plan->rows[q] : plan->end[q];
+        sum_grown<P, DYN>(a, c, gb, ge, a.cls[q].kind <= kRowThread ? kGrownLane : kGrown, t);
+        __syncwarp();
+        *grown_flag() = 0;
+        __syncwarp();
       }
     }
     u = nw + __shfl_sync(kFull, nx, 0);

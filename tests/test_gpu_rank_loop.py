@@ -129,3 +129,39 @@ def test_every_run_gives_the_same_bits(graph, kw, call):
     for Rk, stk, dVk in out[1:]:
         assert torch.equal(R, Rk) and torch.equal(dV, dVk)
         assert st.iterations == stk.iterations and st.iterations_fp32 == stk.iterations_fp32
+
+
+@pytest.mark.parametrize("old", [1, 2, 6, 20, 60])
+def test_a_row_that_outgrew_its_class(old):
+    """A vertex of `old` in-edges gains 100,000 in a batch that keeps the numbering. Its row is walked by as many lanes
+    as in the class of a warp per row, so a solve takes no longer than twice that of a graph built with the row there
+    (the rest of a sweep is the same; a lane or a few of them alone take up to fifty times as long), in Static and in
+    DF, whose ranks and flags are those of the fresh graph."""
+    n, s, d = synth.rmat(19, 1 << 23, seed=81)
+    keep = d != 5
+    s, d = s[keep], d[keep]
+    src = np.arange(n - 200000, n, dtype=np.int32)
+    s = np.concatenate([s, src[:old - 1]]).astype(np.int32)
+    d = np.concatenate([d, np.full(old - 1, 5, np.int32)]).astype(np.int32)
+    g = prdf().Graph(n, dev(s), dev(d))
+    new = dev(src[1000:101000])
+    e = torch.zeros(0, dtype=torch.int32, device="cuda")
+    g.apply_batch(e, e, new, torch.full_like(new, 5))
+    assert g.m > 6 << 20
+    fresh = prdf().Graph(n, torch.cat([dev(s), new]), torch.cat([dev(d), torch.full_like(new, 5)]))
+    fresh.set_thresholds(prdf().PRDF_IN, [1, 4, 16, 32, 128, 1 << 30])
+    assert fresh.m == g.m
+    ms = {}
+    for name, x in (("grown", g), ("fresh", fresh)):
+        for precision in (0, 1):
+            x.pagerank_static(precision=precision)
+            ms[name, precision] = min(x.pagerank_static(precision=precision)[1].ms_iterate for _ in range(3))
+    Rg, stg = g.pagerank_static()
+    Rf, stf = fresh.pagerank_static()
+    assert torch.equal(Rg, Rf) and stg.iterations == stf.iterations
+    for precision in (0, 1):
+        assert ms["grown", precision] <= 2 * ms["fresh", precision]
+    (Rg, stg, dVg), (Rf, stf, dVf) = (x.pagerank_dfp(e, e, new, Rf, want_dV=True, prune=0, tol=1e-14, tau_f=1e-9)
+                                      for x in (g, fresh))
+    assert torch.equal(Rg, Rf) and torch.equal(dVg, dVf) and stg.iterations == stf.iterations
+    assert stg.affected_initial == stf.affected_initial
