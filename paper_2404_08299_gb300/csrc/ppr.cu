@@ -5,13 +5,15 @@
 // rounded up to a multiple of four (padding columns stay zero), so one index
 // and weight fetch serves a tile of columns, four of them per lane.
 //
-// FP32 sweeps sum the products of up to eight edges with FMAs and fold each
+// FP32 sweeps sum the products of up to four edges with FMAs and fold each
 // such sum into a compensated pair (TwoSum), so the rounding error does not
-// grow with the row length. The FP64 stage is mixed-precision iterative
-// refinement: an FP64 sweep computes the Jacobi step T(R) and the residual
-// T(R) - R; an FP32 solve of E = alpha P^T E + residual gives the correction.
-// The stop rule is the same as Static's: the L-inf change of an FP64 Jacobi
-// step <= tol.
+// grow with the row length. (Eight at a time lose most of what follows a large
+// product in a row of eight; four cost 1 % of the K = 32 forward and backward,
+// 34.8 -> 35.2 ms, and nothing at K = 64.) The FP64 stage is mixed-precision
+// iterative refinement: an FP64 sweep computes the Jacobi step T(R) and the
+// residual T(R) - R; an FP32 solve of E = alpha P^T E + residual gives the
+// correction. The stop rule is the same as Static's: the L-inf change of an
+// FP64 Jacobi step <= tol.
 //
 // One persistent kernel per solve (k_ppr_loop, a cooperative launch), as in
 // sweep.cu: units of rows and row chunks of every column tile, a grid barrier
@@ -68,7 +70,7 @@ struct Sum64 {
   }
 };
 
-// Column accumulator: products go to b; fold() ends a block of at most eight
+// Column accumulator: products go to b; fold() ends a block of at most four
 // of them; sum(folded) is the total (folded: any block was ended before).
 struct Col32 {
   using Sum = Dot2;
@@ -313,7 +315,7 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q].prod(w, r[k].v[q]);
       }
-      if ((e0 / U) % 2 == 1 && (more || e0 + U < most)) {
+      if (more || e0 + U < most) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q].fold();
         folded = true;
@@ -525,10 +527,8 @@ __device__ __forceinline__ void unit_chunks(const PprArgs<T>& a, const Ctx<T>& c
 #pragma unroll
         for (int q = 0; q < Q; ++q) acc[q].prod(w, r[i].v[q]);
       }
-      if ((i0 / U) % 2 == 1 || kPer == U) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) acc[q].fold();
-      }
+      for (int q = 0; q < Q; ++q) acc[q].fold();
       if (i0 + U < kPer && (i0 + U) * kSlots < here) {
 #pragma unroll
         for (int i = 0; i < U; ++i) {
