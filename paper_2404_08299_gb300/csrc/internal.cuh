@@ -229,7 +229,8 @@ struct SweepArgs {
 int launch_rank_loop(const SweepArgs<double>& a, const PartThr& t, const int64_t* cb, bool exact, bool dynamic,
                      cudaStream_t s);
 int launch_rank_loop(const SweepArgs<float>& a, const PartThr& t, const int64_t* cb, bool dynamic, cudaStream_t s);
-// Chunk table of the rows [begin, n) longer than `above` entries (above = 0: of every row).
+// Chunk table of the rows [begin, n) longer than `above` entries (above = 0: of every row). With above > 0 the number of
+// chunks is read back (max_chunks is exact), else the table has room for the most there can be.
 int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int size, int above, SweepChunks& t,
                  Workspace& ws, cudaStream_t s);
 // initialAffected (Alg. affected) in the sweep numbering: dV, dN and the frontier list of the first push

@@ -1476,18 +1476,27 @@ int build_chunks(const int64_t* off, int64_t begin, int64_t n, int64_t m, int si
     t.rows = 0;
     return PRDF_OK;
   }
-  // the number of chunks stays on the device; the table has room for the most there can be
-  t.max_chunks = (above > 0 ? m / above : t.rows) + m / size + 1;
+  PRDF_TRY(t.cnt.reserve((size_t)t.rows, s));
+  PRDF_TRY(t.first.reserve((size_t)t.rows + 1, s));
+  k_chunk_count<<<grid_for(t.rows, 256), 256, 0, s>>>(off, begin, t.rows, size, above, t.cnt.p);
+  PRDF_LAUNCH_CHECK();
+  PRDF_TRY(exclusive_scan_u32(t.cnt.p, t.rows, t.first.p, ws, s));
+  if (above > 0) {
+    // the K-column calls keep a partial sum per chunk and column: room for as
+    // many chunks as there are (2^22 vertices, K = 64: 158 K chunks, 81 MB; the
+    // bound m / above + m / size would be 859 K, 440 MB)
+    PRDF_CUDA(cudaMemcpyAsync(ws.host_i64, t.first.p + t.rows, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    PRDF_CUDA(cudaStreamSynchronize(s));
+    t.max_chunks = ws.host_i64[0];
+  } else {
+    // the rank sweep's 16 bytes a chunk: room for the most there can be, so that a call after a batch waits for nothing
+    t.max_chunks = t.rows + m / size + 1;
+  }
   if (t.max_chunks >= INT32_MAX) {
     set_error("too many row chunks");
     return PRDF_EINVAL;
   }
-  PRDF_TRY(t.cnt.reserve((size_t)t.rows, s));
-  PRDF_TRY(t.first.reserve((size_t)t.rows + 1, s));
-  PRDF_TRY(t.chunks.reserve((size_t)t.max_chunks, s));
-  k_chunk_count<<<grid_for(t.rows, 256), 256, 0, s>>>(off, begin, t.rows, size, above, t.cnt.p);
-  PRDF_LAUNCH_CHECK();
-  PRDF_TRY(exclusive_scan_u32(t.cnt.p, t.rows, t.first.p, ws, s));
+  PRDF_TRY(t.chunks.reserve((size_t)(t.max_chunks > 0 ? t.max_chunks : 1), s));
   k_chunk_fill<<<grid_for(t.rows * 32, 256), 256, 0, s>>>(off, begin, t.rows, size, t.first.p, t.chunks.p);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;

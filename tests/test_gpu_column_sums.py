@@ -1,4 +1,4 @@
-"""K-column calls: how finely FP32 products are folded into the compensated sums."""
+"""K-column calls: how finely FP32 products are folded into the compensated sums, and the memory a call takes."""
 import numpy as np
 import pytest
 import torch
@@ -43,3 +43,24 @@ def test_fp32_products_are_folded_by_fours(deg, K):
     err = (got - term.sum()).abs().max().item() / 2.0 ** -23
     lost = 3 * 0.4
     assert err <= lost + 0.5 + deg * 2.0 ** -23
+
+
+def test_memory_of_a_call_without_long_rows():
+    """Rows of at most 90 entries, so no chunks of long rows: an FP64 call takes the state (24 bytes a vertex and column)
+    and its tables (16 bytes a vertex, 4 more a vertex and tile of 64 columns), and no room for partial sums of chunks.
+    64 MB are left for the pool's granularity."""
+    n, deg, K = 20000, 90, 2048
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    i = torch.arange(n, device="cuda")
+    src = torch.cat([(i + int(k)) % n for k in torch.randperm(n - 1, device="cuda", generator=gen)[:deg - 1] + 1])
+    g = prdf().Graph(n, src.int(), i.repeat(deg - 1).int(), torch.ones(src.numel(), device="cuda"))
+    S = torch.rand(n, K, dtype=torch.float64, device="cuda", generator=gen)
+    g.pagerank_ppr(S[:, :3].contiguous(), max_iter=2)
+    R = torch.empty(n, K, dtype=torch.float64, device="cuda")
+    del R  # (the result's memory is there: torch hands the block out again)
+    prdf().release_cached_memory()
+    before = torch.cuda.mem_get_info()[0]
+    R, _ = g.pagerank_ppr(S, max_iter=2)
+    prdf().release_cached_memory()
+    used = before - torch.cuda.mem_get_info()[0]
+    assert used <= 24 * n * K + 16 * n + 4 * n * (K // 64) + (64 << 20), used
