@@ -294,6 +294,74 @@ __global__ void __launch_bounds__(kRT) k_uniq_count(const uint64_t* __restrict__
   if (lane == 0) cnt[gw] = c;
 }
 
+// ---- row offsets of long runs of empty rows ----
+// The lane of a key writes the offsets of its row and of the empty rows before
+// it, runs of fewer than kGapLane rows that is (and those after the last key).
+// Longer runs are left to far_gaps, which a warp that saw one calls in the end:
+// the warp writes them, or lists those of kGapWarp rows and more for
+// k_fill_gaps, the whole GPU's. One lane took 140 ms for the 16 M rows after the
+// last used one (1 M edges; the whole build 145.6 ms, 2.0 now).
+constexpr int64_t kGapLane = 64;
+constexpr int64_t kGapWarp = 1 << 16;
+struct Gap {
+  int64_t first, last, pos;  // off[first..last] = pos
+};
+struct Gaps {
+  Gap* list;  // room for n / kGapWarp + 1
+  unsigned int* count;
+};
+
+// the runs at the warp's keys [base, base + 32 * kRK) of k[0..M), the first new one of which has position pos
+__device__ __forceinline__ void far_gaps(const uint64_t* __restrict__ k, int64_t M, int B, int32_t n, int64_t base,
+                                      int64_t pos, int64_t* __restrict__ off, const Gaps gaps) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = lanemask_lt();
+#pragma unroll 1
+  for (int r = 0; r < kRK; ++r) {
+    const int64_t i = base + r * 32 + lane;
+    const uint64_t key = i < M ? k[i] : ~0ull, prev = i > 0 && i < M ? k[i - 1] : ~0ull;
+    const bool f = i < M && (i == 0 || key != prev);
+    const uint32_t bal = __ballot_sync(0xffffffffu, f);
+    const int64_t row = (int64_t)(key >> B);
+    // the rows before a new key, and those after the last key
+#pragma unroll 1
+    for (int after = 0; after < 2; ++after) {
+      int64_t first = 1, last = 0, at = 0;
+      if (after == 0 && f) {
+        first = i == 0 ? 0 : (int64_t)(prev >> B) + 1;
+        last = row;
+        at = pos + __popc(bal & lt);
+      } else if (after == 1 && i == M - 1) {
+        first = row + 1;
+        last = n;
+        at = pos + __popc(bal);
+      }
+      uint32_t todo = __ballot_sync(0xffffffffu, last - first >= kGapLane);
+      while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const Gap g = {__shfl_sync(0xffffffffu, first, l), __shfl_sync(0xffffffffu, last, l),
+                       __shfl_sync(0xffffffffu, at, l)};
+        if (g.last - g.first >= kGapWarp) {
+          if (lane == 0) gaps.list[atomicAdd(gaps.count, 1u)] = g;
+        } else {
+          for (int64_t q = g.first + lane; q <= g.last; q += 32) off[q] = g.pos;
+        }
+      }
+    }
+    pos += __popc(bal);
+  }
+}
+
+__global__ void k_fill_gaps(const Gaps gaps, int64_t* __restrict__ off) {
+  const unsigned int c = *gaps.count;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (unsigned int k = 0; k < c; ++k) {
+    const Gap g = gaps.list[k];
+    for (int64_t q = g.first + tid; q <= g.last; q += step) off[q] = g.pos;
+  }
+}
+
 // Columns of the unique keys, and off[r] = position of row r's first unique
 // key (rows without keys take the next row's start; off[n] = total).
 // woff = exclusive scan of the per-warp counts, woff[nw] = total. kt (or null)
@@ -307,8 +375,9 @@ __global__ void __launch_bounds__(kRT) k_uniq_count(const uint64_t* __restrict__
 __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ k, int64_t M, int B, int32_t n,
                                                    const int64_t* __restrict__ woff, int64_t nw,
                                                    int32_t* __restrict__ adj, int64_t* __restrict__ off,
-                                                   int32_t* __restrict__ urow, uint64_t* __restrict__ kt,
-                                                   const float* __restrict__ w, uint32_t* __restrict__ uw) {
+                                                   int32_t* __restrict__ urow, const Gaps gaps,
+                                                   uint64_t* __restrict__ kt, const float* __restrict__ w,
+                                                   uint32_t* __restrict__ uw) {
   const int lane = threadIdx.x & 31;
   const int64_t gw = ((int64_t)blockIdx.x * kRT + threadIdx.x) >> 5;
   const int64_t base = gw * (32 * kRK);
@@ -331,6 +400,7 @@ __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ 
   }
   const uint64_t after = base + 32 * kRK < M ? k[base + 32 * kRK] : ~0ull;  // the next warp's first key
   int64_t pos = gw < nw ? woff[gw] : 0;
+  bool far = false;
 #pragma unroll
   for (int r = 0; r < kRK; ++r) {
     const int64_t i = base + r * 32 + lane;
@@ -358,15 +428,22 @@ __global__ void __launch_bounds__(kRT) k_uniq_emit(const uint64_t* __restrict__ 
         urow[p] = (int32_t)row;
       } else {
         const int64_t first = i == 0 ? 0 : (int64_t)(prev >> B) + 1;  // rows after the previous key's
-        for (int64_t q = first; q <= row; ++q) off[q] = p;
+        if (row - first < kGapLane)
+          for (int64_t q = first; q <= row; ++q) off[q] = p;
+        else
+          far = true;
       }
     }
     if (!urow && i == M - 1) {
-      const int64_t total = woff[nw];
-      for (int64_t q = (int64_t)(key[r] >> B) + 1; q <= n; ++q) off[q] = total;
+      const int64_t total = woff[nw], first = (int64_t)(key[r] >> B) + 1;
+      if (n - first < kGapLane)
+        for (int64_t q = first; q <= n; ++q) off[q] = total;
+      else
+        far = true;
     }
     pos += __popc(bal);
   }
+  if (__any_sync(0xffffffffu, far)) far_gaps(k, M, B, n, base, woff[gw], off, gaps);
 }
 
 // off[r] = first position whose row is >= r (urow ascending, length mu): one
@@ -386,7 +463,7 @@ __global__ void k_offsets_from_rows(const int32_t* __restrict__ urow, int64_t mu
 // 32 * kRK keys, all loaded before the first is written (one key at a time a
 // thread before: 0.73 ms for 285 M keys, 4.6 TB/s)
 __global__ void __launch_bounds__(kRT) k_emit(const uint64_t* __restrict__ k, int64_t m, int B, int32_t n,
-                                              int32_t* __restrict__ adj, int64_t* __restrict__ off) {
+                                              int32_t* __restrict__ adj, int64_t* __restrict__ off, const Gaps gaps) {
   const uint64_t cmask = (1ull << B) - 1;
   const int lane = threadIdx.x & 31;
   const int64_t base = (((int64_t)blockIdx.x * kRT + threadIdx.x) >> 5) * (32 * kRK);
@@ -398,6 +475,7 @@ __global__ void __launch_bounds__(kRT) k_emit(const uint64_t* __restrict__ k, in
     key[r] = i < m ? __ldcs(reinterpret_cast<const unsigned long long*>(k) + i) : ~0ull;
   }
   int64_t row = base > 0 ? (int64_t)(k[base - 1] >> B) : -1;  // of the key before the round's first
+  bool far = false;
 #pragma unroll
   for (int r = 0; r < kRK; ++r) {
     const int64_t i = base + r * 32 + lane;
@@ -407,11 +485,20 @@ __global__ void __launch_bounds__(kRT) k_emit(const uint64_t* __restrict__ k, in
     row = __shfl_sync(0xffffffffu, mine, 31);
     if (i < m) adj[i] = (int32_t)(key[r] & cmask);
     // rows after the previous key's start here; past the last key (i = m) they are empty and end there
-    if (i <= m)
-      for (int64_t q = prev + 1; q <= mine; ++q) off[q] = i;
+    if (i <= m) {
+      if (mine - (prev + 1) < kGapLane)
+        for (int64_t q = prev + 1; q <= mine; ++q) off[q] = i;
+      else
+        far = true;
+    }
   }
-  if (base + 32 * kRK == m && lane == 31)  // no lane had i = m
-    for (int64_t q = row + 1; q <= n; ++q) off[q] = m;
+  if (base + 32 * kRK == m && lane == 31) {  // no lane had i = m
+    if (n - (row + 1) < kGapLane)
+      for (int64_t q = row + 1; q <= n; ++q) off[q] = m;
+    else
+      far = true;
+  }
+  if (__any_sync(0xffffffffu, far)) far_gaps(k, m, B, n, base, base, off, gaps);
 }
 
 template <bool FIRST>
@@ -519,12 +606,19 @@ int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols,
   // a list much shorter than n leaves long runs of empty rows: their offsets
   // are found row-parallel instead of by the lanes that emit the keys
   const bool sparse = M * 16 < (int64_t)n;
+  DBuf<Gap> gap_list;
+  DBuf<unsigned int> gap_count;
+  PRDF_TRY(gap_list.alloc((size_t)(n / kGapWarp + 1), s));
+  PRDF_TRY(gap_count.alloc(1, s));
+  const Gaps gaps{gap_list.p, gap_count.p};
+  PRDF_CUDA(cudaMemsetAsync(gap_count.p, 0, sizeof(unsigned int), s));
   DBuf<int32_t> urow;
   if (sparse) PRDF_TRY(urow.alloc(room, s));
   k_uniq_emit<<<(unsigned)ntiles, kRT, 0, s>>>(cur, M, B, n, woff.p, nw, out.adj.p, out.off.p,
-                                               sparse ? urow.p : nullptr, in ? nxt : nullptr, wcur,
+                                               sparse ? urow.p : nullptr, gaps, in ? nxt : nullptr, wcur,
                                                w ? reinterpret_cast<uint32_t*>(out.w.p) : nullptr);
   if (sparse) k_offsets_from_rows<<<grid_for((int64_t)n + 1, kRT), kRT, 0, s>>>(urow.p, out.m, n, out.off.p);
+  else if (n >= kGapWarp) k_fill_gaps<<<grid_for(n, 8 * kRT, kSMs * 8), kRT, 0, s>>>(gaps, out.off.p);
   PRDF_LAUNCH_CHECK();
   if (!in) return PRDF_OK;
   swap(cur, nxt);  // the transposed keys
@@ -543,7 +637,9 @@ int build_radix(int32_t n, int64_t m0, const int32_t* rows, const int32_t* cols,
     swap(cur, nxt);
     swap(wcur, wnxt);
   }
-  k_emit<<<(unsigned)((m + kRTile - 1) / kRTile), kRT, 0, s>>>(cur, m, B, n, in->adj.p, in->off.p);
+  PRDF_CUDA(cudaMemsetAsync(gap_count.p, 0, sizeof(unsigned int), s));
+  k_emit<<<(unsigned)((m + kRTile - 1) / kRTile), kRT, 0, s>>>(cur, m, B, n, in->adj.p, in->off.p, gaps);
+  if (n >= kGapWarp) k_fill_gaps<<<grid_for(n, 8 * kRT, kSMs * 8), kRT, 0, s>>>(gaps, in->off.p);
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }
