@@ -1,0 +1,64 @@
+"""Calls whose rows, thresholds or options are not the usual ones: their results against the usual form of the same call,
+and their times, which stay within a factor of it."""
+import time
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+from helpers import dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2404_08299_gb300 import build
+    build.build()
+    torch.cuda.init()
+
+
+def prdf():
+    import paper_2404_08299_gb300 as p
+    return p
+
+
+def best_ms(call, runs=4):
+    call()
+    best = 1e9
+    for _ in range(runs):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        call()
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t)
+    return 1e3 * best
+
+
+def hubs(n, k, deg):
+    """k vertices with deg in-edges each among others with about four."""
+    rng = np.random.default_rng(7)
+    s = rng.integers(0, n, k * deg + 4 * n).astype(np.int32)
+    return n, s, np.concatenate([np.repeat(np.arange(k, dtype=np.int32), deg),
+                                 rng.integers(0, n, 4 * n).astype(np.int32)])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_pull_rounds_on_a_few_long_rows(precision):
+    """DF-P whose expansion rounds all pull, on 40 rows of 50,000 in-entries: the flags and ranks are those of push
+    rounds, and the call takes at most eight times as long (32 rows of that length on one warp take thirty times)."""
+    n, s, d = hubs(300000, 40, 50000)
+    g = prdf().Graph(n, dev(s), dev(d))
+    R0, _ = g.pagerank_static()
+    e, ins = torch.zeros(0, dtype=torch.int32, device="cuda"), (dev(np.array([x], np.int32)) for x in (17, 4711))
+    isrc, idst = ins
+    g.apply_batch(e, e, isrc, idst)
+    ms, out = {}, {}
+    for form in (0.0, 2.0):
+        def call():
+            out[form] = g.pagerank_dfp(e, e, isrc, R0, want_dV=True, expand_pull=form, precision=precision)
+        ms[form] = best_ms(call)
+    (Ra, sa, dVa), (Rb, sb, dVb) = out[0.0], out[2.0]
+    assert torch.equal(dVa, dVb) and torch.equal(Ra, Rb) and sa.iterations == sb.iterations
+    assert ms[0.0] <= 8 * ms[2.0], ms
