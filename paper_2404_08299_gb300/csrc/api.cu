@@ -471,7 +471,7 @@ int nonempty_classes(const int64_t* cb, int nclass) {
 //     check_every sweeps ahead of each residual read; sweeps launched past
 //     convergence exit at once on the device. Each sweep is bracketed by CUDA
 //     events.
-constexpr int64_t kChunkSmallM = 6ll << 20;
+constexpr int64_t kChunkSmallM = 6ll << 20, kChunkSmallRow = 32;
 
 struct Loop {
   bool fp32 = false, dynamic = false, expand = false, exact = true;
@@ -569,12 +569,15 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
 // (a warp per row otherwise, up to 4096 edges) is cut as well, into chunks of
 // 512 edges: R-MAT 2^16 (1.0 M edges) 16 -> 13 us a sweep, 2^18 (4.4 M) 39 ->
 // 30, but 2^19 (8.9 M) 44 -> 47 and 2^20 64 -> 84 (a unit of one chunk costs
-// about 4 us whatever its length).
+// about 4 us whatever its length). Only a class of rows above kChunkSmallRow
+// entries: with thresholds that put short rows there a chunk, and with it a
+// unit, held a few edges (bounds of 1 and 64 on a 2^17 R-MAT: 5.0 ms a solve,
+// 4.3 in batches of a warp per row).
 int ensure_sweep_chunks(prdf_graph* g, const int64_t* cb, cudaStream_t s) {
   SweepChunks& t = g->sweep_chunks;
   if (!t.valid || t.version != g->rl.version) {
     const int C = g->rl.thr.n + 1;
-    const bool small = g->rl.in.m < kChunkSmallM && C >= 3;
+    const bool small = g->rl.in.m < kChunkSmallM && C >= 3 && g->rl.thr.thr[C - 3] >= kChunkSmallRow;
     t.valid = false;
     t.first_class = small ? C - 2 : C - 1;
     t.size = small ? 512 : (int)kHubChunk;

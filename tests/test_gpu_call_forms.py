@@ -62,3 +62,24 @@ def test_pull_rounds_on_a_few_long_rows(precision):
     (Ra, sa, dVa), (Rb, sb, dVb) = out[0.0], out[2.0]
     assert torch.equal(dVa, dVb) and torch.equal(Ra, Rb) and sa.iterations == sb.iterations
     assert ms[0.0] <= 8 * ms[2.0], ms
+
+
+@pytest.mark.parametrize("graph", ["random", "hubs"])
+def test_thresholds_that_leave_short_rows_in_the_last_classes(graph):
+    """Thresholds 1 and 64: every row above one entry is in the last classes. The ranks are those of the default
+    classes, and a solve takes at most five times as long (with a chunk and a unit to each of those rows: eight)."""
+    rng = np.random.default_rng(3)
+    if graph == "hubs":
+        n, s, d = hubs(300000, 40, 50000)
+    else:
+        n = 100000
+        s, d = (rng.integers(0, n, 3 * n).astype(np.int32) for _ in range(2))
+    g = prdf().Graph(n, dev(s), dev(d))
+    ms, R = [], []
+    for thr in (None, [1, 64]):
+        if thr:
+            g.set_thresholds(prdf().PRDF_IN, thr)
+        ms.append(best_ms(lambda: g.pagerank_static()))
+        R.append(g.pagerank_static()[0])
+    assert torch.equal(R[0], R[1])
+    assert ms[1] <= 5 * ms[0], ms
