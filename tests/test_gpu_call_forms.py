@@ -104,3 +104,29 @@ def test_push_rounds_on_rows_of_all_lengths():
     (Ra, sa, dVa), (Rb, sb, dVb) = out["push"], out["default"]
     assert torch.equal(dVa, dVb) and torch.equal(Ra, Rb) and sa.iterations == sb.iterations
     assert ms["push"] <= 2.2 * ms["default"], ms
+
+
+def test_weights_of_one_long_row():
+    """New weights on 2 M edges that enter one vertex, and on 2 M edges between random ones: at most ten times as long
+    (a block of threads for the long row takes 25 times), and every weight in its place: the K-column result is that of
+    a graph built with them."""
+    n = 2000000
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    i = torch.arange(1, n, dtype=torch.int32, device="cuda")
+    graphs = {"star": (i, torch.zeros_like(i)),
+              "random": tuple(torch.randint(n, (n,), device="cuda", generator=gen, dtype=torch.int32)
+                              for _ in range(2))}
+    ms = {}
+    for name, (s, d) in graphs.items():
+        g = prdf().Graph(n, s, d, torch.ones(len(s), device="cuda"))
+        w = torch.rand(g.m, device="cuda", generator=gen) + 0.5
+        g.set_weights(w)
+        ms[name] = best_ms(lambda: g.set_weights(w))
+        off, adj, got = g.export_csr(prdf().PRDF_OUT)
+        assert torch.equal(got, w)
+        rows = torch.repeat_interleave(torch.arange(n, device="cuda", dtype=torch.int32), off.diff())
+        fresh = prdf().Graph(n, rows, adj, w, self_loops=False)
+        S = torch.zeros(n, 4, dtype=torch.float64, device="cuda")
+        S[:64] = 1 / 64
+        assert torch.equal(g.pagerank_ppr(S)[0], fresh.pagerank_ppr(S)[0])
+    assert ms["star"] <= 10 * ms["random"], ms
