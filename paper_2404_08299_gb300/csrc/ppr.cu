@@ -926,13 +926,17 @@ int launch_grad_w(const int64_t* off, const int32_t* adj, const int32_t* perm, c
   DBuf<double> bu;
   PRDF_TRY(bu.alloc((size_t)n, s));
   const int grid = grid_for((m + kGradChunk - 1) / kGradChunk * 32, 256);
-  if (K > 8) {
+  if (K > 8)
     k_grad_rows<8><<<grid_for((int64_t)n * 8, 256), 256, 0, s>>>(lam, Gs, g_scale, Rr, n, K, bu.p);
-    k_grad_w<8><<<grid, 256, 0, s>>>(off, adj, perm, orig_off, lam, bu.p, Rr, W, n, m, K, alpha, grad_w);
-  } else {
+  else
     k_grad_rows<2><<<grid_for((int64_t)n * 2, 256), 256, 0, s>>>(lam, Gs, g_scale, Rr, n, K, bu.p);
+  // Lanes per edge: as few as keep the gathered rows of lambda in flight, since every lane past the columns is idle
+  // and the lanes' sums cost additions. Gradient part, ms, 8 lanes -> 2: R-MAT 2^19 (8 M edges) K = 12 0.78 -> 0.45,
+  // K = 32 1.05 -> 0.82; 12 M edges in rows of 200 0.90 -> 0.49, 1.23 -> 0.89; 8 -> 4 at K = 64: 1.66 -> 1.47.
+  if (K > 32)
+    k_grad_w<4><<<grid, 256, 0, s>>>(off, adj, perm, orig_off, lam, bu.p, Rr, W, n, m, K, alpha, grad_w);
+  else
     k_grad_w<2><<<grid, 256, 0, s>>>(off, adj, perm, orig_off, lam, bu.p, Rr, W, n, m, K, alpha, grad_w);
-  }
   PRDF_LAUNCH_CHECK();
   return PRDF_OK;
 }
