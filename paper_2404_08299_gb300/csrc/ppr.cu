@@ -35,7 +35,10 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int64_t kShortMean = 4;  // K of 1 or 2: 2 lanes a row in units of at most this mean length, else 8
+// K of 1 or 2: 2 lanes a row in units of at most this mean length, else 4. (2 up to a mean of 4 and 8 lanes above it
+// left most lanes without an edge on rows of 5 to 20. K = 2, ms a solve, FP64 and mixed: 10^6-vertex grid 22.3 -> 5.4
+// and 11.1 -> 3.9, 8.7 M random edges 21.8 -> 7.1 and 9.2 -> 5.3, 2^22 R-MAT 59.4 -> 47.6 and 39.2 -> 35.)
+constexpr int64_t kShortMean = 20;
 
 // Compensated FP32 sum (s + e): TwoSum folds each term's rounding error into e.
 struct Dot2 {
@@ -643,7 +646,7 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
       } else {
         const int64_t len = __ldg(a.off + ve) - __ldg(a.off + vb);
         if (len <= kShortMean * (ve - vb)) unit_rows_narrow<T, Q, 2>(a, c, (int32_t)vb, (int32_t)ve, pk);
-        else unit_rows_narrow<T, Q, 8>(a, c, (int32_t)vb, (int32_t)ve, pk);
+        else unit_rows_narrow<T, Q, 4>(a, c, (int32_t)vb, (int32_t)ve, pk);
       }
     }
     x = nw + __shfl_sync(kFull, nx, 0);
