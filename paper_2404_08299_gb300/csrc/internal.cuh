@@ -358,7 +358,7 @@ struct prdf_graph {
   bool ppr_valid = false;
   prdf::DBuf<double> wsum;           // sum of out-weights per vertex (sweep numbering)
   prdf::DBuf<double> pin64;          // P on the in-edge slots of rl.in
-  prdf::DBuf<float> pin32;
+  prdf::DBuf<float> pin32;  // m + kAdjPad, the padding zero, as pout32
   prdf::DBuf<double> pout64;         // P on the out-edge slots of rl.out (adjoint)
   prdf::DBuf<float> pout32;
   // K-column scratch

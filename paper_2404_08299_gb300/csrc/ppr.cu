@@ -84,6 +84,14 @@ struct Col32 {
     d.add(b);
     b = 0.f;
   }
+  // a whole block at once
+  template <class R>
+  __device__ __forceinline__ void block(const float (&p)[4], const R (&r)[4], int q) {
+    float x = p[0] * r[0].v[q];
+#pragma unroll
+    for (int k = 1; k < 4; ++k) x = fmaf(p[k], r[k].v[q], x);
+    d.add(x);
+  }
   __device__ __forceinline__ Dot2 sum(bool folded) {
     if (!folded) {
       d.s = b;
@@ -170,6 +178,12 @@ __device__ __forceinline__ float ld_weight(const float* p, uint64_t pol) {
   return v;
 }
 __device__ __forceinline__ double ld_weight(const double* p, uint64_t pol) { return ld_stream_f64(p, pol); }
+// four weights from a 16-byte boundary
+__device__ __forceinline__ void ld_weights4(const float* p, uint64_t pol, float (&w)[4]) {
+  asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
+      : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3])
+      : "l"(p), "l"(pol));
+}
 
 // Largest |T(R) - R| and |T(R)| a thread saw (bits).
 struct Peak {
@@ -275,7 +289,7 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
   load_win(b, rem);
   load_off(v + kSlots, bn, ln);
   typename Traits<T>::Col acc[4];
-  bool todo = rem >= 0, folded = false;
+  bool todo = rem >= 0;
   for (int32_t v0 = vb; v0 < ve;) {
     const int here = rem < kE ? rem : kE;
     const int most = __reduce_max_sync(kFull, here);
@@ -309,19 +323,23 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
 #pragma unroll
     for (int e0 = 0; e0 < kE; e0 += U) {
       if (e0 >= most) break;
+      if constexpr (sizeof(T) == 4) {
+        // (no partial block is kept from step to step: K = 32 on 17 M edges 130.3 -> 128.6, 10^6-vertex grid 17.7 -> 16.9 ms)
+        T w[U];
 #pragma unroll
-      for (int k = 0; k < U; ++k) {
-        // FP64 products are what a step is short of, and an instruction costs its 32 lanes whatever they hold:
-        // those past the longest row are left out (K = 8 on 17 M edges: 37.3 -> 34.2 ms)
-        if (sizeof(T) == 8 && k > 0 && e0 + k >= most) break;
-        const T w = __shfl_sync(kFull, cp[(e0 + k) / LPE], slot0 + (e0 + k) % LPE);
+        for (int k = 0; k < U; ++k) w[k] = __shfl_sync(kFull, cp[(e0 + k) / LPE], slot0 + (e0 + k) % LPE);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].prod(w, r[k].v[q]);
-      }
-      if (more || e0 + U < most) {
+        for (int q = 0; q < 4; ++q) acc[q].block(w, r, q);
+      } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].fold();
-        folded = true;
+        for (int k = 0; k < U; ++k) {
+          // FP64 products are what a step is short of, and an instruction costs its 32 lanes whatever they hold:
+          // those past the longest row are left out (K = 8 on 17 M edges: 37.3 -> 34.2 ms)
+          if (k > 0 && e0 + k >= most) break;
+          const T w = __shfl_sync(kFull, cp[(e0 + k) / LPE], slot0 + (e0 + k) % LPE);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[q].prod(w, r[k].v[q]);
+        }
       }
       if (e0 + U < kE && e0 + U < most) {
 #pragma unroll
@@ -335,16 +353,94 @@ __device__ __forceinline__ void unit_rows(const PprArgs<T>& a, const Ctx<T>& c, 
       if (done) {
         T t[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = acc[q].sum(folded).value();
+        for (int q = 0; q < 4; ++q) t[q] = acc[q].d.value();
         Own<T, 4> own;
         load_own<T, 4>(a, c, vdone, own);
         finish_row<T, 4>(a, c, vdone, t, own, pk);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[q] = typename Traits<T>::Col();
-      folded = false;
       v0 += kSlots;
     }
+  }
+}
+
+// The same rows for FP32 tiles of up to 16 columns (LPE lanes a row, 1, 2 or
+// 4): every lane of a slot loads the row's next four indices and weights
+// itself, one 16-byte load each (from the 16-byte boundary at or before the
+// row, so the first and last may hold neighbours' entries: adj and the weights
+// end in padding), which leaves out the window's registers and its shuffles.
+// The indices of the next step load while this step's gathers are on their
+// way; the weights come with the gathers. The
+// block of four products goes straight into the compensated pair. Ms a mixed
+// solve, windows and this form: 10^6-vertex grid K = 4 5.8 and 4.1, K = 8 6.5
+// and 5.6, K = 16 11.9 and 9.8; 8.7 M random edges 8.2 and 5.7, 8.7 and 7.2, 14.7
+// and 12.8; 2^22 R-MAT 51.8 and 41.0, 54.3 and 51.8, 88.9 and 83.0. At 32
+// columns and above the windows' loads, one entry a lane, are the cheaper ones.
+// (The teleport and the previous rank load with the step's gathers; with one
+// lane a row that cost more: K = 4 on the random edges 6.53 against 6.43.)
+template <int LPE>
+__device__ __forceinline__ void unit_rows_direct(const PprArgs<float>& a, const Ctx<float>& c, int32_t vb, int32_t ve,
+                                                 Peak& pk) {
+  constexpr int kSlots = 32 / LPE;
+  const int slot = c.lane / LPE;
+  auto load_off = [&](int32_t v, int64_t& b, int& len) {
+    b = 0;
+    len = -1;
+    if (v < ve && v >= 0) {
+      b = ld_stream_i64(a.off + v, c.pf);
+      const int64_t d = ld_stream_i64(a.off + v + 1, c.pf) - b;
+      len = d <= a.row_max ? (int)d : -1;
+    }
+  };
+  int32_t v = vb + slot;
+  int64_t b, bn;
+  int len, ln;
+  load_off(v, b, len);
+  load_off(v + kSlots, bn, ln);
+  int j = -(int)(b & 3);  // the step's first entry, counted from the row's
+  int4 u = make_int4(0, 0, 0, 0);
+  if (j < len) u = ld_stream_i32x4(a.adj + b + j, c.pf);
+  Dot2 acc[4];
+  float w[4] = {};
+  for (int32_t v0 = vb; v0 < ve;) {
+    Vec<float, 4> r[4];
+    const int32_t id[4] = {u.x, u.y, u.z, u.w};
+    if (j < len) ld_weights4(a.P + b + j, c.pf, w);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) gather<4>(c, a.K, id[k], j + k >= 0 && j + k < len, r[k]);
+    j += 4;
+    const bool more = __any_sync(kFull, j < len);
+    const int32_t vdone = v;
+    const bool fin = len >= 0 && !more;
+    Own<float, 4> own;
+    if (LPE > 1 && fin) load_own<float, 4>(a, c, vdone, own);
+    if (!more) {
+      v += kSlots;
+      b = bn;
+      len = ln;
+      j = -(int)(b & 3);
+      load_off(v + kSlots, bn, ln);
+    }
+    if (j < len) u = ld_stream_i32x4(a.adj + b + j, c.pf);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float x = w[0] * r[0].v[q];
+#pragma unroll
+      for (int k = 1; k < 4; ++k) x = fmaf(w[k], r[k].v[q], x);
+      acc[q].add(x);
+    }
+    if (more) continue;
+    if (fin) {
+      if (LPE == 1) load_own<float, 4>(a, c, vdone, own);
+      float t[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) t[q] = acc[q].value();
+      finish_row<float, 4>(a, c, vdone, t, own, pk);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = Dot2();
+    v0 += kSlots;
   }
 }
 
@@ -604,7 +700,7 @@ __device__ __forceinline__ bool stopped(unsigned long long resid, float tol) {
 }
 
 // LPE lanes of four columns each side by side (Q = 4); LPE = 1: a lane has the
-// whole row, Q columns.
+// whole row, Q columns (FP32: 1, 2 or 4, FP64: 1 or 2).
 template <class T, int LPE, int Q>
 __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
   Ctx<T> c;
@@ -641,7 +737,9 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
       // from the highest class down: long rows first
       const int64_t ve = a.row_end - (int64_t)un * a.rows_per_unit;
       const int64_t vb = ve > a.rows_per_unit ? ve - a.rows_per_unit : 0;
-      if constexpr (LPE > 1) {
+      if constexpr (sizeof(T) == 4 && Q == 4 && LPE <= 4) {
+        unit_rows_direct<LPE>(a, c, (int32_t)vb, (int32_t)ve, pk);
+      } else if constexpr (LPE > 1) {
         unit_rows<T, LPE>(a, c, (int32_t)vb, (int32_t)ve, pk);
       } else {
         const int64_t len = __ldg(a.off + ve) - __ldg(a.off + vb);
@@ -881,7 +979,7 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
     return PRDF_ECUDA;
   }
   const int max_b = per * sms;
-  constexpr int kSlots = LPE > 1 ? 32 / LPE : 16;
+  constexpr int kSlots = Q == 4 ? 32 / LPE : 16;
   a.tiles = (a.K + Q * LPE - 1) / (Q * LPE);
   // rows of a unit: about an eighth of a warp's share, a few steps at least
   int64_t rows = kSlots;
@@ -910,6 +1008,8 @@ template <class T>
 int run_ppr(const PprArgs<T>& a, int tile, int64_t n, cudaStream_t s) {
   if (a.K == 1) return run_tile<T, 1, 1>(a, n, s);
   if (a.K == 2) return run_tile<T, 1, 2>(a, n, s);
+  if constexpr (sizeof(T) == 4)
+    if (a.K == 4) return run_tile<T, 1, 4>(a, n, s);
   switch (tile) {
     case 8: return run_tile<T, 2, 4>(a, n, s);
     case 16: return run_tile<T, 4, 4>(a, n, s);

@@ -329,9 +329,12 @@ int build_ppr_weights(prdf_graph* g, cudaStream_t s) {
   const int64_t m = r.in.m;
   PRDF_TRY(g->wsum.reserve((size_t)n, s));
   PRDF_TRY(g->pin64.reserve((size_t)m, s));
-  PRDF_TRY(g->pin32.reserve((size_t)m, s));
+  PRDF_TRY(g->pin32.reserve((size_t)m + kAdjPad, s));
   PRDF_TRY(g->pout64.reserve((size_t)m, s));
-  PRDF_TRY(g->pout32.reserve((size_t)m, s));
+  PRDF_TRY(g->pout32.reserve((size_t)m + kAdjPad, s));
+  // (read with the last entries and multiplied by zeros: not to be a NaN)
+  PRDF_CUDA(cudaMemsetAsync(g->pin32.p + m, 0, kAdjPad * sizeof(float), s));
+  PRDF_CUDA(cudaMemsetAsync(g->pout32.p + m, 0, kAdjPad * sizeof(float), s));
   DBuf<int32_t> longs;
   DBuf<unsigned int> cnt;
   PRDF_TRY(longs.alloc((size_t)n, s));
