@@ -783,11 +783,12 @@ struct KOp {
 // chunks for whole warps. A narrow tile has many short slots (2 or 4 lanes) and
 // its long rows would be walked a few entries a step: measured on 0.7 M edges,
 // K = 5 in FP64, 32 / 48 / 64: 2.86 / 2.73 / 3.03 ms; wide tiles, 8.9 M edges,
-// K = 32, 80 / 96 / 128: 35.1 / 35.0 / 39.8 ms (forward and backward). FP64
-// loops on graphs large enough to hide the walk save the additions that merge a
-// chunk's slots: K = 8, 48 / 96 / 128: 17.1 / 15.7 / 17.8 ms on 8.7 M edges,
-// 122.9 / 104.9 / 106.6 on 69 M, but 2.74 / 3.30 / 3.39 on 0.7 M.
-int ppr_long_row(int tile, bool fp64, int64_t m) { return tile > 16 || (fp64 && m >= (1ll << 22)) ? 96 : 48; }
+// K = 32, 80 / 96 / 128: 35.1 / 35.0 / 39.8 ms (forward and backward). Graphs
+// large enough to hide the walk save the units of the chunks and the additions
+// that merge their slots: K = 8 in FP64, 48 / 96 / 128: 17.1 / 15.7 / 17.8 ms on
+// 8.7 M edges, 122.9 / 104.9 / 106.6 on 69 M, but 2.74 / 3.30 / 3.39 on 0.7 M;
+// mixed, 48 / 96: 4.7 / 2.0 ms on 12 M edges in rows of 60, 1.6 / 2.0 on 0.7 M.
+int ppr_long_row(int tile, int64_t m) { return tile > 16 || m >= (1ll << 22) ? 96 : 48; }
 // Chunks of 256 edges shorten the chains of small graphs (0.7 M edges, K = 33
 // mixed: 5.6 -> 4.6 ms), 512 cost less on larger ones, and 1024 on large ones
 // where the tile is narrow (K = 8 mixed, 512 / 1024: 7.95 / 7.82 ms on 8.7 M
@@ -796,8 +797,8 @@ int ppr_long_row(int tile, bool fp64, int64_t m) { return tile > 16 || (fp64 && 
 int ppr_chunk(int64_t m, int tile) {
   return m < (1ll << 22) ? 256 : m >= (12ll << 20) && tile <= 32 ? 1024 : 512;
 }
-int ensure_ppr_chunks(prdf_graph* g, const Csr& c, int tile, bool fp64, SweepChunks& t, cudaStream_t s) {
-  const int above = ppr_long_row(tile, fp64, c.m), size = ppr_chunk(c.m, tile);
+int ensure_ppr_chunks(prdf_graph* g, const Csr& c, int tile, SweepChunks& t, cudaStream_t s) {
+  const int above = ppr_long_row(tile, c.m), size = ppr_chunk(c.m, tile);
   if (t.valid && t.version == g->rl.version && t.above == above && t.size == size) return PRDF_OK;
   t.valid = false;
   t.size = size;
@@ -1697,7 +1698,7 @@ int prdf_pagerank_ppr(prdf_graph* g, const double* S, int K, double* R, const pr
   k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(S, g->rl.perm.p, g->n, K, Kp, 1.0, g->S64.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_TRY(ensure_ppr_chunks(g, g->rl.in, tile, p->precision == PRDF_FP64, g->ppr_chunks_in, s));
+  PRDF_TRY(ensure_ppr_chunks(g, g->rl.in, tile, g->ppr_chunks_in, s));
   const KOp op{g->rl.in.off.p, g->rl.in.adj.p, g->pin32.p, g->pin64.p, &g->ppr_chunks_in, g->S64.p, true};
   KSolve ks;
   ks.kernels = 1;
@@ -1804,7 +1805,7 @@ int prdf_pagerank_backward(prdf_graph* g, const double* R, const double* G, int 
   k_rows_gather<<<grid_for(cnt, kThreads), kThreads, 0, s>>>(G, g->rl.perm.p, g->n, K, Kp, 1.0 / beta, g->S64.p);
   PRDF_LAUNCH_CHECK();
   PRDF_CUDA(cudaEventRecord(t.e[1], s));
-  PRDF_TRY(ensure_ppr_chunks(g, g->rl.out, tile, p->precision == PRDF_FP64, g->ppr_chunks_out, s));
+  PRDF_TRY(ensure_ppr_chunks(g, g->rl.out, tile, g->ppr_chunks_out, s));
   const KOp op{g->rl.out.off.p, g->rl.out.adj.p, g->pout32.p, g->pout64.p, &g->ppr_chunks_out, g->S64.p, false};
   KSolve ks;
   ks.kernels = 1;

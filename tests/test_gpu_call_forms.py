@@ -226,3 +226,19 @@ def test_mixed_share_of_the_fp64_time(graph, K, share):
     S[torch.arange(0, n, n // 64, device="cuda")[:64]] = 1 / 64
     ms = [best_ms(lambda: g.pagerank_ppr(S, precision=p)) for p in (0, 1)]
     assert ms[1] <= share * ms[0], ms
+
+
+def test_mixed_time_of_rows_above_48_entries():
+    """12 M edges in rows of 60 or of 40 entries, K = 8 in mixed precision: about the same time (within 1.5 times; a
+    chunk and a unit for each row of 60 takes more than twice)."""
+    ms = {}
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    for deg in (40, 60):
+        n = 12000000 // deg
+        d = torch.arange(n, dtype=torch.int32, device="cuda").repeat_interleave(deg)
+        s = torch.randint(n, (n * deg,), device="cuda", generator=gen, dtype=torch.int32)
+        g = prdf().Graph(n, s, d, torch.rand(n * deg, device="cuda", generator=gen) + 0.5)
+        S = torch.zeros(n, 8, dtype=torch.float64, device="cuda")
+        S[torch.arange(0, n, n // 64, device="cuda")[:64]] = 1 / 64
+        ms[deg] = best_ms(lambda: g.pagerank_ppr(S, precision=1))
+    assert ms[60] <= 1.5 * ms[40], ms
