@@ -530,7 +530,6 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
   const SweepChunks& ch = g->sweep_chunks;
   a.chunks = ch.chunks.p;
   a.nchunk = ch.rows > 0 ? ch.first.p + ch.rows : nullptr;
-  a.max_chunks = ch.max_chunks;
   a.chunk_class = ch.first_class;
   a.chunk_size = ch.size;
   // four chunks a unit: 2^24 R-MAT 58.7 against 60.0 ms with one, 59.4 with two
@@ -831,7 +830,7 @@ int ppr_args(prdf_graph* g, const KOp& op, const prdf_params* p, int Kp, int til
   a.tol = sizeof(T) == 4 ? (T)p->tol_fp32_rel : (T)p->tol;
   a.max_iter = max_iter;
   a.m = g->m;
-  a.row_end = g->n;
+  a.n = g->n;
   a.row_max = ch.above;
   a.chunks = ch.chunks.p;
   a.nchunk = ch.rows > 0 ? ch.first.p + ch.rows : nullptr;

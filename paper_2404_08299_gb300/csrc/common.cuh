@@ -14,11 +14,6 @@ namespace prdf {
 
 void set_error(const char* fmt, ...);
 
-struct Status {
-  int code = PRDF_OK;
-  bool ok() const { return code == PRDF_OK; }
-};
-
 #define PRDF_CUDA(call)                                                                             \
   do {                                                                                              \
     cudaError_t e__ = (call);                                                                       \
@@ -200,14 +195,6 @@ struct Fix4 {
         : "r"(t0), "r"(t1), "r"(t2));
   }
 
-  __device__ __forceinline__ void add_words(const uint32_t* s) { add4(s[0], s[1], s[2], s[3]); }
-  __device__ __forceinline__ void store(uint32_t* s) const {
-    s[0] = w0;
-    s[1] = w1;
-    s[2] = w2;
-    s[3] = w3;
-  }
-
   template <int G>
   __device__ __forceinline__ void group_reduce() {
 #pragma unroll
@@ -287,22 +274,6 @@ __device__ __forceinline__ int64_t ld_stream_i64(const int64_t* p, uint64_t pol)
 __device__ __forceinline__ double ld_stream_f64(const double* p, uint64_t pol) {
   double v;
   asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
-  return v;
-}
-// gathered FP64 value returned as its bit pattern (stays on the integer pipes)
-__device__ __forceinline__ uint64_t ld_gather_b64(const double* p, uint64_t pol) {
-  uint64_t v;
-  asm("ld.global.nc.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ double ld_gather_f64(const double* p, uint64_t pol) {
-  double v;
-  asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ float ld_gather_f32(const float* p, uint64_t pol) {
-  float v;
-  asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
   return v;
 }
 

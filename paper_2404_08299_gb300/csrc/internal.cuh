@@ -202,7 +202,6 @@ struct SweepArgs {
   // and an arrival counter (zero between sweeps) per row
   const SweepChunk* chunks;
   const int64_t* nchunk;   // number of chunks (device), null: none
-  int64_t max_chunks;
   int chunk_class, chunk_size;
   uint32_t chunks_per_unit;
   uint4* hub_part;
@@ -261,8 +260,8 @@ struct PprArgs {
   int max_iter, mode, it0, it_first;  // as in SweepArgs
   LoopSlot* slot;
   LoopCtl* ctl;
-  // rows [0, row_end) of at most row_max entries one by one, the others in the chunk table
-  int64_t row_end;
+  // the n rows of at most row_max entries one by one, the others in the chunk table
+  int64_t n;
   int row_max;
   int rows_per_unit;
   const SweepChunk* chunks;

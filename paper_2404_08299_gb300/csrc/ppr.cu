@@ -713,7 +713,7 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
   const unsigned int nw = gridDim.x * kWarps;
   const unsigned int nchunk = a.nchunk ? (unsigned int)__ldg(a.nchunk) : 0u;
   const unsigned int cu = (nchunk + a.chunks_per_unit - 1) / a.chunks_per_unit;
-  const unsigned int ru = (unsigned int)((a.row_end + a.rows_per_unit - 1) / a.rows_per_unit);
+  const unsigned int ru = (unsigned int)((a.n + a.rows_per_unit - 1) / a.rows_per_unit);
   const unsigned int per_tile = cu + ru;
   const unsigned int total = per_tile * a.tiles;
   const bool counted = total > 4 * nw;
@@ -735,7 +735,7 @@ __device__ __forceinline__ void ppr_sweep(const PprArgs<T>& a, int it) {
       unit_chunks<T, LPE, Q>(a, c, cb, (int)cnt, tile_no, pk);
     } else {
       // from the highest class down: long rows first
-      const int64_t ve = a.row_end - (int64_t)un * a.rows_per_unit;
+      const int64_t ve = a.n - (int64_t)un * a.rows_per_unit;
       const int64_t vb = ve > a.rows_per_unit ? ve - a.rows_per_unit : 0;
       if constexpr (sizeof(T) == 4 && Q == 4 && LPE <= 4) {
         unit_rows_direct<LPE>(a, c, (int32_t)vb, (int32_t)ve, pk);
@@ -823,12 +823,12 @@ __global__ void k_grad_rows(const double* __restrict__ lam, const double* __rest
 }
 
 // A warp takes kGradChunk consecutive out-slots; L lanes (a slot) per edge,
-// columns over the lanes, four edges of a slot at a time, whose dot products
-// meet by exchanging halves (four additions for four edges instead of one per
-// edge and level: FP64 additions are what this kernel is short of after its
-// multiplications). The rows of long and short vertices cost the same per
-// edge (a lane per edge and a warp per row before: a serial walk over the
-// columns, and the longest row's walk at the end).
+// columns over the lanes, L edges of a slot at a time, whose dot products meet
+// by exchanging halves (fewer additions than one per edge and level: FP64
+// additions are what this kernel is short of after its multiplications). The
+// rows of long and short vertices cost the same per edge (a lane per edge and a
+// warp per row before: a serial walk over the columns, and the longest row's
+// walk at the end).
 constexpr int64_t kGradChunk = 512;
 template <int L>
 __global__ void __launch_bounds__(256) k_grad_w(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
@@ -837,7 +837,6 @@ __global__ void __launch_bounds__(256) k_grad_w(const int64_t* __restrict__ off,
                                                 const double* __restrict__ Rr, const double* __restrict__ W, int32_t n,
                                                 int64_t m, int K, double alpha, double* __restrict__ grad_w) {
   constexpr int kSlots = 32 / L;
-  constexpr int kE = L < 4 ? L : 4;  // edges of a slot at a time
   const int lane = threadIdx.x & 31, sub = lane & (L - 1), slot = lane / L;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -847,14 +846,14 @@ __global__ void __launch_bounds__(256) k_grad_w(const int64_t* __restrict__ off,
     int64_t r = 0, z = n;
     while (z - r > 1) {
       const int64_t mid = (r + z) >> 1;
-      if (off[mid] <= p0 + slot * kE) r = mid; else z = mid;
+      if (off[mid] <= p0 + slot * L) r = mid; else z = mid;
     }
-    for (int64_t q0 = p0; q0 < pe; q0 += kSlots * kE) {
-      double d[kE];
-      int64_t row[kE];
+    for (int64_t q0 = p0; q0 < pe; q0 += kSlots * L) {
+      double d[L];
+      int64_t row[L];
 #pragma unroll
-      for (int k = 0; k < kE; ++k) {
-        const int64_t p = q0 + slot * kE + k;
+      for (int k = 0; k < L; ++k) {
+        const int64_t p = q0 + slot * L + k;
         d[k] = 0;
         row[k] = -1;
         if (p < pe) {
@@ -886,37 +885,31 @@ __global__ void __launch_bounds__(256) k_grad_w(const int64_t* __restrict__ off,
           }
         }
       }
-      // lane sub of the slot ends with the sum of edge sub % kE: exchange halves while several
-      // edges are left, then plain butterflies
-      int have = kE;
-      int mine = 0;
+      // lane sub of the slot ends with the sum of its edge sub
+      int have = L;
 #pragma unroll
-      for (int o = 1; o < kE; o <<= 1) {
+      for (int o = 1; o < L; o <<= 1) {
         have >>= 1;
         const bool hi = sub & o;
 #pragma unroll
-        for (int k = 0; k < kE / 2; ++k) {
+        for (int k = 0; k < L / 2; ++k) {
           if (k < have) {
             const double keep = hi ? d[2 * k + 1] : d[2 * k], give = hi ? d[2 * k] : d[2 * k + 1];
             d[k] = keep + __shfl_xor_sync(kFull, give, o);
           }
         }
-        if (hi) mine += o;
       }
-#pragma unroll
-      for (int o = kE; o < L; o <<= 1) d[0] += __shfl_xor_sync(kFull, d[0], o);
-      const int64_t p = q0 + slot * kE + mine;
+      const int64_t p = q0 + slot * L + sub;
       int64_t rw = row[0];
 #pragma unroll
-      for (int k = 1; k < kE; ++k)
-        if (mine == k) rw = row[k];
-      if (sub < kE && rw >= 0 && p < pe)
+      for (int k = 1; k < L; ++k)
+        if (sub == k) rw = row[k];
+      if (rw >= 0 && p < pe)
         grad_w[orig_off[perm[rw]] + (p - off[rw])] = (alpha * d[0] - bu[rw]) * (1.0 / W[rw]);
     }
   }
 }
 
-// R64 += (double) E32
 // rows of a [n, K] matrix with a non-zero entry (flag per row)
 __global__ void k_row_nonzero(const double* __restrict__ S, int64_t n, int K, uint32_t* __restrict__ flag) {
   const int lane = threadIdx.x & 31;
@@ -988,7 +981,7 @@ int run_tile(PprArgs<T> a, int64_t n, cudaStream_t s) {
   // four chunks a unit on large graphs (K = 64 at 2^22: 218 against 222 ms), one
   // where that leaves warps idle (K = 32 at 2^19, 8.9 M edges: 35 against 53 ms)
   a.chunks_per_unit = a.m >= (1ll << 25) ? 4 : 1;
-  const int64_t work = (a.row_end / rows + 1 + a.max_chunks / a.chunks_per_unit + 1) * a.tiles;
+  const int64_t work = (a.n / rows + 1 + a.max_chunks / a.chunks_per_unit + 1) * a.tiles;
   if (work * 2 >= (int64_t)UINT32_MAX) {
     set_error("too many work units");
     return PRDF_EINVAL;
