@@ -84,7 +84,12 @@ typedef struct {
                           loop (a residual read every check_every sweeps); 0 (default): every sweep
                           loop (Static, DF, DF-P, DT, and the FP32 stage of each) runs as one
                           cooperative launch with the convergence test on the device, no host round
-                          trips, and so do the K-column loops. Both give identical results. */
+                          trips, and so do the K-column loops. Both give identical results. Such a
+                          launch is as wide as the GPU and holds every SM until the loop ends: it
+                          starts when the kernels of other streams have left room for all of its
+                          blocks, and kernels issued after it wait for the whole solve. A caller
+                          that overlaps streams with a solve sets 1, where other kernels run
+                          between its launches. */
   int tile;            /* K-column calls: columns per index fetch (8, 16, 32, 64); 0 = automatic */
   double expand_pull;  /* DF / DF-P: an expansion round after a sweep runs in pull form (each vertex
                           outside the affected set looks for a frontier in-neighbour in G') when the

@@ -570,8 +570,8 @@ int loop_args(prdf_graph* g, const prdf_params* p, const Loop& L, int max_iter, 
 // 30, but 2^19 (8.9 M) 44 -> 47 and 2^20 64 -> 84 (a unit of one chunk costs
 // about 4 us whatever its length). Only a class of rows above kChunkSmallRow
 // entries: with thresholds that put short rows there a chunk, and with it a
-// unit, held a few edges (bounds of 1 and 64 on a 2^17 R-MAT: 5.0 ms a solve,
-// 4.3 in batches of a warp per row).
+// unit, held a few edges (bounds of 1 and 64 on a 2^17 R-MAT: 4.7 ms a solve,
+// 2.1 in batches).
 int ensure_sweep_chunks(prdf_graph* g, const int64_t* cb, cudaStream_t s) {
   SweepChunks& t = g->sweep_chunks;
   if (!t.valid || t.version != g->rl.version) {

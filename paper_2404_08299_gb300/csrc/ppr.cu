@@ -8,8 +8,8 @@
 // FP32 sweeps sum the products of up to four edges with FMAs and fold each
 // such sum into a compensated pair (TwoSum), so the rounding error does not
 // grow with the row length. (Eight at a time lose most of what follows a large
-// product in a row of eight; four cost 1 % of the K = 32 forward and backward,
-// 34.8 -> 35.2 ms, and nothing at K = 64.) The FP64 stage is mixed-precision
+// product in a row of eight; four cost 1 % of the K = 32 forward and backward
+// and nothing at K = 64.) The FP64 stage is mixed-precision
 // iterative refinement: an FP64 sweep computes the Jacobi step T(R) and the
 // residual T(R) - R; an FP32 solve of E = alpha P^T E + residual gives the
 // correction. The stop rule is the same as Static's: the L-inf change of an
@@ -20,10 +20,11 @@
 // between sweeps, the stop test on the device. What bounds a sweep is the
 // 16-byte gathers of the rows of R (K * 4 bytes per edge through L2), so the
 // kernel is built to keep them in flight: the indices and weights of the next
-// step load (one per lane, handed round by shuffles) while this step's
-// gathers are on their way, across row and chunk bounds. At 2^22 and K = 64 (69
-// M edges, 17.8 GB of gathered rows) an FP32 sweep takes 2.3-2.4 ms; four
-// kernels per sweep with unpipelined loads took 3.07 ms.
+// step load (one per lane, handed round by shuffles; in narrow FP32 tiles four
+// per lane, the same in every lane of a row) while this step's gathers are on
+// their way, across row and chunk bounds. At 2^22 and K = 64 (69 M edges, 17.8
+// GB of gathered rows) an FP32 sweep takes 2.3 ms; four kernels per sweep with
+// unpipelined loads took 3.07 ms.
 #include <cstring>
 
 #include "loop.cuh"

@@ -160,9 +160,9 @@ __device__ __forceinline__ void rank_keys(const uint64_t (&key)[kRK], int shift,
 }
 
 // Stable scatter of one tile by digit; goff = exclusive scan of hist. W: the
-// weights move with their keys. Bound by shared memory (the data pipe 73 %
+// weights move with their keys. Bound by shared memory (the data pipe 85 %
 // busy: counters by digit and the staged keys are hit at random banks) and by
-// issue (57 %, the ballots), not by DRAM (3.4 of 6.7 TB/s). So a digit's start
+// issue (60 %, the ballots), not by DRAM (4.0 of 6.7 TB/s). So a digit's start
 // is folded into the warps' counters (one random read less a key), and full
 // tiles take a branch-free path: all loads are in flight before the first
 // key is ranked, and no round tests for a missing key. 285 M keys to two CSRs:
